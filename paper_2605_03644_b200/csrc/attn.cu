@@ -70,6 +70,12 @@ struct Sched {
   long long Lj[kMaxPairs];           // context length of the pair's probe (clamped to ctx_cap)
   int n_ctx[kMaxPairs];
   int n_su[kMaxPairs];
+  int n_cut;                         // units that a range boundary cuts; their pieces are merged afterwards
+  struct Cut {
+    int bpj, g;                      // (b * nl + l) * P + j and KV head of the unit
+    int gang, n;                     // its pieces lie with gangs gang .. gang + n - 1
+    int which;                       // slot of the first piece (the others are their gangs' first pieces)
+  } cut[kMaxCtas];
 };
 
 struct AttnParams {
@@ -159,14 +165,16 @@ __global__ void __launch_bounds__(256) attn_prep_kernel(const PrepParams p) {
 
   if (blockIdx.x == gridDim.x - 1) {
     // the schedule, by a block of its own (beside the rotation, not in front of a share of it);
-    // intermediate values stay in shared memory
-    __shared__ long long s_pre[kMaxPairs + 1], s_vpre[kMaxPairs + 1];
-    __shared__ int s_nsu[kMaxPairs];
+    // intermediate values stay in shared memory.  One pair per thread (kMaxPairs = blockDim.x): the
+    // prefix sums are a block scan.
+    __shared__ long long s_pre[kMaxPairs + 1], s_vpre[kMaxPairs + 1], s_start[kMaxCtas + 1], s_warp[2][8];
+    __shared__ int s_nsu[kMaxPairs], s_fp[kMaxCtas + 1], s_ncut;
     Sched* sc = p.sched;
-    const int n_pairs = p.P * p.B;
+    const int n_pairs = p.P * p.B, pi = threadIdx.x;
     const int n_own = (p.To + kTileN - 1) / kTileN;
     const long long units_per_pair = (long long)p.nl * p.Hkv;
-    for (int pi = threadIdx.x; pi < n_pairs; pi += blockDim.x) {
+    long long len = 0, vlen = 0;
+    if (pi < n_pairs) {
       const int j = p.P - 1 - pi / p.B, b = pi % p.B;
       long long Lj = p.ctx_off[(long long)b * (p.k + 1) + probe_shots(p, b, j)];
       Lj = Lj > p.ctx_cap ? p.ctx_cap : (Lj < 0 ? 0 : Lj);
@@ -175,28 +183,39 @@ __global__ void __launch_bounds__(256) attn_prep_kernel(const PrepParams p) {
       sc->n_ctx[pi] = n_ctx;
       sc->n_su[pi] = n_ctx + n_own;
       s_nsu[pi] = n_ctx + n_own;
+      len = (n_ctx + n_own) * units_per_pair;
+      vlen = (n_ctx + n_own + kUnitCost) * units_per_pair;
     }
+    if (pi == 0) s_ncut = 0;
+    long long in_l = len, in_v = vlen;                // inclusive scans
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long a = __shfl_up_sync(0xffffffffu, in_l, o), c = __shfl_up_sync(0xffffffffu, in_v, o);
+      if (lane >= o) { in_l += a; in_v += c; }
+    }
+    if (lane == 31) { s_warp[0][pi >> 5] = in_l; s_warp[1][pi >> 5] = in_v; }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      long long acc = 0, vacc = 0;
-      for (int pi = 0; pi < n_pairs; ++pi) {
-        s_pre[pi] = acc;
-        s_vpre[pi] = vacc;
-        sc->prefix[pi] = acc;
-        acc += (long long)s_nsu[pi] * units_per_pair;
-        vacc += (long long)(s_nsu[pi] + kUnitCost) * units_per_pair;
+    for (int w = 0; w < (pi >> 5); ++w) { in_l += s_warp[0][w]; in_v += s_warp[1][w]; }
+    if (pi < n_pairs) {
+      s_pre[pi] = in_l - len;
+      s_vpre[pi] = in_v - vlen;
+      sc->prefix[pi] = in_l - len;
+      if (pi == n_pairs - 1) {
+        s_pre[n_pairs] = in_l;
+        s_vpre[n_pairs] = in_v;
+        sc->prefix[n_pairs] = in_l;
+        sc->total = in_l;
       }
-      s_pre[n_pairs] = acc;
-      s_vpre[n_pairs] = vacc;
-      sc->prefix[n_pairs] = acc;
-      sc->total = acc;
     }
     __syncthreads();
     // Range q starts where the cost sequence (every unit preceded by kUnitCost virtual tiles)
-    // reaches q / n_gangs of its length: threads q = 0 .. n_gangs, independently.
+    // reaches q / n_ranges of its length: threads q = 0 .. n_gangs, independently.  A range is at least
+    // kUnitCost + 1 long, so that it holds a real tile: a call with less work leaves gangs without any.
     const long long vtotal = s_vpre[n_pairs];
+    const long long fit = vtotal / (kUnitCost + 1);
+    const int n_ranges = (int)(fit < 1 ? 1 : (fit < p.n_gangs ? fit : p.n_gangs));
     for (int q = threadIdx.x; q <= p.n_gangs; q += blockDim.x) {
-      const long long v = (long long)q * vtotal / p.n_gangs;
+      const long long v = q < n_ranges ? q * vtotal / n_ranges : vtotal;
       long long real = s_pre[n_pairs];
       int fp = n_pairs - 1;
       if (v < vtotal) {
@@ -213,7 +232,30 @@ __global__ void __launch_bounds__(256) attn_prep_kernel(const PrepParams p) {
       }
       sc->start[q] = real;
       sc->first_pair[q] = fp;
+      s_start[q] = real;
+      s_fp[q] = fp;
     }
+    __syncthreads();
+    // The units to merge: gang q lists the unit that its range's end cuts, if the unit starts in that range.
+    for (int q = threadIdx.x; q + 1 < n_ranges; q += blockDim.x) {
+      const long long cut = s_start[q + 1];
+      const int pr = s_fp[q + 1];
+      const long long nsu = s_nsu[pr], rel = cut - s_pre[pr];
+      const long long su = rel / nsu, s_u = s_pre[pr] + su * nsu;
+      if (s_u == cut || s_u < s_start[q]) continue;   // between two units; or an earlier gang holds its first piece
+      int n = 2;                                      // gangs whose range begins inside the unit, and this one
+      while (q + n < n_ranges && s_start[q + n] < s_u + nsu) ++n;
+      Sched::Cut c;
+      const int l = (int)(su / p.Hkv);
+      c.bpj = ((pr % p.B) * p.nl + l) * p.P + p.P - 1 - pr / p.B;
+      c.g = (int)(su % p.Hkv);
+      c.gang = q;
+      c.n = n;
+      c.which = s_start[q] >= s_u ? 0 : 1;
+      sc->cut[atomicAdd(&s_ncut, 1)] = c;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) sc->n_cut = s_ncut;
     return;
   }
   const long long gw = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -383,15 +425,6 @@ __device__ __forceinline__ PairInfo pair_info(const Sched* sc, const SchedCache*
     pi.n_ctx = sc->n_ctx[pair]; pi.n_su = sc->n_su[pair];
   }
   return pi;
-}
-
-__device__ __forceinline__ int find_pair(const Sched* sc, int n_pairs, long long x) {
-  int lo = 0, hi = n_pairs;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (sc->prefix[mid] <= x) lo = mid; else hi = mid;
-  }
-  return lo;
 }
 
 __device__ __forceinline__ bool next_piece(const Sched* sc, const SchedCache* cache, int n_pairs, Walker& wk,
@@ -1232,82 +1265,81 @@ struct CombineParams {
   const float* ml_part;
   __nv_bfloat16* out;   // [B][nl][P][Tq][Hq][D]
   float* lse;           // [B][nl][P][Hq][Tq] or null
-  int B, P, Tq, Hq, Hkv, G, nl, n_mp, n_gangs;
+  int Tq, Hq, G, n_mp;
 };
 
 constexpr int kCombineRows = 8;      // rows per warp
+constexpr int kCombineSteps = 2;     // 16-column steps per warp (blockIdx.z covers the others)
 
-// Block (q, y): if the range of gang q ends inside a unit that starts in that range, the
-// unit was cut; its pieces sit with gangs q .. q_last.  One warp merges eight rows.
+// Block x merges the x-th of the units that a range boundary cut (listed by the schedule block, so that
+// nothing has to be searched for here).  Latency- and L2-bound: one query of one layer (26 MB of partials)
+// took 14.6 us when every block searched the schedule and merged piece after piece, 8.8 us now; in front of
+// a cache of 12 K tokens, cut into eighteen pieces per unit, 19.4 and 7.4 us.  A warp merges 8 rows: lane = (row r_sub, 4-column chunk c_sub of the 16 columns of one step),
+// so that a load is 8 rows x 16 bytes contiguous per chunk in the partial layout ([D/4][128 rows][4] per
+// M tile) and a store fills one 32-byte sector per row.
 template <int D>
 __global__ void __launch_bounds__(256) attn_combine_kernel(const CombineParams p) {
   const Sched* sc = p.sched;
-  const int q = blockIdx.x;
-  const long long total = sc->total;
-  const long long cut = sc->start[q + 1];
-  if (cut >= total) return;
-  const int n_pairs = p.P * p.B;
-  const int pair = find_pair(sc, n_pairs, cut);
-  const int nsu = sc->n_su[pair];
-  const long long rel = cut - sc->prefix[pair];
-  if (rel % nsu == 0) return;                       // the cut falls between two units
-  const int su = (int)(rel / nsu);
-  const long long s_u = sc->prefix[pair] + (long long)su * nsu, e_u = s_u + nsu;
-  if (s_u < sc->start[q]) return;                   // an earlier gang holds the unit's first piece
-  int q_last = q + 1;                               // last gang whose range begins inside the unit
-  while (q_last + 1 < p.n_gangs && sc->start[q_last + 1] < e_u) ++q_last;
-
+  if (blockIdx.x >= sc->n_cut) return;
+  const Sched::Cut c = sc->cut[blockIdx.x];
   const int lane = threadIdx.x & 31;
-  const int j = p.P - 1 - pair / p.B, b = pair % p.B;
-  const int l = su / p.Hkv, g = su % p.Hkv;
-  const long long bpj = ((long long)b * p.nl + l) * p.P + j;
-  // A warp merges 8 rows: lane = (row r_sub, 4-column chunk c_sub of the 16 columns of one
-  // step), so that a load is 8 rows x 16 bytes contiguous per chunk in the partial layout
-  // ([D/4][128 rows][4] per M tile) and a store fills one 32-byte sector per row.
   const int r_sub = lane & 7, c_sub = lane >> 3;
   const int m = (blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kCombineRows + r_sub;
   if (m >= p.Tq * p.G) return;
   const int mt = m / kTileM, r = m % kTileM, mp = mt >> 1, x = mt & 1;
-  const int t = m / p.G, hh = m % p.G, h = g * p.G + hh;
-  auto slot_tile = [&](int qq) -> long long {
-    const int which = sc->start[qq] >= s_u ? 0 : 1;           // the gang's first piece, or its last
-    return ((long long)(2 * qq + which) * p.n_mp + mp) * 2 + x;
+  const int t = m / p.G, hh = m % p.G, h = c.g * p.G + hh;
+  const long long bpj = c.bpj;
+  auto slot_tile = [&](int i) -> long long {        // tile of piece i
+    return ((long long)(2 * (c.gang + i) + (i == 0 ? c.which : 0)) * p.n_mp + mp) * 2 + x;
   };
-  // (when there are fewer tiles than gangs, empty ranges lie between the pieces)
-  auto has_piece = [&](int qq) -> bool { return sc->start[qq] < sc->start[qq + 1]; };
-  float M = kNegSentinel;
-  for (int qq = q; qq <= q_last; ++qq)
-    if (has_piece(qq)) M = fmaxf(M, p.ml_part[(slot_tile(qq) * kTileM + r) * 2]);
   const float4* o4 = reinterpret_cast<const float4*>(p.o_part);
-  float4 acc[D / 16];
+  const int it0 = blockIdx.z * kCombineSteps;
+  float4 acc[kCombineSteps];
 #pragma unroll
-  for (int it = 0; it < D / 16; ++it) acc[it] = make_float4(0.f, 0.f, 0.f, 0.f);
-  float lsum = 0.f;
-  for (int qq = q; qq <= q_last; ++qq) {
-    if (!has_piece(qq)) continue;
-    const long long tile = slot_tile(qq);
-    const float* ml = p.ml_part + (tile * kTileM + r) * 2;
-    const float wgt = exp2f(ml[0] - M);
-    lsum += ml[1] * wgt;
-    float4 v[D / 16];
+  for (int it = 0; it < kCombineSteps; ++it) acc[it] = make_float4(0.f, 0.f, 0.f, 0.f);
+  float M = kNegSentinel, lsum = 0.f;
+  // the loads of four pieces are issued before any is merged (running maximum, one pass)
+  for (int i0 = 0; i0 < c.n; i0 += 4) {
+    float2 ml[4];
+    float4 v[4][kCombineSteps];
 #pragma unroll
-    for (int it = 0; it < D / 16; ++it) v[it] = o4[(tile * (D / 4) + it * 4 + c_sub) * kTileM + r];
+    for (int u = 0; u < 4; ++u) {
+      const bool use = i0 + u < c.n;
+      const long long tile = slot_tile(use ? i0 + u : 0);
+      ml[u] = use ? *reinterpret_cast<const float2*>(p.ml_part + (tile * kTileM + r) * 2) : make_float2(kNegSentinel, 0.f);
 #pragma unroll
-    for (int it = 0; it < D / 16; ++it) {
-      acc[it].x += v[it].x * wgt; acc[it].y += v[it].y * wgt;
-      acc[it].z += v[it].z * wgt; acc[it].w += v[it].w * wgt;
+      for (int it = 0; it < kCombineSteps; ++it)
+        v[u][it] = use ? o4[(tile * (D / 4) + (it0 + it) * 4 + c_sub) * kTileM + r] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    const float m_new = fmaxf(fmaxf(M, fmaxf(ml[0].x, ml[1].x)), fmaxf(ml[2].x, ml[3].x));
+    const float keep = exp2f(M - m_new);
+    M = m_new;
+    lsum *= keep;
+#pragma unroll
+    for (int it = 0; it < kCombineSteps; ++it) {
+      acc[it].x *= keep; acc[it].y *= keep; acc[it].z *= keep; acc[it].w *= keep;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float wgt = exp2f(ml[u].x - M);
+      lsum += ml[u].y * wgt;
+#pragma unroll
+      for (int it = 0; it < kCombineSteps; ++it) {
+        acc[it].x += v[u][it].x * wgt; acc[it].y += v[u][it].y * wgt;
+        acc[it].z += v[u][it].z * wgt; acc[it].w += v[u][it].w * wgt;
+      }
     }
   }
   const float inv = 1.f / lsum;
   __nv_bfloat16* dst = p.out + (((bpj * p.Tq + t) * p.Hq) + h) * (long long)D;
 #pragma unroll
-  for (int it = 0; it < D / 16; ++it) {
+  for (int it = 0; it < kCombineSteps; ++it) {
     uint2 packed;
     packed.x = pack_bf16x2(acc[it].x * inv, acc[it].y * inv);
     packed.y = pack_bf16x2(acc[it].z * inv, acc[it].w * inv);
-    *reinterpret_cast<uint2*>(dst + (it * 4 + c_sub) * 4) = packed;
+    *reinterpret_cast<uint2*>(dst + ((it0 + it) * 4 + c_sub) * 4) = packed;
   }
-  if (p.lse != nullptr && c_sub == 0)
+  if (p.lse != nullptr && c_sub == 0 && blockIdx.z == 0)
     p.lse[(bpj * p.Hq + h) * p.Tq + t] = (M + log2f(lsum)) * kLn2;
 }
 
@@ -1536,9 +1568,9 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
   CombineParams cp;
   cp.sched = sched; cp.o_part = o_part; cp.ml_part = ml_part;
   cp.out = ap.out; cp.lse = lse;
-  cp.B = B; cp.P = P; cp.Tq = Tq; cp.Hq = Hq; cp.Hkv = Hkv; cp.G = G; cp.nl = nl;
-  cp.n_mp = pl.n_mp; cp.n_gangs = n_gangs;
-  const dim3 grid((unsigned)n_gangs, (unsigned)((Tq * G + 8 * kCombineRows - 1) / (8 * kCombineRows)));
+  cp.Tq = Tq; cp.Hq = Hq; cp.G = G; cp.n_mp = pl.n_mp;
+  const dim3 grid((unsigned)n_gangs, (unsigned)((Tq * G + 8 * kCombineRows - 1) / (8 * kCombineRows)),
+                  D / (16 * kCombineSteps));
   attn_combine_kernel<D><<<grid, 256, 0, st>>>(cp);
   return ads_launch_status();
 }

@@ -179,3 +179,13 @@ def test_a_range_that_spans_more_pairs_than_the_schedule_cache_holds():
         want.append(o_want)
         assert abs(float(lse[b, 0, j, h, t]) - l_want) <= hp.lse_bound()
     hp.assert_attn_close(np.stack(got), np.stack(want))
+
+
+@pytest.mark.parametrize("n_shots", [1, 5, 86, 87, 88])
+def test_number_of_ranges_follows_the_work(n_shots):
+    # A range holds at least five tiles' worth of cost (four of them a unit's fixed cost): eight units of one
+    # context tile fill nine ranges, units of 87 and 88 context tiles lie on either side of one range per CTA
+    # (148); most units are cut, into two to nineteen pieces.
+    w = wl.CONFIGS["cfg2"].scaled(n_shots=n_shots, len_dist="const", len_lo=128, len_hi=128, batch=1, k=n_shots, t_q=3,
+                                  n_q_heads=8, n_kv_heads=8, head_dim=64, seed=28)
+    _run_case(w, np.arange(n_shots, dtype=np.int32)[None, ::-1].copy(), [n_shots], 1)
