@@ -57,6 +57,28 @@ static inline int ads_set_max_smem(Kernel kernel, int bytes, bool* done) {
   return ADAPSHOT_OK;
 }
 
+// Programmatic dependent launch: the kernel may be started while the one in front of it in the stream still
+// runs, so that its launch and its set-up cost no gap.  Every kernel launched this way calls ads_dependency_wait()
+// before it touches global memory (in every block: what completes a kernel is the completion of its blocks, and a
+// block that did not wait would not stand for the kernels before), and ads_dependency_trigger() as early as it likes.
+template <typename... KArgs, typename... Args>
+static inline int ads_launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                       Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...) == cudaSuccess ? ads_launch_status() : ADAPSHOT_ECUDA;
+}
+__device__ __forceinline__ void ads_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void ads_dependency_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Device: record an error code once; later codes do not overwrite the first.
 __device__ __forceinline__ void ads_set_status(int32_t* status, int32_t code) {
   if (status != nullptr) atomicCAS(status, 0, code);
@@ -81,6 +103,15 @@ __device__ __forceinline__ double ads_key_score(unsigned long long k) {
 size_t ads_topk_scratch_bytes(int N, int B, int k);
 int ads_topk_from_keys(const unsigned long long* keys, const int* ids, int N, int B, int k, void* cand,
                        int32_t* sel_idx, float* sel_score, cudaStream_t st);
+
+// Decoding with few rows per KV head (decode.cu): whether a call's rows fit, its scratch, and the call itself
+// (arguments checked by the caller).
+bool ads_decode_rows_fit(const adapshot_model_t* model, int T_new);
+size_t ads_decode_rows_workspace(const adapshot_model_t* model, int B);
+int ads_decode_rows(const adapshot_model_t* model, const void* k_ctx, const void* v_ctx, int64_t ctx_cap,
+                    const int64_t* ctx_off, int B, int k, const int32_t* n_shots, const void* q_new, const void* k_own,
+                    const void* v_own, int T_new, int T_own, int nl, void* out, float* lse, void* ws, int32_t* status,
+                    cudaStream_t st);
 
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll

@@ -133,3 +133,46 @@ def test_decode_reports_a_shot_count_outside_the_selection():
                             v_own, 0, nl, out, None, ws, st)
     torch.cuda.synchronize()
     assert st.item() == ab.EINDEX
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("hq,d,batch,n_shots,t_new,t_own", [
+    (16, 128, 1, 1, 1, 64),        # G = 16 rows exactly (one row block); own tokens fill one tile
+    (17, 64, 2, 3, 1, 65),         # 17 rows (two row blocks); one own token in a second tile
+    (8, 128, 3, 2, 4, 5),          # 32 rows, the most the kernel takes; rows of four tokens, causal
+    (11, 64, 1, 2, 3, 3),          # 33 rows: the prefill kernels
+    (2, 64, 1, 150, 1, 1),         # one request over 150 tiles: every unit is cut into many pieces
+    (1, 128, 70, 1, 2, 130),       # more requests than one prefix scan of 64, three own tiles, short contexts
+])
+def test_decode_row_counts_and_range_cuts(hq, d, batch, n_shots, t_new, t_own):
+    # one KV head; shots of 63, 64 and 65 tokens put the context's end on either side of a 64-key tile
+    ab = hp.gpu_binding()
+    w = wl.CONFIGS["cfg2"].scaled(n_shots=n_shots, len_lo=63, len_hi=65, batch=batch, k=n_shots, probes=(n_shots,),
+                                  t_q=t_own, n_q_heads=hq, n_kv_heads=1, head_dim=d, seed=76)
+    ab, pool, qs, sel_np, off_np, model, cap, kc, vc, off = _setup(w, 1, 12)
+    n_star = np.random.default_rng(13).integers(1, n_shots + 1, size=batch).astype(np.int32)
+    n_star[0] = n_shots
+    q_new = qs["q"][:, :, 0, t_own - t_new:].contiguous().cuda()
+    k_own, v_own = qs["kq"][:, :, 0].contiguous().cuda(), qs["vq"][:, :, 0].contiguous().cuda()
+    out = torch.full_like(q_new, 9.0)
+    lse = torch.zeros((batch, 1, hq, t_new), dtype=torch.float32, device="cuda")
+    ws = torch.empty(ab.adapshot_decode_workspace_bytes(model, batch, t_new, t_own, 1), dtype=torch.uint8, device="cuda")
+    st = hp.new_status()
+    ab.adapshot_decode_attn(model, kc, vc, cap, off, n_shots, torch.from_numpy(n_star).cuda(), q_new, k_own, v_own, 0, 1,
+                            out, lse, ws, st)
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    kp, vp = hp.f64(pool["k"][:1]), hp.f64(pool["v"][:1])
+    got, want = [], []
+    for b in sorted({0, batch // 2, batch - 1}):
+        k_ctx, v_ctx, _ = orc.assemble_kv(kp, vp, pool["shot_off"], sel_np[b], w.rope_base)
+        ko, vo = hp.f64(qs["kq"][b, 0, 0]), hp.f64(qs["vq"][b, 0, 0])
+        for t in range(t_new):
+            u = t_own - t_new + t
+            for h in range(hq):
+                o_want, l_want = orc.decode_row(hp.f64(q_new[b, 0, t, h].cpu()), ko[:u + 1], vo[:u + 1], k_ctx[0], v_ctx[0],
+                                                int(off_np[b, n_star[b]]), 0, w.rope_base)
+                got.append(out[b, 0, t, h].cpu().double().numpy())
+                want.append(o_want)
+                assert abs(float(lse[b, 0, h, t]) - l_want) <= hp.lse_bound()
+    hp.assert_attn_close(np.stack(got), np.stack(want))
