@@ -19,13 +19,14 @@
 //                 memory into whole row segments); a range that cuts a unit stores
 //                 un-normalised partials;
 //   attn_combine  log-sum-exp merge of the partials of the cut units.
-// The fused variant (adapshot_query_attn_fused) adds attn_fused_plan (row map and rotary
-// table, once per call) and runs attn_main with two loader warps that copy the context
-// K/V tiles from the pool and re-encode K (Eq. 7) in shared memory, instead of TMA loads
-// from an assembled cache.  The V-from-pool variant (adapshot_query_attn_vpool) sits between
-// the two: K tiles come by TMA from a cache that holds the re-encoded K only, V tiles (which
-// Eq. 7 leaves as they are) are copied from the pool through the row map, so that the gather
-// moves half the bytes.
+// Two variants take tiles straight from the pool, through a row map written once per call (attn_row_map): the
+// V-from-pool variant (adapshot_query_attn_vpool) reads K from a cache that holds the re-encoded K only and
+// V, which Eq. 7 leaves as it is, from the pool, so that the gather moves half the bytes; the fused variant
+// (adapshot_query_attn_fused) reads both from the pool and re-encodes K (Eq. 7) in shared memory.  One warp per
+// operand stitches a tile from the runs of pool rows it consists of; four warps rotate K where it landed.
+// (Fused, 2 queries x 2 layers x 16.4 K tokens, probes of 64 and 128 shots: 1396 us with two warps that copied K
+// and V element-wise and rotated K from a table, 535 us with four warps that rotated K on its way through
+// registers (16 KB in flight per SM, latency-bound), 325 us as it is now.)
 #include <cuda.h>
 #include <float.h>
 
@@ -45,12 +46,17 @@ constexpr int kUnitCost = 4;          // fixed cost of starting a unit, in tiles
 constexpr int kTileM = 128;          // query rows per M tile (TMEM lanes)
 constexpr int kTileN = 128;          // keys per tile
 constexpr int kAttnThreads = 320;    // warp 0 TMA, warp 1 MMA, warps 2-5 softmax A, warps 6-9 softmax B
-constexpr int kFusedThreads = 384;   // fused variant: warps 2-3 load and rotate K/V, softmax on warps 4-11
+constexpr int kFusedThreads = 512;   // fused variant: warps 2-3 gather V and K, softmax on warps 4-11, K rotated by warps 12-15
 constexpr int kVPoolThreads = 352;   // V-from-pool variant: the cache variant's warps plus warp 10, which gathers V
 constexpr int kModeCache = 0;        // K and V tiles by TMA from the assembled cache
 constexpr int kModeFused = 1;        // K and V tiles from the pool, K re-encoded in shared memory
 constexpr int kModeVPool = 2;        // K tiles by TMA from a K-only cache, V tiles from the pool
-constexpr int kLoaders = 64;         // threads of the two loader warps
+constexpr int kRotateWarp0 = 12;     // fused variant: first of the four warps that rotate K
+constexpr int kRotateWarps = 4;
+// Registers per thread of the fused variant's warpgroups (issue and gather, softmax twice, rotation): together
+// what 512 threads are launched with, 4 x 128.
+constexpr int kFusedRegsIssue = 64, kFusedRegsSoftmax = 176, kFusedRegsRotate = 96;
+static_assert(kFusedRegsIssue + 2 * kFusedRegsSoftmax + kFusedRegsRotate <= 4 * 128, "register split");
 constexpr uint32_t kTmemCols = 512;
 constexpr float kRescaleThreshold = 8.f;   // log2 units: rescale O only when the max grows by 2^8
 constexpr float kNegSentinel = -1.0e30f;
@@ -89,18 +95,13 @@ struct AttnParams {
   int To;                     // own tokens per probe (>= Tq): the Tq rows are the last Tq of them
   int n_mt, n_mp, gang, n_gangs;
   float scale_log2;           // softmax_scale * log2(e)
-  // fused variant only: K/V tiles come from the pool (and from the probe's own rotated keys)
-  const __nv_bfloat16* k_pool;   // [n_layers][pool_tokens][Hkv][D]
-  const __nv_bfloat16* v_pool;
-  const __nv_bfloat16* kq_rot;   // [B*nl*P][To][Hkv][D], rotated by the prep kernel
-  const __nv_bfloat16* vq;
+  // K or V from the pool
   const int* row_map;            // [B][ctx_cap]: pool token of every context position, -1 beyond L
   const int* off_map;            // [B][ctx_cap]: first position of the shot a position lies in (k_pos_mode 1)
   int k_pos_mode;                // 0: angle = position; 1: angle = the shot's first position (Eq. 7 as printed)
-  const float2* rope_tab;        // [ctx_cap rounded up to 128][D/2]: (cos, sin) of position * theta_i
-  long long pool_tokens, ctx_cap;
+  long long ctx_cap;
   int layer_begin;
-  double rope_base_f;
+  double theta[64];
 };
 
 struct PrepParams {
@@ -310,63 +311,57 @@ __global__ void __launch_bounds__(256) attn_prep_kernel(const PrepParams p) {
   }
 }
 
-// Fused variant, once per call: the pool token behind every context position of every query
-// (the gather's plan lookup, stored instead of applied) and the rotary table of the context
-// positions, (cos, sin)(p * theta_i) from fp64 angles.
-struct FusedPlanParams {
+// V-from-pool and fused variants, once per call: the pool token behind every context position of every query
+// (the gather's plan lookup, stored instead of applied) and, for keys stored rotated, the first position of its
+// shot.  Positions from L to the end of the last 128-token tile get -1; nothing beyond them is read.
+struct RowMapParams {
   const long long* ctx_off;   // [B][k+1]
   const int32_t* sel_idx;     // [B][k]
   const long long* shot_off;  // [n_shots+1]
   int* row_map;               // [B][ctx_cap]
-  int* off_map;               // [B][ctx_cap]: first position of the position's shot
-  float2* rope_tab;           // [tab_rows][D/2]
-  long long ctx_cap, tab_rows;
-  int B, k, n_shots, half_d;
-  double rope_base;
+  int* off_map;               // [B][ctx_cap] or null
+  long long ctx_cap;
+  int B, k, n_shots;
 };
 
-__global__ void __launch_bounds__(256) attn_fused_plan_kernel(const FusedPlanParams p) {
-  const long long n_map = (long long)p.B * p.ctx_cap;
-  const long long n_tab = p.tab_rows * p.half_d;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long u = (long long)blockIdx.x * blockDim.x + threadIdx.x; u < n_map + n_tab; u += stride) {
-    if (u < n_map) {
-      const int b = (int)(u / p.ctx_cap);
-      const long long pos = u % p.ctx_cap;
-      const long long* off = p.ctx_off + (long long)b * (p.k + 1);
-      int row = -1, first = 0;
-      if (pos < off[p.k]) {
-        int lo = 0, hi = p.k;          // shot slot with off[lo] <= pos < off[lo+1]
-        while (hi - lo > 1) {
-          const int mid = (lo + hi) >> 1;
-          if (off[mid] <= pos) lo = mid; else hi = mid;
-        }
-        const int s = p.sel_idx[(long long)b * p.k + lo];
-        if (s >= 0 && s < p.n_shots) row = (int)(p.shot_off[s] + (pos - off[lo]));
-        first = (int)off[lo];
-      }
-      p.row_map[u] = row;
-      p.off_map[u] = first;
-    } else {
-      const long long v = u - n_map;
-      const long long pos = v / p.half_d;
-      const int i = (int)(v % p.half_d);
-      const double theta = pow(p.rope_base, -(double)i / (double)p.half_d);
-      float sn, cs;
-      rope_sincos((double)pos, theta, &sn, &cs);
-      p.rope_tab[v] = make_float2(cs, sn);
+// One warp per selected shot: its run of positions is written with whole lines (a search per position
+// took 38 us for 32 queries of 66 K positions and 8.3 us for 8 of 33 K; 3 us for those now).
+__global__ void __launch_bounds__(256) attn_row_map_kernel(const RowMapParams p) {
+  const int lane = threadIdx.x & 31;
+  const long long w = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (w >= (long long)p.B * p.k) return;
+  const int b = (int)(w / p.k), r = (int)(w % p.k);
+  const long long* off = p.ctx_off + (long long)b * (p.k + 1);
+  const long long o0 = off[r], o1 = off[r + 1];
+  const int s = p.sel_idx[w];
+  int* rows = p.row_map + (long long)b * p.ctx_cap;
+  int* firsts = p.off_map == nullptr ? nullptr : p.off_map + (long long)b * p.ctx_cap;
+  const long long end = min(o1, p.ctx_cap);
+  const bool known = s >= 0 && s < p.n_shots;        // (an unknown shot is reported by the plan and has no positions)
+  const long long src = known ? p.shot_off[s] - o0 : 0;
+  for (long long pos = o0 + lane; pos < end; pos += 32) {
+    rows[pos] = known ? (int)(src + pos) : -1;
+    if (firsts != nullptr) firsts[pos] = (int)o0;
+  }
+  if (r == p.k - 1) {
+    const long long pad = min((o1 + kTileN - 1) / kTileN * kTileN, p.ctx_cap);
+    for (long long pos = o1 + lane; pos < pad; pos += 32) {
+      rows[pos] = -1;
+      if (firsts != nullptr) firsts[pos] = 0;
     }
   }
 }
 
 // Shared-memory plan.  Every operand tile is made of [128 rows][128 bytes] sub-tiles
 // written by TMA with the 128-byte swizzle; D = 128 needs two of them per tile.
-// The fused variant's loader warps take the stages of tile i+1 before they hand over tile i,
-// which needs a third V stage; the room goes at the expense of the read-out staging.
+// The fused variant has a third K stage (one tile landing, one being rotated, one in use) in the place of
+// the read-out staging.
+__host__ __device__ constexpr int sched_cache_pairs(int mode) { return mode == kModeFused ? 16 : 40; }
+__host__ __device__ constexpr uint32_t sched_cache_bytes(int mode) { return mode == kModeFused ? 512 : 1024; }
 template <int D, int MODE>
 struct AttnSmem {
-  static constexpr int kKStages = 2;
-  static constexpr int kVStages = MODE == kModeFused ? 3 : 2;
+  static constexpr int kKStages = MODE == kModeFused ? 3 : 2;
+  static constexpr int kVStages = 2;
   static constexpr uint32_t kStageBytes = MODE == kModeFused ? 0 : 4096;  // per softmax warp: 32 rows x 128 bytes
   static constexpr uint32_t kTileBytes = (D / 64) * 16384u;
   static constexpr uint32_t kOffQ = 0;                                    // Q of M tile A, then of M tile B
@@ -374,15 +369,16 @@ struct AttnSmem {
   static constexpr uint32_t kOffV = kOffK + kKStages * kTileBytes;
   static constexpr uint32_t kOffStage = kOffV + kVStages * kTileBytes;    // read-out staging of the 8 softmax warps
   static constexpr uint32_t kOffBar = kOffStage + 8 * kStageBytes;
-  static constexpr uint32_t kOffRows = kOffBar + 256 + 1024;              // V-from-pool variant: pool rows of a tile
-  static constexpr uint32_t kTotal = kOffRows + (MODE == kModeVPool ? 512 : 0) + 1024;   // + alignment slack
+  static constexpr uint32_t kOffRows = kOffBar + 256 + sched_cache_bytes(MODE);   // pool rows of a tile, per gather warp
+  static constexpr uint32_t kTotal = kOffRows + (MODE == kModeVPool ? 512 : MODE == kModeFused ? 1024 : 0) + 1024;   // + alignment slack
 };
 
 // mbarrier slots (8 bytes each)
 enum Bar {
   kBarQFull = 0, kBarQEmpty = 2, kBarKFull = 4, kBarKEmpty = 7, kBarVFull = 10, kBarVEmpty = 13,
   kBarSFull = 16, kBarPFull = 18, kBarOFull = 20, kBarOEmpty = 22, kBarDrain = 24,
-  kNumBars = 25
+  kBarKRot = 25,                 // fused variant: K tile rotated
+  kNumBars = 28
 };
 
 // A piece = the part of one unit (pair, layer, kv head) that falls into a gang's range.
@@ -400,7 +396,7 @@ struct Walker {
 // The part of the schedule a CTA walks, copied to shared memory once: the pairs from the
 // one its range starts in.  Pairs beyond the copy (a range that spans more than
 // kCachePairs pairs) are read from the workspace.
-constexpr int kCachePairs = 40;
+template <int kCachePairs>
 struct SchedCache {
   long long prefix[kCachePairs + 1];
   long long Lj[kCachePairs];
@@ -409,12 +405,14 @@ struct SchedCache {
   long long begin, end;
   int p0, n;
 };
-static_assert(sizeof(SchedCache) <= 1024, "the schedule cache has 1 KiB of shared memory");
+static_assert(sizeof(SchedCache<sched_cache_pairs(kModeCache)>) <= sched_cache_bytes(kModeCache) &&
+              sizeof(SchedCache<sched_cache_pairs(kModeFused)>) <= sched_cache_bytes(kModeFused), "room of the schedule cache");
 struct PairInfo {
   long long prefix, next_prefix, Lj;
   int n_ctx, n_su;
 };
-__device__ __forceinline__ PairInfo pair_info(const Sched* sc, const SchedCache* c, int pair) {
+template <typename Cache>
+__device__ __forceinline__ PairInfo pair_info(const Sched* sc, const Cache* c, int pair) {
   PairInfo pi;
   const int k = pair - c->p0;
   if (k >= 0 && k < c->n) {
@@ -427,7 +425,8 @@ __device__ __forceinline__ PairInfo pair_info(const Sched* sc, const SchedCache*
   return pi;
 }
 
-__device__ __forceinline__ bool next_piece(const Sched* sc, const SchedCache* cache, int n_pairs, Walker& wk,
+template <typename Cache>
+__device__ __forceinline__ bool next_piece(const Sched* sc, const Cache* cache, int n_pairs, Walker& wk,
                                            Piece& pc) {
   if (wk.x >= wk.end) return false;
   PairInfo pi = pair_info(sc, cache, wk.pair);
@@ -483,23 +482,22 @@ __device__ __forceinline__ void make_item(const AttnParams& p, const Piece& pc, 
   w.slot = ((long long)(2 * gang_id + (pc.first_of_gang ? 0 : 1)) * p.n_mp + mp);
 }
 
-// V-from-pool variant: maps over the pool's V with boxes of 1, 2, 4, ..., 128 rows, from which a
-// tile is stitched run by run (a run = consecutive context positions that are consecutive pool rows).
-struct VPoolMaps {
+// Maps over the pool's V (or K) with boxes of 1, 2, 4, ..., 128 rows, from which a tile is stitched run by
+// run (a run = consecutive context positions that are consecutive pool rows).
+struct PoolMaps {
   CUtensorMap m[8];
 };
 
 // TMEM: S/P of M tile A at columns 0..127, of M tile B at 128..255 (P, as packed bf16,
 // overwrites the S tile it was computed from); O accumulators at 256 and 384.
-// FUSED: the context K/V tiles are read from the pool through the row map (per-thread async
-// copies into the swizzled tile layout) and K is rotated in shared memory by two loader warps,
-// so that no re-encoded cache is ever written to HBM; TMA then only brings Q.
+// VPOOL and FUSED: V tiles are stitched from the pool by a gather warp.  FUSED: so are the K tiles, by a second
+// one; four warps then re-encode them (Eq. 7) where they lie, so that no re-encoded cache is ever written to HBM.
 template <int D, int MODE>
 __global__ void __launch_bounds__(MODE == kModeFused ? kFusedThreads : (MODE == kModeVPool ? kVPoolThreads : kAttnThreads), 1)
 attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kctx,
                  const __grid_constant__ CUtensorMap tm_vctx, const __grid_constant__ CUtensorMap tm_kown,
-                 const __grid_constant__ CUtensorMap tm_vown, const __grid_constant__ VPoolMaps vmaps,
-                 const AttnParams p) {
+                 const __grid_constant__ CUtensorMap tm_vown, const __grid_constant__ PoolMaps vmaps,
+                 const __grid_constant__ PoolMaps kmaps, const __grid_constant__ AttnParams p) {
   constexpr bool FUSED = MODE == kModeFused;
   constexpr bool VPOOL = MODE == kModeVPool;
   using SM = AttnSmem<D, MODE>;
@@ -510,7 +508,8 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   constexpr uint32_t kIdescPV = idesc_bf16_f32(kTileM, D, 1);
   constexpr uint32_t kTmemS = 0, kTmemO = 256;
   constexpr int kSoftmaxWarp0 = FUSED ? 4 : 2;          // first of the eight softmax warps
-  constexpr int kGatherWarp = kSoftmaxWarp0 + 8;        // V-from-pool variant: the warp that gathers the V tiles
+  constexpr int kGatherWarp = FUSED ? 2 : kSoftmaxWarp0 + 8;   // the warp that gathers the V tiles (fused: K by the next one)
+  constexpr int kBarKReady = FUSED ? kBarKRot : kBarKFull;
 
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw_addr = smem_u32(smem_raw);
@@ -536,9 +535,10 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       mbar_init(bar(kBarOEmpty + i), 128);
     }
     for (int i = 0; i < 3; ++i) {
-      mbar_init(bar(kBarKFull + i), FUSED ? kLoaders : 1);
+      mbar_init(bar(kBarKFull + i), 1);
       mbar_init(bar(kBarKEmpty + i), 1);
-      mbar_init(bar(kBarVFull + i), FUSED ? kLoaders : 1);
+      mbar_init(bar(kBarVFull + i), 1);
+      mbar_init(bar(kBarKRot + i), kRotateWarps);
       mbar_init(bar(kBarVEmpty + i), 1);
     }
     mbar_init(bar(kBarDrain), 1);
@@ -551,7 +551,8 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     tmem_relinquish();
   }
   // the CTA's part of the schedule, fetched by two otherwise idle warps while the rest is set up
-  SchedCache* cache = reinterpret_cast<SchedCache*>(base_ptr + SM::kOffBar + 256);
+  constexpr int kCachePairs = sched_cache_pairs(MODE);
+  SchedCache<kCachePairs>* cache = reinterpret_cast<SchedCache<kCachePairs>*>(base_ptr + SM::kOffBar + 256);
   if (warp >= 2 && warp < 4) {
     const int p0 = sc->first_pair[gang_id];
     const int n = min(kCachePairs, n_pairs - p0);
@@ -581,7 +582,7 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   wk0.x = wk0.begin;
   wk0.pair = cache->p0;
 
-  if (warp == 0) {
+  auto role_tma = [&]() {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
       tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_kctx); tma_prefetch_desc(&tm_vctx);
@@ -647,7 +648,8 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       }
     }
     __syncwarp();
-  } else if (warp == 1) {
+  };
+  auto role_mma = [&]() {
     // -------------------------------------------------------------- MMA issuer
     if (lane == 0) {
       // The tensor pipe takes only a few UMMAs ahead of the one it runs: whatever this thread
@@ -709,7 +711,7 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           // S of the first tile for both M tiles
           ok = mbar_wait(bar(kBarQFull + 0), ni0 & 1, abort_flag);
           if (ok && w.has_b) ok = mbar_wait(bar(kBarQFull + 1), ni1 & 1, abort_flag);
-          if (ok) ok = mbar_wait(bar(kBarKFull + tk % KS), (tk / KS) & 1, abort_flag);
+          if (ok) ok = mbar_wait(bar(kBarKReady + tk % KS), (tk / KS) & 1, abort_flag);
           if (!ok) break;
           tc_fence_after();
           issue_qk(0, tk % KS);
@@ -723,7 +725,7 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           for (int i = 0; i < w.n_tiles && ok; ++i) {
             const bool next = i + 1 < w.n_tiles;
             const uint32_t k_stage = tk % KS, v_stage = tv % VS;
-            if (next) ok = mbar_wait(bar(kBarKFull + k_stage), (tk / KS) & 1, abort_flag);
+            if (next) ok = mbar_wait(bar(kBarKReady + k_stage), (tk / KS) & 1, abort_flag);
             if (ok) ok = mbar_wait(bar(kBarVFull + v_stage), (tv / VS) & 1, abort_flag);
             if (ok) ok = chain(0, np0, ni0, i, w.n_tiles, k_stage, v_stage);
             if (ok && w.has_b) ok = chain(1, np1, ni1, i, w.n_tiles, k_stage, v_stage);
@@ -745,155 +747,109 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       }
     }
     __syncwarp();
-  } else if (FUSED && warp < 4) {
-    // ------------------------------------------- loader: K/V tiles straight from the pool
-    // A thread owns the same rotary pairs of every tile: pair c = lt + 64 u is row c / PPR,
-    // 16-byte chunk jj = c % PPR of the low half and chunk jj + PPR of the high half, so its
-    // eight frequencies never change and consecutive pairs are kRowStep positions apart: the
-    // (cos, sin) of the first row come from the table, the others by one complex
-    // multiplication with (cos, sin)(kRowStep * theta).  Copies are per-thread async copies
-    // (no registers, zero fill for rows beyond the context), written in the 128-byte swizzle
-    // the UMMA descriptors expect; K is rotated in place by the thread that copied it.
+  };
+  auto role_rotate_k = [&]() {
+    // ------------------------------------------- K tiles re-encoded where they landed
+    // A thread owns the same rotary pairs of every tile: 16-byte chunk jj of the low half of a row and
+    // chunk jj + PPR of the high half, rows row0, row0 + kRowStep, ...: its eight frequencies never change,
+    // and neither does the swizzle (kRowStep is a multiple of 8).  Angles: fp64 once per tile (or per shot, when
+    // the keys are stored rotated), then kRowStep positions further by one complex multiplication.
     constexpr int PPR = D / 16;
-    constexpr int kRowStep = kLoaders / PPR;
-    constexpr int PAIRS = kTileN / kRowStep;
-    const int lt = threadIdx.x - 64;
-    const int jj = lt % PPR, row0 = lt / PPR;
-    uint32_t dst_off[2];                              // tile offsets of row 0's two chunks, before the row term
+    constexpr int kRowStep = 32 * kRotateWarps / PPR;
+    constexpr int kUnits = kTileN / kRowStep;
+    constexpr int RPW = 32 / PPR;                     // rows of one unit in a warp
+    static_assert(kRowStep % 8 == 0, "the swizzle of a thread's rows must not change");
+    const int lw = warp - kRotateWarp0;
+    const int jj = lane % PPR, row0 = lw * RPW + lane / PPR;
+    const int map_row = (lane / RPW) * kRowStep + lw * RPW + lane % RPW;     // the row whose map entry this lane loads
+    const uint32_t off_lo = (jj / 8) * 16384u + row0 * 128u + (((jj & 7) ^ (row0 & 7)) << 4);
+    const uint32_t off_hi = ((jj + PPR) / 8) * 16384u + row0 * 128u + ((((jj + PPR) & 7) ^ (row0 & 7)) << 4);
+    const double* theta = p.theta + jj * 8;
+    const bool per_shot = p.k_pos_mode == 1;          // the angle is that of the shot's first position
+    float2 step_c[4], step_s[4];                      // (cos, sin) of kRowStep positions, two frequencies each
 #pragma unroll
-    for (int h = 0; h < 2; ++h) dst_off[h] = ((jj + h * PPR) / 8) * 16384u;
-    float2 step[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const double theta = pow((double)p.rope_base_f, -(double)(jj * 8 + e) / (double)(D / 2));
-      float sn, cs;
-      rope_sincos((double)kRowStep, theta, &sn, &cs);
-      step[e] = make_float2(cs, sn);
+    for (int e = 0; e < 4; ++e) {
+      rope_sincos((double)kRowStep, theta[2 * e], &step_s[e].x, &step_c[e].x);
+      rope_sincos((double)kRowStep, theta[2 * e + 1], &step_s[e].y, &step_c[e].y);
     }
-    uint32_t tk = 0, tv = 0;
+    float2 c2[4], s2[4];                              // (cos, sin) of the current row
+    auto set_angles = [&](double delta) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        rope_sincos_fast(delta, theta[2 * e], &s2[e].x, &c2[e].x);
+        rope_sincos_fast(delta, theta[2 * e + 1], &s2[e].y, &c2[e].y);
+      }
+    };
+    auto rotate_unit = [&](unsigned char* kt, int u, bool step) {
+      uint4* lo = reinterpret_cast<uint4*>(kt + off_lo + u * kRowStep * 128u);
+      uint4* hi = reinterpret_cast<uint4*>(kt + off_hi + u * kRowStep * 128u);
+      const uint4 xl = *lo, yl = *hi;
+      const uint32_t xw[4] = {xl.x, xl.y, xl.z, xl.w}, yw[4] = {yl.x, yl.y, yl.z, yl.w};
+      uint32_t xo[4], yo[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 x = make_float2(__uint_as_float(xw[e] << 16), __uint_as_float(xw[e] & 0xffff0000u));
+        const float2 y = make_float2(__uint_as_float(yw[e] << 16), __uint_as_float(yw[e] & 0xffff0000u));
+        const float2 ns = make_float2(-s2[e].x, -s2[e].y);
+        const float2 xr = __ffma2_rn(y, ns, __fmul2_rn(x, c2[e]));
+        const float2 yr = __ffma2_rn(x, s2[e], __fmul2_rn(y, c2[e]));
+        xo[e] = pack_bf16x2(xr.x, xr.y);
+        yo[e] = pack_bf16x2(yr.x, yr.y);
+        if (step) {
+          const float2 c = __ffma2_rn(ns, step_s[e], __fmul2_rn(c2[e], step_c[e]));
+          s2[e] = __ffma2_rn(c2[e], step_s[e], __fmul2_rn(s2[e], step_c[e]));
+          c2[e] = c;
+        }
+      }
+      *lo = make_uint4(xo[0], xo[1], xo[2], xo[3]);
+      *hi = make_uint4(yo[0], yo[1], yo[2], yo[3]);
+    };
+    uint32_t tk = 0;
     bool ok = true;
     Walker wk = wk0;
     Piece pc;
-    auto chunk_addr = [&](int row, int h) -> uint32_t {
-      const int j = (jj + h * PPR) & 7;
-      return dst_off[h] + row * 128u + ((j ^ (row & 7)) << 4);
-    };
-    auto issue = [&](const Item& w, int i, uint32_t sk, uint32_t sv) {
-      const bool own = i >= w.n_ctx;
-      const uint32_t k_base = base + SM::kOffK + sk * kTileBytes, v_base = base + SM::kOffV + sv * kTileBytes;
-      long long src[PAIRS];                            // element offset of the row's head, -1: zero fill
-#pragma unroll
-      for (int u = 0; u < PAIRS; ++u) {
-        const int row = row0 + u * kRowStep;
-        if (!own) {
-          const long long pos = (long long)(w.ctx_begin + i) * kTileN + row;
-          const int r = pos < p.ctx_cap ? p.row_map[(long long)w.b * p.ctx_cap + pos] : -1;
-          src[u] = r < 0 ? -1 : (((long long)(p.layer_begin + w.l) * p.pool_tokens + r) * p.Hkv + w.g) * D;
-        } else {
-          const int t = (w.own_begin + i - w.n_ctx) * kTileN + row;
-          src[u] = t >= p.To ? -1 : (((long long)w.outer_own * p.To + t) * p.Hkv + w.g) * D;
-        }
-      }
-      const __nv_bfloat16* kb = own ? p.kq_rot : p.k_pool;
-      const __nv_bfloat16* vb = own ? p.vq : p.v_pool;
-#pragma unroll
-      for (int u = 0; u < PAIRS; ++u) {
-        const int row = row0 + u * kRowStep;
-        const uint32_t n = src[u] < 0 ? 0u : 16u;
-        const __nv_bfloat16* g = kb + (src[u] < 0 ? 0 : src[u]) + jj * 8;
-        cp_async16(k_base + chunk_addr(row, 0), g, n);
-        cp_async16(k_base + chunk_addr(row, 1), g + D / 2, n);
-      }
-      cp_async_commit();
-#pragma unroll
-      for (int u = 0; u < PAIRS; ++u) {
-        const int row = row0 + u * kRowStep;
-        const uint32_t n = src[u] < 0 ? 0u : 16u;
-        const __nv_bfloat16* g = vb + (src[u] < 0 ? 0 : src[u]) + jj * 8;
-        cp_async16(v_base + chunk_addr(row, 0), g, n);
-        cp_async16(v_base + chunk_addr(row, 1), g + D / 2, n);
-      }
-      cp_async_commit();
-    };
-    auto rotate = [&](const Item& w, int i, uint32_t sk) {
-      unsigned char* kt = base_ptr + SM::kOffK + sk * kTileBytes;
-      const long long pos0 = (long long)(w.ctx_begin + i) * kTileN + row0;
-      float2 cur[8];
-      auto load_angles = [&](long long table_row) {
-        const float4* tab = reinterpret_cast<const float4*>(p.rope_tab + table_row * (D / 2) + jj * 8);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float4 t4 = tab[e];
-          cur[2 * e] = make_float2(t4.x, t4.y);
-          cur[2 * e + 1] = make_float2(t4.z, t4.w);
-        }
-      };
-      const bool per_shot = p.k_pos_mode == 1;     // the angle is that of the shot's first position
-      if (!per_shot) load_angles(pos0);
-#pragma unroll
-      for (int u = 0; u < PAIRS; ++u) {
-        const int row = row0 + u * kRowStep;
-        uint4* lo = reinterpret_cast<uint4*>(kt + chunk_addr(row, 0));
-        uint4* hi = reinterpret_cast<uint4*>(kt + chunk_addr(row, 1));
-        if (per_shot) {
-          const long long pos = pos0 + u * kRowStep;
-          load_angles(pos < p.ctx_cap ? p.off_map[(long long)w.b * p.ctx_cap + pos] : 0);
-        }
-        float x[8], y[8], xr[8], yr[8];
-        bf16x8_unpack(*lo, x);
-        bf16x8_unpack(*hi, y);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          xr[e] = x[e] * cur[e].x - y[e] * cur[e].y;
-          yr[e] = y[e] * cur[e].x + x[e] * cur[e].y;
-        }
-        *lo = bf16x8_pack(xr);
-        *hi = bf16x8_pack(yr);
-        if (!per_shot && u + 1 < PAIRS) {
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const float c = cur[e].x * step[e].x - cur[e].y * step[e].y;
-            const float sn = cur[e].y * step[e].x + cur[e].x * step[e].y;
-            cur[e] = make_float2(c, sn);
-          }
-        }
-      }
-    };
     while (ok && next_piece(sc, cache, n_pairs, wk, pc)) {
       for (int mp = rank; mp < p.n_mp && ok; mp += p.gang) {
         Item w;
         make_item(p, pc, gang_id, mp, w);
-        if (w.n_tiles == 0) continue;
-        ok = mbar_wait(bar(kBarKEmpty + tk % KS), ((tk / KS) & 1) ^ 1, abort_flag) &&
-             mbar_wait(bar(kBarVEmpty + tv % VS), ((tv / VS) & 1) ^ 1, abort_flag);
-        if (!ok) break;
-        issue(w, 0, tk % KS, tv % VS);
-        for (int i = 0; i < w.n_tiles; ++i) {
-          const uint32_t sk = tk % KS, sv = tv % VS;
-          const bool next = i + 1 < w.n_tiles;
-          if (next) {
-            ok = mbar_wait(bar(kBarKEmpty + (tk + 1) % KS), (((tk + 1) / KS) & 1) ^ 1, abort_flag) &&
-                 mbar_wait(bar(kBarVEmpty + (tv + 1) % VS), (((tv + 1) / VS) & 1) ^ 1, abort_flag);
-            if (!ok) break;
-            issue(w, i + 1, (tk + 1) % KS, (tv + 1) % VS);
-            cp_async_wait<3>();                         // K of tile i has landed
-          } else {
-            cp_async_wait<1>();
+        const int* omap = p.off_map + (long long)w.b * p.ctx_cap;
+        auto first_of = [&](int i) -> int {           // first position of the shot that map_row of tile i lies in
+          const long long pos = (long long)(w.ctx_begin + i) * kTileN + map_row;
+          return per_shot && i < w.n_ctx && pos < p.ctx_cap ? omap[pos] : 0;
+        };
+        int first = first_of(0), first_cur = -1;
+        for (int i = 0; i < w.n_tiles; ++i, ++tk) {
+          const uint32_t sk = tk % KS;
+          unsigned char* kt = base_ptr + SM::kOffK + sk * kTileBytes;
+          const bool ctx = i < w.n_ctx;               // (the probe's own keys were rotated by the prep kernel)
+          const int first_next = first_of(i + 1);
+          if (ctx && !per_shot) set_angles((double)((long long)(w.ctx_begin + i) * kTileN + row0));
+          ok = __all_sync(0xffffffffu, mbar_wait(bar(kBarKFull + sk), (tk / KS) & 1, abort_flag));
+          if (!ok) break;
+          if (ctx && !per_shot) {
+#pragma unroll
+            for (int u = 0; u < kUnits; ++u) rotate_unit(kt, u, u + 1 < kUnits);
+          } else if (ctx) {
+#pragma unroll 2
+            for (int u = 0; u < kUnits; ++u) {
+              const int o = __shfl_sync(0xffffffffu, first, u * RPW + lane / PPR);
+              if (o != first_cur) {
+                set_angles((double)o);
+                first_cur = o;
+              }
+              rotate_unit(kt, u, false);
+            }
           }
-          if (i < w.n_ctx) rotate(w, i, sk);
           fence_proxy_async_smem();
-          mbar_arrive(bar(kBarKFull + sk));
-          if (next) cp_async_wait<2>(); else cp_async_wait<0>();   // V of tile i
-          fence_proxy_async_smem();
-          mbar_arrive(bar(kBarVFull + sv));
-          ++tk;
-          ++tv;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar(kBarKRot + sk));
+          first = first_next;
         }
       }
     }
-    cp_async_wait<0>();
-  } else if (VPOOL && warp == kGatherWarp) {
-    // ----------------------------------------------- V tiles straight from the pool, stitched by TMA
+  };
+  auto role_gather = [&]() {
+    // ----------------------------------------------- V (fused: K, too) tiles straight from the pool, stitched by TMA
     // Eq. 7 corrects K only, so V needs no assembled copy.  The 128 context positions of a tile map
     // to a few runs of consecutive pool rows (one per selected shot the tile touches): the lanes look
     // the positions up and mark where a run ends; every run is brought as one or two power-of-two boxes
@@ -901,32 +857,39 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     // address only has to be 128-byte aligned), one box per lane, all found before the stage is waited
     // for.  Positions beyond the context continue the last run (their P is exactly zero; rows outside
     // the pool arrive as zeros).  The probe's own tokens are one run of the own-token tensor.
-    int* rows_s = reinterpret_cast<int*>(base_ptr + SM::kOffRows);
+    const bool is_k = FUSED && warp != kGatherWarp;
+    int* rows_s = reinterpret_cast<int*>(base_ptr + SM::kOffRows + (is_k ? 512 : 0));
+    const uint32_t n_st = is_k ? KS : VS;
+    const uint32_t tiles0 = base + (is_k ? SM::kOffK : SM::kOffV);
+    const uint32_t full0 = bar(is_k ? kBarKFull : kBarVFull), empty0 = bar(is_k ? kBarKEmpty : kBarVEmpty);
+    const PoolMaps* maps = is_k ? &kmaps : &vmaps;
+    const CUtensorMap* own_map = is_k ? &tm_kown : &tm_vown;
+    uint32_t sv = 0, phase = 0;                  // stage and parity of tile tv
     uint32_t tv = 0;
     bool ok = true;
     Walker wk = wk0;
     Piece pc;
     if (lane == 0) {
-      tma_prefetch_desc(&tm_vown);
+      tma_prefetch_desc(own_map);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) tma_prefetch_desc(&vmaps.m[e]);
+      for (int e = 0; e < 8; ++e) tma_prefetch_desc(&maps->m[e]);
     }
     while (ok && next_piece(sc, cache, n_pairs, wk, pc)) {
       for (int mp = rank; mp < p.n_mp && ok; mp += p.gang) {
         Item w;
         make_item(p, pc, gang_id, mp, w);
-        for (int i = 0; i < w.n_tiles; ++i, ++tv) {
-          const uint32_t sv = tv % VS;
-          const uint32_t v_dst = base + SM::kOffV + sv * kTileBytes;
+        for (int i = 0; i < w.n_tiles; ++i, ++tv, phase ^= (sv + 1 == n_st), sv = sv + 1 == n_st ? 0 : sv + 1) {
+          const uint32_t v_dst = tiles0 + sv * kTileBytes;
+          const uint32_t full = full0 + 8u * sv;
           if (i >= w.n_ctx) {
             // own tokens: one tiled box (rows beyond the last own token arrive as zeros)
             if (lane == 0) {
-              ok = mbar_wait(bar(kBarVEmpty + sv), ((tv / VS) & 1) ^ 1, abort_flag);
+              ok = mbar_wait(empty0 + 8u * sv, phase ^ 1, abort_flag);
               if (ok) {
-                mbar_arrive_expect_tx(bar(kBarVFull + sv), kTileBytes);
+                mbar_arrive_expect_tx(full, kTileBytes);
 #pragma unroll
                 for (int s2 = 0; s2 < SUB; ++s2)
-                  tma_load_4d(v_dst + s2 * 16384u, &tm_vown, bar(kBarVFull + sv), s2 * 64, w.g,
+                  tma_load_4d(v_dst + s2 * 16384u, own_map, full, s2 * 64, w.g,
                               (w.own_begin + i - w.n_ctx) * kTileN, w.outer_own);
               }
             }
@@ -1004,8 +967,8 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           if (my_pidx >= 0) my_row = rows_s[my_pidx];
           // (tiles of more than 32 boxes - many one-token shots - take further rounds of the same walk)
           if (lane == 0) {
-            ok = mbar_wait(bar(kBarVEmpty + sv), ((tv / VS) & 1) ^ 1, abort_flag);
-            if (ok) mbar_arrive_expect_tx(bar(kBarVFull + sv), tile_bytes);
+            ok = mbar_wait(empty0 + 8u * sv, phase ^ 1, abort_flag);
+            if (ok) mbar_arrive_expect_tx(full, tile_bytes);
           }
           ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
           if (!ok) break;
@@ -1013,7 +976,7 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           if (my_pidx >= 0) {
 #pragma unroll
             for (int s2 = 0; s2 < SUB; ++s2)
-              tma_load_4d(v_dst + s2 * 16384u + (uint32_t)my_pidx * 128u, &vmaps.m[my_lg], bar(kBarVFull + sv), s2 * 64,
+              tma_load_4d(v_dst + s2 * 16384u + (uint32_t)my_pidx * 128u, &maps->m[my_lg], full, s2 * 64,
                           w.g, my_row, layer);
           }
           for (int round = 1; round * 32 < n_boxes; ++round) {      // rare: more than 32 boxes in the tile
@@ -1039,7 +1002,7 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
               const int brow = rows_s[bp];
 #pragma unroll
               for (int s2 = 0; s2 < SUB; ++s2)
-                tma_load_4d(v_dst + s2 * 16384u + (uint32_t)bp * 128u, &vmaps.m[bl], bar(kBarVFull + sv), s2 * 64, w.g,
+                tma_load_4d(v_dst + s2 * 16384u + (uint32_t)bp * 128u, &maps->m[bl], full, s2 * 64, w.g,
                             brow, layer);
             }
           }
@@ -1049,11 +1012,12 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     }
     if (!ok && lane == 0) {
       // gave up: let the copies already in flight land before the CTA retires
-      for (uint32_t t = tv > (uint32_t)VS ? tv - VS : 0; t < tv; ++t)
-        mbar_wait(bar(kBarVFull + t % VS), (t / VS) & 1, abort_flag + 1);
+      for (uint32_t t = tv > n_st ? tv - n_st : 0; t < tv; ++t)
+        mbar_wait(full0 + 8u * (t % n_st), (t / n_st) & 1, abort_flag + 1);
     }
     __syncwarp();
-  } else {
+  };
+  auto role_softmax = [&]() {
     // ---------------------------------------------------- softmax + read-out of O
     const int x = (warp - kSoftmaxWarp0) >> 2;     // 0: M tile A, 1: M tile B
     const int quarter = warp & 3;                  // TMEM lanes this warp may touch
@@ -1079,7 +1043,8 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           if (!ok) break;
           tc_fence_after();
           float s[kTileN];
-          tmem_ld128(s_addr, reinterpret_cast<uint32_t*>(s));
+          if constexpr (FUSED) tmem_ld4x32(s_addr, reinterpret_cast<uint32_t*>(s));
+          else tmem_ld128(s_addr, reinterpret_cast<uint32_t*>(s));
 
           // mask: context keys at or beyond L_j; own keys after the row's token (causal).
           // Only the last context tile and the own-token tiles can hide anything.
@@ -1113,19 +1078,32 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           const float2 scale2 = make_float2(p.scale_log2, p.scale_log2);
           const float2 neg_m2 = make_float2(-m_used, -m_used);
           float2 part[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-          // the packed pair c2 goes into the register that held score c2 (already consumed:
-          // c2 <= 2 c2), so the row never needs more than its 128 registers
-          uint32_t* pk = reinterpret_cast<uint32_t*>(s);
-#pragma unroll
-          for (int c2 = 0; c2 < kTileN / 2; ++c2) {
+          auto exp_pair = [&](int c2) -> uint32_t {
             const float2 xs = __ffma2_rn(make_float2(s[2 * c2], s[2 * c2 + 1]), scale2, neg_m2);
             const float2 e = make_float2(ex2_approx(xs.x), ex2_approx(xs.y));
             part[c2 & 3] = __fadd2_rn(part[c2 & 3], e);
-            pk[c2] = pack_bf16x2(e.x, e.y);
+            return pack_bf16x2(e.x, e.y);
+          };
+          if constexpr (FUSED) {
+            // 32 keys at a time: their 16 packed columns are stored while the next ones are computed
+#pragma unroll
+            for (int c0 = 0; c0 < kTileN / 2; c0 += 16) {
+              uint32_t pk[16];
+#pragma unroll
+              for (int c = 0; c < 16; ++c) pk[c] = exp_pair(c0 + c);
+              tmem_st16_nowait(s_addr + c0, pk);
+            }
+            tmem_st_wait();
+          } else {
+            // the packed pair c2 goes into the register that held score c2 (already consumed:
+            // c2 <= 2 c2), so the row never needs more than its 128 registers
+            uint32_t* pk = reinterpret_cast<uint32_t*>(s);
+#pragma unroll
+            for (int c2 = 0; c2 < kTileN / 2; ++c2) pk[c2] = exp_pair(c2);
+            tmem_st64(s_addr, pk);
           }
           const float2 tot = __fadd2_rn(__fadd2_rn(part[0], part[1]), __fadd2_rn(part[2], part[3]));
           l_sum += tot.x + tot.y;
-          tmem_st64(s_addr, pk);
           if (i > 0 && __any_sync(0xffffffffu, need)) {
             // S(i) is complete, so PV(i-1), issued before it, is complete too; PV(i) waits for
             // the arrival below: O is quiescent here.
@@ -1248,6 +1226,26 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         ++ni;
       }
     }
+  };
+
+  if constexpr (FUSED) {                     // registers go where they are needed, one warpgroup at a time
+    if (warp < 4) {
+      regs_lower<kFusedRegsIssue>();
+      if (warp == 0) role_tma();
+      else if (warp == 1) role_mma();
+      else role_gather();
+    } else if (warp < kRotateWarp0) {
+      regs_raise<kFusedRegsSoftmax>();
+      role_softmax();
+    } else {
+      regs_lower<kFusedRegsRotate>();
+      role_rotate_k();
+    }
+  } else {
+    if (warp == 0) role_tma();
+    else if (warp == 1) role_mma();
+    else if (VPOOL && warp == kGatherWarp) role_gather();
+    else role_softmax();
   }
 
   tc_fence_before();
@@ -1380,8 +1378,7 @@ cudaEvent_t g_profile_ev[2] = {nullptr, nullptr};
 
 struct AttnPlan {
   int n_mt, n_mp, gang;
-  size_t off_qrot, off_kqrot, off_sched, off_opart, off_ml, off_rowmap, off_offmap, off_tab, total;
-  long long tab_rows;
+  size_t off_qrot, off_kqrot, off_sched, off_opart, off_ml, off_rowmap, off_offmap, total;
 };
 
 // Own tokens beyond the query rows, and a per-query shot count on the device (decode calls).
@@ -1399,8 +1396,7 @@ struct FusedSrc {
 
 // The gang (CTAs that walk the same K/V tiles, one M pair each per round) is the number of
 // M pairs when that is at most kMaxGang, else the M pairs are dealt out in rounds.
-AttnPlan make_plan(const adapshot_model_t* model, int B, int P, int Tq, int nl, long long fused_ctx_cap = 0,
-                   bool with_table = true, int To = 0) {
+AttnPlan make_plan(const adapshot_model_t* model, int B, int P, int Tq, int nl, long long map_ctx_cap = 0, int To = 0) {
   if (To < Tq) To = Tq;
   AttnPlan pl;
   const int G = model->n_q_heads / model->n_kv_heads;
@@ -1416,14 +1412,8 @@ AttnPlan make_plan(const adapshot_model_t* model, int B, int P, int Tq, int nl, 
   pl.off_sched = off; off += ads_round_up(sizeof(Sched), 256);
   pl.off_opart = off; off += ads_round_up(slots * 2 * kTileM * D * 4, 256);
   pl.off_ml = off;    off += ads_round_up(slots * 2 * kTileM * 2 * 4, 256);
-  pl.off_rowmap = pl.off_offmap = pl.off_tab = off;
-  pl.tab_rows = 0;
-  if (fused_ctx_cap > 0) {
-    pl.tab_rows = with_table ? (fused_ctx_cap + kTileN - 1) / kTileN * kTileN : 0;
-    pl.off_rowmap = off; off += ads_round_up((size_t)B * fused_ctx_cap * 4, 256);
-    pl.off_offmap = off; off += ads_round_up((size_t)B * fused_ctx_cap * 4, 256);
-    pl.off_tab = off;    off += ads_round_up((size_t)pl.tab_rows * (D / 2) * 8, 256);
-  }
+  pl.off_rowmap = off; off += ads_round_up((size_t)B * map_ctx_cap * 4, 256);
+  pl.off_offmap = off; off += ads_round_up((size_t)B * map_ctx_cap * 4, 256);
   pl.total = off;
   return pl;
 }
@@ -1477,36 +1467,33 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
     if (!make_map(&tm_kown, kq_rot, 4, dims, str, box)) return ADAPSHOT_ECUDA;
     if (!make_map(&tm_vown, vq, 4, dims, str, box)) return ADAPSHOT_ECUDA;
   }
-  VPoolMaps vmaps;
-  for (int e = 0; e < 8; ++e) vmaps.m[e] = tm_q;       // (unused outside the V-from-pool variant)
-  if (mode == kModeVPool) {
-    // the pool's V with boxes of 1, 2, ..., 128 rows (the layout of the cache maps, over the pool)
+  PoolMaps vmaps, kmaps;
+  for (int e = 0; e < 8; ++e) vmaps.m[e] = kmaps.m[e] = tm_q;       // (unused where nothing comes from the pool)
+  if (mode != kModeCache) {
+    // the pool's V (fused: K, too) with boxes of 1, 2, ..., 128 rows (the layout of the cache maps, over the pool)
     const uint64_t pt = (uint64_t)fused->pool->pool_tokens;
     const uint64_t dims[4] = {(uint64_t)D, (uint64_t)Hkv, pt, (uint64_t)model->n_layers};
     const uint64_t str[3] = {(uint64_t)D * 2, (uint64_t)Hkv * D * 2, pt * Hkv * D * 2};
     for (int e = 0; e < 8; ++e) {
       const uint32_t box[4] = {64, 1, 1u << e, 1};
       if (!make_map(&vmaps.m[e], fused->pool->v, 4, dims, str, box)) return ADAPSHOT_ECUDA;
+      if (mode == kModeFused && !make_map(&kmaps.m[e], fused->pool->k, 4, dims, str, box)) return ADAPSHOT_ECUDA;
     }
   }
 
-  // ---- fused variant: row map and rotary table
+  // ---- K or V from the pool: row map
   int* row_map = reinterpret_cast<int*>(wsb + pl.off_rowmap);
   int* off_map = reinterpret_cast<int*>(wsb + pl.off_offmap);
-  float2* rope_tab = reinterpret_cast<float2*>(wsb + pl.off_tab);
   if (fused != nullptr) {
-    FusedPlanParams fp;
-    fp.ctx_off = reinterpret_cast<const long long*>(ctx_off);
-    fp.sel_idx = fused->sel_idx;
-    fp.shot_off = reinterpret_cast<const long long*>(fused->pool->shot_off);
-    fp.row_map = row_map; fp.off_map = off_map; fp.rope_tab = rope_tab;
-    fp.ctx_cap = ctx_cap; fp.tab_rows = pl.tab_rows;
-    fp.B = B; fp.k = k; fp.n_shots = fused->pool->n_shots; fp.half_d = D / 2;
-    fp.rope_base = model->rope_base;
-    const long long work = (long long)B * ctx_cap + pl.tab_rows * (D / 2);
-    long long blocks = (work + 255) / 256;
-    if (blocks > n_sm * 16) blocks = n_sm * 16;
-    attn_fused_plan_kernel<<<(unsigned)blocks, 256, 0, st>>>(fp);
+    RowMapParams rm;
+    rm.ctx_off = reinterpret_cast<const long long*>(ctx_off);
+    rm.sel_idx = fused->sel_idx;
+    rm.shot_off = reinterpret_cast<const long long*>(fused->pool->shot_off);
+    rm.row_map = row_map;
+    rm.off_map = mode == kModeFused && model->k_pos_mode == 1 ? off_map : nullptr;
+    rm.ctx_cap = ctx_cap;
+    rm.B = B; rm.k = k; rm.n_shots = fused->pool->n_shots;
+    attn_row_map_kernel<<<(unsigned)(((long long)B * k + 7) / 8), 256, 0, st>>>(rm);
     if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
   }
 
@@ -1533,29 +1520,26 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
   const float scale = model->softmax_scale > 0.f ? model->softmax_scale : 1.0f / sqrtf((float)D);
   ap.scale_log2 = scale * 1.4426950408889634f;
   // the same request for D = 64 as for D = 128: one CTA per SM in every variant
-  const int smem = mode == kModeVPool ? (int)AttnSmem<128, kModeVPool>::kTotal : (int)AttnSmem<128, kModeCache>::kTotal;
+  const int smem = mode == kModeVPool ? (int)AttnSmem<128, kModeVPool>::kTotal
+                   : mode == kModeFused ? (int)AttnSmem<128, kModeFused>::kTotal : (int)AttnSmem<128, kModeCache>::kTotal;
   static bool attr_done[3][kAdsMaxDevices] = {{false}, {false}, {false}};   // per template instance (D, mode) and device
   if (g_profile) ADS_CHECK_CUDA(cudaEventRecord(g_profile_ev[0], st));
   if (mode == kModeCache) {
     if (ads_set_max_smem(attn_main_kernel<D, kModeCache>, smem, attr_done[0]) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
     attn_main_kernel<D, kModeCache><<<(unsigned)(n_gangs * pl.gang), kAttnThreads, smem, st>>>(
-        tm_q, tm_kctx, tm_vctx, tm_kown, tm_vown, vmaps, ap);
+        tm_q, tm_kctx, tm_vctx, tm_kown, tm_vown, vmaps, kmaps, ap);
   } else {
-    ap.k_pool = static_cast<const __nv_bfloat16*>(fused->pool->k);
-    ap.v_pool = static_cast<const __nv_bfloat16*>(fused->pool->v);
-    ap.kq_rot = kq_rot;
-    ap.vq = static_cast<const __nv_bfloat16*>(vq);
-    ap.row_map = row_map; ap.off_map = off_map; ap.k_pos_mode = model->k_pos_mode; ap.rope_tab = rope_tab;
-    ap.pool_tokens = fused->pool->pool_tokens; ap.ctx_cap = ctx_cap;
-    ap.layer_begin = fused->layer_begin; ap.rope_base_f = model->rope_base;
+    ap.row_map = row_map; ap.off_map = off_map; ap.k_pos_mode = model->k_pos_mode;
+    ap.ctx_cap = ctx_cap; ap.layer_begin = fused->layer_begin;
+    for (int i = 0; i < D / 2; ++i) ap.theta[i] = pp.theta[i];
     if (mode == kModeFused) {
       if (ads_set_max_smem(attn_main_kernel<D, kModeFused>, smem, attr_done[1]) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
       attn_main_kernel<D, kModeFused><<<(unsigned)(n_gangs * pl.gang), kFusedThreads, smem, st>>>(
-          tm_q, tm_kctx, tm_vctx, tm_kown, tm_vown, vmaps, ap);
+          tm_q, tm_kctx, tm_vctx, tm_kown, tm_vown, vmaps, kmaps, ap);
     } else {
       if (ads_set_max_smem(attn_main_kernel<D, kModeVPool>, smem, attr_done[2]) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
       attn_main_kernel<D, kModeVPool><<<(unsigned)(n_gangs * pl.gang), kVPoolThreads, smem, st>>>(
-          tm_q, tm_kctx, tm_vctx, tm_kown, tm_vown, vmaps, ap);
+          tm_q, tm_kctx, tm_vctx, tm_kown, tm_vown, vmaps, kmaps, ap);
     }
   }
   if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
@@ -1671,7 +1655,7 @@ extern "C" size_t adapshot_attn_vpool_workspace_bytes(const adapshot_model_t* mo
   if (model == nullptr || !attn_shape_ok(model) || B <= 0 || P <= 0 || Tq <= 0 || n_layers_in_call <= 0 ||
       ctx_cap <= 0)
     return 0;
-  return make_plan(model, B, P, Tq, n_layers_in_call, ctx_cap, false).total;
+  return make_plan(model, B, P, Tq, n_layers_in_call, ctx_cap).total;
 }
 
 extern "C" int adapshot_query_attn_vpool(const adapshot_model_t* model, const adapshot_pool_t* pool,
@@ -1700,7 +1684,7 @@ extern "C" int adapshot_query_attn_vpool(const adapshot_model_t* model, const ad
     return ADAPSHOT_EALIGN;
   if (ctx_cap > (1ll << 31) - 256 || pool->pool_tokens > (1ll << 31) - 1) return ADAPSHOT_ESHAPE;
   const int nl = layer_end - layer_begin;
-  const AttnPlan pl = make_plan(model, B, P, Tq, nl, ctx_cap, false);
+  const AttnPlan pl = make_plan(model, B, P, Tq, nl, ctx_cap);
   if (ws_bytes < pl.total) return ADAPSHOT_ECAPACITY;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   FusedSrc src;
@@ -1787,7 +1771,7 @@ extern "C" size_t adapshot_decode_workspace_bytes(const adapshot_model_t* model,
   if (model == nullptr || !attn_shape_ok(model) || B <= 0 || T_new <= 0 || T_own < T_new || n_layers_in_call <= 0)
     return 0;
   if (ads_decode_rows_fit(model, T_new)) return ads_decode_rows_workspace(model, B);
-  return make_plan(model, B, 1, T_new, n_layers_in_call, 0, true, T_own).total;
+  return make_plan(model, B, 1, T_new, n_layers_in_call, 0, T_own).total;
 }
 
 extern "C" int adapshot_decode_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_ctx,
@@ -1818,7 +1802,7 @@ extern "C" int adapshot_decode_attn(const adapshot_model_t* model, const void* k
     return ads_decode_rows(model, k_ctx, v_ctx, ctx_cap, ctx_off, B, k, n_shots, q_new, k_own, v_own, T_new, T_own, nl,
                            out, lse, ws, status, static_cast<cudaStream_t>(stream));
   }
-  const AttnPlan pl = make_plan(model, B, 1, T_new, nl, 0, true, T_own);
+  const AttnPlan pl = make_plan(model, B, 1, T_new, nl, 0, T_own);
   if (ws_bytes < pl.total) return ADAPSHOT_ECAPACITY;
   AttnExtra extra;
   extra.To = T_own;

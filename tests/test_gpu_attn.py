@@ -189,3 +189,37 @@ def test_number_of_ranges_follows_the_work(n_shots):
     w = wl.CONFIGS["cfg2"].scaled(n_shots=n_shots, len_dist="const", len_lo=128, len_hi=128, batch=1, k=n_shots, t_q=3,
                                   n_q_heads=8, n_kv_heads=8, head_dim=64, seed=28)
     _run_case(w, np.arange(n_shots, dtype=np.int32)[None, ::-1].copy(), [n_shots], 1)
+
+
+@pytest.mark.parametrize("k_pos_mode", [0, 1])
+@pytest.mark.parametrize("d,lens,k,t_q,probes", [
+    (128, (127, 129), 7, 1, (1, 7)),       # shots that end on either side of a 128-key tile
+    (64, (1, 1), 150, 129, (128, 150)),    # one-token shots: more than 32 copies per tile; two tiles of own tokens
+    (128, (1, 9), 60, 70, (3, 60)),        # many short runs; two M tiles of which the second is nearly empty (G = 2)
+    (64, (300, 300), 6, 33, (6,)),         # a shot spans several tiles
+])
+def test_keys_re_encoded_on_the_way_to_the_tensor_cores(d, lens, k, t_q, probes, k_pos_mode):
+    # the fused call against the oracle's assembled context, for keys stored bare and stored rotated at local positions
+    ab = hp.gpu_binding()
+    w = wl.CONFIGS["cfg2"].scaled(n_shots=k + 3, len_lo=lens[0], len_hi=lens[1], batch=2, k=k, probes=probes, t_q=t_q,
+                                  n_q_heads=4, n_kv_heads=2, head_dim=d, seed=29)
+    pool, qs = wl.make_pool(w, n_layers=1), wl.make_queries(w, n_layers=1)
+    rng = np.random.default_rng(6)
+    sel = np.stack([rng.permutation(k + 3)[:k] for _ in range(2)]).astype(np.int32)
+    dp, model = hp.dev_pool(ab, pool), hp.model_of(ab, w, n_layers=1, k_pos_mode=k_pos_mode)
+    off_np = orc.plan_offsets(sel, pool["shot_off"])
+    cap = int(off_np[:, -1].max()) + 5
+    sel_d, off = torch.from_numpy(sel).cuda(), torch.from_numpy(off_np).cuda()
+    out = torch.full_like(qs["q"].cuda(), 9.0)
+    ws = torch.empty(ab.adapshot_attn_fused_workspace_bytes(model, 2, len(probes), t_q, 1, cap), dtype=torch.uint8,
+                     device="cuda")
+    st = hp.new_status()
+    ab.adapshot_query_attn_fused(model, dp, sel_d, off, cap, list(probes), qs["q"].cuda(), qs["kq"].cuda(),
+                                 qs["vq"].cuda(), 0, 1, out, None, ws, st)
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    for b in range(2):
+        kc, vc, _ = orc.assemble_kv(hp.f64(pool["k"]), hp.f64(pool["v"]), pool["shot_off"], sel[b], w.rope_base, k_pos_mode)
+        want, _ = orc.query_attn(hp.f64(qs["q"][b, 0]), hp.f64(qs["kq"][b, 0]), hp.f64(qs["vq"][b, 0]), kc[0], vc[0],
+                                 [int(off_np[b, n]) for n in probes], w.rope_base)
+        hp.assert_attn_close(out[b, 0].cpu().double().numpy(), want, what=b)
