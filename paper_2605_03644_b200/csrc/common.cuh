@@ -98,11 +98,9 @@ __device__ __forceinline__ double ads_key_score(unsigned long long k) {
 }
 
 // Top k of N candidates per query from their sort keys (select.cu): keys [B][N] as ads_desc_key
-// writes them, ids [B][N] = 0..N-1 (read only when N needs the chunked sort), cand = scratch of
-// ads_topk_scratch_bytes(N, B, k) bytes.  Enqueues on st; returns an ADAPSHOT_* code.
-size_t ads_topk_scratch_bytes(int N, int B, int k);
-int ads_topk_from_keys(const unsigned long long* keys, const int* ids, int N, int B, int k, void* cand,
-                       int32_t* sel_idx, float* sel_score, cudaStream_t st);
+// writes them; equal keys by the lower index.  Enqueues on st; returns an ADAPSHOT_* code.
+int ads_topk_from_keys(const unsigned long long* keys, int N, int B, int k, int32_t* sel_idx, float* sel_score,
+                       cudaStream_t st);
 
 // Decoding with few rows per KV head (decode.cu): whether a call's rows fit, its scratch, and the call itself
 // (arguments checked by the caller).

@@ -336,23 +336,22 @@ __global__ void __launch_bounds__(128) rel_merge_kernel(const float* __restrict_
   lse2[unit * kTile + r] = l > 0.f ? M + log2f(l) : 0.f;
 }
 
-// score[b][i] = mass[b][i] / (T_q * Hq) (and / T_i with per_token); writes the sort keys and the ids.
+// score[b][i] = mass[b][i] / (T_q * Hq) (and / T_i with per_token); writes the sort keys.
 __global__ void __launch_bounds__(256) rel_scores_kernel(const double* __restrict__ mass,
                                                          const long long* __restrict__ shot_off, int B, int n_shots,
                                                          double inv_rows, int per_token,
-                                                         unsigned long long* __restrict__ keys, int* __restrict__ ids) {
+                                                         unsigned long long* __restrict__ keys) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long long)B * n_shots) return;
   const int shot = (int)(i % n_shots);
   double s = mass[i] * inv_rows;
   if (per_token) s /= (double)(shot_off[shot + 1] - shot_off[shot]);
   keys[i] = ads_desc_key(s);
-  ids[i] = shot;
 }
 
 struct RelPlan {
   int G, n_mt, rows, rows_pad, n_tiles, splits, tiles_per_split;
-  size_t off_qpack, off_ml, off_lse, off_tokshot, off_mass, off_keys, off_ids, off_cand, total;
+  size_t off_qpack, off_ml, off_lse, off_tokshot, off_mass, off_keys, total;
 };
 
 RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int B, int Tq, int k) {
@@ -389,8 +388,6 @@ RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int
   pl.off_tokshot = off; off += ads_round_up((size_t)pool->pool_tokens * 4, 256);
   pl.off_mass = off;    off += ads_round_up((size_t)B * pool->n_shots * 8, 256);
   pl.off_keys = off;    off += ads_round_up((size_t)B * pool->n_shots * 8, 256);
-  pl.off_ids = off;     off += ads_round_up((size_t)B * pool->n_shots * 4, 256);
-  pl.off_cand = off;    off += ads_topk_scratch_bytes(pool->n_shots, B, k);
   pl.total = off;
   return pl;
 }
@@ -412,7 +409,6 @@ int rel_launch(const adapshot_model_t* model, const adapshot_pool_t* pool, int l
   int* tok_shot = reinterpret_cast<int*>(wsb + pl.off_tokshot);
   double* mass = reinterpret_cast<double*>(wsb + pl.off_mass);
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(wsb + pl.off_keys);
-  int* ids = reinterpret_cast<int*>(wsb + pl.off_ids);
   const long long units = (long long)B * pl.n_mt * Hkv;
 
   CUtensorMap tm_q, tm_k;
@@ -461,9 +457,9 @@ int rel_launch(const adapshot_model_t* model, const adapshot_pool_t* pool, int l
   const long long n_sc = (long long)B * pool->n_shots;
   rel_scores_kernel<<<(unsigned)((n_sc + 255) / 256), 256, 0, st>>>(
       mass, reinterpret_cast<const long long*>(pool->shot_off), B, pool->n_shots, 1.0 / ((double)Tq * Hq),
-      (flags & ADAPSHOT_RELEVANCE_PER_TOKEN) ? 1 : 0, keys, ids);
+      (flags & ADAPSHOT_RELEVANCE_PER_TOKEN) ? 1 : 0, keys);
   if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-  return ads_topk_from_keys(keys, ids, pool->n_shots, B, k, wsb + pl.off_cand, sel_idx, sel_score, st);
+  return ads_topk_from_keys(keys, pool->n_shots, B, k, sel_idx, sel_score, st);
 }
 
 }  // namespace

@@ -1,32 +1,34 @@
 // Semantic shot selection (paper Sec. 4.1 ranking, Sec. 4.2 "rank in descending
 // order and select the top k"): cosine of the query embedding against every cached
-// shot embedding, then the top k with ties broken by the lower shot id (by rank counting
-// for pools of up to 4096 shots, by chunked block-wide sorts beyond).
+// shot embedding, then the top k with ties broken by the lower shot id.
 //
 // The ranking must equal that of an fp64 evaluation of the same formula, so the
 // fp32 products (exact in fp64) are accumulated in fp64 and scores are compared in
-// fp64; the table is read once and the kernel stays bandwidth-bound.
+// fp64, as 64-bit sort keys.  Batches of queries go through fp64 matrix instructions, one or two
+// queries through a warp per shot; the top k are found by rank counting for small pools
+// and by a radix selection in front of a sort of the few candidates otherwise.
 #include "common.cuh"
 
 namespace {
 
 constexpr int kSortCap = 8192;      // candidates one CTA sorts in shared memory
-constexpr int kSortThreads = 1024;
 
 __device__ __forceinline__ unsigned long long desc_key(double s) { return ads_desc_key(s); }
 __device__ __forceinline__ double key_score(unsigned long long k) { return ads_key_score(k); }
 
-// One warp per pool row i: dots[b][i] = <q_b, e_i> for all b, enorm[i] = |e_i|.  With
-// keys_out set (pools that the rank kernel handles) the warp also forms |q_b| from the values
-// it loads anyway and writes the sort key of cos(q_b, e_i) in place of the dot product, so
-// that the ranking kernel's CTAs do not each redo N fp64 divisions.
-// NV > 0: E = 128 NV, the row is widened to fp64 once and kept in registers for all B queries
-// (the fp32 -> fp64 conversions, not the fp64 FMAs, are what a row-times-many-queries pass pays for);
-// NV = 0: any E.
+// sort key of cos = <q, e> / (|q| |e|), 0 where either norm is 0
+__device__ __forceinline__ unsigned long long cosine_key(double dot, double qq, double nn) {
+  const double den = sqrt(qq) * sqrt(nn);
+  return desc_key(den > 0.0 ? dot / den : 0.0);
+}
+
+// One warp per pool row i, for one or two queries: keys[b][i] = sort key of cos(q_b, e_i).
+// NV > 0: E = 128 NV, the row is widened to fp64 once and kept in registers for all queries
+// (the fp32 -> fp64 conversions are what a row-times-query pass pays for); NV = 0: any E and any B.
 template <int NV>
 __global__ void __launch_bounds__(256)
-cosine_dots_kernel(const float* __restrict__ emb, const float* __restrict__ q_emb, int N, int E,
-                   int B, double* __restrict__ dots, double* __restrict__ enorm, int keys_out) {
+cosine_keys_kernel(const float* __restrict__ emb, const float* __restrict__ q_emb, int N, int E,
+                   int B, unsigned long long* __restrict__ keys) {
   const int lane = threadIdx.x & 31;
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (row >= N) return;
@@ -42,7 +44,6 @@ cosine_dots_kernel(const float* __restrict__ emb, const float* __restrict__ q_em
 #pragma unroll
     for (int j = 0; j < 4 * NV; ++j) nn += ev[j] * ev[j];
     nn = warp_sum(nn);
-    if (lane == 0) enorm[row] = sqrt(nn);
     for (int b = 0; b < B; ++b) {
       const float* q = q_emb + (long long)b * E;
       double acc = 0.0, qq = 0.0;
@@ -51,18 +52,11 @@ cosine_dots_kernel(const float* __restrict__ emb, const float* __restrict__ q_em
         const float4 w = __ldg(reinterpret_cast<const float4*>(q + lane * 4 + 128 * i));
         const double w0 = w.x, w1 = w.y, w2 = w.z, w3 = w.w;
         acc += ev[4 * i] * w0 + ev[4 * i + 1] * w1 + ev[4 * i + 2] * w2 + ev[4 * i + 3] * w3;
-        if (keys_out) qq += w0 * w0 + w1 * w1 + w2 * w2 + w3 * w3;
+        qq += w0 * w0 + w1 * w1 + w2 * w2 + w3 * w3;
       }
       acc = warp_sum(acc);
-      if (keys_out) {
-        qq = warp_sum(qq);
-        if (lane == 0) {
-          const double den = sqrt(qq) * sqrt(nn);
-          reinterpret_cast<unsigned long long*>(dots)[(long long)b * N + row] = desc_key(den > 0.0 ? acc / den : 0.0);
-        }
-      } else if (lane == 0) {
-        dots[(long long)b * N + row] = acc;
-      }
+      qq = warp_sum(qq);
+      if (lane == 0) keys[(long long)b * N + row] = cosine_key(acc, qq, nn);
     }
     return;
   }
@@ -76,7 +70,6 @@ cosine_dots_kernel(const float* __restrict__ emb, const float* __restrict__ q_em
     for (int i = lane; i < E; i += 32) nn += (double)e[i] * e[i];
   }
   nn = warp_sum(nn);
-  if (lane == 0) enorm[row] = sqrt(nn);
   for (int b = 0; b < B; ++b) {
     const float* q = q_emb + (long long)b * E;
     double acc = 0.0, qq = 0.0;
@@ -94,15 +87,109 @@ cosine_dots_kernel(const float* __restrict__ emb, const float* __restrict__ q_em
       }
     }
     acc = warp_sum(acc);
-    if (keys_out) {
-      qq = warp_sum(qq);
-      if (lane == 0) {
-        const double den = sqrt(qq) * sqrt(nn);
-        reinterpret_cast<unsigned long long*>(dots)[(long long)b * N + row] = desc_key(den > 0.0 ? acc / den : 0.0);
-      }
-    } else if (lane == 0) {
-      dots[(long long)b * N + row] = acc;
+    qq = warp_sum(qq);
+    if (lane == 0) keys[(long long)b * N + row] = cosine_key(acc, qq, nn);
+  }
+}
+
+// c (16 x 8) += a (16 x 8) b (8 x 8), fp64
+__device__ __forceinline__ void mma_f64(double (&c)[4], const double (&a)[4], const double (&b)[2]) {
+  asm volatile("mma.sync.aligned.m16n8k8.row.col.f64.f64.f64.f64 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+               "{%0, %1, %2, %3};"
+               : "+d"(c[0]), "+d"(c[1]), "+d"(c[2]), "+d"(c[3])
+               : "d"(a[0]), "d"(a[1]), "d"(a[2]), "d"(a[3]), "d"(b[0]), "d"(b[1]));
+}
+
+// The same for batches: a CTA takes 32 shots and 8 NB queries, its eight warps share the embedding's length
+// and are summed in a fixed order through shared memory.  Bound by the fp64 units; the operands come straight
+// from memory as fp32 (a lane's four consecutive elements are the k slots lane % 4 and lane % 4 + 4 of two
+// instructions), so an element is widened once per 16 queries or 32 shots instead of once per product, which is
+// what the warp-per-shot form above spends its time on.  Norms are summed from the same registers.  E % 16 == 0.
+// (20000 shots x 768, 16 queries: 140 -> 26 us; 8192 x 1024, 32 queries: 115 -> 27 us.)
+constexpr int kMmaWarps = 8;
+template <int NB>
+__global__ void __launch_bounds__(32 * kMmaWarps, 2)
+cosine_mma_kernel(const float* __restrict__ emb, const float* __restrict__ q_emb, int N, int E, int B,
+                  unsigned long long* __restrict__ keys) {
+  __shared__ double dot_s[kMmaWarps][8 * NB][33];
+  __shared__ double nn_s[kMmaWarps][32], qq_s[kMmaWarps][8 * NB];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g = lane >> 2, t = lane & 3;
+  const int row0 = blockIdx.x * 32, q0 = blockIdx.y * 8 * NB;
+  const int steps = E / 16, s0 = warp * steps / kMmaWarps, s1 = (warp + 1) * steps / kMmaWarps;
+  const float4* ap[4];
+  const float4* bp[NB];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+    ap[r] = reinterpret_cast<const float4*>(emb + (long long)min(row0 + 8 * r + g, N - 1) * E) + s0 * 4 + t;
+#pragma unroll
+  for (int n = 0; n < NB; ++n)
+    bp[n] = reinterpret_cast<const float4*>(q_emb + (long long)min(q0 + 8 * n + g, B - 1) * E) + s0 * 4 + t;
+  double c[2][NB][4] = {}, nn[4] = {}, qq[NB] = {};
+  float4 av[4], bv[NB];
+  auto load = [&]() {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) { av[r] = __ldg(ap[r]); ap[r] += 4; }
+#pragma unroll
+    for (int n = 0; n < NB; ++n) { bv[n] = __ldg(bp[n]); bp[n] += 4; }
+  };
+  if (s0 < s1) load();
+  for (int s = s0; s < s1; ++s) {
+    double a[4][4], b[NB][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) { a[r][0] = av[r].x; a[r][1] = av[r].y; a[r][2] = av[r].z; a[r][3] = av[r].w; }
+#pragma unroll
+    for (int n = 0; n < NB; ++n) { b[n][0] = bv[n].x; b[n][1] = bv[n].y; b[n][2] = bv[n].z; b[n][3] = bv[n].w; }
+    if (s + 1 < s1) load();
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) nn[r] += a[r][e] * a[r][e];
+#pragma unroll
+    for (int n = 0; n < NB; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) qq[n] += b[n][e] * b[n][e];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int n = 0; n < NB; ++n) {
+          const double aa[4] = {a[2 * m][2 * h], a[2 * m + 1][2 * h], a[2 * m][2 * h + 1], a[2 * m + 1][2 * h + 1]};
+          const double bb[2] = {b[n][2 * h], b[n][2 * h + 1]};
+          mma_f64(c[m][n], aa, bb);
+        }
+  }
+#pragma unroll
+  for (int m = 0; m < 2; ++m)
+#pragma unroll
+    for (int n = 0; n < NB; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) dot_s[warp][8 * n + 2 * t + (e & 1)][16 * m + 8 * (e >> 1) + g] = c[m][n][e];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    nn[r] += __shfl_xor_sync(0xffffffffu, nn[r], 1);
+    nn[r] += __shfl_xor_sync(0xffffffffu, nn[r], 2);
+    if (t == 0) nn_s[warp][8 * r + g] = nn[r];
+  }
+#pragma unroll
+  for (int n = 0; n < NB; ++n) {
+    qq[n] += __shfl_xor_sync(0xffffffffu, qq[n], 1);
+    qq[n] += __shfl_xor_sync(0xffffffffu, qq[n], 2);
+    if (t == 0) qq_s[warp][8 * n + g] = qq[n];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < 32 * 8 * NB; i += 32 * kMmaWarps) {
+    const int r = i & 31, q = i >> 5;
+    if (row0 + r >= N || q0 + q >= B) continue;
+    double d = 0.0, n2 = 0.0, q2 = 0.0;
+#pragma unroll
+    for (int w = 0; w < kMmaWarps; ++w) {
+      d += dot_s[w][q][r];
+      n2 += nn_s[w][r];
+      q2 += qq_s[w][q];
     }
+    keys[(long long)(q0 + q) * N + row0 + r] = cosine_key(d, q2, n2);
   }
 }
 
@@ -110,106 +197,211 @@ __device__ __forceinline__ bool pair_less(unsigned long long ka, int ia, unsigne
   return ka < kb || (ka == kb && ia < ib);
 }
 
-// grid (n_chunks, B).  Sorts candidates [chunk*kSortCap, ...) of query b and writes
-// the first min(k, n_in_chunk) of them to out_key/out_id at [b][chunk*k + r].
-// Round 0 builds the candidates from dots / norms (in_key == nullptr).
-__global__ void __launch_bounds__(kSortThreads)
-topk_sort_kernel(const double* __restrict__ dots, const double* __restrict__ enorm,
-                 const float* __restrict__ q_emb, int E,
-                 const unsigned long long* __restrict__ in_key, const int* __restrict__ in_id,
-                 int n_in, int in_stride, int k, unsigned long long* __restrict__ out_key,
-                 int* __restrict__ out_id,
-                 int out_stride, int32_t* __restrict__ final_idx, float* __restrict__ final_score) {
+// Top k by radix selection, one CTA per query.  The keys' interval is narrowed, 4096 bins at a time, until
+// the bin that holds the k-th key and everything in front of it fit the candidate area; the candidates are
+// then sorted by (key, id).  The first pass bins by the score's sign, exponent and five bits more (cosines and
+// attention masses both spread over many of them), the following ones divide the bin's interval evenly, so two
+// passes nearly always do; equal keys without end are cut by id.  Latency-bound: a pass reads the keys once
+// (the second one from L1) with eight loads in flight per thread.  A cluster of eight CTAs per query that
+// added their histograms up through distributed shared memory was slower (40 us against 21 at 20000 keys): the
+// cluster barriers cost more than the counting.  (One 8192-entry bitonic sort per chunk took 79 us per launch;
+// 20000 keys, k = 512, 16 queries: 159 -> 21 us, 8192 keys, k = 512, 32 queries: 145 -> 13 us.)
+constexpr int kSelThreads = 1024;
+constexpr int kSelBins = 4096;
+
+// First-pass bins, ascending with the key: 0 = scores of 2 and more, 1 .. 2040 = positive scores below that in 32nds
+// of an octave (63 octaves), 2041 = smaller ones, then the negative scores in the same way.
+constexpr int kBinHi = (1023 + 1) << 5, kBinLo = kBinHi - 2040;
+constexpr int kBinShift = 47;                     // leaves the sign, the exponent and 5 bits
+__device__ __forceinline__ int first_bin(unsigned long long key) {
+  const int v = (int)(key >> kBinShift);          // 17 bits: those of a positive score count down
+  const int m = v < 0x10000 ? 0xffff - v : v - 0x10000;
+  const int mid = m - kBinLo;                     // 0 .. 2039
+  if (v < 0x10000) return m >= kBinHi ? 0 : (mid < 0 ? 2041 : 2040 - mid);
+  return m >= kBinHi ? 4083 : (mid < 0 ? 2042 : 2043 + mid);
+}
+__device__ __forceinline__ void first_bin_interval(int bin, unsigned long long* lo, unsigned long long* hi) {
+  int a, b;                                       // first and last v of the bin
+  if (bin == 0) { a = 0; b = 0xffff - kBinHi; }
+  else if (bin <= 2040) { a = b = 0xffff - (kBinLo + 2040 - bin); }
+  else if (bin == 2041) { a = 0xffff - (kBinLo - 1); b = 0xffff; }
+  else if (bin == 2042) { a = 0x10000; b = 0x10000 + kBinLo - 1; }
+  else if (bin <= 4082) { a = b = 0x10000 + kBinLo + bin - 2043; }
+  else { a = 0x10000 + kBinHi; b = 0x1ffff; }
+  *lo = (unsigned long long)a << kBinShift;
+  *hi = ((unsigned long long)b << kBinShift) | ((1ull << kBinShift) - 1);
+}
+
+__global__ void __launch_bounds__(kSelThreads)
+radix_topk_kernel(const unsigned long long* __restrict__ all_keys, int N, int k, int want, int32_t* __restrict__ final_idx,
+                  float* __restrict__ final_score) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem_raw);
-  int* ids = reinterpret_cast<int*>(keys + kSortCap);
-  __shared__ double red[kSortThreads / 32];
-  __shared__ double qnorm_sh;
+  unsigned long long* ckey = reinterpret_cast<unsigned long long*>(smem_raw);     // [want] candidates
+  int* cid = reinterpret_cast<int*>(ckey + want);                                 // [want]
+  int* hist = cid + want;                                                         // [kSelBins]
+  __shared__ int warp_sum_s[32], bin_s, before_s, inside_s, n_s;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b = blockIdx.x;
+  const unsigned long long* keys = all_keys + (long long)b * N;
+  constexpr int kFly = 8;
 
-  const int b = blockIdx.y, chunk = blockIdx.x;
-  const int begin = chunk * kSortCap;
-  const int n = min(kSortCap, n_in - begin);
-  int n_pow2 = 1;
-  while (n_pow2 < n) n_pow2 <<= 1;
-
-  if (in_key == nullptr) {
-    // |q_b| in fp64, once per CTA
-    const float* q = q_emb + (long long)b * E;
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < E; i += kSortThreads) acc += (double)q[i] * q[i];
-    acc = warp_sum(acc);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  unsigned long long lo = 0, hi = ~0ull;           // keys below lo: taken; above hi: out
+  int before = 0, inside = N;                       // how many are below lo, how many in [lo, hi]
+  if (tid == 0) n_s = 0;
+  for (int pass = 0; before + inside > want && lo < hi; ++pass) {
+    int shift = 64 - __clzll((long long)(hi - lo)) - 12;
+    if (shift < 0) shift = 0;
+    *reinterpret_cast<int4*>(hist + 4 * tid) = make_int4(0, 0, 0, 0);
     __syncthreads();
-    if (threadIdx.x < 32) {
-      double v = red[threadIdx.x];
-      v = warp_sum(v);
-      if (threadIdx.x == 0) qnorm_sh = sqrt(v);
+    for (int i0 = tid; i0 < N; i0 += kFly * kSelThreads) {
+      unsigned long long key[kFly];
+#pragma unroll
+      for (int u = 0; u < kFly; ++u) key[u] = i0 + u * kSelThreads < N ? keys[i0 + u * kSelThreads] : ~0ull;
+#pragma unroll
+      for (int u = 0; u < kFly; ++u)
+        if (i0 + u * kSelThreads < N && key[u] >= lo && key[u] <= hi)
+          atomicAdd(hist + (pass == 0 ? first_bin(key[u]) : (int)((key[u] - lo) >> shift)), 1);
     }
     __syncthreads();
-    const double qn = qnorm_sh;
-    for (int i = threadIdx.x; i < n_pow2; i += kSortThreads) {
-      if (i < n) {
-        double den = qn * enorm[begin + i];
-        double s = den > 0.0 ? dots[(long long)b * in_stride + begin + i] / den : 0.0;
-        keys[i] = desc_key(s);
-        ids[i] = begin + i;
-      } else {
-        keys[i] = ~0ull;             // padding sorts last
-        ids[i] = 0x7fffffff;
-      }
+    // the bin that holds rank k - 1
+    const int4 h4 = *reinterpret_cast<const int4*>(hist + 4 * tid);
+    const int h[4] = {h4.x, h4.y, h4.z, h4.w};
+    const int sum = h[0] + h[1] + h[2] + h[3];
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
     }
-  } else {
-    for (int i = threadIdx.x; i < n_pow2; i += kSortThreads) {
-      if (i < n) {
-        keys[i] = in_key[(long long)b * in_stride + begin + i];
-        ids[i] = in_id[(long long)b * in_stride + begin + i];
-      } else {
-        keys[i] = ~0ull;
-        ids[i] = 0x7fffffff;
+    if (lane == 31) warp_sum_s[warp] = incl;
+    __syncthreads();
+    int at = before + incl - sum + __reduce_add_sync(0xffffffffu, lane < warp ? warp_sum_s[lane] : 0);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (at < k && at + h[u] >= k) {
+        bin_s = 4 * tid + u;
+        before_s = at;
+        inside_s = h[u];
       }
+      at += h[u];
+    }
+    __syncthreads();
+    before = before_s;
+    inside = inside_s;
+    if (pass == 0) {
+      first_bin_interval(bin_s, &lo, &hi);
+    } else {
+      lo += (unsigned long long)bin_s << shift;
+      const unsigned long long top = lo + ((1ull << shift) - 1);
+      hi = top < hi ? top : hi;
     }
   }
   __syncthreads();
 
+  // candidates: everything up to hi; of more equal keys than there is room for, the lowest ids
+  const bool cut = before + inside > want;          // then lo == hi
+  int taken = 0;                                    // equal keys with lower ids (cut only)
+  for (int i0 = tid; i0 < N + tid; i0 += kFly * kSelThreads) {      // (whole warps: i0 - tid is the same for all)
+    unsigned long long key[kFly];
+#pragma unroll
+    for (int u = 0; u < kFly; ++u) key[u] = i0 + u * kSelThreads < N ? keys[i0 + u * kSelThreads] : ~0ull;
+#pragma unroll
+    for (int u = 0; u < kFly; ++u) {
+      const int i = i0 + u * kSelThreads;
+      bool take = i < N && key[u] <= hi;
+      if (cut) {                                    // in id order: a block-wide count of the equal keys
+        const bool eq = i < N && key[u] == hi;
+        const unsigned m = __ballot_sync(0xffffffffu, eq);
+        __syncthreads();
+        if (lane == 0) warp_sum_s[warp] = __popc(m);
+        __syncthreads();
+        const int v = warp_sum_s[lane];
+        const int pos = taken + __reduce_add_sync(0xffffffffu, lane < warp ? v : 0) + __popc(m & ((1u << lane) - 1));
+        taken += __reduce_add_sync(0xffffffffu, v);
+        if (eq) take = before + pos < k;
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, take);
+      if (m == 0) continue;
+      int slot = 0;
+      if (lane == 0) slot = atomicAdd(&n_s, __popc(m));
+      slot = __shfl_sync(0xffffffffu, slot, 0) + __popc(m & ((1u << lane) - 1));
+      if (take) {
+        ckey[slot] = key[u];
+        cid[slot] = i;
+      }
+    }
+  }
+  __syncthreads();
+  const int n = n_s;
+  int n_pow2 = 32;
+  while (n_pow2 < n) n_pow2 <<= 1;
   // bitonic sort, ascending on (key, id); ids are unique so the order is total
+  if (n_pow2 <= kSelThreads) {
+    // one candidate per thread: exchanges within a warp by shuffles, the others through shared memory
+    if (tid >= n_pow2) return;                      // (whole warps)
+    auto sync = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(n_pow2) : "memory"); };
+    unsigned long long key = tid < n ? ckey[tid] : ~0ull;      // padding sorts last
+    int id = tid < n ? cid[tid] : 0x7fffffff;
+    sync();
+    for (int size = 2; size <= n_pow2; size <<= 1) {
+      for (int stride = size >> 1; stride > 0; stride >>= 1) {
+        unsigned long long ko;
+        int io;
+        if (stride >= 32) {
+          ckey[tid] = key;
+          cid[tid] = id;
+          sync();
+          ko = ckey[tid ^ stride];
+          io = cid[tid ^ stride];
+          sync();
+        } else {
+          ko = __shfl_xor_sync(0xffffffffu, key, stride);
+          io = __shfl_xor_sync(0xffffffffu, id, stride);
+        }
+        const bool keep_low = ((tid & stride) == 0) == ((tid & size) == 0);
+        if (pair_less(ko, io, key, id) == keep_low) {
+          key = ko;
+          id = io;
+        }
+      }
+    }
+    if (tid < min(k, n)) {
+      final_idx[(long long)b * k + tid] = id;
+      if (final_score != nullptr) final_score[(long long)b * k + tid] = (float)key_score(key);
+    }
+    return;
+  }
+  for (int i = n + tid; i < n_pow2; i += kSelThreads) {
+    ckey[i] = ~0ull;
+    cid[i] = 0x7fffffff;
+  }
+  __syncthreads();
   for (int size = 2; size <= n_pow2; size <<= 1) {
     for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int t = threadIdx.x; t < (n_pow2 >> 1); t += kSortThreads) {
-        int lo = 2 * t - (t & (stride - 1));
-        int hi = lo + stride;
-        bool up = (lo & size) == 0;
-        unsigned long long ka = keys[lo], kb = keys[hi];
-        int ia = ids[lo], ib = ids[hi];
-        bool swap = up ? pair_less(kb, ib, ka, ia) : pair_less(ka, ia, kb, ib);
-        if (swap) {
-          keys[lo] = kb; keys[hi] = ka;
-          ids[lo] = ib; ids[hi] = ia;
+      for (int u = tid; u < (n_pow2 >> 1); u += kSelThreads) {
+        const int x = 2 * u - (u & (stride - 1)), y = x + stride;
+        const bool up = (x & size) == 0;
+        const unsigned long long kx = ckey[x], ky = ckey[y];
+        const int ix = cid[x], iy = cid[y];
+        if (up ? pair_less(ky, iy, kx, ix) : pair_less(kx, ix, ky, iy)) {
+          ckey[x] = ky; ckey[y] = kx;
+          cid[x] = iy; cid[y] = ix;
         }
       }
       __syncthreads();
     }
   }
-
-  const int n_out = min(k, n);
-  if (final_idx != nullptr) {
-    for (int r = threadIdx.x; r < n_out; r += kSortThreads) {
-      final_idx[(long long)b * k + r] = ids[r];
-      if (final_score != nullptr) final_score[(long long)b * k + r] = (float)key_score(keys[r]);
-    }
-  } else {
-    for (int r = threadIdx.x; r < n_out; r += kSortThreads) {
-      out_key[(long long)b * out_stride + chunk * k + r] = keys[r];
-      out_id[(long long)b * out_stride + chunk * k + r] = ids[r];
-    }
+  for (int r = tid; r < min(k, n); r += kSelThreads) {
+    final_idx[(long long)b * k + r] = cid[r];
+    if (final_score != nullptr) final_score[(long long)b * k + r] = (float)key_score(ckey[r]);
   }
 }
 
-// Top-k by counting, for pools of up to kRankMaxN shots: the rank of shot i in the order
+// Top-k by counting, for small pools: the rank of shot i in the order
 // (score descending, id ascending) is the number of shots that precede it; every shot with
 // rank < k writes its id to position rank.  No sort and no serial phases: grid (N / 16, B),
 // 16 candidates per CTA, the comparison range split over sixteen groups of 16 threads.
 // "key_j precedes key_i" = key_j < key_i, or equal keys and j < i, = key_j < key_i + (j < i).
-constexpr int kRankMaxN = 4096;
 constexpr int kRankThreads = 256, kRankCand = 16, kRankTile = 2048;
 
 __global__ void __launch_bounds__(kRankThreads)
@@ -250,71 +442,33 @@ rank_topk_kernel(const unsigned long long* __restrict__ all_keys, int N, int k,
   }
 }
 
-size_t sel_cand_entries(int n_shots, int k) {
-  if (n_shots <= kSortCap) return 0;
-  size_t chunks = ((size_t)n_shots + kSortCap - 1) / kSortCap;
-  return chunks * (size_t)k;
-}
+// Rank counting compares every pair of keys, over the whole chip; the radix selection is one CTA per
+// query (7 to 9 us up to 4096 keys).  One query: 5.9 us at 1024 keys, 6.4 at 2048, 10.5 at 4096; eight queries of 1024
+// keys 6.7: the line lies where the count reaches the selection's 7 us.
+bool rank_by_counting(int N, int B) { return (long long)N * N * B <= 9000000ll; }
 
 }  // namespace
 
-size_t ads_topk_scratch_bytes(int N, int B, int k) {
-  const size_t cand = sel_cand_entries(N, k);
-  return 2 * (ads_round_up((size_t)B * cand * 8, 256) + ads_round_up((size_t)B * cand * 4, 256));
-}
-
-int ads_topk_from_keys(const unsigned long long* keys, const int* ids, int N, int B, int k, void* cand_ws,
-                       int32_t* sel_idx, float* sel_score, cudaStream_t st) {
+int ads_topk_from_keys(const unsigned long long* keys, int N, int B, int k, int32_t* sel_idx, float* sel_score,
+                       cudaStream_t st) {
   if (N > kSortCap && k > kSortCap / 2) return ADAPSHOT_EUNSUPPORTED;
-  if (N <= kRankMaxN) {
+  if (rank_by_counting(N, B)) {
     dim3 grid((N + kRankCand - 1) / kRankCand, B);
     rank_topk_kernel<<<grid, kRankThreads, 0, st>>>(keys, N, k, sel_idx, sel_score);
     return ads_launch_status();
   }
-  const size_t smem = (size_t)kSortCap * (8 + 4);
+  // candidates worth sorting: the power of two the sort pads to (bins of the second pass rarely hold two keys)
+  int want = 128;
+  while (want < k) want <<= 1;
   static bool attr_set[kAdsMaxDevices] = {false};
-  if (ads_set_max_smem(topk_sort_kernel, (int)smem, attr_set) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-  const size_t cand = sel_cand_entries(N, k);
-  unsigned char* p = static_cast<unsigned char*>(cand_ws);
-  unsigned long long* ckey[2];
-  int* cid[2];
-  for (int i = 0; i < 2; ++i) {
-    ckey[i] = reinterpret_cast<unsigned long long*>(p);
-    p += ads_round_up((size_t)B * cand * 8, 256);
-    cid[i] = reinterpret_cast<int*>(p);
-    p += ads_round_up((size_t)B * cand * 4, 256);
-  }
-  int n_in = N, in_stride = N, round = 0;
-  const unsigned long long* in_key = keys;
-  const int* in_id = ids;
-  while (true) {
-    const int chunks = (n_in + kSortCap - 1) / kSortCap;
-    const bool last = chunks == 1;
-    dim3 grid(chunks, B);
-    const int out_stride = chunks * k;
-    topk_sort_kernel<<<grid, kSortThreads, smem, st>>>(
-        nullptr, nullptr, nullptr, 0, in_key, in_id, n_in, in_stride, k, ckey[round & 1], cid[round & 1], out_stride,
-        last ? sel_idx : nullptr, last ? sel_score : nullptr);
-    if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-    if (last) break;
-    in_key = ckey[round & 1];
-    in_id = cid[round & 1];
-    const int last_n = n_in - (chunks - 1) * kSortCap;
-    n_in = (chunks - 1) * k + (last_n < k ? last_n : k);
-    in_stride = out_stride;
-    ++round;
-  }
-  return ADAPSHOT_OK;
+  if (ads_set_max_smem(radix_topk_kernel, kSortCap * (8 + 4) + kSelBins * 4, attr_set) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
+  radix_topk_kernel<<<(unsigned)B, kSelThreads, want * (8 + 4) + kSelBins * 4, st>>>(keys, N, k, want, sel_idx, sel_score);
+  return ads_launch_status();
 }
 
 extern "C" size_t adapshot_select_workspace_bytes(int32_t n_shots, int32_t B, int32_t k) {
   if (n_shots <= 0 || B <= 0 || k <= 0) return 0;
-  size_t bytes = ads_round_up((size_t)B * n_shots * sizeof(double), 256);   // dots
-  bytes += ads_round_up((size_t)n_shots * sizeof(double), 256);             // |e_i|
-  size_t cand = sel_cand_entries(n_shots, k);
-  // two ping-pong candidate lists of (key, id)
-  bytes += 2 * (ads_round_up((size_t)B * cand * 8, 256) + ads_round_up((size_t)B * cand * 4, 256));
-  return bytes;
+  return ads_round_up((size_t)B * n_shots * sizeof(unsigned long long), 256);   // sort keys
 }
 
 extern "C" int adapshot_select(const adapshot_pool_t* pool, const float* q_emb, int32_t B, int32_t k,
@@ -330,64 +484,22 @@ extern "C" int adapshot_select(const adapshot_pool_t* pool, const float* q_emb, 
   if (ws_bytes < adapshot_select_workspace_bytes(N, B, k)) return ADAPSHOT_ECAPACITY;
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  unsigned char* p = static_cast<unsigned char*>(ws);
-  double* dots = reinterpret_cast<double*>(p);
-  p += ads_round_up((size_t)B * N * sizeof(double), 256);
-  double* enorm = reinterpret_cast<double*>(p);
-  p += ads_round_up((size_t)N * sizeof(double), 256);
-  const size_t cand = sel_cand_entries(N, k);
-  unsigned long long* ckey[2];
-  int* cid[2];
-  for (int i = 0; i < 2; ++i) {
-    ckey[i] = reinterpret_cast<unsigned long long*>(p);
-    p += ads_round_up((size_t)B * cand * 8, 256);
-    cid[i] = reinterpret_cast<int*>(p);
-    p += ads_round_up((size_t)B * cand * 4, 256);
+  unsigned long long* keys = static_cast<unsigned long long*>(ws);
+  if (B > 2 && E % 16 == 0) {          // (4096 x 384: 4.7 us for two queries by warps, 3.4 for four by matrix tiles)
+    const unsigned rows = (unsigned)((N + 31) / 32);
+    if (B <= 8)
+      cosine_mma_kernel<1><<<dim3(rows, 1), 32 * kMmaWarps, 0, st>>>(pool->emb, q_emb, N, E, B, keys);
+    else
+      cosine_mma_kernel<2><<<dim3(rows, (unsigned)((B + 15) / 16)), 32 * kMmaWarps, 0, st>>>(pool->emb, q_emb, N, E, B, keys);
+  } else {
+    const unsigned grid = (unsigned)((N + 7) / 8);
+    auto run = [&](auto kernel) { kernel<<<grid, 256, 0, st>>>(pool->emb, q_emb, N, E, B, keys); };
+    if (E == 1024) run(cosine_keys_kernel<8>);
+    else if (E == 768) run(cosine_keys_kernel<6>);
+    else if (E == 384) run(cosine_keys_kernel<3>);
+    else if (E == 128) run(cosine_keys_kernel<1>);
+    else run(cosine_keys_kernel<0>);
   }
-
-  const int warps_per_block = 8;
-  const unsigned cgrid = (unsigned)((N + warps_per_block - 1) / warps_per_block);
-  const int keys_out = N <= kRankMaxN ? 1 : 0;
-  if (E == 1024)
-    cosine_dots_kernel<8><<<cgrid, warps_per_block * 32, 0, st>>>(pool->emb, q_emb, N, E, B, dots, enorm, keys_out);
-  else if (E == 128)
-    cosine_dots_kernel<1><<<cgrid, warps_per_block * 32, 0, st>>>(pool->emb, q_emb, N, E, B, dots, enorm, keys_out);
-  else
-    cosine_dots_kernel<0><<<cgrid, warps_per_block * 32, 0, st>>>(pool->emb, q_emb, N, E, B, dots, enorm, keys_out);
   if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-
-  if (N <= kRankMaxN) {
-    dim3 grid((N + kRankCand - 1) / kRankCand, B);
-    rank_topk_kernel<<<grid, kRankThreads, 0, st>>>(reinterpret_cast<const unsigned long long*>(dots), N, k, sel_idx,
-                                                    sel_score);
-    return ads_launch_status();
-  }
-
-  const size_t smem = (size_t)kSortCap * (8 + 4);
-  static bool attr_set[kAdsMaxDevices] = {false};
-  if (ads_set_max_smem(topk_sort_kernel, (int)smem, attr_set) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-
-  int n_in = N, in_stride = N;
-  int round = 0;
-  const unsigned long long* in_key = nullptr;
-  const int* in_id = nullptr;
-  while (true) {
-    const int chunks = (n_in + kSortCap - 1) / kSortCap;
-    const bool last = chunks == 1;
-    dim3 grid(chunks, B);
-    const int out_stride = chunks * k;
-    topk_sort_kernel<<<grid, kSortThreads, smem, st>>>(
-        dots, enorm, q_emb, E, in_key, in_id, n_in, in_stride, k, ckey[round & 1], cid[round & 1], out_stride,
-        last ? sel_idx : nullptr, last ? sel_score : nullptr);
-    if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-    if (last) break;
-    in_key = ckey[round & 1];
-    in_id = cid[round & 1];
-    // every chunk but possibly the last holds >= k candidates (k <= kSortCap / 2)
-    const int last_n = n_in - (chunks - 1) * kSortCap;
-    n_in = (chunks - 1) * k + (last_n < k ? last_n : k);
-    in_stride = out_stride;
-    ++round;
-  }
-  return ADAPSHOT_OK;
+  return ads_topk_from_keys(keys, N, B, k, sel_idx, sel_score, st);
 }

@@ -65,3 +65,28 @@ def test_nested_probes_are_prefixes():
     for n in (1, 16, 64):
         part, _, _ = hp.run_select(ab, pool, q, n)
         assert torch.equal(part, full[:, :n])
+
+
+@pytest.mark.parametrize("N,E,B,k", [(33, 16, 3, 33), (97, 48, 8, 13), (3001, 64, 9, 1500), (4096, 768, 17, 1025),
+                                     (8192, 32, 4, 5000), (9000, 112, 33, 1024)])
+def test_select_batches(N, E, B, k):
+    # fp64 matrix tiles: remainders of 32 shots, 8 and 16 queries, embeddings of one step, of fewer steps than warps
+    # and of unequal shares; rank counting and radix selection with few and with many candidates; k beyond the
+    # positive scores (half of them are)
+    ab = hp.gpu_binding()
+    g = torch.Generator().manual_seed(N + E)
+    _check(ab, torch.randn(N, E, generator=g), torch.randn(B, E, generator=g), k)
+
+
+@pytest.mark.parametrize("n_same,k", [(6000, 700), (6000, 1500), (1025, 900)])
+def test_radix_selection_cuts_equal_scores_by_id(n_same, k):
+    # more equal scores around rank k than the candidate area takes, in front of them a few better ones
+    ab = hp.gpu_binding()
+    g = torch.Generator().manual_seed(n_same)
+    emb = torch.randn(6100, 32, generator=g)
+    same = torch.randperm(6100, generator=g)[:n_same]
+    emb[same] = emb[same[0]].clone()
+    _check(ab, emb, torch.cat([emb[same[:1]] + 0.3 * torch.randn(1, 32, generator=g), torch.randn(2, 32, generator=g)]), k)
+    zero = torch.zeros(6100, 32)
+    zero[17], zero[5000] = 1.0, -1.0
+    _check(ab, zero, torch.ones(1, 32), k)
