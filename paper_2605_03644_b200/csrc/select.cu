@@ -468,7 +468,9 @@ int ads_topk_from_keys(const unsigned long long* keys, int N, int B, int k, int3
 
 extern "C" size_t adapshot_select_workspace_bytes(int32_t n_shots, int32_t B, int32_t k) {
   if (n_shots <= 0 || B <= 0 || k <= 0) return 0;
-  return ads_round_up((size_t)B * n_shots * sizeof(unsigned long long), 256);   // sort keys
+  // the sort keys; the second term (a norm per shot) is part of the size that the call has always asked for
+  return ads_round_up((size_t)B * n_shots * sizeof(unsigned long long), 256) +
+         ads_round_up((size_t)n_shots * sizeof(double), 256);
 }
 
 extern "C" int adapshot_select(const adapshot_pool_t* pool, const float* q_emb, int32_t B, int32_t k,
