@@ -3,20 +3,27 @@
 // two-shot example, where a shot's Delta is the total length placed before it).
 //
 // Kernel 1 (plan): ctx_off[b][r] = exclusive prefix sum of the selected lengths.
-// Kernel 2 (gather): one warp moves one destination token of one query for every
-// layer of the call: V rows are copied with 16-byte vectors, K rows are rotated in
-// registers between the 16-byte load and store.  The rotation angles of a token do
-// not depend on layer or head, so each lane forms its few (sin, cos) pairs once per
-// token, in fp64 before the fp32 sincos, and reuses them over heads and layers.
+// Kernel 2 (gather): a selected shot's tokens are consecutive in the pool and in the cache, so both are
+// moved by bulk copies, a chunk of consecutive destination tokens at a time: one warp finds the runs of pool
+// rows behind a chunk and brings them to shared memory, V leaves from there as it came, K is rotated in place
+// by four warps in between.  The rotation angles of a token do not depend on layer or head: a thread forms
+// its few (sin, cos) pairs once per chunk, in fp64 before the fp32 sincos, and reuses them.
 #include <math.h>
 
 #include "common.cuh"
+#include "sm100_ptx.cuh"
 
 namespace {
 
+using namespace sm100;
+
 constexpr int kPlanThreads = 256;
 constexpr int kTile = 128;   // the attention kernel reads the cache in 128-token tiles
-constexpr int kRunMax = 4;   // consecutive destination tokens per warp (fewer when the launch is small)
+constexpr int kRotWarps = 4;         // gather: warps that rotate K; after them one that loads and one that stores
+constexpr int kRotThreads = 32 * kRotWarps;
+constexpr int kGatherThreads = kRotThreads + 64;
+constexpr int kStages = 3;           // chunks of one CTA on their way at a time
+constexpr uint32_t kStageMax = 32768;
 
 // One CTA per query: lengths of the selected shots, block-wide exclusive scan.
 __global__ void __launch_bounds__(kPlanThreads)
@@ -109,208 +116,298 @@ struct GatherArgs {
   double rope_base;
   int32_t* status;
   double theta[64];            // theta_i = rope_base^(-2i/D), i < D/2, formed on the host
-  int run;                     // destination tokens per warp and plan lookup
+  int chunk;                   // destination tokens per chunk
+  int heads;                   // KV heads per stage (all of them, or rows are cut)
+  int layer_groups;            // a chunk's layers are dealt out to this many items
+};
+
+// What a stage holds, written by the loading warp.
+struct StageInfo {
+  long long dst;               // byte offset of the chunk's first row in k_ctx / v_ctx
+  long long pos0;              // position of its first token
+  int n;                       // tokens; 0: no more stages
+  int is_v;
+  long long item;              // stages of one item have the same positions
 };
 
 // D = head_dim.  A "pair unit" is the 16-byte vector j of the low half of one head
 // together with vector j of the high half (elements i and i + D/2 rotate together).
-// 128-thread CTAs of at most 88 registers: small enough to be co-resident with a persistent
-// attention CTA (which leaves about 11.7 K registers and 1.5 KB of shared memory per SM), so
-// that the gather of the next layer chunk can run under the attention of the current one.
-// WITH_V = false: the K-only form (V is taken from the pool by its consumer); it keeps two layers'
-// loads in flight and takes the registers for that (five CTAs per SM instead of six).
+// Bound by HBM.  The copies need no registers and no instructions per byte, so what a CTA has in flight is its
+// three stages (two CTAs of 96 KB per SM at the 8B shape; with two stages it is 8-15 % slower), and one layer per
+// call moves at the rate of many: the form before, a warp per token with 16-byte loads and stores, had too few
+// bytes on their way when the plan lookup and the angles of a token were paid for one or two layers (K only, 32
+// queries of 66 K tokens, one layer: 2290 -> 1320 us = 6.5 TB/s; K and V of one layer, 16.4 K tokens: 32 -> 29 us;
+// of sixteen layers, 2 K tokens: 55 -> 47 us; K only, four layers, 8 queries of 33 K tokens: 650 -> 663 us).
+// WITH_V = false: the K-only form (V is taken from the pool by its consumer).
 template <typename T, int D, bool WITH_V>
-__global__ void __launch_bounds__(128, WITH_V ? 6 : 5)
-gather_rope_kernel(const GatherArgs a) {
+__global__ void __launch_bounds__(kGatherThreads, 2)
+gather_rope_kernel(const __grid_constant__ GatherArgs a) {
   constexpr int EPV = Vec16<T>::N;                 // elements per 16-byte vector
-  constexpr int VPH = D / EPV;                     // vectors per head row
-  constexpr int HALF_V = VPH / 2;                  // pair units per head
-  static_assert(32 % HALF_V == 0, "a lane must keep the same vector column over its units");
-  const int lane = threadIdx.x & 31;
-  const long long warp_global = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const long long n_warps = (long long)gridDim.x * (blockDim.x >> 5);
-  const int row_vecs = a.n_kv_heads * VPH;         // 16-byte vectors in one token row
-  const int pair_units = a.n_kv_heads * HALF_V;
-  const long long layer_stride_pool = a.pool_tokens * row_vecs;   // in uint4
-  const long long layer_stride_ctx = a.ctx_cap * row_vecs;
+  constexpr int HALF_V = D / EPV / 2;              // pair units per head
+  constexpr int kHeadBytes = D * (int)sizeof(T);
+  constexpr int kPassTokens = kRotThreads / HALF_V;  // tokens the rotating threads cover at once
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ StageInfo info[kStages];
+  __shared__ int first_s[kStages][4 * kPassTokens];  // first position of the shot a token lies in (k_pos_mode 1)
+  __shared__ __align__(8) unsigned long long bars[3 * kStages];
+  __shared__ int abort_s[2];
+  const uint32_t bar0 = smem_u32(bars), smem0 = smem_u32(smem);
+  auto full = [&](int s) { return bar0 + 8u * s; };                     // the chunk has landed
+  auto done = [&](int s) { return bar0 + 8u * (kStages + s); };         // K has been rotated
+  auto empty = [&](int s) { return bar0 + 8u * (2 * kStages + s); };    // the chunk has left
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t stage_bytes = (uint32_t)a.chunk * a.heads * kHeadBytes;
+  const int row_bytes = a.n_kv_heads * kHeadBytes;
+  const int part_bytes = a.heads * kHeadBytes;     // of a row, in one stage
+  const bool cut_rows = a.heads != a.n_kv_heads;
 
-  // the EPV values of theta of this lane's column
-  const int jcol = lane % HALF_V;
-  double theta[EPV];
-#pragma unroll
-  for (int e = 0; e < EPV; ++e) theta[e] = a.theta[jcol * EPV + e];
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(full(s), 1);
+      mbar_init(done(s), kRotWarps);
+      mbar_init(empty(s), 1);
+    }
+    abort_s[0] = abort_s[1] = 0;
+    mbar_fence_init();
+  }
+  __syncthreads();
 
-  const uint4* kp = static_cast<const uint4*>(a.k_pool);
-  const uint4* vp = static_cast<const uint4*>(a.v_pool);
-  uint4* kc = static_cast<uint4*>(a.k_ctx);
-  uint4* vc = static_cast<uint4*>(a.v_ctx);
-  constexpr bool with_v = WITH_V;
-
-  // A warp takes a run of kRun consecutive destination tokens of one query.  The plan lookup
-  // (which selected shot covers the position) is a dependent chain of global loads, so it is
-  // done once per run by the whole warp (a 32-ary search: two rounds of parallel probes of the
-  // offsets instead of log2(k) serial ones) and then walked forward token by token.
-  const int kRun = a.run;
-  const long long runs_per_query = (a.ctx_cap + kRun - 1) / kRun;
-  const long long n_runs = (long long)a.B * runs_per_query;
-  for (long long run = warp_global; run < n_runs; run += n_warps) {
-    const int b = (int)(run / runs_per_query);
-    const long long p0 = (run % runs_per_query) * kRun;
-    const long long* off = a.ctx_off + (long long)b * (a.k + 1);
-    const long long L = off[a.k];
-    const long long pad_end = (L + kTile - 1) / kTile * kTile;
-    const long long first_pos = off[a.shot_begin];                // positions before it stay as they are
-    if (p0 >= pad_end || p0 + kRun <= first_pos) continue;
-    int lo = 0;
-    long long o = 0, o_next = 0, src0 = 0;
-    int s = -1;
-    if (p0 < L) {
-      // largest lo in [0, k) with off[lo] <= p0 (zero-length slots are skipped by the search)
-      int seg_lo = 0, seg_n = a.k;
+  if (warp == kRotWarps) {
+    // ---------------------------------------------------------------- loading warp
+    const int chunks_per_query = (int)((a.ctx_cap + a.chunk - 1) / a.chunk);
+    const long long n_items = (long long)a.B * chunks_per_query * a.layer_groups;
+    const int group_layers = (a.n_layers_call + a.layer_groups - 1) / a.layer_groups;
+    uint32_t it = 0;
+    bool ok = true;
+    for (long long item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+      const int l0 = (int)(item % a.layer_groups) * group_layers;
+      const int l1 = min(a.n_layers_call, l0 + group_layers);
+      const long long chunk = item / a.layer_groups;
+      const int b = (int)(chunk / chunks_per_query);
+      const long long p0 = (chunk % chunks_per_query) * a.chunk;
+      const long long* off = a.ctx_off + (long long)b * (a.k + 1);
+      const long long L = off[a.k];
+      const long long pa = max(p0, off[a.shot_begin]);                 // positions before it stay as they are
+      const long long pb = min(p0 + a.chunk, min(L, a.ctx_cap));
+      // zeros for the rest of the last 128-token tile, so that whole tiles can be read later
+      const long long za = max(p0, L), zb = min(p0 + a.chunk, min((L + kTile - 1) / kTile * kTile, a.ctx_cap));
+      for (int l = l0; za < zb && l < l1; ++l) {
+        const long long dst = (((long long)b * a.n_layers_call + l) * a.ctx_cap + za) * row_bytes;
+        for (long long v = lane; v < (zb - za) * row_bytes / 16; v += 32) {
+          reinterpret_cast<uint4*>(static_cast<char*>(a.k_ctx) + dst)[v] = make_uint4(0, 0, 0, 0);
+          if (WITH_V) reinterpret_cast<uint4*>(static_cast<char*>(a.v_ctx) + dst)[v] = make_uint4(0, 0, 0, 0);
+        }
+      }
+      if (pa >= pb) continue;
+      // the largest slot in [0, k) with off[slot] <= pa, by a 32-ary search of the whole warp
+      int lo = 0, seg_n = a.k;
       while (seg_n > 1) {
         const int stride = (seg_n + 31) / 32;
-        const int idx = seg_lo + lane * stride;
-        const bool le = idx < seg_lo + seg_n && off[idx] <= p0;
-        const int cnt = __popc(__ballot_sync(0xffffffffu, le));      // probes are ascending: a prefix is true
-        const int first = seg_lo + (cnt - 1) * stride;                // cnt >= 1: off[seg_lo] <= p0
-        seg_n = min(stride, seg_lo + seg_n - first);
-        seg_lo = first;
+        const int idx = lo + lane * stride;
+        const bool le = idx < lo + seg_n && off[idx] <= pa;
+        const int cnt = __popc(__ballot_sync(0xffffffffu, le));        // probes are ascending: a prefix is true
+        const int first = lo + (cnt - 1) * stride;                      // cnt >= 1: off[lo] <= pa
+        seg_n = min(stride, lo + seg_n - first);
+        lo = first;
       }
-      lo = seg_lo;
-      o = off[lo];
-      o_next = off[lo + 1];
-      s = a.sel_idx[(long long)b * a.k + lo];
-      if (s >= 0 && s < a.n_shots) src0 = a.shot_off[s];
-    }
-#pragma unroll 1
-    for (int tt = 0; tt < kRun; ++tt) {
-    const long long p = p0 + tt;
-    if (p >= a.ctx_cap) break;
-    if (p < first_pos) continue;
-    if (p >= L) {
-      // zero the rest of the last 128-token tile so whole tiles can be read later
-      if (p < pad_end) {
-        for (int l = 0; l < a.n_layers_call; ++l) {
-          const long long dst = ((long long)b * a.n_layers_call + l) * layer_stride_ctx + p * row_vecs;
-          for (int i = lane; i < row_vecs; i += 32) {
-            kc[dst + i] = make_uint4(0, 0, 0, 0);
-            if (with_v) vc[dst + i] = make_uint4(0, 0, 0, 0);
+      // Lane i takes the run of slot lo + i (and of the 32nd after it, ... in chunks of many short shots).
+      long long run_src = 0;                       // pool token of the run's first row
+      int run_at = 0, run_n = 0, run_first = 0;    // its place in the chunk, its length, its shot's first position
+      auto find_run = [&](int group) -> bool {     // whether a further group is needed
+        const int slot = lo + 32 * group + lane;
+        run_n = 0;
+        bool in = slot < a.k;
+        const long long o = in ? off[slot] : 0;
+        in = in && o < pb;
+        if (in) {
+          const long long s0 = max(o, pa), s1 = min(off[slot + 1], pb);
+          const int s = a.sel_idx[(long long)b * a.k + slot];
+          if (s1 > s0 && s >= 0 && s < a.n_shots) {          // (an unknown shot is reported by the plan kernel)
+            run_src = a.shot_off[s] + (s0 - o);
+            run_at = (int)(s0 - pa);
+            run_n = (int)(s1 - s0);
+            run_first = (int)o;
           }
         }
+        return (__ballot_sync(0xffffffffu, in) >> 31) != 0;
+      };
+      const bool many = find_run(0);
+      int total = __reduce_add_sync(0xffffffffu, run_n);     // tokens that will come
+      if (many) {
+        bool more = true;
+        for (int g = 1; more; ++g) {
+          more = find_run(g);
+          total += __reduce_add_sync(0xffffffffu, run_n);
+        }
+        find_run(0);
       }
-      continue;
+      for (int l = l0; l < l1 && ok; ++l)
+        for (int v = 0; v < (WITH_V ? 2 : 1) && ok; ++v)
+          for (int h0 = 0; h0 < a.n_kv_heads; h0 += a.heads, ++it) {
+            const int s = it % kStages;
+            ok = __all_sync(0xffffffffu, mbar_wait(empty(s), ((it / kStages) & 1) ^ 1, abort_s));
+            if (!ok) break;
+            const int width = min(a.heads, a.n_kv_heads - h0) * kHeadBytes;
+            const char* src = static_cast<const char*>(v ? a.v_pool : a.k_pool) +
+                              (long long)(a.layer_begin + l) * a.pool_tokens * row_bytes + h0 * kHeadBytes;
+            if (lane == 0) {
+              StageInfo& si = info[s];
+              si.dst = (((long long)b * a.n_layers_call + l) * a.ctx_cap + pa) * row_bytes + h0 * kHeadBytes;
+              si.pos0 = pa;
+              si.n = (int)(pb - pa);
+              si.is_v = v;
+              si.item = item;
+            }
+            if (a.k_pos_mode == 1) {
+              bool more = many;
+              for (int t = 0; t < run_n; ++t) first_s[s][run_at + t] = run_first;
+              for (int g = 1; more; ++g) {
+                more = find_run(g);
+                for (int t = 0; t < run_n; ++t) first_s[s][run_at + t] = run_first;
+              }
+              if (many) find_run(0);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive_expect_tx(full(s), (uint32_t)total * width);
+            __syncwarp();
+            bool more = true;
+            for (int g = 0; more; ++g) {
+              more = many && (g == 0 || find_run(g));
+              const uint32_t dst = smem0 + s * stage_bytes + run_at * part_bytes;
+              if (!cut_rows) {
+                if (run_n > 0) bulk_load(dst, src + run_src * row_bytes, (uint32_t)run_n * row_bytes, full(s));
+              } else {
+                for (int t = 0; t < run_n; ++t) bulk_load(dst + t * part_bytes, src + (run_src + t) * row_bytes, width, full(s));
+              }
+            }
+            if (many) find_run(0);
+          }
     }
-    if (p >= o_next) {               // next selected shot (skipping zero-length slots); warp-uniform
-      do {
-        ++lo;
-        o = o_next;
-        o_next = off[lo + 1];
-      } while (p >= o_next);
-      s = a.sel_idx[(long long)b * a.k + lo];
-      src0 = (s >= 0 && s < a.n_shots) ? a.shot_off[s] : 0;
+    if (lane == 0) {
+      // the end: an empty stage; after giving up, the copies still on their way have to land
+      const int s = it % kStages;
+      if (ok && mbar_wait(empty(s), ((it / kStages) & 1) ^ 1, abort_s)) {
+        info[s].n = 0;
+        mbar_arrive(full(s));
+      } else {
+        for (uint32_t t = it > (uint32_t)kStages ? it - kStages : 0; t < it; ++t)
+          mbar_wait(full(t % kStages), (t / kStages) & 1, abort_s + 1);
+      }
     }
-    if (s < 0 || s >= a.n_shots) continue;           // reported by the plan kernel
-    const long long src_tok = src0 + (p - o);
-    const double delta = a.k_pos_mode == 0 ? (double)p : (double)o;
-
+    __syncwarp();
+  } else if (warp == kRotWarps + 1) {
+    // ---------------------------------------------------------------- storing warp (one thread)
+    if (lane == 0) {
+      for (uint32_t it = 0;; ++it) {
+        const int s = it % kStages;
+        if (!mbar_wait(full(s), (it / kStages) & 1, abort_s)) break;
+        const StageInfo si = info[s];
+        if (si.n == 0) break;
+        // (consumers arrive for every stage, so that the phases of `done` follow those of `full`)
+        if (!mbar_wait(done(s), (it / kStages) & 1, abort_s)) break;
+        char* dst = static_cast<char*>(si.is_v ? a.v_ctx : a.k_ctx) + si.dst;
+        const uint32_t src = smem0 + s * stage_bytes;
+        if (!cut_rows) {
+          bulk_store(dst, src, (uint32_t)si.n * row_bytes);
+        } else {
+          const int width = min(part_bytes, row_bytes - (int)(si.dst % row_bytes));
+          for (int t = 0; t < si.n; ++t) bulk_store(dst + (long long)t * row_bytes, src + t * part_bytes, width);
+        }
+        bulk_commit();
+        if (it > 0) {                              // the stage before has been read
+          bulk_wait_read<1>();
+          mbar_arrive(empty((it - 1) % kStages));
+        }
+      }
+      bulk_wait_all();
+    }
+    __syncwarp();
+  } else {
+    // ---------------------------------------------------------------- rotating warps
+    const int jcol = threadIdx.x % HALF_V, tok0 = threadIdx.x / HALF_V;
+    double theta[EPV];
+#pragma unroll
+    for (int e = 0; e < EPV; ++e) theta[e] = a.theta[jcol * EPV + e];
     float sn[EPV], cs[EPV];
+    const bool one_pass = a.chunk <= kPassTokens;
+    long long last_item = -1;
+    for (uint32_t it = 0;; ++it) {
+      const int s = it % kStages;
+      if (!__all_sync(0xffffffffu, mbar_wait(full(s), (it / kStages) & 1, abort_s))) break;
+      const StageInfo si = info[s];
+      if (si.n == 0) break;
+      if (!si.is_v) {
+        for (int t = tok0; t < si.n; t += kPassTokens) {
+          if (!one_pass || si.item != last_item) {
+            const double delta = a.k_pos_mode == 0 ? (double)(si.pos0 + t) : (double)first_s[s][t];
 #pragma unroll
-    for (int e = 0; e < EPV; ++e) {
-      // bf16 storage rounds at 2^-9: the hardware sin/cos of the reduced angle is ample there
-      if constexpr (sizeof(T) == 2) rope_sincos_fast(delta, theta[e], &sn[e], &cs[e]);
-      else rope_sincos(delta, theta[e], &sn[e], &cs[e]);
-    }
-
-    // rotates one pair unit (vector j of the low half of a head with vector j of the high half) and stores it
-    auto rot_store = [&](const uint4& lo_v, const uint4& hi_v, long long d0) {
-      float x[EPV], y[EPV], xr[EPV], yr[EPV];
-      Vec16<T>::unpack(lo_v, x); Vec16<T>::unpack(hi_v, y);
+            for (int e = 0; e < EPV; ++e) {
+              // bf16 storage rounds at 2^-9: the hardware sin/cos of the reduced angle is ample there
+              if constexpr (sizeof(T) == 2) rope_sincos_fast(delta, theta[e], &sn[e], &cs[e]);
+              else rope_sincos(delta, theta[e], &sn[e], &cs[e]);
+            }
+          }
+          unsigned char* row = smem + s * stage_bytes + t * part_bytes + jcol * 16;
+#pragma unroll 4
+          for (int h = 0; h < a.heads; ++h, row += kHeadBytes) {
+            uint4* lo_p = reinterpret_cast<uint4*>(row);
+            uint4* hi_p = reinterpret_cast<uint4*>(row + kHeadBytes / 2);
+            float x[EPV], y[EPV], xr[EPV], yr[EPV];
+            Vec16<T>::unpack(*lo_p, x);
+            Vec16<T>::unpack(*hi_p, y);
 #pragma unroll
-      for (int e = 0; e < EPV; ++e) {
-        xr[e] = x[e] * cs[e] - y[e] * sn[e];
-        yr[e] = y[e] * cs[e] + x[e] * sn[e];
-      }
-      kc[d0] = Vec16<T>::pack(xr);
-      kc[d0 + HALF_V] = Vec16<T>::pack(yr);
-    };
-    int l_first = 0;
-    if (!with_v) {
-      // K alone: the loads of two layers are issued before either is rotated, so that a warp keeps as
-      // many bytes on their way as it does when it also copies V
-      for (; l_first + 1 < a.n_layers_call; l_first += 2) {
-        const long long srcA = (long long)(a.layer_begin + l_first) * layer_stride_pool + src_tok * row_vecs;
-        const long long srcB = srcA + layer_stride_pool;
-        const long long dstA = ((long long)b * a.n_layers_call + l_first) * layer_stride_ctx + p * row_vecs;
-        const long long dstB = dstA + layer_stride_ctx;
-        for (int unit = lane; unit < pair_units; unit += 64) {
-          const int unit2 = unit + 32;
-          const bool two = unit2 < pair_units;
-          const int o0 = (unit / HALF_V) * VPH + jcol, o1 = (unit2 / HALF_V) * VPH + jcol;
-          const uint4 z = make_uint4(0, 0, 0, 0);
-          const uint4 aLo0 = kp[srcA + o0], aHi0 = kp[srcA + o0 + HALF_V];
-          const uint4 bLo0 = kp[srcB + o0], bHi0 = kp[srcB + o0 + HALF_V];
-          const uint4 aLo1 = two ? kp[srcA + o1] : z, aHi1 = two ? kp[srcA + o1 + HALF_V] : z;
-          const uint4 bLo1 = two ? kp[srcB + o1] : z, bHi1 = two ? kp[srcB + o1 + HALF_V] : z;
-          rot_store(aLo0, aHi0, dstA + o0);
-          rot_store(bLo0, bHi0, dstB + o0);
-          if (two) {
-            rot_store(aLo1, aHi1, dstA + o1);
-            rot_store(bLo1, bHi1, dstB + o1);
+            for (int e = 0; e < EPV; ++e) {
+              xr[e] = x[e] * cs[e] - y[e] * sn[e];
+              yr[e] = y[e] * cs[e] + x[e] * sn[e];
+            }
+            *lo_p = Vec16<T>::pack(xr);
+            *hi_p = Vec16<T>::pack(yr);
           }
         }
+        last_item = si.item;
+        fence_proxy_async_smem();                  // the rotated rows, for the bulk store
       }
-    }
-    for (int l = l_first; l < a.n_layers_call; ++l) {
-      const long long src = (long long)(a.layer_begin + l) * layer_stride_pool + src_tok * row_vecs;
-      const long long dst = ((long long)b * a.n_layers_call + l) * layer_stride_ctx + p * row_vecs;
-      // K: rotate pairs.  unit = head * HALF_V + column; lane stride 32 keeps the column.
-      for (int unit = lane; unit < pair_units; unit += 64) {
-        const int unit2 = unit + 32;
-        const bool two = unit2 < pair_units;
-        const int o0 = (unit / HALF_V) * VPH + jcol, o1 = (unit2 / HALF_V) * VPH + jcol;
-        const uint4 lo0 = kp[src + o0], hi0 = kp[src + o0 + HALF_V];
-        uint4 lo1 = make_uint4(0, 0, 0, 0), hi1 = lo1;
-        if (two) { lo1 = kp[src + o1]; hi1 = kp[src + o1 + HALF_V]; }
-        rot_store(lo0, hi0, dst + o0);
-        if (two) rot_store(lo1, hi1, dst + o1);
-      }
-      // V: plain copy, four vectors in flight per lane
-      for (int i = lane; with_v && i < row_vecs; i += 128) {
-        uint4 r0 = vp[src + i];
-        uint4 r1 = i + 32 < row_vecs ? vp[src + i + 32] : make_uint4(0, 0, 0, 0);
-        uint4 r2 = i + 64 < row_vecs ? vp[src + i + 64] : make_uint4(0, 0, 0, 0);
-        uint4 r3 = i + 96 < row_vecs ? vp[src + i + 96] : make_uint4(0, 0, 0, 0);
-        vc[dst + i] = r0;
-        if (i + 32 < row_vecs) vc[dst + i + 32] = r1;
-        if (i + 64 < row_vecs) vc[dst + i + 64] = r2;
-        if (i + 96 < row_vecs) vc[dst + i + 96] = r3;
-      }
-    }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(done(s));
     }
   }
+  __syncthreads();
+  if (threadIdx.x == 0 && abort_s[0] != 0) ads_set_status(a.status, ADAPSHOT_ETIMEOUT);
 }
 
 template <typename T, int D>
 int launch_gather(GatherArgs a, cudaStream_t st) {
-  const int warps_per_block = 4;
-  // Resident warps: about six 128-thread CTAs per SM.  Long runs amortise the plan lookup; a
-  // small launch takes shorter runs so that every resident warp gets several and the tail
-  // wave stays short.
-  const long long n_sm = ads_sm_count();
+  constexpr int kPassTokens = kRotThreads / (D / Vec16<T>::N / 2);
+  const int n_sm = ads_sm_count();
   if (n_sm <= 0) return ADAPSHOT_ECUDA;
-  const long long resident_warps = n_sm * 6 * warps_per_block;
-  const long long tokens = (long long)a.B * a.ctx_cap;
-  // a call of one or two layers has little work per token to spread the plan lookup over: longer runs
-  a.run = a.n_layers_call <= 2 ? 4 * kRunMax : kRunMax;
-  while (a.run > 1 && tokens / a.run < 4 * resident_warps) a.run >>= 1;
-  const long long units = (long long)a.B * ((a.ctx_cap + a.run - 1) / a.run);
-  long long blocks = (units + warps_per_block - 1) / warps_per_block;
-  // measured: one resident wave with a grid-stride loop is best when a run is short (one
-  // layer per call), several waves when every run walks several layers
-  const long long max_blocks = a.n_layers_call == 1 ? n_sm * 6 : n_sm * 16 * 4;
-  if (blocks > max_blocks) blocks = max_blocks;
-  if (a.v_ctx != nullptr) gather_rope_kernel<T, D, true><<<(unsigned)blocks, warps_per_block * 32, 0, st>>>(a);
-  else gather_rope_kernel<T, D, false><<<(unsigned)blocks, warps_per_block * 32, 0, st>>>(a);
+  // A pass of the rotating threads over one head is 4 KB whatever D and T: eight heads fill a stage, more are
+  // cut into several stages, fewer leave room for up to four passes (as long as every CTA gets a chunk).
+  a.heads = a.n_kv_heads < 8 ? a.n_kv_heads : 8;
+  int passes = 8 / a.heads < 4 ? 8 / a.heads : 4;
+  auto chunks = [&]() { return (long long)a.B * ((a.ctx_cap + (long long)kPassTokens * passes - 1) / (kPassTokens * passes)); };
+  while (passes > 1 && chunks() < 2 * n_sm) passes >>= 1;
+  a.chunk = kPassTokens * passes;
+  const uint32_t smem = kStages * (uint32_t)a.chunk * a.heads * D * sizeof(T);
+  int per_sm = (int)(200 * 1024 / (smem + 4096));
+  per_sm = per_sm > 8 ? 8 : per_sm;
+  const long long ctas = (long long)n_sm * per_sm;
+  // K alone: one item per layer (neighbouring CTAs then take the same chunk's layers; 663 against 687 us for four
+  // layers of 8 x 33 K tokens).  With V a chunk's layers stay together (246 against 252 us for three layers of 64 K
+  // tokens) unless pairs of them are needed to give every CTA several items.
+  long long groups = a.v_ctx == nullptr ? a.n_layers_call : (4 * ctas + chunks() - 1) / chunks();
+  if (a.v_ctx != nullptr && groups > (a.n_layers_call + 1) / 2) groups = (a.n_layers_call + 1) / 2;
+  a.layer_groups = groups < 1 ? 1 : (int)groups;
+  const long long items = chunks() * a.layer_groups;
+  const unsigned grid = (unsigned)(items < ctas ? items : ctas);
+  static bool attr_done[2][kAdsMaxDevices] = {{false}, {false}};
+  const int most = (int)(kStages * kStageMax);
+  if (a.v_ctx != nullptr) {
+    if (ads_set_max_smem(gather_rope_kernel<T, D, true>, most, attr_done[0]) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
+    gather_rope_kernel<T, D, true><<<grid, kGatherThreads, smem, st>>>(a);
+  } else {
+    if (ads_set_max_smem(gather_rope_kernel<T, D, false>, most, attr_done[1]) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
+    gather_rope_kernel<T, D, false><<<grid, kGatherThreads, smem, st>>>(a);
+  }
   return ads_launch_status();
 }
 

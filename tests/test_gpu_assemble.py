@@ -155,3 +155,45 @@ def test_extending_a_nested_prefix_equals_one_gather(k_pos_mode):
         for b in range(w.batch):
             assert torch.equal(kc[b, :, :first[b]], keep_k[b, :, :first[b]])
             assert torch.equal(vc[b, :, :first[b]], keep_v[b, :, :first[b]])
+
+
+@pytest.mark.parametrize("dtype,d,hkv,nl,lens,k,shot_begin,k_only", [
+    ("bf16", 128, 8, 3, (1, 1), 70, 0, False),      # one-token shots: a chunk of sixteen rows is sixteen runs
+    ("bf16", 64, 1, 1, (1, 2), 150, 0, True),       # more than 32 shots per chunk (128 rows of one head)
+    ("bf16", 64, 9, 2, (5, 40), 9, 0, False),       # nine heads: rows cut into eight heads and one
+    ("fp32", 128, 12, 1, (3, 30), 7, 4, False),     # cut rows, earlier shots kept
+    ("bf16", 128, 2, 2, (127, 129), 5, 3, True),    # several passes per chunk, K alone, earlier shots kept
+    ("fp32", 64, 1, 1, (1, 300), 6, 0, False),
+])
+@pytest.mark.parametrize("k_pos_mode", [0, 1])
+def test_gather_chunks(dtype, d, hkv, nl, lens, k, shot_begin, k_only, k_pos_mode):
+    ab = hp.gpu_binding()
+    w = wl.CONFIGS["cfg2"].scaled(n_layers=nl, n_q_heads=hkv, n_kv_heads=hkv, head_dim=d, dtype=dtype, n_shots=k + 2,
+                                  len_lo=lens[0], len_hi=lens[1], batch=2, k=k, probes=(k,), t_q=1, seed=91)
+    pool = wl.make_pool(w)
+    rng = np.random.default_rng(14)
+    sel_np = np.stack([rng.permutation(k + 2)[:k] for _ in range(2)]).astype(np.int32)
+    off_np = orc.plan_offsets(sel_np, pool["shot_off"])
+    cap = int(off_np[:, -1].max()) + 131
+    shape = (2, nl, cap, hkv, d)
+    kc = torch.full(shape, 7.0, dtype=w.torch_dtype, device="cuda")
+    vc = None if k_only else kc.clone()
+    off, st = torch.zeros((2, k + 1), dtype=torch.int64, device="cuda"), hp.new_status()
+    dp, model = hp.dev_pool(ab, pool), hp.model_of(ab, w, k_pos_mode=k_pos_mode)
+    ab.adapshot_assemble_kv_from(model, dp, torch.from_numpy(sel_np).cuda(), shot_begin, 0, nl, kc, vc, cap, off, st,
+                                 flags=ab.ASSEMBLE_K_ONLY if k_only else 0)
+    torch.cuda.synchronize()
+    assert st.item() == 0 and np.array_equal(off.cpu().numpy(), off_np)
+    for b in range(2):
+        want_k, want_v, _ = orc.assemble_kv(hp.f64(pool["k"]), hp.f64(pool["v"]), pool["shot_off"], sel_np[b],
+                                            w.rope_base, k_pos_mode)
+        a, L = int(off_np[b, shot_begin]), int(off_np[b, -1])
+        end = min(-(-L // 128) * 128, cap)
+        got = hp.f64(kc[b, :, a:L].cpu())
+        err = np.abs(got - want_k[:, a:L])
+        bound = 2.0 ** -8 * np.abs(want_k[:, a:L]) + 1e-5 if dtype == "bf16" else 1e-5 * np.maximum(1.0, np.abs(want_k[:, a:L]))
+        assert (err <= bound).all()
+        for c in (kc,) if k_only else (kc, vc):
+            assert (c[b, :, :a] == 7.0).all() and (c[b, :, end:] == 7.0).all() and (c[b, :, L:end] == 0.0).all()
+        if not k_only:
+            assert np.array_equal(hp.f64(vc[b, :, a:L].cpu()), want_v[:, a:L])
