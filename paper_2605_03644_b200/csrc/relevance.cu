@@ -5,14 +5,16 @@
 // shot's relevance being the attention mass that falls on its tokens, averaged over query tokens
 // and heads (optionally divided by T_i).  Q and K enter as stored; 1/sqrt(d) scaling as in Eq. 5.
 //
-// Two passes over the pool's K of that layer, both on the tensor cores (tcgen05, S in TMEM, tiles
-// staged by TMA), because the normaliser of a row is only known after all keys have been seen:
-//   pass 1  S = Q K^T, one thread per query row (TMEM lane): running maximum and sum of exponentials
-//           over the CTA's range of key tiles; a small kernel merges the ranges into log2-sum-exp;
-//   pass 2  S^T = K Q^T (the same two shared-memory tiles with their roles swapped), one thread per
-//           KEY: p = 2^(s c - lse(row)) summed over the query rows of the tile is the key's mass
-//           from these rows; keys are folded into their shots by a segmented warp sum and one fp64
-//           atomic per (warp, shot).
+// One pass over the pool's K of that layer, on the tensor cores (tcgen05, S in TMEM, tiles staged by TMA).  The
+// normaliser of a row is only known after all keys have been seen, so the pass leaves, for every query row and shot,
+// the log2 of the row's un-normalised mass on the shot:
+//   pass    S = Q K^T, one thread per query row (TMEM lane): running maximum, exponentials, and their sum over
+//           every shot of the CTA's range of keys, written as maximum + log2(sum) at the shot's end;
+//   merge   the ranges' (maximum, sum) pairs -> log2-sum-exp of every row;
+//   reduce  mass of a shot = sum over rows of 2^(its log2 mass - the row's log2-sum-exp), a warp per shot.
+// (A second pass over the keys, with the normalisers known, used to take the reduce step's place: it cost as much as
+// the first, 813 of 1580 us for 2 queries x 128 tokens and 328 K pool tokens.)  What lies between the steps is 4
+// bytes per row and shot; the rows are taken in batches that keep it below kPieceBytes.
 // The scores then go through the same top-k as the embedding selector (ties -> lower shot id).
 #include <float.h>
 
@@ -58,14 +60,14 @@ __device__ __forceinline__ float2 rel_ex2_poly2(float2 x) {
                      __uint_as_float(__float_as_uint(p.y) + (__float_as_uint(t.y) << 23)));
 }
 
+// A unit is an M tile (of a query) and a KV head; units of a batch of M tiles are numbered from 0.
 struct RelParams {
-  float* ml_part;               // pass 1 out: [unit][split][128][2] (max in log2 units, sum)
-  const float* lse2;            // pass 2 in:  [unit][128] log2-sum-exp of every query row
-  double* mass;                 // pass 2 out: [B][n_shots], zeroed before the pass
-  const int* tok_shot;          // [pool_tokens] shot of every pool token
+  float* ml_part;               // [unit][split][128][2] (max in log2 units, sum)
+  float* pieces;                // [unit][n_shots + splits][128]: log2 mass of row on shot i in range s, at slot s + i
+  const long long* shot_off;
   int32_t* status;
   long long pool_tokens;
-  int B, Hkv, n_mt, rows, n_shots, layer;   // rows = T_q * G query rows per (query, kv head)
+  int Hkv, n_mt, n_shots, layer, tile0;     // tile0: first of the batch's M tiles (b * n_mt + mt)
   int n_tiles, splits, tiles_per_split;
   float scale_log2;
 };
@@ -94,19 +96,6 @@ __global__ void __launch_bounds__(256) rel_pack_q_kernel(const __nv_bfloat16* __
   reinterpret_cast<uint4*>(q_pack)[i] = val;
 }
 
-// tok_shot[t] = shot that owns pool token t (one thread per token, binary search of the offsets).
-__global__ void __launch_bounds__(256) rel_token_shot_kernel(const long long* __restrict__ shot_off, int n_shots,
-                                                             long long pool_tokens, int* __restrict__ tok_shot) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= pool_tokens) return;
-  int lo = 0, hi = n_shots;                          // shot with shot_off[lo] <= t < shot_off[lo + 1]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (shot_off[mid] <= t) lo = mid; else hi = mid;
-  }
-  tok_shot[t] = lo;
-}
-
 enum RelBar { kRQFull = 0, kRKFull = 1, kRKEmpty = 5, kRSFull = 9, kRSEmpty = 11, kRDrain = 13, kRNumBars = 14 };
 
 template <int D>
@@ -115,13 +104,12 @@ struct RelSmem {
   static constexpr uint32_t kOffQ = 0;
   static constexpr uint32_t kOffK = kTileBytes;
   static constexpr uint32_t kOffBar = kOffK + kKStages<D> * kTileBytes;
-  static constexpr uint32_t kOffLse = kOffBar + 128;
-  static constexpr uint32_t kTotal = kOffLse + 512 + 1024;      // + alignment slack
+  static constexpr uint32_t kTotal = kOffBar + 128 + 1024;      // + alignment slack
 };
 
-// grid (B * n_mt, splits, Hkv): the CTAs that differ only in (query, M tile) walk the same key tiles
+// grid (M tiles of the batch, splits, Hkv): the CTAs that differ only in (query, M tile) walk the same key tiles
 // at the same time, so the pool's K layer is read from DRAM about once and from L2 otherwise.
-template <int D, int PASS>
+template <int D>
 __global__ void __launch_bounds__(kRelThreads, 2)
 rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                 const RelParams p) {
@@ -138,12 +126,11 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   auto bar = [&](int i) { return bar0 + 8u * i; };
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + SM::kOffBar + 8 * kRNumBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + SM::kOffBar + 8 * kRNumBars + 8);
-  float* lse_s = reinterpret_cast<float*>(base_ptr + SM::kOffLse);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b = blockIdx.x / p.n_mt, mt = blockIdx.x % p.n_mt;
+  const int b = (p.tile0 + blockIdx.x) / p.n_mt, mt = (p.tile0 + blockIdx.x) % p.n_mt;
   const int split = blockIdx.y, g = blockIdx.z;
-  const int unit = (b * p.Hkv + g) * p.n_mt + mt;
+  const long long unit = (long long)blockIdx.x * p.Hkv + g;
   const int t0 = split * p.tiles_per_split;
   const int t1 = min(p.n_tiles, t0 + p.tiles_per_split);
   const int n_it = max(0, t1 - t0);
@@ -166,11 +153,6 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   if (warp == 0) {
     tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), 256);
     tmem_relinquish();
-  }
-  if (PASS == 2 && threadIdx.x >= 64) {
-    // -lse per query row; rows of the M tile that do not exist get -inf: their 2^(s c - lse) is exactly zero
-    const int c = threadIdx.x - 64;
-    lse_s[c] = c < min(kTile, p.rows - mt * kTile) ? -p.lse2[(long long)unit * kTile + c] : -INFINITY;
   }
   tc_fence_before();
   __syncthreads();
@@ -221,8 +203,7 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks) {
           const uint32_t o = ((ks / 4) * 16384u + (ks % 4) * 32u) >> 4;
-          if (PASS == 1) umma_ss_lohi(d, q_lo + o, kHi, k_lo + o, kHi, kIdesc, ks > 0 ? 1u : 0u);   // rows = queries
-          else umma_ss_lohi(d, k_lo + o, kHi, q_lo + o, kHi, kIdesc, ks > 0 ? 1u : 0u);             // rows = keys
+          umma_ss_lohi(d, q_lo + o, kHi, k_lo + o, kHi, kIdesc, ks > 0 ? 1u : 0u);
         }
         umma_commit(bar(kRSFull + sb));
         umma_commit(bar(kRKEmpty + st));
@@ -236,9 +217,32 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   } else {
     // --------------------------------------------------------------- consumers
     const int quarter = warp & 3;
-    const int r = quarter * 32 + lane;                      // TMEM lane: query row (pass 1) or key of the tile (pass 2)
+    const int r = quarter * 32 + lane;                      // TMEM lane: query row
     const uint32_t lane_addr = static_cast<uint32_t>(quarter * 32) << 16;
-    float m_run = -1.0e30f, l_run = 0.f;
+    float m_run = -1.0e30f, l_run = 0.f, acc = 0.f;         // running maximum, sum of the shots so far, of the current one
+    // the current shot and where it and the next one end (the last one with the pool); the same in every lane
+    auto shot_end = [&](int i) -> long long {
+      return i + 1 < p.n_shots ? p.shot_off[i + 1] : i + 1 == p.n_shots ? p.pool_tokens : (1ll << 62);
+    };
+    int shot = 0;
+    {
+      int hi = p.n_shots;
+      while (hi - shot > 1) {
+        const int mid = (shot + hi) >> 1;
+        if (p.shot_off[mid] <= (long long)t0 * kTile) shot = mid; else hi = mid;
+      }
+    }
+    long long end = shot_end(shot), end_next = shot_end(shot + 1);
+    float* piece = p.pieces + ((unit * (p.n_shots + p.splits) + split + shot) * kTile + r);
+    auto flush = [&]() {                                    // the current shot is complete (in this range)
+      *piece = m_run + __log2f(acc);
+      l_run += acc;
+      acc = 0.f;
+      piece += kTile;
+      ++shot;
+      end = end_next;
+      end_next = shot_end(shot + 1);
+    };
     bool ok = true;
     for (int i = 0; i < n_it; ++i) {
       const int sb = i & 1;
@@ -250,63 +254,73 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       tc_fence_before();
       mbar_arrive(bar(kRSEmpty + sb));                      // the scores are in registers: the buffer is free
       const long long key0 = (long long)(t0 + i) * kTile;
-      if (PASS == 1) {
-        const int limit = (int)min((long long)kTile, p.pool_tokens - key0);   // keys of this tile that exist
-        if (limit < kTile) {                       // only the pool's last tile: keys beyond it count as -inf
+      const int limit = (int)min((long long)kTile, p.pool_tokens - key0);   // keys of this tile that exist
+      if (limit < kTile) {                       // only the pool's last tile: keys beyond it count as -inf
 #pragma unroll
-          for (int c = 0; c < kTile; ++c) s[c] = c < limit ? s[c] : -INFINITY;
-        }
-        float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+        for (int c = 0; c < kTile; ++c) s[c] = c < limit ? s[c] : -INFINITY;
+      }
+      float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-        for (int c = 0; c < kTile; c += 8) {
+      for (int c = 0; c < kTile; c += 8) {
 #pragma unroll
-          for (int u = 0; u < 4; ++u) mx4[u] = fmax3(mx4[u], s[c + 2 * u], s[c + 2 * u + 1]);
-        }
-        const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * p.scale_log2;
-        if (mx > m_run) {
-          l_run *= rel_ex2(m_run - mx);
-          m_run = mx;
-        }
-        // two scores per FMA / add instruction; the exponentials themselves are one MUFU operation each
-        const float2 scale2 = make_float2(p.scale_log2, p.scale_log2), neg_m2 = make_float2(-m_run, -m_run);
-        float2 part[2] = {{0.f, 0.f}, {0.f, 0.f}};
+        for (int u = 0; u < 4; ++u) mx4[u] = fmax3(mx4[u], s[c + 2 * u], s[c + 2 * u + 1]);
+      }
+      const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * p.scale_log2;
+      if (mx > m_run) {
+        const float keep = rel_ex2(m_run - mx);
+        l_run *= keep;
+        acc *= keep;
+        m_run = mx;
+      }
+      // two scores per FMA / add instruction; the exponentials themselves are one MUFU operation each
+      const float2 scale2 = make_float2(p.scale_log2, p.scale_log2), neg_m2 = make_float2(-m_run, -m_run);
+      float group[kTile / 16];                              // sums of 16 keys
 #pragma unroll
-        for (int c = 0; c < kTile; c += 2) {
+      for (int c0 = 0; c0 < kTile; c0 += 16) {
+        float2 part = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int c = c0; c < c0 + 16; c += 2) {
           const float2 a = __ffma2_rn(make_float2(s[c], s[c + 1]), scale2, neg_m2);
           const float2 e = ((c >> 1) & 3) == 3 ? rel_ex2_poly2(a) : make_float2(rel_ex2(a.x), rel_ex2(a.y));
-          part[(c >> 1) & 1] = __fadd2_rn(part[(c >> 1) & 1], e);
+          s[c] = e.x;
+          s[c + 1] = e.y;
+          part = c == c0 ? e : __fadd2_rn(part, e);
         }
-        l_run += (part[0].x + part[0].y) + (part[1].x + part[1].y);
+        group[c0 / 16] = part.x + part.y;
+      }
+      // sums per shot (the branches are the same in every lane): a tile within one shot, else group by group, the
+      // keys of a group one by one only where a shot ends in it
+      const long long left = end - key0;
+      if (left > kTile) {
+        acc += ((group[0] + group[1]) + (group[2] + group[3])) + ((group[4] + group[5]) + (group[6] + group[7]));
       } else {
-        const long long key = key0 + r;
-        const float2 scale2 = make_float2(p.scale_log2, p.scale_log2);
-        float2 part[2] = {{0.f, 0.f}, {0.f, 0.f}};
-        const float4* lse4 = reinterpret_cast<const float4*>(lse_s);
+        int ce = (int)left;                                 // columns left of the current shot
 #pragma unroll
-        for (int c4 = 0; c4 < kTile / 4; ++c4) {
-          const float4 l4 = lse4[c4];                     // the same address for every lane: a broadcast
-          const float2 a0 = __ffma2_rn(make_float2(s[4 * c4], s[4 * c4 + 1]), scale2, make_float2(l4.x, l4.y));
-          const float2 a1 = __ffma2_rn(make_float2(s[4 * c4 + 2], s[4 * c4 + 3]), scale2, make_float2(l4.z, l4.w));
-          part[0] = __fadd2_rn(part[0], make_float2(rel_ex2(a0.x), rel_ex2(a0.y)));
-          part[1] = __fadd2_rn(part[1], (c4 & 1) ? rel_ex2_poly2(a1) : make_float2(rel_ex2(a1.x), rel_ex2(a1.y)));
-        }
-        float v = (part[0].x + part[0].y) + (part[1].x + part[1].y);
-        int id = -1;
-        if (key < p.pool_tokens) id = p.tok_shot[key]; else v = 0.f;
-        // shots are runs of consecutive keys: segmented inclusive sum along the lanes, the last
-        // lane of every run adds the run's mass to its shot
+        for (int c0 = 0; c0 < kTile; c0 += 16) {
+          if (ce > c0 + 16) {
+            acc += group[c0 / 16];
+          } else {
+            int from = c0;
+            while (from < c0 + 16) {
+              const int to = min(ce, c0 + 16);
+              float sum[2] = {0.f, 0.f};
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const float u = __shfl_up_sync(0xffffffffu, v, o);
-          const int iu = __shfl_up_sync(0xffffffffu, id, o);
-          if (lane >= o && iu == id) v += u;
+              for (int c = 0; c < 16; ++c) sum[c & 1] += c0 + c >= from && c0 + c < to ? s[c0 + c] : 0.f;
+              acc += sum[0] + sum[1];
+              if (to == ce) {
+                flush();
+                ce = end - key0 > 4096 ? 4096 : (int)(end - key0);
+              }
+              from = to;
+            }
+          }
         }
-        const int idn = __shfl_down_sync(0xffffffffu, id, 1);
-        if (id >= 0 && (lane == 31 || idn != id)) atomicAdd(p.mass + (long long)b * p.n_shots + id, (double)v);
       }
     }
-    if (PASS == 1 && ok) {
-      float* out = p.ml_part + (((long long)unit * p.splits + split) * kTile + r) * 2;
+    if (ok && n_it > 0) {
+      // the shot that goes on in the next range
+      if (shot < p.n_shots && (shot == 0 || (long long)t1 * kTile > p.shot_off[shot])) flush();
+      float* out = p.ml_part + ((unit * p.splits + split) * kTile + r) * 2;
       out[0] = m_run;
       out[1] = l_run;
     }
@@ -321,11 +335,13 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   if (threadIdx.x == 0 && *abort_flag != 0) ads_set_status(p.status, ADAPSHOT_ETIMEOUT);
 }
 
-// lse2[unit][row] = log2 sum_keys 2^(s c) from the per-range (max, sum) pairs; one thread per row.
-__global__ void __launch_bounds__(128) rel_merge_kernel(const float* __restrict__ ml_part, int splits,
-                                                        float* __restrict__ lse2) {
+// lse2[unit][row] = log2 sum_keys 2^(s c) from the per-range (max, sum) pairs, +inf for rows that do not exist (so
+// that they add nothing); one thread per row.
+__global__ void __launch_bounds__(128) rel_merge_kernel(const float* __restrict__ ml_part, int splits, int Hkv, int tile0,
+                                                        int n_mt, int rows, float* __restrict__ lse2) {
   const long long unit = blockIdx.x;
   const int r = threadIdx.x;
+  const int mt = (int)((tile0 + unit / Hkv) % n_mt);
   float M = -1.0e30f;
   for (int s = 0; s < splits; ++s) M = fmaxf(M, ml_part[((unit * splits + s) * kTile + r) * 2]);
   float l = 0.f;
@@ -333,7 +349,41 @@ __global__ void __launch_bounds__(128) rel_merge_kernel(const float* __restrict_
     const float* ml = ml_part + ((unit * splits + s) * kTile + r) * 2;
     l += ml[1] * exp2f(ml[0] - M);
   }
-  lse2[unit * kTile + r] = l > 0.f ? M + log2f(l) : 0.f;
+  lse2[unit * kTile + r] = mt * kTile + r >= rows ? INFINITY : l > 0.f ? M + log2f(l) : 0.f;
+}
+
+// mass[b][i] (+)= sum over the batch's rows of query b of 2^(piece - lse); grid (shots / 8, queries), a warp per shot.
+__global__ void __launch_bounds__(256) rel_reduce_kernel(const float* __restrict__ pieces, const float* __restrict__ lse2,
+                                                         const long long* __restrict__ shot_off, int n_shots, int Hkv,
+                                                         int n_mt, int tile0, int n_tiles_m, int splits,
+                                                         int tiles_per_split, long long pool_tokens, int b0,
+                                                         double* __restrict__ mass) {
+  const int lane = threadIdx.x & 31, b = b0 + blockIdx.y;
+  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (i >= n_shots) return;
+  const int first = max(tile0, b * n_mt), last = min(tile0 + n_tiles_m, (b + 1) * n_mt);   // M tiles of this query
+  const long long o0 = i > 0 ? shot_off[i] : 0, o1 = i + 1 < n_shots ? shot_off[i + 1] : pool_tokens;
+  const int s0 = (int)(o0 / kTile) / tiles_per_split, s1 = (int)((o1 - 1) / kTile) / tiles_per_split;
+  double sum = 0.0;
+  for (int m = first; m < last; ++m) {
+    const float4* lse = reinterpret_cast<const float4*>(lse2 + (long long)(m - tile0) * Hkv * kTile) + lane;
+    for (int s = s0; s <= s1; ++s) {
+      const float4* pc = reinterpret_cast<const float4*>(
+          pieces + (((long long)(m - tile0) * Hkv * (n_shots + splits)) + s + i) * kTile) + lane;
+      float part = 0.f;
+#pragma unroll 8
+      for (int g = 0; g < Hkv; ++g) {
+        const float4 v = pc[(long long)g * (n_shots + splits) * (kTile / 4)], n = lse[g * (kTile / 4)];
+        part += (rel_ex2(v.x - n.x) + rel_ex2(v.y - n.y)) + (rel_ex2(v.z - n.z) + rel_ex2(v.w - n.w));
+      }
+      sum += (double)part;
+    }
+  }
+  sum = warp_sum(sum);
+  if (lane == 0) {
+    double* out = mass + (long long)b * n_shots + i;
+    *out = first == b * n_mt ? sum : *out + sum;
+  }
 }
 
 // score[b][i] = mass[b][i] / (T_q * Hq) (and / T_i with per_token); writes the sort keys.
@@ -349,12 +399,15 @@ __global__ void __launch_bounds__(256) rel_scores_kernel(const double* __restric
   keys[i] = ads_desc_key(s);
 }
 
+constexpr size_t kPieceBytes = 256u << 20;
+
 struct RelPlan {
   int G, n_mt, rows, rows_pad, n_tiles, splits, tiles_per_split;
-  size_t off_qpack, off_ml, off_lse, off_tokshot, off_mass, off_keys, total;
+  int batch;                    // M tiles per launch of the pass
+  size_t off_qpack, off_ml, off_lse, off_pieces, off_mass, off_keys, total;
 };
 
-RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int B, int Tq, int k) {
+RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int B, int Tq) {
   RelPlan pl;
   const int D = model->head_dim, Hkv = model->n_kv_heads;
   pl.G = model->n_q_heads / Hkv;
@@ -362,12 +415,18 @@ RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int
   pl.n_mt = (pl.rows + kTile - 1) / kTile;
   pl.rows_pad = pl.n_mt * kTile;
   pl.n_tiles = (int)((pool->pool_tokens + kTile - 1) / kTile);
+  const int most = (pl.n_tiles + 7) / 8 < 256 ? (pl.n_tiles + 7) / 8 : 256;
+  // M tiles whose pieces fit, in batches of equal size
+  const long long m_tiles = (long long)B * pl.n_mt;
+  const size_t per_tile = (size_t)Hkv * ((size_t)pool->n_shots + most) * kTile * 4;
+  const long long fit = (long long)(kPieceBytes / per_tile) > 1 ? (long long)(kPieceBytes / per_tile) : 1;
+  const long long n_batches = (m_tiles + fit - 1) / fit;
+  pl.batch = (int)((m_tiles + n_batches - 1) / n_batches);
   // Key ranges per unit: units * splits CTAs run in waves of 296 (two per SM on 148 SMs; a fixed
   // figure, so that the workspace size does not depend on the device), each CTA costs its tiles plus
   // about four tiles' time of start-up; the split with the cheapest waves * (tiles + 4) is taken,
   // every range at least eight key tiles.
-  const long long units = (long long)B * pl.n_mt * Hkv;
-  const int most = (pl.n_tiles + 7) / 8 < 256 ? (pl.n_tiles + 7) / 8 : 256;
+  const long long units = (long long)pl.batch * Hkv;
   int best_s = 1;
   long long best_cost = 0;
   for (int sp = 1; sp <= most; ++sp) {
@@ -385,7 +444,7 @@ RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int
   pl.off_qpack = off;   off += ads_round_up((size_t)B * Hkv * pl.rows_pad * D * 2, 256);
   pl.off_ml = off;      off += ads_round_up((size_t)units * pl.splits * kTile * 2 * 4, 256);
   pl.off_lse = off;     off += ads_round_up((size_t)units * kTile * 4, 256);
-  pl.off_tokshot = off; off += ads_round_up((size_t)pool->pool_tokens * 4, 256);
+  pl.off_pieces = off;  off += ads_round_up((size_t)units * ((size_t)pool->n_shots + pl.splits) * kTile * 4, 256);
   pl.off_mass = off;    off += ads_round_up((size_t)B * pool->n_shots * 8, 256);
   pl.off_keys = off;    off += ads_round_up((size_t)B * pool->n_shots * 8, 256);
   pl.total = off;
@@ -406,10 +465,9 @@ int rel_launch(const adapshot_model_t* model, const adapshot_pool_t* pool, int l
   __nv_bfloat16* q_pack = reinterpret_cast<__nv_bfloat16*>(wsb + pl.off_qpack);
   float* ml_part = reinterpret_cast<float*>(wsb + pl.off_ml);
   float* lse2 = reinterpret_cast<float*>(wsb + pl.off_lse);
-  int* tok_shot = reinterpret_cast<int*>(wsb + pl.off_tokshot);
+  float* pieces = reinterpret_cast<float*>(wsb + pl.off_pieces);
   double* mass = reinterpret_cast<double*>(wsb + pl.off_mass);
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(wsb + pl.off_keys);
-  const long long units = (long long)B * pl.n_mt * Hkv;
 
   CUtensorMap tm_q, tm_k;
   {
@@ -429,34 +487,36 @@ int rel_launch(const adapshot_model_t* model, const adapshot_pool_t* pool, int l
   rel_pack_q_kernel<D><<<(unsigned)((n_vec + 255) / 256), 256, 0, st>>>(static_cast<const __nv_bfloat16*>(q), q_pack, B,
                                                                        Tq, Hq, Hkv, pl.rows_pad);
   if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-  rel_token_shot_kernel<<<(unsigned)((pool->pool_tokens + 255) / 256), 256, 0, st>>>(
-      reinterpret_cast<const long long*>(pool->shot_off), pool->n_shots, pool->pool_tokens, tok_shot);
-  if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-  ADS_CHECK_CUDA(cudaMemsetAsync(mass, 0, (size_t)B * pool->n_shots * 8, st));
-
+  const long long* shot_off = reinterpret_cast<const long long*>(pool->shot_off);
   RelParams rp;
-  rp.ml_part = ml_part; rp.lse2 = lse2; rp.mass = mass; rp.tok_shot = tok_shot; rp.status = status;
+  rp.ml_part = ml_part; rp.pieces = pieces; rp.shot_off = shot_off; rp.status = status;
   rp.pool_tokens = pool->pool_tokens;
-  rp.B = B; rp.Hkv = Hkv; rp.n_mt = pl.n_mt; rp.rows = pl.rows; rp.n_shots = pool->n_shots; rp.layer = layer;
+  rp.Hkv = Hkv; rp.n_mt = pl.n_mt; rp.n_shots = pool->n_shots; rp.layer = layer;
   rp.n_tiles = pl.n_tiles; rp.splits = pl.splits; rp.tiles_per_split = pl.tiles_per_split;
   const float scale = model->softmax_scale > 0.f ? model->softmax_scale : 1.0f / sqrtf((float)D);
   rp.scale_log2 = scale * 1.4426950408889634f;
 
   const int smem = (int)RelSmem<D>::kTotal;
-  static bool attr_done[2][kAdsMaxDevices] = {{false}, {false}};
-  if (ads_set_max_smem(rel_pass_kernel<D, 1>, smem, attr_done[0]) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-  if (ads_set_max_smem(rel_pass_kernel<D, 2>, smem, attr_done[1]) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-  const dim3 grid((unsigned)(B * pl.n_mt), (unsigned)pl.splits, (unsigned)Hkv);
-  rel_pass_kernel<D, 1><<<grid, kRelThreads, smem, st>>>(tm_q, tm_k, rp);
-  if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-  rel_merge_kernel<<<(unsigned)units, 128, 0, st>>>(ml_part, pl.splits, lse2);
-  if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-  rel_pass_kernel<D, 2><<<grid, kRelThreads, smem, st>>>(tm_q, tm_k, rp);
-  if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
+  static bool attr_done[kAdsMaxDevices] = {false};
+  if (ads_set_max_smem(rel_pass_kernel<D>, smem, attr_done) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
+  const int m_tiles = B * pl.n_mt;
+  for (int t0 = 0; t0 < m_tiles; t0 += pl.batch) {
+    const int n = m_tiles - t0 < pl.batch ? m_tiles - t0 : pl.batch;
+    rp.tile0 = t0;
+    rel_pass_kernel<D><<<dim3((unsigned)n, (unsigned)pl.splits, (unsigned)Hkv), kRelThreads, smem, st>>>(tm_q, tm_k, rp);
+    if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
+    rel_merge_kernel<<<(unsigned)(n * Hkv), 128, 0, st>>>(ml_part, pl.splits, Hkv, t0, pl.n_mt, pl.rows, lse2);
+    if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
+    const int b0 = t0 / pl.n_mt, b1 = (t0 + n - 1) / pl.n_mt;       // queries with rows in the batch
+    rel_reduce_kernel<<<dim3((unsigned)((pool->n_shots + 7) / 8), (unsigned)(b1 - b0 + 1)), 256, 0, st>>>(
+        pieces, lse2, shot_off, pool->n_shots, Hkv, pl.n_mt, t0, n, pl.splits, pl.tiles_per_split, pool->pool_tokens, b0,
+        mass);
+    if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
+  }
 
   const long long n_sc = (long long)B * pool->n_shots;
   rel_scores_kernel<<<(unsigned)((n_sc + 255) / 256), 256, 0, st>>>(
-      mass, reinterpret_cast<const long long*>(pool->shot_off), B, pool->n_shots, 1.0 / ((double)Tq * Hq),
+      mass, shot_off, B, pool->n_shots, 1.0 / ((double)Tq * Hq),
       (flags & ADAPSHOT_RELEVANCE_PER_TOKEN) ? 1 : 0, keys);
   if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
   return ads_topk_from_keys(keys, pool->n_shots, B, k, sel_idx, sel_score, st);
@@ -469,7 +529,7 @@ extern "C" size_t adapshot_select_attn_workspace_bytes(const adapshot_model_t* m
   if (model == nullptr || pool == nullptr || !rel_shape_ok(model) || B <= 0 || Tq <= 0 || k <= 0 ||
       pool->n_shots <= 0 || pool->pool_tokens <= 0)
     return 0;
-  return rel_plan(model, pool, B, Tq, k).total;
+  return rel_plan(model, pool, B, Tq).total;
 }
 
 extern "C" int adapshot_select_attn(const adapshot_model_t* model, const adapshot_pool_t* pool, int32_t layer,
@@ -489,7 +549,7 @@ extern "C" int adapshot_select_attn(const adapshot_model_t* model, const adapsho
   if (pool->pool_tokens > (1ll << 31) - 256) return ADAPSHOT_ESHAPE;
   if (!ads_aligned16(pool->k) || !ads_aligned16(q) || ((uintptr_t)ws & 255u) || ((uintptr_t)pool->shot_off & 7u))
     return ADAPSHOT_EALIGN;
-  const RelPlan pl = rel_plan(model, pool, B, Tq, k);
+  const RelPlan pl = rel_plan(model, pool, B, Tq);
   if ((long long)B * pl.n_mt > 0x7fffffffll || pl.splits > 65535 || model->n_kv_heads > 65535) return ADAPSHOT_ESHAPE;
   if (ws_bytes < pl.total) return ADAPSHOT_ECAPACITY;
   cudaStream_t st = static_cast<cudaStream_t>(stream);

@@ -95,3 +95,28 @@ def test_identical_shots_get_equal_masses():
     sel, score = _run(ab, hp.model_of(ab, w, n_layers=1), dp, 0, q, n_rep)
     assert np.allclose(score, 1.0 / n_rep, rtol=1e-4)
     assert sorted(sel[0].tolist()) == list(range(n_rep))
+
+
+@pytest.mark.parametrize("lens,n_shots,t_q,batch", [((128, 128), 40, 3, 1), ((1, 1), 700, 2, 2), ((15, 17), 130, 33, 1),
+                                                   ((900, 1100), 9, 1, 3)])
+def test_masses_per_shot_at_tile_and_range_edges(lens, n_shots, t_q, batch):
+    # shots that end with the 128-key tiles, shots of one key, shots around the 16-key groups, shots that span several
+    # ranges of keys
+    w = wl.CONFIGS["cfg2"].scaled(n_shots=n_shots, len_lo=lens[0], len_hi=lens[1], batch=batch, k=n_shots, t_q=t_q,
+                                  n_q_heads=8, n_kv_heads=2, seed=86)
+    _check(w, 1, 0, n_shots)
+
+
+def test_rows_in_several_batches():
+    # 8 KV heads, 20000 one-token shots: a tile of 128 rows leaves 82 MB of pieces, so the four M tiles go two by two:
+    # each query's two tiles apart from the other's
+    w = wl.CONFIGS["cfg2"].scaled(n_shots=20000, len_lo=1, len_hi=1, batch=2, k=64, t_q=40, n_q_heads=32, n_kv_heads=8,
+                                  head_dim=64, seed=87)
+    _check(w, 1, 0, 64)
+
+
+def test_a_query_whose_rows_are_cut_by_a_batch():
+    # as above with three M tiles per query: batches of two tiles, so a query's masses are summed over two launches
+    w = wl.CONFIGS["cfg2"].scaled(n_shots=24000, len_lo=1, len_hi=1, batch=1, k=64, t_q=70, n_q_heads=32, n_kv_heads=8,
+                                  head_dim=64, seed=88)
+    _check(w, 1, 0, 64)
