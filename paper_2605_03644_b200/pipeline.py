@@ -106,14 +106,15 @@ class ReusePath:
         return self.k_bufs[buf][:n].view(shape), (None if self.vpool else self.v_bufs[buf][:n].view(shape))
 
     def assemble(self, layer_begin: int, layer_end: int, buf: int = 0, keep_plan: bool = False):
-        k_ctx, v_ctx = self.ctx_views(layer_end - layer_begin, buf)
+        # (the calls take the buffers as they are: the view's shape is ctx_cap's and the layer range's business)
+        k_ctx, v_ctx = self.k_bufs[buf], (None if self.vpool else self.v_bufs[buf])
         flags = (ab.ASSEMBLE_KEEP_PLAN if keep_plan else 0) | (ab.ASSEMBLE_K_ONLY if self.vpool else 0)
         ab.adapshot_assemble_kv(self.model, self.pool, self.sel_idx, layer_begin, layer_end,
                                 k_ctx, v_ctx, self.ctx_cap, self.ctx_off, self.status, flags=flags)
 
     def attend(self, q, kq, vq, out, layer_begin: int, layer_end: int, buf: int = 0, probes=None):
         """Attention of the probes (default: all of them; a sub-list must be ascending) over the cache."""
-        k_ctx, v_ctx = self.ctx_views(layer_end - layer_begin, buf)
+        k_ctx, v_ctx = self.k_bufs[buf], (None if self.vpool else self.v_bufs[buf])
         probes = self.probes if probes is None else list(probes)
         if self.vpool:
             ab.adapshot_query_attn_vpool(self.model, self.pool, self.sel_idx, k_ctx, self.ctx_cap, self.ctx_off,
@@ -136,7 +137,7 @@ class ReusePath:
         """One pass of the whole path; everything is enqueued on the current stream (the
         gathers of a multi-chunk pass on the side stream, ordered by events).
         q_chunks[i] / kq_chunks[i] / vq_chunks[i] belong to layer chunk self.chunks[i]."""
-        main = torch.cuda.current_stream()
+        main = torch.cuda.current_stream() if self.entropy_overlap or self.overlap else None
         if self.entropy_overlap:
             self.ev_begin.record(main)
             self.side.wait_event(self.ev_begin)
@@ -149,9 +150,8 @@ class ReusePath:
             for i, (lb, le) in enumerate(self.chunks):
                 self.attend_fused(q_chunks[i], kq_chunks[i], vq_chunks[i], self.out[i], lb, le)
         elif not self.overlap:
-            self.plan()
             for i, (lb, le) in enumerate(self.chunks):
-                self.assemble(lb, le, keep_plan=True)
+                self.assemble(lb, le, keep_plan=i > 0)         # the first chunk's call writes the plan
                 self.attend(q_chunks[i], kq_chunks[i], vq_chunks[i], self.out[i], lb, le)
         else:
             self.plan()
