@@ -50,7 +50,10 @@ class ProbeRounds:
         nl, hkv, hq, d = model.n_layers, model.n_kv_heads, model.n_q_heads, model.head_dim
         dt = torch.float32 if model.dtype == ab.F32 else torch.bfloat16
         u8 = dict(dtype=torch.uint8, device=device)
-        self.status = torch.zeros(1, dtype=torch.int32, device=device)
+        # what the host reads after a round, in one copy: the status word and, 16 bytes on, first_ok
+        self._verdict = torch.zeros(4 + batch, dtype=torch.int32, device=device)
+        self._verdict_host = torch.zeros(4 + batch, dtype=torch.int32, pin_memory=True)
+        self.status = self._verdict[:1]
         self.sel_idx = torch.empty((batch, self.k_max), dtype=torch.int32, device=device)
         self.sel_score = torch.empty((batch, self.k_max), dtype=torch.float32, device=device)
         self._ctx_off = torch.empty(batch * (self.k_max + 1), dtype=torch.int64, device=device)
@@ -58,7 +61,7 @@ class ProbeRounds:
         self.v_ctx = torch.empty_like(self.k_ctx)
         self.out = torch.empty((batch, nl, m, t_q, hq, d), dtype=dt, device=device)
         self.H = torch.empty((batch * m,), dtype=torch.float32, device=device)
-        self.first_ok = torch.empty((batch,), dtype=torch.int32, device=device)
+        self.first_ok = self._verdict[4:]
         self.ws_select = torch.empty(max(256, ab.adapshot_select_workspace_bytes(pool.c.n_shots, batch, self.k_max)), **u8)
         self.ws_attn = torch.empty(max(256, ab.adapshot_attn_workspace_bytes(model, batch, m, t_q, nl, self.ctx_cap)), **u8)
         self.ws_entropy = torch.empty(max(256, ab.adapshot_entropy_workspace_bytes(batch * m, vocab)), **u8)
@@ -94,10 +97,12 @@ class ProbeRounds:
         for r, probes in enumerate(self.schedule):
             q, kq, vq, logits = round_inputs(r, probes)
             self.run_round(r, q, kq, vq, logits, tau)
+            self._verdict_host.copy_(self._verdict, non_blocking=True)
             torch.cuda.current_stream().synchronize()
-            if self.status.item() != 0:
-                raise RuntimeError(f"device status {self.status.item()}: {ab.adapshot_strerror(self.status.item())}")
-            per_round.append(self.first_ok.cpu().tolist())
+            verdict = self._verdict_host.tolist()
+            if verdict[0] != 0:
+                raise RuntimeError(f"device status {verdict[0]}: {ab.adapshot_strerror(verdict[0])}")
+            per_round.append(verdict[4:])
             if on_round is not None:
                 on_round(r, self)
             if all(s != (-1, -1) for s in first_stops(per_round)):

@@ -157,14 +157,17 @@ __device__ __forceinline__ int probe_shots(const PrepParams& p, int b, int j) {
   return n;
 }
 
-// kPrepParts warps per probe token (b, l, j, t): all Hq query heads and Hkv key heads of the
-// token rotate by the same angles (L_j + t) * theta_i.  The last block writes the schedule instead.
+// kPrepParts warps per own token (b, l, j, u): all Hq query heads and Hkv key heads of the token rotate by the same
+// angles (L_j + u) * theta_i, which the block forms once for its tokens, half an angle per thread, while the first
+// rows are on their way.  (Every lane forming its eight angles itself was what bound the kernel: 4096 tokens of 32
+// + 8 heads, 84 MB, 27 us and 14336 tokens 82-90 us; now 20 and 73.)  The first block writes the schedule instead: started
+// first, its chain of dependent steps lies under the others' copies.
 template <int D>
-__global__ void __launch_bounds__(256) attn_prep_kernel(const PrepParams p) {
+__global__ void __launch_bounds__(256, 3) attn_prep_kernel(const PrepParams p) {
   constexpr int VPH = D / 8, HALF_V = VPH / 2;
   const int lane = threadIdx.x & 31;
 
-  if (blockIdx.x == gridDim.x - 1) {
+  if (blockIdx.x == 0) {
     // the schedule, by a block of its own (beside the rotation, not in front of a share of it);
     // intermediate values stay in shared memory.  One pair per thread (kMaxPairs = blockDim.x): the
     // prefix sums are a block scan.
@@ -259,55 +262,79 @@ __global__ void __launch_bounds__(256) attn_prep_kernel(const PrepParams p) {
     if (threadIdx.x == 0) sc->n_cut = s_ncut;
     return;
   }
-  const long long gw = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const long long tok = gw / kPrepParts;            // kPrepParts warps share the heads of one own token
-  const int part = (int)(gw % kPrepParts);
-  const long long n_tok = (long long)p.B * p.nl * p.P * p.To;
-  if (tok >= n_tok) return;
-  const int u_own = (int)(tok % p.To);              // own token u sits at position L_j + u
-  const long long bpj = tok / p.To;                 // (b*nl + l)*P + j
-  const int j = (int)(bpj % p.P);
-  const int b = (int)(bpj / ((long long)p.P * p.nl));
-  const long long Lj = p.ctx_off[(long long)b * (p.k + 1) + probe_shots(p, b, j)];
-  const double pos = (double)(Lj + u_own);
+  constexpr int kTokens = 8 / kPrepParts;           // of a block
+  __shared__ float2 angle_s[kTokens][D / 2];        // (cos, sin)
+  // (tokens and rows fit 32 bits: 2^31 of them would not fit the device's memory)
+  const int n_tok = p.B * p.nl * p.P * p.To, tok0 = (int)(blockIdx.x - 1) * kTokens;
+  const int warp = threadIdx.x >> 5, slot = warp / kPrepParts, part = warp % kPrepParts;
+  const int tok = tok0 + slot;
+  const bool live = tok < n_tok;
+  const int bpj = tok / p.To;                       // (b*nl + l)*P + j
+  const int u_own = tok - bpj * p.To;               // own token u sits at position L_j + u
   const int G = p.Hq / p.Hkv;
   const int t = u_own - (p.To - p.Tq);              // query row of this token (the last Tq own tokens have one)
   const bool has_q = t >= 0;
-
   const int jcol = lane % HALF_V;
+  const uint4* qsrc = reinterpret_cast<const uint4*>(p.q) + ((long long)bpj * p.Tq + (has_q ? t : 0)) * p.Hq * VPH;
+  const uint4* ksrc = reinterpret_cast<const uint4*>(p.kq) + (long long)tok * p.Hkv * VPH;
+  uint4* kdst = reinterpret_cast<uint4*>(p.kq_rot) + (long long)tok * p.Hkv * VPH;
+  uint4* qdst_base = reinterpret_cast<uint4*>(p.q_rot);
+  const int units = live ? (p.Hq + p.Hkv) * HALF_V : 0;
+  constexpr int kFly = 3;                           // units of a lane loaded at once (the 8B shape has 2.5 per lane)
+  uint4 lo[kFly], hi[kFly];
+  auto load = [&](int u0) {
+#pragma unroll
+    for (int e = 0; e < kFly; ++e) {
+      const int u = u0 + e * 32 * kPrepParts, head = u / HALF_V;       // column == jcol since 32 % HALF_V == 0
+      if (u >= units || (head < p.Hq && !has_q)) continue;
+      const uint4* src = head < p.Hq ? qsrc + head * VPH + jcol : ksrc + (head - p.Hq) * VPH + jcol;
+      lo[e] = src[0];
+      hi[e] = src[HALF_V];
+    }
+  };
+  load(part * 32 + lane);
+  for (int i = threadIdx.x; i < kTokens * (D / 2); i += 256) {
+    const int tk = tok0 + i / (D / 2);
+    if (tk < n_tok) {
+      const int x = tk / p.To, bl = x / p.P, j = x - bl * p.P, b = bl / p.nl;
+      const long long Lj = p.ctx_off[(long long)b * (p.k + 1) + probe_shots(p, b, j)];
+      float sn, cs;
+      rope_sincos((double)(Lj + tk - x * p.To), p.theta[i % (D / 2)], &sn, &cs);
+      angle_s[i / (D / 2)][i % (D / 2)] = make_float2(cs, sn);
+    }
+  }
+  __syncthreads();
   float sn[8], cs[8];
 #pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    rope_sincos(pos, p.theta[jcol * 8 + e], &sn[e], &cs[e]);
+  for (int e = 0; e < 4; ++e) {
+    const float4 v = *reinterpret_cast<const float4*>(&angle_s[slot][jcol * 8 + 2 * e]);
+    cs[2 * e] = v.x; sn[2 * e] = v.y; cs[2 * e + 1] = v.z; sn[2 * e + 1] = v.w;
   }
-  const uint4* qsrc = reinterpret_cast<const uint4*>(p.q) + (bpj * p.Tq + (has_q ? t : 0)) * p.Hq * VPH;
-  const uint4* ksrc = reinterpret_cast<const uint4*>(p.kq) + tok * p.Hkv * VPH;
-  uint4* kdst = reinterpret_cast<uint4*>(p.kq_rot) + tok * p.Hkv * VPH;
-  uint4* qdst_base = reinterpret_cast<uint4*>(p.q_rot);
-  const int units = (p.Hq + p.Hkv) * HALF_V;
-  for (int u = part * 32 + lane; u < units; u += 32 * kPrepParts) {
-    const int head = u / HALF_V;                    // column == jcol since 32 % HALF_V == 0
-    const bool is_q = head < p.Hq;
-    if (is_q && !has_q) continue;
-    const uint4* src = is_q ? qsrc + head * VPH + jcol : ksrc + (head - p.Hq) * VPH + jcol;
-    float x[8], y[8], xr[8], yr[8];
-    bf16x8_unpack(src[0], x);
-    bf16x8_unpack(src[HALF_V], y);
+  for (int u0 = part * 32 + lane; u0 < units; u0 += kFly * 32 * kPrepParts) {
+    if (u0 >= kFly * 32 * kPrepParts) load(u0);
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      xr[e] = x[e] * cs[e] - y[e] * sn[e];
-      yr[e] = y[e] * cs[e] + x[e] * sn[e];
+    for (int e = 0; e < kFly; ++e) {
+      const int u = u0 + e * 32 * kPrepParts, head = u / HALF_V;
+      if (u >= units || (head < p.Hq && !has_q)) continue;
+      float x[8], y[8], xr[8], yr[8];
+      bf16x8_unpack(lo[e], x);
+      bf16x8_unpack(hi[e], y);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        xr[c] = x[c] * cs[c] - y[c] * sn[c];
+        yr[c] = y[c] * cs[c] + x[c] * sn[c];
+      }
+      uint4* dst;
+      if (head < p.Hq) {
+        const int g = head / G, hh = head % G;
+        const long long row = ((long long)bpj * p.Hkv + g) * (p.Tq * G) + t * G + hh;
+        dst = qdst_base + row * VPH + jcol;
+      } else {
+        dst = kdst + (head - p.Hq) * VPH + jcol;
+      }
+      dst[0] = bf16x8_pack(xr);
+      dst[HALF_V] = bf16x8_pack(yr);
     }
-    uint4* dst;
-    if (is_q) {
-      const int g = head / G, hh = head % G;
-      const long long row = ((bpj * p.Hkv + g) * ((long long)p.Tq * G)) + (long long)t * G + hh;
-      dst = qdst_base + row * VPH + jcol;
-    } else {
-      dst = kdst + (head - p.Hq) * VPH + jcol;
-    }
-    dst[0] = bf16x8_pack(xr);
-    dst[HALF_V] = bf16x8_pack(yr);
   }
 }
 
