@@ -45,14 +45,17 @@ constexpr int kMaxGang = 8;          // CTAs that share one range of K/V tiles
 constexpr int kUnitCost = 4;          // fixed cost of starting a unit, in tiles (measured: about 10 k clocks)
 constexpr int kTileM = 128;          // query rows per M tile (TMEM lanes)
 constexpr int kTileN = 128;          // keys per tile
-constexpr int kAttnThreads = 320;    // warp 0 TMA, warp 1 MMA, warps 2-5 softmax A, warps 6-9 softmax B
+constexpr int kAttnThreads = 384;    // warp 0 TMA, warp 1 MMA, warp 2 gathers V (V from the pool), softmax of M tile A on warps 4-7, B on 8-11
 constexpr int kFusedThreads = 512;   // fused variant: warps 2-3 gather V and K, softmax on warps 4-11, K rotated by warps 12-15
-constexpr int kVPoolThreads = 352;   // V-from-pool variant: the cache variant's warps plus warp 10, which gathers V
 constexpr int kModeCache = 0;        // K and V tiles by TMA from the assembled cache
 constexpr int kModeFused = 1;        // K and V tiles from the pool, K re-encoded in shared memory
 constexpr int kModeVPool = 2;        // K tiles by TMA from a K-only cache, V tiles from the pool
 constexpr int kRotateWarp0 = 12;     // fused variant: first of the four warps that rotate K
 constexpr int kRotateWarps = 4;
+// Registers per thread of the warpgroups (TMA / MMA / gather, softmax twice): together what 384 threads are launched
+// with, 3 x 168.
+constexpr int kRegsIssue = 120, kRegsSoftmax = 192;
+static_assert(kRegsIssue + 2 * kRegsSoftmax <= 3 * 168, "register split");
 // Registers per thread of the fused variant's warpgroups (issue and gather, softmax twice, rotation): together
 // what 512 threads are launched with, 4 x 128.
 constexpr int kFusedRegsIssue = 64, kFusedRegsSoftmax = 176, kFusedRegsRotate = 96;
@@ -520,7 +523,7 @@ struct PoolMaps {
 // VPOOL and FUSED: V tiles are stitched from the pool by a gather warp.  FUSED: so are the K tiles, by a second
 // one; four warps then re-encode them (Eq. 7) where they lie, so that no re-encoded cache is ever written to HBM.
 template <int D, int MODE>
-__global__ void __launch_bounds__(MODE == kModeFused ? kFusedThreads : (MODE == kModeVPool ? kVPoolThreads : kAttnThreads), 1)
+__global__ void __launch_bounds__(MODE == kModeFused ? kFusedThreads : kAttnThreads, 1)
 attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kctx,
                  const __grid_constant__ CUtensorMap tm_vctx, const __grid_constant__ CUtensorMap tm_kown,
                  const __grid_constant__ CUtensorMap tm_vown, const __grid_constant__ PoolMaps vmaps,
@@ -534,8 +537,8 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   constexpr uint32_t kIdescQK = idesc_bf16_f32(kTileM, kTileN, 0);
   constexpr uint32_t kIdescPV = idesc_bf16_f32(kTileM, D, 1);
   constexpr uint32_t kTmemS = 0, kTmemO = 256;
-  constexpr int kSoftmaxWarp0 = FUSED ? 4 : 2;          // first of the eight softmax warps
-  constexpr int kGatherWarp = FUSED ? 2 : kSoftmaxWarp0 + 8;   // the warp that gathers the V tiles (fused: K by the next one)
+  constexpr int kSoftmaxWarp0 = 4;          // first of the eight softmax warps
+  constexpr int kGatherWarp = 2;   // the warp that gathers the V tiles (fused: K by the next one)
   constexpr int kBarKReady = FUSED ? kBarKRot : kBarKFull;
 
   extern __shared__ unsigned char smem_raw[];
@@ -1255,24 +1258,18 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     }
   };
 
-  if constexpr (FUSED) {                     // registers go where they are needed, one warpgroup at a time
-    if (warp < 4) {
-      regs_lower<kFusedRegsIssue>();
-      if (warp == 0) role_tma();
-      else if (warp == 1) role_mma();
-      else role_gather();
-    } else if (warp < kRotateWarp0) {
-      regs_raise<kFusedRegsSoftmax>();
-      role_softmax();
-    } else {
-      regs_lower<kFusedRegsRotate>();
-      role_rotate_k();
-    }
-  } else {
+  // registers go where they are needed, one warpgroup at a time
+  if (warp < 4) {
+    regs_lower<FUSED ? kFusedRegsIssue : kRegsIssue>();
     if (warp == 0) role_tma();
     else if (warp == 1) role_mma();
-    else if (VPOOL && warp == kGatherWarp) role_gather();
-    else role_softmax();
+    else if (FUSED || (VPOOL && warp == kGatherWarp)) role_gather();
+  } else if (!FUSED || warp < kRotateWarp0) {
+    regs_raise<FUSED ? kFusedRegsSoftmax : kRegsSoftmax>();
+    role_softmax();
+  } else if constexpr (FUSED) {
+    regs_lower<kFusedRegsRotate>();
+    role_rotate_k();
   }
 
   tc_fence_before();
@@ -1565,7 +1562,7 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
           tm_q, tm_kctx, tm_vctx, tm_kown, tm_vown, vmaps, kmaps, ap);
     } else {
       if (ads_set_max_smem(attn_main_kernel<D, kModeVPool>, smem, attr_done[2]) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-      attn_main_kernel<D, kModeVPool><<<(unsigned)(n_gangs * pl.gang), kVPoolThreads, smem, st>>>(
+      attn_main_kernel<D, kModeVPool><<<(unsigned)(n_gangs * pl.gang), kAttnThreads, smem, st>>>(
           tm_q, tm_kctx, tm_vctx, tm_kown, tm_vown, vmaps, kmaps, ap);
     }
   }
