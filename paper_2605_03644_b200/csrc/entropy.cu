@@ -47,12 +47,18 @@ __device__ __forceinline__ float ent_max3(float a, float b, float c) {   // one 
 constexpr float kEntFloor = -1.5845632502852868e29f;
 constexpr uint32_t kEntFloorBf16x2 = 0xF000F000u;
 
+// A thread's running state: two interleaved sums each, so that pairs of logits go through the two-wide fp32
+// instructions and nothing is added across a pair before the end.
+struct EntRun {
+  float m;
+  float2 s, t;
+};
+
 // Adds N logits (already raised to kEntFloor) to a state.  d = x - m is formed exactly (the row
 // maximum itself gives d = 0 and e = 1), e = 2^(d log2 e) is one multiply and one MUFU operation,
-// t accumulates e * d.  Pairs of logits go through the two-wide fp32 add / multiply / FMA forms,
-// which halves the instructions around the exponential.
+// t accumulates e * d.
 template <int N>
-__device__ __forceinline__ void ent_accumulate(EntState& st, const float (&x)[N]) {
+__device__ __forceinline__ void ent_accumulate(EntRun& st, const float (&x)[N]) {
   constexpr float kLog2e = 1.4426950408889634f;
   float vm = x[0];
   {
@@ -62,32 +68,30 @@ __device__ __forceinline__ void ent_accumulate(EntState& st, const float (&x)[N]
     if (i < N) vm = fmaxf(vm, x[i]);
   }
   if (vm > st.m) {
-    float e = __expf(st.m - vm);
-    st.t = st.s > 0.f ? (st.t + st.s * (st.m - vm)) * e : 0.f;
-    st.s *= e;
+    const float d = st.m - vm, e = __expf(d);
+    st.t.x = st.s.x > 0.f ? (st.t.x + st.s.x * d) * e : 0.f;
+    st.t.y = st.s.y > 0.f ? (st.t.y + st.s.y * d) * e : 0.f;
+    st.s.x *= e;
+    st.s.y *= e;
     st.m = vm;
   }
   if constexpr (N % 2 == 0) {
-    const float2 neg_m = make_float2(-st.m, -st.m);
-    const float2 l2e = make_float2(kLog2e, kLog2e);
-    float2 s2 = make_float2(0.f, 0.f), t2 = make_float2(0.f, 0.f);
+    const float2 neg_m = make_float2(-st.m, -st.m), l2e = make_float2(kLog2e, kLog2e);
 #pragma unroll
     for (int i = 0; i < N; i += 2) {
       const float2 d = __fadd2_rn(make_float2(x[i], x[i + 1]), neg_m);
       const float2 a = __fmul2_rn(d, l2e);
       const float2 e = make_float2(ent_ex2(a.x), ent_ex2(a.y));
-      s2 = __fadd2_rn(s2, e);
-      t2 = __ffma2_rn(e, d, t2);
+      st.s = __fadd2_rn(st.s, e);
+      st.t = __ffma2_rn(e, d, st.t);
     }
-    st.s += s2.x + s2.y;
-    st.t += t2.x + t2.y;
   } else {
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       const float d = x[i] - st.m;
       const float e = ent_ex2(d * kLog2e);
-      st.s += e;
-      st.t = fmaf(e, d, st.t);
+      st.s.x += e;
+      st.t.x = fmaf(e, d, st.t.x);
     }
   }
 }
@@ -110,7 +114,7 @@ constexpr int kEntThreads = 256;
 // bound by the 65535 limit of the other grid dimensions).
 // partial[(r * n_split + s)] = state of slice s of row r.
 template <typename T>
-__global__ void __launch_bounds__(kEntThreads, 6)
+__global__ void __launch_bounds__(kEntThreads, 5)
 entropy_partial_kernel(const T* __restrict__ logits, int V, long long row_stride, int slice, int n_split,
                        float* __restrict__ partial) {
   constexpr int kVec = 16 / sizeof(T);
@@ -119,7 +123,7 @@ entropy_partial_kernel(const T* __restrict__ logits, int V, long long row_stride
   const T* row = logits + (long long)r * row_stride;
   const int begin = sp * slice;
   const int end = V - begin <= slice ? V : begin + slice;      // (begin + slice may not fit an int)
-  EntState st{kEntFloor, 0.f, 0.f};    // every logit is at least the floor, so m starts there
+  EntRun st{kEntFloor, {0.f, 0.f}, {0.f, 0.f}};    // every logit is at least the floor, so m starts there
 
   const int n_vec = (end - begin) / kVec;                        // slice is a multiple of kVec
   auto widen = [](const uint4& raw, float (&x)[kVec]) {
@@ -194,7 +198,8 @@ entropy_partial_kernel(const T* __restrict__ logits, int V, long long row_stride
   for (int w = 1; w < kEntThreads / 32; ++w) M = fmaxf(M, sh_m[w]);
   const float d = fmaxf(st.m - M, -1.0e30f);          // <= 0; the clamp keeps s * d finite
   const float e = ent_ex2(d * kLog2e);
-  float ss = st.s * e, tt = fmaf(st.s, d, st.t) * e;
+  const float s_all = st.s.x + st.s.y;
+  float ss = s_all * e, tt = fmaf(s_all, d, st.t.x + st.t.y) * e;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     ss += __shfl_xor_sync(0xffffffffu, ss, o);
@@ -309,15 +314,17 @@ entropy_subset_finish_kernel(const float* __restrict__ partial, int n_split, int
 
 // A fixed figure rather than the SM count of the current device, so that the workspace size
 // can be asked for without a device and does not change from one GPU to another: one resident
-// wave of 256-thread CTAs at 40 registers (six per SM) on 148 SMs.
-constexpr int kEntTargetCtas = 888;
+// wave of 256-thread CTAs at 48 registers (five per SM) on 148 SMs.  (Six per SM at 40 registers, with
+// sums added across each vector: 51.9 us for 1024 rows of 128 256 bf16 logits, 188 us for 4096; now 48.7
+// and 171 us = 6.1 TB/s.)
+constexpr int kEntTargetCtas = 740;
 constexpr int kEntSliceUnit = 8192;      // entries: what a CTA's unrolled loop takes per trip (bf16)
 constexpr int kEntCtaOverhead = 2048;    // fixed cost of a CTA (start, state merge, store) in entries
 
 // Rows are cut into slices of j * kEntSliceUnit entries (the last one shorter).  A call's CTAs run
 // in ceil(R * n / kEntTargetCtas) waves of about equal length (slice + overhead), so the j that
-// minimises waves * (slice + overhead) is taken: 2048 rows of 128 256 run as 2 slices each (4.6
-// waves) rather than whole (2.3 waves, the third one a third full), 224 rows as 3 slices (one wave).  `max_states` bounds R * n (the fixed scratch of the static entry point).
+// minimises waves * (slice + overhead) is taken: 1024 rows of 128 256 run as 2 slices each (2.8
+// waves) rather than whole (1.4 waves, the second one two fifths full), 224 rows as 3 slices (one wave).  `max_states` bounds R * n (the fixed scratch of the static entry point).
 struct EntSplit { int slice, n; };
 EntSplit ent_split(int R, int V, long long max_states = 0x7fffffffll) {
   const long long unit = kEntSliceUnit;
