@@ -113,7 +113,6 @@ NCU_TRAFFIC = {
     # workload: (attn_main bytes per captured launch, layers x queries in that capture,
     #            gather bytes per captured launch, layers x queries in that capture), for the variant
     #            that `--variant auto` picks for the workload
-    "cfg2": (102.0e6, 1, 119.6e6, 1),             # profiles/attn_main_kernel_cfg2.md, profiles/gather_rope_kernel.md
     "cfg3": (2.2323e9, 16, 2.113e9, 16),          # profiles/attn_main_kernel_cfg3_2layers.md (2 layers x 8 queries, K-only cache)
     "cfg5": (2.049e9, 4, 1.0660e9, 4),            # profiles/attn_main_and_gather_cfg5_1layer_4queries.md (K-only cache)
 }
@@ -163,15 +162,12 @@ def layers_per_call_for(w: wl.Workload, ctx_cap: int, device_bytes: float = 0.0,
 
 
 def choose_variant(w: wl.Workload, ctx_cap: int, variant: str = "auto", layers_per_call: int = 0):
-    """(vpool, layers per call) of a run.  auto (the rule of ReusePath(vpool=None)): the K-only cache, V taken
-    from the pool, when the full cache of one call would be larger than L2 and a KV head has at most 1024 query
-    rows (with more rows the gather is a small share of the call and the dearer V tiles cost more than half a
-    gather saves); the full cache otherwise."""
+    """(vpool, layers per call) of a run.  auto: the rule of ReusePath(vpool=None), for the full cache of one call."""
+    from paper_2605_03644_b200.pipeline import v_from_pool_pays
     vpool = variant == "vpool"
     if variant == "auto":
         lpc_full = layers_per_call or layers_per_call_for(w, ctx_cap)
-        vpool = (w.batch * lpc_full * ctx_cap * w.bytes_per_token_layer > (128 << 20)
-                 and w.t_q * w.group <= 1024)
+        vpool = v_from_pool_pays(w.batch * lpc_full * ctx_cap * w.bytes_per_token_layer, float(wl.shot_lengths(w).mean()))
     return vpool, (layers_per_call or layers_per_call_for(w, ctx_cap, k_only=vpool))
 
 
@@ -827,7 +823,7 @@ def main():
                     help="materialise: gather + re-encode K and V into a contiguous cache, then attend; "
                          "vpool: gather + re-encode K only, attention takes V tiles from the pool; "
                          "fused: attention reads the pool and re-encodes K in shared memory; "
-                         "auto (default): vpool when a call's cache is larger than L2, else materialise")
+                         "auto (default): vpool where a call's cache is large enough for it (v_from_pool_pays), else materialise")
     ap.add_argument("--k-pos-mode", type=int, default=0, choices=[0, 1],
                     help="0: pool K carries no position (default); 1: pool K rotated at shot-local positions "
                          "(the paper's store), the re-encode is one angle per shot")

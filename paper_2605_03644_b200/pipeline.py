@@ -38,6 +38,16 @@ def layer_chunks(n_layers: int, lpc: int, ramp: bool = False):
     return out
 
 
+def v_from_pool_pays(cache_bytes: float, mean_shot_tokens: float) -> bool:
+    """The measured choice between a K-only cache, V tiles taken from the pool, and a full cache (`cache_bytes` of
+    K and V per call).  Leaving V where it is saves half of the gather and costs the attention 2-3 % (V tiles stitched
+    from runs of pool rows) and one small launch.  One query of one layer: full / K-only 59 / 60 us at 16 shots of 160
+    tokens, 67.6 / 67.5 at 32 (33 MB), 82.7 / 79.3 at 64, 109 / 101 at 128; three layers of 64 K tokens 1712 / 1640.
+    Short shots make many runs per tile: at 24 tokens on average 90 / 95 us (one query, 12 K tokens) and 1395 / 1401
+    (32 queries), at 36 tokens 1042 / 978, at 48 2689 / 2405; at 12 744 / 946."""
+    return cache_bytes > (32 << 20) and mean_shot_tokens >= 32
+
+
 class ReusePath:
     def __init__(self, model: ab.ModelT, pool: ab.Pool, batch: int, k: int, probes: Sequence[int],
                  t_q: int, vocab: int, ctx_cap: int, layers_per_call: Optional[int] = None,
@@ -59,12 +69,8 @@ class ReusePath:
         self.chunks = layer_chunks(self.nl, self.lpc, ramp)
         self.fused = bool(fused)
         if vpool is None:
-            # measured choice: a cache that stays in L2 between the gather and the attention (a single
-            # layer of one query) is cheapest to read in full; anything larger is better off with the
-            # K-only cache, whose gather moves half the bytes - unless a KV head has so many query rows
-            # (more than 1024) that the gather is a small share of the call anyway
-            vpool = (batch * self.lpc * self.ctx_cap * 2 * hkv * d * (4 if model.dtype == ab.F32 else 2) > (128 << 20)
-                     and t_q * (hq // hkv) <= 1024)
+            cache = batch * self.lpc * self.ctx_cap * 2 * hkv * d * (4 if model.dtype == ab.F32 else 2)
+            vpool = v_from_pool_pays(cache, pool.c.pool_tokens / max(1, pool.c.n_shots))
         self.vpool = bool(vpool) and not self.fused and model.dtype != ab.F32
         self.overlap = bool(overlap) and len(self.chunks) > 1 and not self.fused
         n_ctx = batch * self.lpc * self.ctx_cap * hkv * d

@@ -47,3 +47,10 @@ def test_layer_chunks_cover_the_layers_in_order():
     assert [e - b for b, e in layer_chunks(32, 8, True)] == [2, 6, 8, 8, 6, 2]
     assert [e - b for b, e in layer_chunks(32, 32, True)] == [32]
     assert [e - b for b, e in layer_chunks(32, 8, False)] == [8, 8, 8, 8]
+
+
+def test_v_from_pool_rule_on_both_sides_of_its_lines():
+    from paper_2605_03644_b200.pipeline import v_from_pool_pays
+    assert v_from_pool_pays((32 << 20) + 1, 32.0)
+    assert not v_from_pool_pays(32 << 20, 160.0)            # a cache of at most 32 MiB per call stays full
+    assert not v_from_pool_pays(1 << 30, 31.9)              # short shots: too many runs per V tile
