@@ -348,6 +348,49 @@ ADAPSHOT_API int adapshot_entropy_static(const void* logits, int32_t dtype, int3
                             int64_t row_stride, float* H, float tau, int32_t rows_per_group,
                             int32_t* first_ok, int32_t* status, void* stream);
 
+/* ---- Steps 1 to 4 of a pass in one call (no counterpart in the paper: the calls above in the
+ * order of a pass, so that a caller whose pass is a few dozen microseconds of kernels does not
+ * spend more than that on crossing into the library).  Selection, then for every chunk of layers
+ * the gather (the first one writes the plan) and the attention, then the entropies.  The
+ * pointers are those of the calls; q, kq, vq and out are HOST arrays of n_chunks device
+ * pointers, layer_end HOST int32 [n_chunks] (ascending, chunk i begins where chunk i-1 ends).
+ * k_ctx / v_ctx hold one chunk at a time.  variant: ADAPSHOT_PASS_FULL (K and V assembled),
+ * _VPOOL (K only, V from the pool; v_ctx unused) or _FUSED (nothing assembled).  The struct is
+ * read during the call only.  Returns the first error; steps before it have been enqueued.   */
+#define ADAPSHOT_PASS_FULL  0
+#define ADAPSHOT_PASS_VPOOL 1
+#define ADAPSHOT_PASS_FUSED 2
+typedef struct adapshot_pass {
+  const adapshot_model_t* model;
+  const adapshot_pool_t*  pool;
+  const int32_t*          probe_nshots;   /* host [P] */
+  const int32_t*          layer_end;      /* host [n_chunks] */
+  int32_t B, k, P, Tq, n_chunks, variant;
+  int32_t V, logits_dtype;
+  int64_t logits_stride, ctx_cap;
+  const float* q_emb;
+  const void* const* q;
+  const void* const* kq;
+  const void* const* vq;
+  void* const* out;
+  const void* logits;                     /* [B*P][logits_stride] */
+  int32_t* sel_idx;
+  float*   sel_score;                     /* or NULL */
+  int64_t* ctx_off;
+  void*    k_ctx;
+  void*    v_ctx;
+  float*   H;
+  int32_t* first_ok;                      /* or NULL */
+  void*    ws_select;
+  void*    ws_attn;
+  void*    ws_entropy;
+  size_t   ws_select_bytes, ws_attn_bytes, ws_entropy_bytes;
+  int32_t* status;
+  float    tau;
+  int32_t  reserved;
+} adapshot_pass_t;
+ADAPSHOT_API int adapshot_reuse_pass(const adapshot_pass_t* pass, void* stream);
+
 /* ---- Measurement aid (no counterpart in the paper).  adapshot_profile(1) makes every
  * later adapshot_query_attn / adapshot_query_attn_fused call record two CUDA events on the
  * caller's stream around its main (tensor-core) kernel; adapshot_profile_attn_main_ms()

@@ -33,7 +33,7 @@ EXPORTS = [
     "adapshot_attn_vpool_workspace_bytes", "adapshot_query_attn_vpool",
     "adapshot_tree_layout", "adapshot_tree_attn", "adapshot_decode_workspace_bytes", "adapshot_decode_attn",
     "adapshot_entropy_workspace_bytes", "adapshot_entropy", "adapshot_entropy_subset",
-    "adapshot_entropy_static",
+    "adapshot_entropy_static", "adapshot_reuse_pass",
     "adapshot_profile", "adapshot_profile_attn_main_ms", "adapshot_selftest_wait_timeout",
     "adapshot_strerror", "adapshot_version",
 ]
@@ -188,6 +188,61 @@ class Pool:
         tokens = int(k.shape[1]) if k is not None else 0
         self.c = PoolT(n_shots, int(emb.shape[1]) if emb is not None else 0, tokens,
                        _ptr(shot_off), _ptr(k), _ptr(v), _ptr(emb))
+
+
+class PassT(C.Structure):
+    _fields_ = [("model", C.POINTER(ModelT)), ("pool", C.POINTER(PoolT)), ("probe_nshots", C.POINTER(_i32)),
+                ("layer_end", C.POINTER(_i32)), ("B", _i32), ("k", _i32), ("P", _i32), ("Tq", _i32), ("n_chunks", _i32),
+                ("variant", _i32), ("V", _i32), ("logits_dtype", _i32), ("logits_stride", _i64), ("ctx_cap", _i64),
+                ("q_emb", _vp), ("q", C.POINTER(_vp)), ("kq", C.POINTER(_vp)), ("vq", C.POINTER(_vp)),
+                ("out", C.POINTER(_vp)), ("logits", _vp), ("sel_idx", _vp), ("sel_score", _vp), ("ctx_off", _vp),
+                ("k_ctx", _vp), ("v_ctx", _vp), ("H", _vp), ("first_ok", _vp), ("ws_select", _vp), ("ws_attn", _vp),
+                ("ws_entropy", _vp), ("ws_select_bytes", _sz), ("ws_attn_bytes", _sz), ("ws_entropy_bytes", _sz),
+                ("status", _vp), ("tau", _f), ("reserved", _i32)]
+
+
+PASS_FULL, PASS_VPOOL, PASS_FUSED = 0, 1, 2
+_reuse_pass = _sig("adapshot_reuse_pass", C.c_int, [C.POINTER(PassT), _vp])
+
+
+class Pass:
+    """The struct of adapshot_reuse_pass: the fixed part (buffers, sizes) is filled in once; a call sets the pointers
+    of that pass's tensors.  The tensors behind the fixed part belong to the caller, who keeps them."""
+
+    def __init__(self, model: ModelT, pool: Pool, B: int, k: int, probes: Sequence[int], Tq: int, layer_end: Sequence[int],
+                 variant: int, ctx_cap: int, buffers: dict):
+        n = len(layer_end)
+        self.n, self.rows = n, B * len(probes)
+        self._keep = (model, pool, (_i32 * len(probes))(*[int(x) for x in probes]), (_i32 * n)(*[int(x) for x in layer_end]))
+        self.ptrs = {name: (_vp * n)() for name in ("q", "kq", "vq", "out")}
+        layers = [le - lb for lb, le in zip([0, *layer_end[:-1]], layer_end)]
+        row = self.rows * Tq * model.head_dim                       # elements of one head and layer
+        self.sizes = {name: [row * h * l for l in layers] for name, h in
+                      (("q", model.n_q_heads), ("kq", model.n_kv_heads), ("vq", model.n_kv_heads), ("out", model.n_q_heads))}
+        self.c = PassT(model=C.pointer(model), pool=C.pointer(pool.c), probe_nshots=self._keep[2], layer_end=self._keep[3],
+                       B=B, k=k, P=len(probes), Tq=Tq, n_chunks=n, variant=variant, ctx_cap=ctx_cap, **self.ptrs)
+        for name, t in buffers.items():
+            setattr(self.c, name, _ptr(t))
+            if name.startswith("ws_"):
+                setattr(self.c, name + "_bytes", t.numel() * t.element_size())
+        self.ref = C.byref(self.c)
+
+    def __call__(self, q_emb: torch.Tensor, q, kq, vq, out, logits: torch.Tensor, tau: float):
+        c, n = self.c, self.n
+        if logits.stride(1) != 1 or not logits.is_cuda:
+            raise ValueError("logit rows must be contiguous, on the GPU")
+        if logits.shape[0] != self.rows or len(q) < n or len(kq) < n or len(vq) < n or len(out) < n:
+            raise ValueError("one logit row per query and probe, one tensor per layer chunk")
+        for name, ts in (("q", q), ("kq", kq), ("vq", vq), ("out", out)):
+            p, size = self.ptrs[name], self.sizes[name]
+            for i in range(n):
+                if ts[i].numel() != size[i]:
+                    raise ValueError(f"{name}[{i}] has {ts[i].numel()} elements, expected {size[i]}")
+                p[i] = _ptr(ts[i])
+        c.q_emb, c.logits, c.tau = _ptr(q_emb), logits.data_ptr(), tau
+        c.V, c.logits_stride = logits.shape[1], logits.stride(0)
+        c.logits_dtype = F32 if logits.dtype == torch.float32 else BF16
+        _check(_reuse_pass(self.ref, _stream()))
 
 
 def adapshot_select_workspace_bytes(n_shots: int, B: int, k: int) -> int:

@@ -1577,7 +1577,10 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
   cp.sched = sched; cp.o_part = o_part; cp.ml_part = ml_part;
   cp.out = ap.out; cp.lse = lse;
   cp.Tq = Tq; cp.Hq = Hq; cp.G = G; cp.n_mp = pl.n_mp;
-  const dim3 grid((unsigned)n_gangs, (unsigned)((Tq * G + 8 * kCombineRows - 1) / (8 * kCombineRows)),
+  // (at most one cut unit per range, and no more than there are units: a small call would launch mostly empty blocks)
+  const long long units = (long long)B * P * nl * Hkv;
+  const dim3 grid((unsigned)(units < n_gangs ? units : n_gangs),
+                  (unsigned)((Tq * G + 8 * kCombineRows - 1) / (8 * kCombineRows)),
                   D / (16 * kCombineSteps));
   attn_combine_kernel<D><<<grid, 256, 0, st>>>(cp);
   return ads_launch_status();

@@ -93,6 +93,16 @@ class ReusePath:
         self.entropy_overlap = bool(entropy_overlap)
         self.side = torch.cuda.Stream(device=device)
         self.ev_begin, self.ev_entropy = torch.cuda.Event(), torch.cuda.Event()
+        buffers = dict(sel_idx=self.sel_idx, sel_score=self.sel_score, ctx_off=self.ctx_off, H=self.H,
+                       first_ok=self.first_ok, ws_select=self.ws_select, ws_attn=self.ws_attn,
+                       ws_entropy=self.ws_entropy, status=self.status)
+        if not self.fused:
+            buffers["k_ctx"] = self.k_bufs[0]
+            if not self.vpool:
+                buffers["v_ctx"] = self.v_bufs[0]
+        self.whole = ab.Pass(model, pool, batch, k, self.probes, t_q, [le for _, le in self.chunks],
+                             ab.PASS_FUSED if self.fused else ab.PASS_VPOOL if self.vpool else ab.PASS_FULL,
+                             self.ctx_cap, buffers)
         if self.overlap:
             self.ev_plan = torch.cuda.Event()
             self.ev_asm = [torch.cuda.Event() for _ in range(2)]
@@ -143,7 +153,10 @@ class ReusePath:
         """One pass of the whole path; everything is enqueued on the current stream (the
         gathers of a multi-chunk pass on the side stream, ordered by events).
         q_chunks[i] / kq_chunks[i] / vq_chunks[i] belong to layer chunk self.chunks[i]."""
-        main = torch.cuda.current_stream() if self.entropy_overlap or self.overlap else None
+        if not self.entropy_overlap and not self.overlap:      # one stream, the calls in order: one call
+            self.whole(q_emb, q_chunks, kq_chunks, vq_chunks, self.out, logits, tau)
+            return self.out, self.H, self.first_ok
+        main = torch.cuda.current_stream()
         if self.entropy_overlap:
             self.ev_begin.record(main)
             self.side.wait_event(self.ev_begin)
