@@ -32,6 +32,7 @@ plan_offsets_kernel(const int32_t* __restrict__ sel_idx, const long long* __rest
                     long long* __restrict__ ctx_off, int32_t* __restrict__ status) {
   __shared__ long long warp_tot[kPlanThreads / 32];
   __shared__ long long carry_sh;
+  ads_dependency_wait();
   const int b = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) carry_sh = 0;
@@ -171,6 +172,7 @@ gather_rope_kernel(const __grid_constant__ GatherArgs a) {
     mbar_fence_init();
   }
   __syncthreads();
+  ads_dependency_wait();
 
   if (warp == kRotWarps) {
     // ---------------------------------------------------------------- loading warp
@@ -403,10 +405,10 @@ int launch_gather(GatherArgs a, cudaStream_t st) {
   const int most = (int)(kStages * kStageMax);
   if (a.v_ctx != nullptr) {
     if (ads_set_max_smem(gather_rope_kernel<T, D, true>, most, attr_done[0]) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-    gather_rope_kernel<T, D, true><<<grid, kGatherThreads, smem, st>>>(a);
+    ads_launch_dependent(gather_rope_kernel<T, D, true>, grid, kGatherThreads, smem, st, a);
   } else {
     if (ads_set_max_smem(gather_rope_kernel<T, D, false>, most, attr_done[1]) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-    gather_rope_kernel<T, D, false><<<grid, kGatherThreads, smem, st>>>(a);
+    ads_launch_dependent(gather_rope_kernel<T, D, false>, grid, kGatherThreads, smem, st, a);
   }
   return ads_launch_status();
 }
@@ -457,7 +459,7 @@ extern "C" int adapshot_assemble_kv_from(const adapshot_model_t* model, const ad
   }
 
   if (!keep_plan) {
-    plan_offsets_kernel<<<B, kPlanThreads, 0, st>>>(
+    ads_launch_dependent(plan_offsets_kernel, B, kPlanThreads, 0, st,
         sel_idx, reinterpret_cast<const long long*>(pool->shot_off), pool->n_shots, k, ctx_cap, ctx_cap > 0,
         reinterpret_cast<long long*>(ctx_off), status);
     if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;

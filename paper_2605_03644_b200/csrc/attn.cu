@@ -169,6 +169,7 @@ template <int D>
 __global__ void __launch_bounds__(256, 3) attn_prep_kernel(const PrepParams p) {
   constexpr int VPH = D / 8, HALF_V = VPH / 2;
   const int lane = threadIdx.x & 31;
+  ads_dependency_wait();
 
   if (blockIdx.x == 0) {
     // the schedule, by a block of its own (beside the rotation, not in front of a share of it);
@@ -357,6 +358,7 @@ struct RowMapParams {
 // One warp per selected shot: its run of positions is written with whole lines (a search per position
 // took 38 us for 32 queries of 66 K positions and 8.3 us for 8 of 33 K; 3 us for those now).
 __global__ void __launch_bounds__(256) attn_row_map_kernel(const RowMapParams p) {
+  ads_dependency_wait();
   const int lane = threadIdx.x & 31;
   const long long w = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (w >= (long long)p.B * p.k) return;
@@ -580,6 +582,7 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
     tmem_relinquish();
   }
+  ads_dependency_wait();
   // the CTA's part of the schedule, fetched by two otherwise idle warps while the rest is set up
   constexpr int kCachePairs = sched_cache_pairs(MODE);
   SchedCache<kCachePairs>* cache = reinterpret_cast<SchedCache<kCachePairs>*>(base_ptr + SM::kOffBar + 256);
@@ -1301,6 +1304,7 @@ constexpr int kCombineSteps = 2;     // 16-column steps per warp (blockIdx.z cov
 // M tile) and a store fills one 32-byte sector per row.
 template <int D>
 __global__ void __launch_bounds__(256) attn_combine_kernel(const CombineParams p) {
+  ads_dependency_wait();
   const Sched* sc = p.sched;
   if (blockIdx.x >= sc->n_cut) return;
   const Sched::Cut c = sc->cut[blockIdx.x];
@@ -1517,7 +1521,7 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
     rm.off_map = mode == kModeFused && model->k_pos_mode == 1 ? off_map : nullptr;
     rm.ctx_cap = ctx_cap;
     rm.B = B; rm.k = k; rm.n_shots = fused->pool->n_shots;
-    attn_row_map_kernel<<<(unsigned)(((long long)B * k + 7) / 8), 256, 0, st>>>(rm);
+    ads_launch_dependent(attn_row_map_kernel, (unsigned)(((long long)B * k + 7) / 8), 256, 0, st, rm);
     if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
   }
 
@@ -1532,7 +1536,7 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
   for (int i = 0; i < D / 2; ++i) pp.theta[i] = pow(model->rope_base, -2.0 * (double)i / (double)D);
   for (int i = 0; i < kMaxProbes; ++i) pp.nshots[i] = i < P ? probe_nshots[i] : 0;
   const long long n_tok = (long long)B * nl * P * To;
-  attn_prep_kernel<D><<<(unsigned)((n_tok * kPrepParts + 7) / 8) + 1, 256, 0, st>>>(pp);   // + the schedule block
+  ads_launch_dependent(attn_prep_kernel<D>, (unsigned)((n_tok * kPrepParts + 7) / 8) + 1, 256, 0, st, pp);   // + the schedule block
   if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
 
   // ---- main kernel
@@ -1550,7 +1554,7 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
   if (g_profile) ADS_CHECK_CUDA(cudaEventRecord(g_profile_ev[0], st));
   if (mode == kModeCache) {
     if (ads_set_max_smem(attn_main_kernel<D, kModeCache>, smem, attr_done[0]) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-    attn_main_kernel<D, kModeCache><<<(unsigned)(n_gangs * pl.gang), kAttnThreads, smem, st>>>(
+    ads_launch_dependent(attn_main_kernel<D, kModeCache>, (unsigned)(n_gangs * pl.gang), kAttnThreads, smem, st,
         tm_q, tm_kctx, tm_vctx, tm_kown, tm_vown, vmaps, kmaps, ap);
   } else {
     ap.row_map = row_map; ap.off_map = off_map; ap.k_pos_mode = model->k_pos_mode;
@@ -1558,11 +1562,11 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
     for (int i = 0; i < D / 2; ++i) ap.theta[i] = pp.theta[i];
     if (mode == kModeFused) {
       if (ads_set_max_smem(attn_main_kernel<D, kModeFused>, smem, attr_done[1]) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-      attn_main_kernel<D, kModeFused><<<(unsigned)(n_gangs * pl.gang), kFusedThreads, smem, st>>>(
+      ads_launch_dependent(attn_main_kernel<D, kModeFused>, (unsigned)(n_gangs * pl.gang), kFusedThreads, smem, st,
           tm_q, tm_kctx, tm_vctx, tm_kown, tm_vown, vmaps, kmaps, ap);
     } else {
       if (ads_set_max_smem(attn_main_kernel<D, kModeVPool>, smem, attr_done[2]) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-      attn_main_kernel<D, kModeVPool><<<(unsigned)(n_gangs * pl.gang), kAttnThreads, smem, st>>>(
+      ads_launch_dependent(attn_main_kernel<D, kModeVPool>, (unsigned)(n_gangs * pl.gang), kAttnThreads, smem, st,
           tm_q, tm_kctx, tm_vctx, tm_kown, tm_vown, vmaps, kmaps, ap);
     }
   }
@@ -1582,7 +1586,7 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
   const dim3 grid((unsigned)(units < n_gangs ? units : n_gangs),
                   (unsigned)((Tq * G + 8 * kCombineRows - 1) / (8 * kCombineRows)),
                   D / (16 * kCombineSteps));
-  attn_combine_kernel<D><<<grid, 256, 0, st>>>(cp);
+  ads_launch_dependent(attn_combine_kernel<D>, grid, 256, 0, st, cp);
   return ads_launch_status();
 }
 
@@ -1730,6 +1734,7 @@ namespace {
 struct TreePosArgs { int n[kMaxProbes]; };
 __global__ void tree_positions_kernel(const long long* __restrict__ ctx_off, int B, int k, int P, int Tq,
                                            const TreePosArgs a, long long* __restrict__ pos) {
+  ads_dependency_wait();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long long)B * P * Tq) return;
   const int t = (int)(i % Tq), j = (int)((i / Tq) % P), b = (int)(i / ((long long)Tq * P));
@@ -1787,7 +1792,7 @@ extern "C" int adapshot_tree_attn(const adapshot_model_t* model, const void* k_c
   TreePosArgs a;
   for (int i = 0; i < kMaxProbes; ++i) a.n[i] = i < P ? nshots[i] : 0;
   const long long n = (long long)B * P * Tq;
-  tree_positions_kernel<<<(unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+  ads_launch_dependent(tree_positions_kernel, (unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream),
       reinterpret_cast<const long long*>(ctx_off), B, k, P, Tq, a, reinterpret_cast<long long*>(pos_seq));
   return ads_launch_status();
 }

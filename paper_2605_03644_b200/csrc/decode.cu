@@ -589,11 +589,11 @@ int launch(const CUtensorMap* m, const DecodeParams& p, cudaStream_t st) {
   const int smem = (int)DecodeSmem<D>::kTotal;
   static bool attr_done[kAdsMaxDevices] = {false};
   if (ads_set_max_smem(decode_rows_kernel<D, MB>, smem, attr_done) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-  if (ads_launch_dependent(decode_rows_kernel<D, MB>, dim3((unsigned)p.n_cta), dim3(kThreads), smem, st, m[0], m[1], m[2],
-                           m[3], p) != ADAPSHOT_OK)
-    return ADAPSHOT_ECUDA;
+  ads_launch_dependent(decode_rows_kernel<D, MB>, (unsigned)p.n_cta, kThreads, smem, st, m[0], m[1], m[2], m[3], p);
+  if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
   const dim3 grid((unsigned)((long long)p.B * p.nl * p.Hkv), (unsigned)p.rows);
-  return ads_launch_dependent(decode_combine_kernel<D>, grid, dim3(32 * kMergeWarps), 0, st, p);
+  ads_launch_dependent(decode_combine_kernel<D>, grid, 32 * kMergeWarps, 0, st, p);
+  return ads_launch_status();
 }
 
 }  // namespace

@@ -117,6 +117,7 @@ template <typename T>
 __global__ void __launch_bounds__(kEntThreads, 5)
 entropy_partial_kernel(const T* __restrict__ logits, int V, long long row_stride, int slice, int n_split,
                        float* __restrict__ partial) {
+  ads_dependency_wait();
   constexpr int kVec = 16 / sizeof(T);
   constexpr float kLog2e = 1.4426950408889634f;
   const int r = blockIdx.x / n_split, sp = blockIdx.x % n_split;
@@ -221,6 +222,7 @@ entropy_partial_kernel(const T* __restrict__ logits, int V, long long row_stride
 __global__ void __launch_bounds__(256)
 entropy_finish_kernel(const float* __restrict__ partial, int n_split, int R, int rows_per_group,
                       float tau, float* __restrict__ H, int32_t* __restrict__ first_ok) {
+  ads_dependency_wait();
   extern __shared__ float sh_h[];
   const int g = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
@@ -262,6 +264,7 @@ entropy_subset_finish_kernel(const float* __restrict__ partial, int n_split, int
                              const int32_t* __restrict__ subset_ids, int n_subset, int renorm,
                              float tau, float* __restrict__ H, int32_t* __restrict__ first_ok,
                              int32_t* __restrict__ status) {
+  ads_dependency_wait();
   extern __shared__ float sh_h[];
   const int g = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
@@ -378,13 +381,13 @@ extern "C" int adapshot_entropy(const void* logits, int32_t dtype, int32_t R, in
   const unsigned grid = (unsigned)((long long)R * n_split);
   float* partial = static_cast<float*>(ws);
   if (dtype == ADAPSHOT_F32)
-    entropy_partial_kernel<float><<<grid, kEntThreads, 0, st>>>(
+    ads_launch_dependent(entropy_partial_kernel<float>, grid, kEntThreads, 0, st,
         static_cast<const float*>(logits), V, row_stride, slice, n_split, partial);
   else
-    entropy_partial_kernel<__nv_bfloat16><<<grid, kEntThreads, 0, st>>>(
+    ads_launch_dependent(entropy_partial_kernel<__nv_bfloat16>, grid, kEntThreads, 0, st,
         static_cast<const __nv_bfloat16*>(logits), V, row_stride, slice, n_split, partial);
   if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-  entropy_finish_kernel<<<R / rows_per_group, 256, rows_per_group * sizeof(float), st>>>(
+  ads_launch_dependent(entropy_finish_kernel, R / rows_per_group, 256, rows_per_group * sizeof(float), st,
       partial, n_split, R, rows_per_group, tau, H, first_ok);
   return ads_launch_status();
 }
@@ -417,16 +420,16 @@ extern "C" int adapshot_entropy_subset(const void* logits, int32_t dtype, int32_
   const size_t sh = rows_per_group * sizeof(float);
   if (dtype == ADAPSHOT_F32) {
     const float* lg = static_cast<const float*>(logits);
-    entropy_partial_kernel<float><<<grid, kEntThreads, 0, st>>>(lg, V, row_stride, slice, n_split, partial);
+    ads_launch_dependent(entropy_partial_kernel<float>, grid, kEntThreads, 0, st, lg, V, row_stride, slice, n_split, partial);
     if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-    entropy_subset_finish_kernel<float><<<R / rows_per_group, 256, sh, st>>>(
+    ads_launch_dependent(entropy_subset_finish_kernel<float>, R / rows_per_group, 256, sh, st,
         partial, n_split, R, rows_per_group, lg, row_stride, V, subset_ids, n_subset, renorm, tau, H, first_ok,
         status);
   } else {
     const __nv_bfloat16* lg = static_cast<const __nv_bfloat16*>(logits);
-    entropy_partial_kernel<__nv_bfloat16><<<grid, kEntThreads, 0, st>>>(lg, V, row_stride, slice, n_split, partial);
+    ads_launch_dependent(entropy_partial_kernel<__nv_bfloat16>, grid, kEntThreads, 0, st, lg, V, row_stride, slice, n_split, partial);
     if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-    entropy_subset_finish_kernel<__nv_bfloat16><<<R / rows_per_group, 256, sh, st>>>(
+    ads_launch_dependent(entropy_subset_finish_kernel<__nv_bfloat16>, R / rows_per_group, 256, sh, st,
         partial, n_split, R, rows_per_group, lg, row_stride, V, subset_ids, n_subset, renorm, tau, H, first_ok,
         status);
   }
@@ -492,13 +495,13 @@ extern "C" int adapshot_entropy_static(const void* logits, int32_t dtype, int32_
   // every (row, split) state this call reads is written by the first kernel, so
   // nothing in the shared array has to start at zero
   if (dtype == ADAPSHOT_F32)
-    entropy_partial_kernel<float><<<grid, kEntThreads, 0, st>>>(
+    ads_launch_dependent(entropy_partial_kernel<float>, grid, kEntThreads, 0, st,
         static_cast<const float*>(logits), V, row_stride, slice, n_split, partial);
   else
-    entropy_partial_kernel<__nv_bfloat16><<<grid, kEntThreads, 0, st>>>(
+    ads_launch_dependent(entropy_partial_kernel<__nv_bfloat16>, grid, kEntThreads, 0, st,
         static_cast<const __nv_bfloat16*>(logits), V, row_stride, slice, n_split, partial);
   if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-  entropy_finish_kernel<<<R / rows_per_group, 256, rows_per_group * sizeof(float), st>>>(
+  ads_launch_dependent(entropy_finish_kernel, R / rows_per_group, 256, rows_per_group * sizeof(float), st,
       partial, n_split, R, rows_per_group, tau, H, first_ok);
   return ads_launch_status();
 }

@@ -29,6 +29,7 @@ template <int NV>
 __global__ void __launch_bounds__(256)
 cosine_keys_kernel(const float* __restrict__ emb, const float* __restrict__ q_emb, int N, int E,
                    int B, unsigned long long* __restrict__ keys) {
+  ads_dependency_wait();
   const int lane = threadIdx.x & 31;
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (row >= N) return;
@@ -113,6 +114,7 @@ cosine_mma_kernel(const float* __restrict__ emb, const float* __restrict__ q_emb
                   unsigned long long* __restrict__ keys) {
   __shared__ double dot_s[kMmaWarps][8 * NB][33];
   __shared__ double nn_s[kMmaWarps][32], qq_s[kMmaWarps][8 * NB];
+  ads_dependency_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
   const int row0 = blockIdx.x * 32, q0 = blockIdx.y * 8 * NB;
@@ -243,6 +245,7 @@ radix_topk_kernel(const unsigned long long* __restrict__ all_keys, int N, int k,
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x;
   const unsigned long long* keys = all_keys + (long long)b * N;
+  ads_dependency_wait();
   constexpr int kFly = 8;
 
   unsigned long long lo = 0, hi = ~0ull;           // keys below lo: taken; above hi: out
@@ -409,6 +412,7 @@ rank_topk_kernel(const unsigned long long* __restrict__ all_keys, int N, int k,
                  int32_t* __restrict__ final_idx, float* __restrict__ final_score) {
   __shared__ unsigned long long keys[kRankTile];
   __shared__ int part_cnt[kRankThreads];
+  ads_dependency_wait();
   const int b = blockIdx.y;
   const int tid = threadIdx.x;
   const unsigned long long* gkeys = all_keys + (long long)b * N;
@@ -454,7 +458,7 @@ int ads_topk_from_keys(const unsigned long long* keys, int N, int B, int k, int3
   if (N > kSortCap && k > kSortCap / 2) return ADAPSHOT_EUNSUPPORTED;
   if (rank_by_counting(N, B)) {
     dim3 grid((N + kRankCand - 1) / kRankCand, B);
-    rank_topk_kernel<<<grid, kRankThreads, 0, st>>>(keys, N, k, sel_idx, sel_score);
+    ads_launch_dependent(rank_topk_kernel, grid, kRankThreads, 0, st, keys, N, k, sel_idx, sel_score);
     return ads_launch_status();
   }
   // candidates worth sorting: the power of two the sort pads to (bins of the second pass rarely hold two keys)
@@ -462,7 +466,7 @@ int ads_topk_from_keys(const unsigned long long* keys, int N, int B, int k, int3
   while (want < k) want <<= 1;
   static bool attr_set[kAdsMaxDevices] = {false};
   if (ads_set_max_smem(radix_topk_kernel, kSortCap * (8 + 4) + kSelBins * 4, attr_set) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-  radix_topk_kernel<<<(unsigned)B, kSelThreads, want * (8 + 4) + kSelBins * 4, st>>>(keys, N, k, want, sel_idx, sel_score);
+  ads_launch_dependent(radix_topk_kernel, (unsigned)B, kSelThreads, want * (8 + 4) + kSelBins * 4, st, keys, N, k, want, sel_idx, sel_score);
   return ads_launch_status();
 }
 
@@ -490,12 +494,12 @@ extern "C" int adapshot_select(const adapshot_pool_t* pool, const float* q_emb, 
   if (B > 2 && E % 16 == 0) {          // (4096 x 384: 4.7 us for two queries by warps, 3.4 for four by matrix tiles)
     const unsigned rows = (unsigned)((N + 31) / 32);
     if (B <= 8)
-      cosine_mma_kernel<1><<<dim3(rows, 1), 32 * kMmaWarps, 0, st>>>(pool->emb, q_emb, N, E, B, keys);
+      ads_launch_dependent(cosine_mma_kernel<1>, dim3(rows, 1), 32 * kMmaWarps, 0, st, pool->emb, q_emb, N, E, B, keys);
     else
-      cosine_mma_kernel<2><<<dim3(rows, (unsigned)((B + 15) / 16)), 32 * kMmaWarps, 0, st>>>(pool->emb, q_emb, N, E, B, keys);
+      ads_launch_dependent(cosine_mma_kernel<2>, dim3(rows, (unsigned)((B + 15) / 16)), 32 * kMmaWarps, 0, st, pool->emb, q_emb, N, E, B, keys);
   } else {
     const unsigned grid = (unsigned)((N + 7) / 8);
-    auto run = [&](auto kernel) { kernel<<<grid, 256, 0, st>>>(pool->emb, q_emb, N, E, B, keys); };
+    auto run = [&](auto kernel) { ads_launch_dependent(kernel, grid, 256, 0, st, pool->emb, q_emb, N, E, B, keys); };
     if (E == 1024) run(cosine_keys_kernel<8>);
     else if (E == 768) run(cosine_keys_kernel<6>);
     else if (E == 384) run(cosine_keys_kernel<3>);
