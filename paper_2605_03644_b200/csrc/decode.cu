@@ -38,6 +38,7 @@ constexpr int kMaxCtas = 320;                // two per SM, at most this many
 constexpr int kUnitCost = 1;                 // fixed cost of a unit (rotate Q, merge the warps), in tiles
 constexpr int kMinRange = 3;                 // shortest range, in tiles (fixed cost included)
 constexpr int kRows = 32;                    // rows a partial has room for
+constexpr int kMergeRows = 4;                // rows whose states the warps merge at a time
 constexpr float kNegSentinel = -1.0e30f;
 constexpr float kLn2 = 0.6931471805599453f;
 
@@ -59,17 +60,23 @@ struct DecodeParams {
   double theta[64];
 };
 
+// a / b for 0 <= a, 0 < b; the positions of most calls fit 32 bits, where a division is a tenth of the instructions
+__device__ __forceinline__ long long div_nn(long long a, long long b) {
+  if (((a | b) >> 32) == 0) return (uint32_t)a / (uint32_t)b;
+  return a / b;
+}
+
 // The part of the tile sequence a CTA takes: every unit (request, layer, KV head) counts its tiles and
 // kUnitCost more in front of them.
 struct Ranges {
   long long total;
   int n;                       // ranges that are not empty
-  __device__ long long start(long long c) const { return c >= n ? total : c * total / n; }
+  __device__ long long start(long long c) const { return c >= n ? total : div_nn(c * total, n); }
   // the range that holds position x (0 <= x < total)
-  __device__ int holder(long long x) const { return (int)(((x + 1) * n - 1) / total); }
+  __device__ int holder(long long x) const { return (int)div_nn((x + 1) * n - 1, total); }
 };
 __device__ __forceinline__ Ranges make_ranges(long long total, int n_cta) {
-  const long long fit = total / kMinRange;
+  const long long fit = div_nn(total, kMinRange);
   return Ranges{total, (int)(fit < 1 ? 1 : (fit < n_cta ? fit : n_cta))};
 }
 
@@ -111,12 +118,12 @@ struct DecodeSmem {
   static constexpr uint32_t kTileBytes = kTile * D * 2;          // K or V of one tile
   static constexpr uint32_t kStageBytes = 2 * kTileBytes;
   static constexpr int kQStride = D + 8;                         // elements; rows of Q do not share banks
-  static constexpr int kOStride = D + 8;                         // floats
+  static constexpr int kOStride = D + 8;                         // floats; a warp's rows in the merge area
   static constexpr uint32_t kOffQ = kStages<D> * kStageBytes;    // Q of the unit; its read-out merges the warps here
   static constexpr uint32_t kQBytes = kRows * kQStride * 2;
-  static_assert(16 * kOStride * 4 <= kQBytes, "the merge area takes the place of Q");
-  static constexpr uint32_t kOffRed = kOffQ + kQBytes;           // [2][kWarps][16] row maxima and sums
-  static constexpr uint32_t kOffPre = kOffRed + 2 * kWarps * 16 * 4;
+  static_assert(kWarps * kMergeRows * kOStride * 4 <= kQBytes, "the merge area takes the place of Q");
+  static constexpr uint32_t kOffRed = kOffQ + kQBytes;           // [kWarps][kMergeRows] row maxima and sums
+  static constexpr uint32_t kOffPre = kOffRed + kWarps * kMergeRows * 8;
   static constexpr uint32_t kOffLen = kOffPre + (kMaxB + 1) * 8; // context lengths
   static constexpr uint32_t kOffBar = kOffLen + kMaxB * 4;
   static constexpr uint32_t kTotal = kOffBar + 128 + 1024;       // + alignment slack
@@ -136,8 +143,7 @@ decode_rows_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   unsigned char* base_ptr = smem_raw + (base - raw_addr);
   __nv_bfloat16* q_s = reinterpret_cast<__nv_bfloat16*>(base_ptr + SM::kOffQ);
   float* o_s = reinterpret_cast<float*>(base_ptr + SM::kOffQ);
-  float* red_m = reinterpret_cast<float*>(base_ptr + SM::kOffRed);
-  float* red_l = red_m + kWarps * 16;
+  float2* red = reinterpret_cast<float2*>(base_ptr + SM::kOffRed);
   long long* pre = reinterpret_cast<long long*>(base_ptr + SM::kOffPre);
   int* len_s = reinterpret_cast<int*>(base_ptr + SM::kOffLen);
   auto full = [&](int s) { return base + SM::kOffBar + 8u * s; };
@@ -157,36 +163,44 @@ decode_rows_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   }
   ads_dependency_trigger();
   ads_dependency_wait();
-  // costs and context lengths: every CTA forms them for itself (B <= 256)
-  for (int b = threadIdx.x; b < p.B; b += kThreads) {
-    int n = p.n_shots[b];
-    if (n < 1 || n > p.k) {                       // reported and clamped
-      ads_set_status(p.status, ADAPSHOT_EINDEX);
-      n = n < 1 ? 1 : p.k;
-    }
-    long long L = p.ctx_off[(long long)b * (p.k + 1) + n];
-    L = L > p.ctx_cap ? p.ctx_cap : (L < 0 ? 0 : L);
-    len_s[b] = (int)L;
-    pre[b + 1] = (L + kTile - 1) / kTile + n_own + kUnitCost;
-  }
-  if (threadIdx.x == 0) pre[0] = 0;
-  __syncthreads();
+  // context lengths and prefix sums of the requests' costs: every CTA forms them for itself (B <= 256), the loads of
+  // all requests on their way at once
   if (warp == 0) {
+    int n[kMaxB / 32];
+#pragma unroll
+    for (int e = 0; e < kMaxB / 32; ++e) n[e] = e * 32 + lane < p.B ? p.n_shots[e * 32 + lane] : 1;
+    long long L[kMaxB / 32];
+#pragma unroll
+    for (int e = 0; e < kMaxB / 32; ++e) {
+      if (n[e] < 1 || n[e] > p.k) {               // reported and clamped
+        ads_set_status(p.status, ADAPSHOT_EINDEX);
+        n[e] = n[e] < 1 ? 1 : p.k;
+      }
+      const int b = e * 32 + lane;
+      L[e] = b < p.B ? p.ctx_off[(long long)b * (p.k + 1) + n[e]] : 0;
+    }
     long long carry = 0;
-    for (int b0 = 0; b0 < p.B; b0 += 32) {
-      long long v = b0 + lane < p.B ? pre[b0 + lane + 1] : 0;
+    if (lane == 0) pre[0] = 0;
+#pragma unroll
+    for (int e = 0; e < kMaxB / 32; ++e) {
+      const int b = e * 32 + lane;
+      if (e * 32 >= p.B) break;
+      L[e] = L[e] > p.ctx_cap ? p.ctx_cap : (L[e] < 0 ? 0 : L[e]);
+      long long v = b < p.B ? (L[e] + kTile - 1) / kTile + n_own + kUnitCost : 0;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const long long u = __shfl_up_sync(0xffffffffu, v, o);
         if (lane >= o) v += u;
       }
       v += carry;
-      if (b0 + lane < p.B) pre[b0 + lane + 1] = v;
       carry = __shfl_sync(0xffffffffu, v, 31);
+      if (b < p.B) {
+        len_s[b] = (int)L[e];
+        pre[b + 1] = v;
+        if (blockIdx.x == 0) p.prefix[b + 1] = v;
+      }
     }
-    __syncwarp();
-    if (blockIdx.x == 0)
-      for (int b = lane; b <= p.B; b += 32) p.prefix[b] = pre[b];
+    if (blockIdx.x == 0 && lane == 0) p.prefix[0] = 0;
   }
   __syncthreads();
   const Ranges rg = make_ranges(pre[p.B] * upb, p.n_cta);
@@ -207,7 +221,7 @@ decode_rows_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
       }
       const int len = (int)(pre[b + 1] - pre[b]);
       const long long rel = x - pre[b] * upb;
-      const int u = (int)(rel / len), off = (int)(rel % len);
+      const int u = (int)div_nn(rel, len), off = (int)(rel - (long long)u * len);
       const int end = (int)(x1 - x < len - off ? off + (x1 - x) : len);
       const int t0 = off > kUnitCost ? off - kUnitCost : 0, t1 = end - kUnitCost, n_tiles = len - kUnitCost;
       if (t1 > t0)
@@ -422,72 +436,60 @@ decode_rows_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
       }
       if (!consumers_all(ok)) return false;              // (every warp comes here, so none waits for one that gave up)
 
-      // merge of the four warps' states and read-out, 16 rows at a time
+      // merge of the four warps' states and read-out, four rows at a time: 32 threads take a row
       const bool whole = t0 == 0 && t1 == n_tiles;
       const long long slot = 2ll * blockIdx.x + (first ? 0 : 1);
 #pragma unroll
-      for (int mb = 0; mb < MB; ++mb) {
-        if (mb > 0) consumers_sync();
+      for (int mb = 0; mb < MB; ++mb)
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
           float v = l_run[mb][hf];
           v += __shfl_xor_sync(0xffffffffu, v, 1);
-          v += __shfl_xor_sync(0xffffffffu, v, 2);
-          if ((lane & 3) == 0) {
-            red_m[warp * 16 + hf * 8 + r0] = m_run[mb][hf];
-            red_l[warp * 16 + hf * 8 + r0] = v;
-          }
+          l_run[mb][hf] = v + __shfl_xor_sync(0xffffffffu, v, 2);
+        }
+#pragma unroll
+      for (int rb = 0; rb < MB * 16; rb += kMergeRows) {
+        if (rb >= p.rows) break;
+        if (rb > 0) consumers_sync();
+        const int mb = rb / 16, hf = (rb / 8) & 1, half = (rb / kMergeRows) & 1;       // constants
+        if ((r0 >> 2) == half) {
+          float* dst = o_s + (warp * kMergeRows + (r0 & 3)) * SM::kOStride + c0;
+#pragma unroll
+          for (int nb = 0; nb < D / 8; ++nb)
+            *reinterpret_cast<float2*>(dst + nb * 8) = make_float2(o[mb][nb][2 * hf], o[mb][nb][2 * hf + 1]);
+          if ((lane & 3) == 0) red[warp * kMergeRows + (r0 & 3)] = make_float2(m_run[mb][hf], l_run[mb][hf]);
         }
         consumers_sync();
-        auto row_max = [&](int row) {
-          float m = red_m[row];
-#pragma unroll
-          for (int w = 1; w < kWarps; ++w) m = fmaxf(m, red_m[w * 16 + row]);
-          return m;
-        };
-        const float f[2] = {ex2(m_run[mb][0] - row_max(r0)), ex2(m_run[mb][1] - row_max(r0 + 8))};
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) {
-          if (warp == w) {
-#pragma unroll
-            for (int nb = 0; nb < D / 8; ++nb)
-#pragma unroll
-              for (int hf = 0; hf < 2; ++hf) {
-                float2* dst = reinterpret_cast<float2*>(o_s + (hf * 8 + r0) * SM::kOStride + nb * 8 + c0);
-                float2 v = make_float2(o[mb][nb][2 * hf] * f[hf], o[mb][nb][2 * hf + 1] * f[hf]);
-                if (w > 0) {
-                  const float2 a = *dst;
-                  v.x += a.x;
-                  v.y += a.y;
-                }
-                *dst = v;
-              }
-          }
-          consumers_sync();
-        }
-        constexpr int CPT = D / 8;                       // columns per thread: eight threads read a row out
-        const int row = threadIdx.x >> 3, col = (threadIdx.x & 7) * CPT, rr = mb * 16 + row;
+        constexpr int CPT = D / 32;                      // columns per thread
+        const int row = threadIdx.x >> 5, col = (threadIdx.x & 31) * CPT, rr = rb + row;
         if (rr < p.rows) {
-          const float m = row_max(row);
-          float lsum = 0.f;
+          float m = kNegSentinel, lsum = 0.f, acc[CPT] = {};
 #pragma unroll
-          for (int w = 0; w < kWarps; ++w) lsum += red_l[w * 16 + row] * ex2(red_m[w * 16 + row] - m);
-          const float4* src = reinterpret_cast<const float4*>(o_s + row * SM::kOStride + col);
+          for (int w = 0; w < kWarps; ++w) m = fmaxf(m, red[w * kMergeRows + row].x);
+#pragma unroll
+          for (int w = 0; w < kWarps; ++w) {
+            const float2 ml = red[w * kMergeRows + row];
+            const float f = ex2(ml.x - m);
+            lsum += ml.y * f;
+            const float* src = o_s + (w * kMergeRows + row) * SM::kOStride + col;
+#pragma unroll
+            for (int c = 0; c < CPT; c += 2) {
+              const float2 v = *reinterpret_cast<const float2*>(src + c);
+              acc[c] += v.x * f;
+              acc[c + 1] += v.y * f;
+            }
+          }
           if (whole) {
             const int tt = rr / p.G, h = g * p.G + rr % p.G;
             const float inv = 1.f / lsum;
-            uint4* dst = reinterpret_cast<uint4*>(p.out + ((bl * p.T_new + tt) * p.Hq + h) * (long long)D + col);
+            __nv_bfloat16* dst = p.out + ((bl * p.T_new + tt) * p.Hq + h) * (long long)D + col;
 #pragma unroll
-            for (int c = 0; c < CPT / 8; ++c) {
-              const float4 a = src[2 * c], d = src[2 * c + 1];
-              dst[c] = make_uint4(pack2(a.x * inv, a.y * inv), pack2(a.z * inv, a.w * inv), pack2(d.x * inv, d.y * inv),
-                                  pack2(d.z * inv, d.w * inv));
-            }
+            for (int c = 0; c < CPT; c += 2) *reinterpret_cast<uint32_t*>(dst + c) = pack2(acc[c] * inv, acc[c + 1] * inv);
             if (p.lse != nullptr && col == 0) p.lse[(bl * p.Hq + h) * p.T_new + tt] = (m + log2f(lsum)) * kLn2;
           } else {
-            float4* dst = reinterpret_cast<float4*>(p.o_part + (slot * kRows + rr) * D + col);
+            float* dst = p.o_part + (slot * kRows + rr) * D + col;
 #pragma unroll
-            for (int c = 0; c < CPT / 4; ++c) dst[c] = src[c];
+            for (int c = 0; c < CPT; c += 2) *reinterpret_cast<float2*>(dst + c) = make_float2(acc[c], acc[c + 1]);
             if (col == 0) *reinterpret_cast<float2*>(p.ml_part + (slot * kRows + rr) * 2) = make_float2(m, lsum);
           }
         }
@@ -509,10 +511,11 @@ __global__ void __launch_bounds__(32 * kMergeWarps) decode_combine_kernel(const 
   ads_dependency_trigger();
   ads_dependency_wait();
   const long long upb = (long long)p.nl * p.Hkv, u = blockIdx.x;
-  const int b = (int)(u / upb), rr = blockIdx.y;
+  const int b = (int)div_nn(u, upb), rr = blockIdx.y;
   const long long p0 = p.prefix[b], len = p.prefix[b + 1] - p0;
   const Ranges rg = make_ranges(p.prefix[p.B] * upb, p.n_cta);
-  const long long s = p0 * upb + (u % upb) * len;
+  const int ub = (int)(u - (long long)b * upb);      // unit within the request
+  const long long s = p0 * upb + (long long)ub * len;
   int c0 = rg.holder(s);
   const int c1 = rg.holder(s + len - 1);
   if (rg.start(c0 + 1) <= s + kUnitCost) ++c0;      // that range holds none of the unit's tiles
@@ -565,7 +568,7 @@ __global__ void __launch_bounds__(32 * kMergeWarps) decode_combine_kernel(const 
     acc.x += v.x * f; acc.y += v.y * f; acc.z += v.z * f; acc.w += v.w * f;
   }
   const float inv = 1.f / lsum;
-  const int l = (int)(u % upb) / p.Hkv, t = rr / p.G, h = (int)(u % p.Hkv) * p.G + rr % p.G;
+  const int l = ub / p.Hkv, t = rr / p.G, h = (ub % p.Hkv) * p.G + rr % p.G;
   const long long bl = (long long)b * p.nl + l;
   reinterpret_cast<uint2*>(p.out + ((bl * p.T_new + t) * p.Hq + h) * (long long)D)[threadIdx.x] =
       make_uint2(pack2(acc.x * inv, acc.y * inv), pack2(acc.z * inv, acc.w * inv));
