@@ -261,33 +261,43 @@ decode_rows_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   } else {
     // ------------------------------------------------------------- consumers
     const int r0 = lane >> 2, c0 = 2 * (lane & 3);       // this lane's rows r0, r0 + 8 and columns c0, c0 + 1 of an 8-column block
-    double th[D / 64];
-#pragma unroll
-    for (int e = 0; e < D / 64; ++e) th[e] = p.theta[lane + 32 * e];
+    // rotations: a lane owns two neighbouring frequencies, a warp turns RPI rows at a time
+    constexpr int RPI = 128 / D;
+    const int f0 = 2 * (lane % (D / 4)), sub = lane / (D / 4);
+    const double th[2] = {p.theta[f0], p.theta[f0 + 1]};
+    auto angles = [&](double pos, float2& cs, float2& sn) {
+      rope_sincos(pos, th[0], &sn.x, &cs.x);
+      rope_sincos(pos, th[1], &sn.y, &cs.y);
+    };
+    auto turn = [&](uint32_t& lo, uint32_t& hi, const float2& cs, const float2& sn) {
+      const float2 x = make_float2(__uint_as_float(lo << 16), __uint_as_float(lo & 0xffff0000u));
+      const float2 y = make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u));
+      const float2 a = __ffma2_rn(y, make_float2(-sn.x, -sn.y), __fmul2_rn(x, cs));
+      const float2 c = __ffma2_rn(x, sn, __fmul2_rn(y, cs));
+      lo = pack2(a.x, a.y);
+      hi = pack2(c.x, c.y);
+    };
     uint32_t it = 0;
     walk([&](int b, int l, int g, int t0, int t1, int n_tiles, int n_ctx, bool first) {
       const long long L = len_s[b];
       const long long bl = (long long)b * p.nl + l;
       consumers_sync();                                  // the read-out of the previous piece is over
       // Q of the unit, rotated to its positions: row rr = (token t, head hh) of the KV head's group
-      for (int rr = warp; rr < MB * 16; rr += kWarps) {
-        if (rr >= p.rows) {
-#pragma unroll
-          for (int e = 0; e < D / 32; ++e) q_s[rr * SM::kQStride + lane + 32 * e] = __float2bfloat16_rn(0.f);
-          continue;
+#pragma unroll 1
+      for (int rr = warp * RPI + sub; rr < MB * 16; rr += kWarps * RPI) {
+        uint32_t* dst = reinterpret_cast<uint32_t*>(q_s + rr * SM::kQStride + f0);
+        uint32_t lo = 0, hi = 0;
+        if (rr < p.rows) {
+          const int t = rr / p.G, h = g * p.G + rr % p.G;
+          const uint32_t* src = reinterpret_cast<const uint32_t*>(p.q + ((bl * p.T_new + t) * p.Hq + h) * (long long)D + f0);
+          lo = src[0];
+          hi = src[D / 4];
+          float2 cs, sn;
+          angles((double)(L + p.T_own - p.T_new + t), cs, sn);
+          turn(lo, hi, cs, sn);
         }
-        const int t = rr / p.G, h = g * p.G + rr % p.G;
-        const double pos = (double)(L + p.T_own - p.T_new + t);
-        const __nv_bfloat16* src = p.q + ((bl * p.T_new + t) * p.Hq + h) * (long long)D;
-#pragma unroll
-        for (int e = 0; e < D / 64; ++e) {
-          const int i = lane + 32 * e;
-          float sn, cs;
-          rope_sincos(pos, th[e], &sn, &cs);
-          const float x = __bfloat162float(src[i]), y = __bfloat162float(src[i + D / 2]);
-          q_s[rr * SM::kQStride + i] = __float2bfloat16_rn(x * cs - y * sn);
-          q_s[rr * SM::kQStride + i + D / 2] = __float2bfloat16_rn(y * cs + x * sn);
-        }
+        dst[0] = lo;
+        dst[D / 4] = hi;
       }
       consumers_sync();
       const uint32_t q_addr = base + SM::kOffQ + ((lane & 15) * SM::kQStride + (lane >> 4) * 8) * 2;
@@ -313,28 +323,27 @@ decode_rows_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
         const bool own = t >= n_ctx;
         const int own0 = (t - n_ctx) * kTile + warp * 16;          // first own token of this warp's keys
         if (own) {
-          // the own keys are stored un-rotated: this warp turns its 16 rows to L + token, the first row from
-          // fp64 angles, the following ones by a complex multiplication with one position's angle
-          __nv_bfloat16* kt = reinterpret_cast<__nv_bfloat16*>(base_ptr + s * SM::kStageBytes);
-#pragma unroll
-          for (int e = 0; e < D / 64; ++e) {
-            const int i = lane + 32 * e;
-            float sn, cs, sn1, cs1;
-            rope_sincos((double)(L + own0), th[e], &sn, &cs);
-            rope_sincos(1.0, th[e], &sn1, &cs1);
-            const int ih = i + D / 2;
-#pragma unroll
-            for (int r = 0; r < 16; ++r) {
-              const int row = warp * 16 + r;
-              __nv_bfloat16* lo = kt + (i >> 6) * (kTile * 64) + row * 64 + ((((i & 63) >> 3) ^ (row & 7)) << 3) + (i & 7);
-              __nv_bfloat16* hi = kt + (ih >> 6) * (kTile * 64) + row * 64 + ((((ih & 63) >> 3) ^ (row & 7)) << 3) + (ih & 7);
-              const float x = __bfloat162float(*lo), y = __bfloat162float(*hi);
-              *lo = __float2bfloat16_rn(x * cs - y * sn);
-              *hi = __float2bfloat16_rn(y * cs + x * sn);
-              const float c = cs * cs1 - sn * sn1;
-              sn = sn * cs1 + cs * sn1;
-              cs = c;
-            }
+          // the own keys are stored un-rotated: this warp turns its 16 rows to L + token, the first ones from fp64
+          // angles, the others RPI positions further at a time by a complex multiplication
+          unsigned char* kt = base_ptr + s * SM::kStageBytes;
+          float2 cs, sn, cs1, sn1;
+          angles((double)(L + own0 + sub), cs, sn);
+          angles((double)RPI, cs1, sn1);
+          auto at = [&](int c, int row) {
+            return reinterpret_cast<uint32_t*>(kt + (c >> 6) * (kTile * 128) + row * 128 +
+                                               ((((c & 63) >> 3) ^ (row & 7)) << 4) + (c & 7) * 2);
+          };
+#pragma unroll 4
+          for (int r = 0; r < 16; r += RPI) {
+            const int row = warp * 16 + r + sub;
+            uint32_t *lo = at(f0, row), *hi = at(f0 + D / 2, row);
+            uint32_t a = *lo, c = *hi;
+            turn(a, c, cs, sn);
+            *lo = a;
+            *hi = c;
+            const float2 cn = __ffma2_rn(make_float2(-sn.x, -sn.y), sn1, __fmul2_rn(cs, cs1));
+            sn = __ffma2_rn(cs, sn1, __fmul2_rn(sn, cs1));
+            cs = cn;
           }
           fence_proxy_async_smem();
           __syncwarp();
