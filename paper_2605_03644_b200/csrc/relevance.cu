@@ -27,10 +27,12 @@ namespace {
 using namespace sm100;
 
 constexpr int kTile = 128;            // query rows per M tile, keys per tile
-constexpr int kRelThreads = 192;      // warp 0 TMA, warp 1 MMA, warps 2-5 consumers (one thread per TMEM lane)
-// K tiles in flight per CTA: two CTAs share an SM (96 KB each at d = 128), so that one's consumers
-// work while the other's wait for a score tile
-template <int D> constexpr int kKStages = D == 128 ? 2 : 4;
+constexpr int kGroups = 4;            // consumer groups of a CTA: a warpgroup each, one thread per row (TMEM lane) of its score tile
+constexpr int kRelThreads = 128 * (kGroups + 1);      // warp 0 TMA, warp 1 MMA; consumers from warp 4 on
+constexpr int kSmemTiles = 6;         // 128-row tiles in shared memory: the Q tiles, and K tiles in the rest
+// Registers per thread of the first warpgroup and of the consumers; together what 640 threads are launched with, 5 x 96.
+constexpr int kRelRegsIssue = 64, kRelRegsConsumer = 104;
+static_assert(kRelRegsIssue + kGroups * kRelRegsConsumer <= 5 * 96, "register split");
 
 // 2^x by the hardware approximation (one MUFU operation, relative error about 2^-22; 2^-inf = 0)
 __device__ __forceinline__ float rel_ex2(float x) {
@@ -44,8 +46,8 @@ __device__ __forceinline__ float rel_ex2(float x) {
 // x = n + f with n = round(x) taken from the low mantissa bits of x + 1.5 * 2^23, 2^f by a cubic on
 // [-0.5, 0.5] (relative error 7.5e-5, fitted for this build), n added to the exponent field.  The
 // passes send every fourth pair here: the exponential unit (16 results per clock and SM) is what
-// bounds them, the FMA pipe is nine tenths idle (measured: 4 % faster at 8 queries, 13 % at one;
-// every second pair is slower again).
+// bounds it together with instruction issue (856 us with none there, 791 with every fourth,
+// 867 with every second pair).
 __device__ __forceinline__ float2 rel_ex2_poly2(float2 x) {
   const float kMagic = 12582912.f;
   x.x = fmaxf(x.x, -125.f);      // keeps the exponent field of the result positive
@@ -69,6 +71,7 @@ struct RelParams {
   long long pool_tokens;
   int Hkv, n_mt, n_shots, layer, tile0;     // tile0: first of the batch's M tiles (b * n_mt + mt)
   int n_tiles, splits, tiles_per_split;
+  int n_m, m_per_cta;           // M tiles of the batch; how many of them share a CTA's K tiles (1, 2 or 4)
   float scale_log2;
 };
 
@@ -96,26 +99,29 @@ __global__ void __launch_bounds__(256) rel_pack_q_kernel(const __nv_bfloat16* __
   reinterpret_cast<uint4*>(q_pack)[i] = val;
 }
 
-enum RelBar { kRQFull = 0, kRKFull = 1, kRKEmpty = 5, kRSFull = 9, kRSEmpty = 11, kRDrain = 13, kRNumBars = 14 };
+enum RelBar { kRQFull = 0, kRKFull = 1, kRKEmpty = 6, kRSFull = 11, kRSEmpty = 15, kRDrain = 19, kRNumBars = 20 };
 
 template <int D>
 struct RelSmem {
   static constexpr uint32_t kTileBytes = (D / 64) * 16384u;
-  static constexpr uint32_t kOffQ = 0;
-  static constexpr uint32_t kOffK = kTileBytes;
-  static constexpr uint32_t kOffBar = kOffK + kKStages<D> * kTileBytes;
-  static constexpr uint32_t kTotal = kOffBar + 128 + 1024;      // + alignment slack
+  static constexpr uint32_t kOffBar = kSmemTiles * kTileBytes;
+  static constexpr uint32_t kTotal = kOffBar + 256 + 1024;      // + alignment slack
 };
 
-// grid (M tiles of the batch, splits, Hkv): the CTAs that differ only in (query, M tile) walk the same key tiles
-// at the same time, so the pool's K layer is read from DRAM about once and from L2 otherwise.
+// grid (groups of M tiles, groups of key ranges, Hkv).  The four consumer groups of a CTA take m_per_cta M tiles times
+// 4 / m_per_cta key ranges: group x has M tile x % m_per_cta and range x / m_per_cta.  M tiles of a CTA share
+// every K tile; where there are few of them the ranges keep all groups busy.  CTAs that differ in their M tiles only
+// walk the same key tiles at the same time, so the pool's K layer is read from DRAM about once.
+// Bound by the exponential unit (128 x 128 results per score tile, 16 per clock and SM) and, where shots end, by
+// instruction issue: sixteen consumer warps keep both busy under each other's latencies.  (Two CTAs per SM with one M
+// tile and four consumer warps each: 1000 us for 2 queries x 128 tokens, 328 K pool tokens; 790 us now, the exponential unit
+// and the issue slots both two thirds busy.)
 template <int D>
-__global__ void __launch_bounds__(kRelThreads, 2)
+__global__ void __launch_bounds__(kRelThreads, 1)
 rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                const RelParams p) {
+                const __grid_constant__ RelParams p) {
   using SM = RelSmem<D>;
   constexpr int SUB = D / 64;
-  constexpr int kStages = kKStages<D>;
   constexpr uint32_t kTileBytes = SM::kTileBytes;
   constexpr uint32_t kIdesc = idesc_bf16_f32(kTile, kTile, 0);
   extern __shared__ unsigned char smem_raw[];
@@ -128,20 +134,24 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + SM::kOffBar + 8 * kRNumBars + 8);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b = (p.tile0 + blockIdx.x) / p.n_mt, mt = (p.tile0 + blockIdx.x) % p.n_mt;
-  const int split = blockIdx.y, g = blockIdx.z;
-  const long long unit = (long long)blockIdx.x * p.Hkv + g;
-  const int t0 = split * p.tiles_per_split;
-  const int t1 = min(p.n_tiles, t0 + p.tiles_per_split);
-  const int n_it = max(0, t1 - t0);
+  const int g = blockIdx.z;
+  const int m0 = blockIdx.x * p.m_per_cta, n_m = min(p.m_per_cta, p.n_m - m0);      // M tiles of this CTA
+  const int s0 = blockIdx.y * (kGroups / p.m_per_cta), n_s = min(kGroups / p.m_per_cta, p.splits - s0);   // its ranges
+  const int stages = kSmemTiles - p.m_per_cta;
+  const uint32_t k_base = base + p.m_per_cta * kTileBytes;
+  // tiles of range s0 + j: the last range of a call may be shorter than the others
+  auto range_tiles = [&](int j) {
+    return max(0, min(p.n_tiles, (s0 + j + 1) * p.tiles_per_split) - (s0 + j) * p.tiles_per_split);
+  };
+  const int n_it = range_tiles(0);
 
   if (threadIdx.x == 32) {
     mbar_init(bar(kRQFull), 1);
-    for (int i = 0; i < kStages; ++i) {
+    for (int i = 0; i < stages; ++i) {
       mbar_init(bar(kRKFull + i), 1);
       mbar_init(bar(kRKEmpty + i), 1);
     }
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < kGroups; ++i) {
       mbar_init(bar(kRSFull + i), 1);
       mbar_init(bar(kRSEmpty + i), 128);
     }
@@ -151,7 +161,7 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     mbar_fence_init();
   }
   if (warp == 0) {
-    tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), 256);
+    tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -159,64 +169,82 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer
-    if (lane == 0 && n_it > 0) {
+  auto role_tma = [&]() {
+    if (lane == 0) {
       tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k);
-      mbar_arrive_expect_tx(bar(kRQFull), kTileBytes);
-#pragma unroll
-      for (int s = 0; s < SUB; ++s)
-        tma_load_3d(base + SM::kOffQ + s * 16384u, &tm_q, bar(kRQFull), s * 64, mt * kTile, b * p.Hkv + g);
-      bool ok = true;
-      int i = 0;
-      for (; i < n_it && ok; ++i) {
-        const int st = i % kStages;
-        ok = mbar_wait(bar(kRKEmpty + st), ((i / kStages) & 1) ^ 1, abort_flag);
-        if (!ok) break;
-        mbar_arrive_expect_tx(bar(kRKFull + st), kTileBytes);
+      mbar_arrive_expect_tx(bar(kRQFull), n_m * kTileBytes);
+      for (int m = 0; m < n_m; ++m) {
+        const int b = (p.tile0 + m0 + m) / p.n_mt, mt = (p.tile0 + m0 + m) % p.n_mt;
 #pragma unroll
         for (int s = 0; s < SUB; ++s)
-          tma_load_4d(base + SM::kOffK + st * kTileBytes + s * 16384u, &tm_k, bar(kRKFull + st), s * 64, g,
-                      (t0 + i) * kTile, p.layer);
+          tma_load_3d(base + m * kTileBytes + s * 16384u, &tm_q, bar(kRQFull), s * 64, mt * kTile, b * p.Hkv + g);
       }
+      bool ok = true;
+      int st = 0, n = 0;
+      uint32_t phase = 1;
+      for (int i = 0; i < n_it && ok; ++i)
+        for (int j = 0; j < n_s; ++j) {
+          if (i >= range_tiles(j)) continue;
+          ok = mbar_wait(bar(kRKEmpty + st), phase, abort_flag);
+          if (!ok) break;
+          mbar_arrive_expect_tx(bar(kRKFull + st), kTileBytes);
+#pragma unroll
+          for (int s = 0; s < SUB; ++s)
+            tma_load_4d(k_base + st * kTileBytes + s * 16384u, &tm_k, bar(kRKFull + st), s * 64, g,
+                        ((s0 + j) * p.tiles_per_split + i) * kTile, p.layer);
+          ++n;
+          if (++st == stages) { st = 0; phase ^= 1; }
+        }
       if (!ok) {      // gave up: let the copies in flight land before the CTA retires
         mbar_wait(bar(kRQFull), 0, abort_flag + 1);
-        for (int t = max(0, i - kStages); t < i; ++t)
-          mbar_wait(bar(kRKFull + t % kStages), (t / kStages) & 1, abort_flag + 1);
+        for (int t = max(0, n - stages); t < n; ++t)
+          mbar_wait(bar(kRKFull + t % stages), (t / stages) & 1, abort_flag + 1);
       }
     }
     __syncwarp();
-  } else if (warp == 1) {
-    // -------------------------------------------------------------- MMA issuer
-    if (lane == 0 && n_it > 0) {
+  };
+  auto role_mma = [&]() {
+    if (lane == 0) {
       constexpr uint32_t kHi = smem_desc_hi_sw128(1024);
-      const uint32_t q_lo = smem_desc_lo(base + SM::kOffQ, 16);
+      const uint32_t q_lo0 = smem_desc_lo(base, 16), k_lo0 = smem_desc_lo(k_base, 16);
       bool ok = mbar_wait(bar(kRQFull), 0, abort_flag);
-      for (int i = 0; i < n_it && ok; ++i) {
-        const int st = i % kStages, sb = i & 1;
-        ok = mbar_wait(bar(kRKFull + st), (i / kStages) & 1, abort_flag) &&
-             mbar_wait(bar(kRSEmpty + sb), ((i >> 1) & 1) ^ 1, abort_flag);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t k_lo = smem_desc_lo(base + SM::kOffK + st * kTileBytes, 16);
-        const uint32_t d = tmem_base + sb * kTile;
+      int st = 0;
+      uint32_t phase = 0;
+      for (int i = 0; i < n_it && ok; ++i)
+        for (int j = 0; j < n_s && ok; ++j) {
+          if (i >= range_tiles(j)) continue;
+          ok = mbar_wait(bar(kRKFull + st), phase, abort_flag);
+          const uint32_t k_lo = k_lo0 + st * (kTileBytes >> 4);
+          for (int m = 0; m < n_m && ok; ++m) {
+            const int x = j * p.m_per_cta + m;
+            ok = mbar_wait(bar(kRSEmpty + x), (i & 1) ^ 1, abort_flag);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t q_lo = q_lo0 + m * (kTileBytes >> 4), d = tmem_base + x * kTile;
 #pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-          const uint32_t o = ((ks / 4) * 16384u + (ks % 4) * 32u) >> 4;
-          umma_ss_lohi(d, q_lo + o, kHi, k_lo + o, kHi, kIdesc, ks > 0 ? 1u : 0u);
+            for (int ks = 0; ks < D / 16; ++ks) {
+              const uint32_t o = ((ks / 4) * 16384u + (ks % 4) * 32u) >> 4;
+              umma_ss_lohi(d, q_lo + o, kHi, k_lo + o, kHi, kIdesc, ks > 0 ? 1u : 0u);
+            }
+            umma_commit(bar(kRSFull + x));
+          }
+          if (!ok) break;
+          umma_commit(bar(kRKEmpty + st));
+          if (++st == stages) { st = 0; phase ^= 1; }
         }
-        umma_commit(bar(kRSFull + sb));
-        umma_commit(bar(kRKEmpty + st));
-      }
       if (!ok) {      // gave up: the UMMAs already issued must be done before the tensor memory is freed
         umma_commit(bar(kRDrain));
         mbar_wait(bar(kRDrain), 0, abort_flag + 1);
       }
     }
     __syncwarp();
-  } else {
-    // --------------------------------------------------------------- consumers
-    const int quarter = warp & 3;
+  };
+  auto role_consume = [&]() {
+    const int x = (warp >> 2) - 1, quarter = warp & 3;
+    const int m = x % p.m_per_cta, j = x / p.m_per_cta;
+    if (m >= n_m || j >= n_s) return;                       // fewer M tiles or ranges than the CTA has room for
+    const int split = s0 + j, n_mine = range_tiles(j), t0 = split * p.tiles_per_split, t1 = t0 + n_mine;
+    const long long unit = (long long)(m0 + m) * p.Hkv + g;
     const int r = quarter * 32 + lane;                      // TMEM lane: query row
     const uint32_t lane_addr = static_cast<uint32_t>(quarter * 32) << 16;
     float m_run = -1.0e30f, l_run = 0.f, acc = 0.f;         // running maximum, sum of the shots so far, of the current one
@@ -244,93 +272,107 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       end_next = shot_end(shot + 1);
     };
     bool ok = true;
-    for (int i = 0; i < n_it; ++i) {
-      const int sb = i & 1;
-      ok = __all_sync(0xffffffffu, mbar_wait(bar(kRSFull + sb), (i >> 1) & 1, abort_flag));
+    for (int i = 0; i < n_mine; ++i) {
+      ok = __all_sync(0xffffffffu, mbar_wait(bar(kRSFull + x), i & 1, abort_flag));
       if (!ok) break;
       tc_fence_after();
-      float s[kTile];
-      tmem_ld128(tmem_base + lane_addr + sb * kTile, reinterpret_cast<uint32_t*>(s));
-      tc_fence_before();
-      mbar_arrive(bar(kRSEmpty + sb));                      // the scores are in registers: the buffer is free
-      const long long key0 = (long long)(t0 + i) * kTile;
-      const int limit = (int)min((long long)kTile, p.pool_tokens - key0);   // keys of this tile that exist
-      if (limit < kTile) {                       // only the pool's last tile: keys beyond it count as -inf
 #pragma unroll
-        for (int c = 0; c < kTile; ++c) s[c] = c < limit ? s[c] : -INFINITY;
-      }
-      float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-      for (int c = 0; c < kTile; c += 8) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) mx4[u] = fmax3(mx4[u], s[c + 2 * u], s[c + 2 * u + 1]);
-      }
-      const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * p.scale_log2;
-      if (mx > m_run) {
-        const float keep = rel_ex2(m_run - mx);
-        l_run *= keep;
-        acc *= keep;
-        m_run = mx;
-      }
-      // two scores per FMA / add instruction; the exponentials themselves are one MUFU operation each
-      const float2 scale2 = make_float2(p.scale_log2, p.scale_log2), neg_m2 = make_float2(-m_run, -m_run);
-      float group[kTile / 16];                              // sums of 16 keys
-#pragma unroll
-      for (int c0 = 0; c0 < kTile; c0 += 16) {
-        float2 part = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int c = c0; c < c0 + 16; c += 2) {
-          const float2 a = __ffma2_rn(make_float2(s[c], s[c + 1]), scale2, neg_m2);
-          const float2 e = ((c >> 1) & 3) == 3 ? rel_ex2_poly2(a) : make_float2(rel_ex2(a.x), rel_ex2(a.y));
-          s[c] = e.x;
-          s[c + 1] = e.y;
-          part = c == c0 ? e : __fadd2_rn(part, e);
+      for (int half = 0; half < 2; ++half) {
+        constexpr int kCols = kTile / 2;                    // (a whole row at once would not fit the registers)
+        float s[kCols];
+        tmem_ld2x32(tmem_base + lane_addr + x * kTile + half * kCols, reinterpret_cast<uint32_t*>(s));
+        if (half == 1) {                                    // the scores are in registers: the buffer is free
+          tc_fence_before();
+          mbar_arrive(bar(kRSEmpty + x));
         }
-        group[c0 / 16] = part.x + part.y;
-      }
-      // sums per shot (the branches are the same in every lane): a tile within one shot, else group by group, the
-      // keys of a group one by one only where a shot ends in it
-      const long long left = end - key0;
-      if (left > kTile) {
-        acc += ((group[0] + group[1]) + (group[2] + group[3])) + ((group[4] + group[5]) + (group[6] + group[7]));
-      } else {
-        int ce = (int)left;                                 // columns left of the current shot
+        const long long key0 = (long long)(t0 + i) * kTile + half * kCols;
+        if (key0 + kCols > p.pool_tokens) {        // only the pool's last tile: keys beyond it count as -inf
+          const int limit = (int)max(0ll, p.pool_tokens - key0);
 #pragma unroll
-        for (int c0 = 0; c0 < kTile; c0 += 16) {
-          if (ce > c0 + 16) {
-            acc += group[c0 / 16];
-          } else {
-            int from = c0;
-            while (from < c0 + 16) {
-              const int to = min(ce, c0 + 16);
-              float sum[2] = {0.f, 0.f};
+          for (int c = 0; c < kCols; ++c) s[c] = c < limit ? s[c] : -INFINITY;
+        }
+        float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-              for (int c = 0; c < 16; ++c) sum[c & 1] += c0 + c >= from && c0 + c < to ? s[c0 + c] : 0.f;
-              acc += sum[0] + sum[1];
-              if (to == ce) {
-                flush();
-                ce = end - key0 > 4096 ? 4096 : (int)(end - key0);
+        for (int c = 0; c < kCols; c += 8) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) mx4[u] = fmax3(mx4[u], s[c + 2 * u], s[c + 2 * u + 1]);
+        }
+        const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * p.scale_log2;
+        if (mx > m_run) {
+          const float keep = rel_ex2(m_run - mx);
+          l_run *= keep;
+          acc *= keep;
+          m_run = mx;
+        }
+        // two scores per FMA / add instruction; the exponentials themselves are one MUFU operation each
+        const float2 scale2 = make_float2(p.scale_log2, p.scale_log2), neg_m2 = make_float2(-m_run, -m_run);
+        float group[kCols / 16];                            // sums of 16 keys
+#pragma unroll
+        for (int c0 = 0; c0 < kCols; c0 += 16) {
+          float2 part = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int c = c0; c < c0 + 16; c += 2) {
+            const float2 a = __ffma2_rn(make_float2(s[c], s[c + 1]), scale2, neg_m2);
+            const float2 e = ((c >> 1) & 3) == 3 ? rel_ex2_poly2(a) : make_float2(rel_ex2(a.x), rel_ex2(a.y));
+            s[c] = e.x;
+            s[c + 1] = e.y;
+            part = c == c0 ? e : __fadd2_rn(part, e);
+          }
+          group[c0 / 16] = part.x + part.y;
+        }
+        // sums per shot (the branches are the same in every lane): all keys within one shot, else group by group, the
+        // keys of a group one by one only where a shot ends in it
+        const long long left = end - key0;
+        if (left > kCols) {
+          acc += (group[0] + group[1]) + (group[2] + group[3]);
+        } else {
+          int ce = (int)left;                               // columns left of the current shot
+#pragma unroll
+          for (int c0 = 0; c0 < kCols; c0 += 16) {
+            if (ce > c0 + 16) {
+              acc += group[c0 / 16];
+            } else {
+              int from = c0;
+              while (from < c0 + 16) {
+                const int to = min(ce, c0 + 16);
+                float sum[2] = {0.f, 0.f};
+#pragma unroll
+                for (int c = 0; c < 16; ++c) sum[c & 1] += c0 + c >= from && c0 + c < to ? s[c0 + c] : 0.f;
+                acc += sum[0] + sum[1];
+                if (to == ce) {
+                  flush();
+                  ce = end - key0 > 4096 ? 4096 : (int)(end - key0);
+                }
+                from = to;
               }
-              from = to;
             }
           }
         }
       }
     }
-    if (ok && n_it > 0) {
+    if (ok && n_mine > 0) {
       // the shot that goes on in the next range
       if (shot < p.n_shots && (shot == 0 || (long long)t1 * kTile > p.shot_off[shot])) flush();
       float* out = p.ml_part + ((unit * p.splits + split) * kTile + r) * 2;
       out[0] = m_run;
       out[1] = l_run;
     }
+  };
+
+  if (warp < 4) {
+    regs_lower<kRelRegsIssue>();
+    if (warp == 0) role_tma();
+    else if (warp == 1) role_mma();
+  } else {
+    regs_raise<kRelRegsConsumer>();
+    role_consume();
   }
 
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, 256);
+    tmem_dealloc(tmem_base, 512);
   }
   if (threadIdx.x == 0 && *abort_flag != 0) ads_set_status(p.status, ADAPSHOT_ETIMEOUT);
 }
@@ -404,6 +446,7 @@ constexpr size_t kPieceBytes = 256u << 20;
 struct RelPlan {
   int G, n_mt, rows, rows_pad, n_tiles, splits, tiles_per_split;
   int batch;                    // M tiles per launch of the pass
+  int m_per_cta;                // of which share a CTA
   size_t off_qpack, off_ml, off_lse, off_pieces, off_mass, off_keys, total;
 };
 
@@ -422,16 +465,24 @@ RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int
   const long long fit = (long long)(kPieceBytes / per_tile) > 1 ? (long long)(kPieceBytes / per_tile) : 1;
   const long long n_batches = (m_tiles + fit - 1) / fit;
   pl.batch = (int)((m_tiles + n_batches - 1) / n_batches);
-  // Key ranges per unit: units * splits CTAs run in waves of 296 (two per SM on 148 SMs; a fixed
-  // figure, so that the workspace size does not depend on the device), each CTA costs its tiles plus
-  // about four tiles' time of start-up; the split with the cheapest waves * (tiles + 4) is taken,
-  // every range at least eight key tiles.
+  // M tiles per CTA: as many as share without leaving more than a seventh of the places empty
+  pl.m_per_cta = 1;
+  for (int m = 4; m > 1; m >>= 1)
+    if ((pl.batch + m - 1) / m * m * 7 <= pl.batch * 8) {
+      pl.m_per_cta = m;
+      break;
+    }
+  // Key ranges: the CTAs run in waves of 148 (a fixed figure, so that the workspace size does not depend on the
+  // device), each costs its tiles plus about four tiles' time of start-up; the split with the cheapest waves *
+  // (tiles + 4) is taken, every range at least eight key tiles.
   const long long units = (long long)pl.batch * Hkv;
+  const int per_cta = kGroups / pl.m_per_cta;                 // ranges of one CTA
+  const long long ctas = (long long)((pl.batch + pl.m_per_cta - 1) / pl.m_per_cta) * Hkv;
   int best_s = 1;
   long long best_cost = 0;
   for (int sp = 1; sp <= most; ++sp) {
     const long long tiles = (pl.n_tiles + sp - 1) / sp;
-    const long long waves = (units * sp + 295) / 296;
+    const long long waves = (ctas * ((sp + per_cta - 1) / per_cta) + 147) / 148;
     const long long cost = waves * (tiles + 4);
     if (sp == 1 || cost < best_cost) {
       best_s = sp;
@@ -503,7 +554,11 @@ int rel_launch(const adapshot_model_t* model, const adapshot_pool_t* pool, int l
   for (int t0 = 0; t0 < m_tiles; t0 += pl.batch) {
     const int n = m_tiles - t0 < pl.batch ? m_tiles - t0 : pl.batch;
     rp.tile0 = t0;
-    rel_pass_kernel<D><<<dim3((unsigned)n, (unsigned)pl.splits, (unsigned)Hkv), kRelThreads, smem, st>>>(tm_q, tm_k, rp);
+    rp.n_m = n;
+    rp.m_per_cta = pl.m_per_cta;
+    const int per_cta = kGroups / pl.m_per_cta;
+    rel_pass_kernel<D><<<dim3((unsigned)((n + pl.m_per_cta - 1) / pl.m_per_cta), (unsigned)((pl.splits + per_cta - 1) / per_cta),
+                              (unsigned)Hkv), kRelThreads, smem, st>>>(tm_q, tm_k, rp);
     if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
     rel_merge_kernel<<<(unsigned)(n * Hkv), 128, 0, st>>>(ml_part, pl.splits, Hkv, t0, pl.n_mt, pl.rows, lse2);
     if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;

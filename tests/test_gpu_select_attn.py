@@ -120,3 +120,11 @@ def test_a_query_whose_rows_are_cut_by_a_batch():
     w = wl.CONFIGS["cfg2"].scaled(n_shots=24000, len_lo=1, len_hi=1, batch=1, k=64, t_q=70, n_q_heads=32, n_kv_heads=8,
                                   head_dim=64, seed=88)
     _check(w, 1, 0, 64)
+
+
+@pytest.mark.parametrize("t_q,batch", [(200, 1), (20, 2), (64, 1), (100, 3)])
+def test_m_tiles_and_ranges_per_cta(t_q, batch):
+    # 7 M tiles (two CTAs of four, one place empty), 2 M tiles (they share a CTA with two ranges), 2 and 12
+    w = wl.CONFIGS["cfg2"].scaled(n_shots=70, len_lo=10, len_hi=120, batch=batch, k=30, t_q=t_q, n_q_heads=8,
+                                  n_kv_heads=2, seed=89)
+    _check(w, 1, 0, 30)
