@@ -66,6 +66,11 @@ class ProbeRounds:
         self.ws_attn = torch.empty(max(256, ab.adapshot_attn_workspace_bytes(model, batch, m, t_q, nl, self.ctx_cap)), **u8)
         self.ws_entropy = torch.empty(max(256, ab.adapshot_entropy_workspace_bytes(batch * m, vocab)), **u8)
 
+        # per round: the selection's prefix (one query's is a view, several queries' are copied round by round) and
+        # the offsets, made once because the GPU waits for the host between rounds
+        self._rounds = [(self.sel_idx[:, :probes[-1]] if batch == 1 else None, self.ctx_off(probes[-1]))
+                        for probes in self.schedule]
+
     def ctx_off(self, k: int) -> torch.Tensor:
         return self._ctx_off[: self.B * (k + 1)].view(self.B, k + 1)
 
@@ -76,8 +81,9 @@ class ProbeRounds:
         probes = self.schedule[r]
         k_r = probes[-1]
         nl = self.model.n_layers
-        sel_r = self.sel_idx[:, :k_r].contiguous()
-        off_r = self.ctx_off(k_r)
+        sel_r, off_r = self._rounds[r]
+        if sel_r is None:
+            sel_r = self.sel_idx[:, :k_r].contiguous()
         # the earlier rounds' shots are in place already: only the new ones are gathered
         first_new = self.schedule[r - 1][-1] if r > 0 else 0
         ab.adapshot_assemble_kv_from(self.model, self.pool, sel_r, first_new, 0, nl, self.k_ctx, self.v_ctx,
@@ -97,8 +103,7 @@ class ProbeRounds:
         for r, probes in enumerate(self.schedule):
             q, kq, vq, logits = round_inputs(r, probes)
             self.run_round(r, q, kq, vq, logits, tau)
-            self._verdict_host.copy_(self._verdict, non_blocking=True)
-            torch.cuda.current_stream().synchronize()
+            self._verdict_host.copy_(self._verdict)      # returns when the round is done
             verdict = self._verdict_host.tolist()
             if verdict[0] != 0:
                 raise RuntimeError(f"device status {verdict[0]}: {ab.adapshot_strerror(verdict[0])}")
