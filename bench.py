@@ -413,7 +413,7 @@ def measure(args, name: str, steps: int, warmup: int, dev, peaks, dist, rank: in
     q_emb, qc, kqc, vqc, logits = qs["q_emb"], chunk(qs["q"]), chunk(qs["kq"]), chunk(qs["vq"]), qs["logits"]
     del qs
     flush = torch.empty(L2_FLUSH_BYTES, dtype=torch.uint8, device=dev)
-    n_sel = 2 if w.n_shots <= 4096 else (3 if w.n_shots > 8192 else 2)
+    n_sel = 2             # scores as sort keys, top-k
     if fused or vpool:
         launches_per_step = n_sel + 1 + len(path.chunks) * ((1 if vpool else 0) + 4) + 2
     else:

@@ -1826,7 +1826,7 @@ extern "C" int adapshot_decode_attn(const adapshot_model_t* model, const void* k
     return ADAPSHOT_EALIGN;
   if (ctx_cap > (1ll << 31) - 256) return ADAPSHOT_ESHAPE;
   const int nl = layer_end - layer_begin;
-  // Up to 32 rows per KV head: the kernel that streams K/V through warp-level tiles (decode.cu): 253 against
+  // Up to 32 rows per KV head: the kernel that streams K/V through warp-level tiles (decode.cu): 256 against
   // 376 us at 4 rows and 32 requests.  The line is where its accumulators stop fitting two CTAs per SM; more rows
   // fill the 128-row tiles of the prefill kernels better as well.
   if (ads_decode_rows_fit(model, T_new)) {

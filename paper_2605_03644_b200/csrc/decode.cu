@@ -16,9 +16,9 @@
 //     preparation kernel and no schedule in memory.
 // A unit that a range boundary cuts leaves un-normalised partials, merged by decode_combine_kernel.
 // Measured at 32 query / 8 KV heads, d = 128, one layer per call, against the prefill kernels that took these
-// calls before: 32 requests of 6 to 16 K tokens (1.6 GB of K/V) 376 -> 253 us = 6.4 TB/s, the copy bandwidth; one request
-// (50 MB) 50 -> 21 us per call, of which the streaming kernel is 16 (start-up and merge, not bytes, are most
-// of it there) and the merge, started under its tail, 4.
+// calls before: 32 requests of 6 to 16 K tokens (1.6 GB of K/V) 376 -> 256 us = 6.4 TB/s, the copy bandwidth; one request
+// (50 MB) 50 -> 18 us per call, 13 of them a chain of latencies that no size makes shorter: launch, the unit's
+// look-up, first tiles from DRAM, merge.
 #include <cuda.h>
 #include <math.h>
 

@@ -13,7 +13,7 @@
 //   merge   the ranges' (maximum, sum) pairs -> log2-sum-exp of every row;
 //   reduce  mass of a shot = sum over rows of 2^(its log2 mass - the row's log2-sum-exp), a warp per shot.
 // (A second pass over the keys, with the normalisers known, used to take the reduce step's place: it cost as much as
-// the first, 813 of 1580 us for 2 queries x 128 tokens and 328 K pool tokens.)  What lies between the steps is 4
+// the first: 1842 us for both, 1113 with one, for 2 queries x 128 tokens and 328 K pool tokens.)  What lies between the steps is 4
 // bytes per row and shot; the rows are taken in batches that keep it below kPieceBytes.
 // The scores then go through the same top-k as the embedding selector (ties -> lower shot id).
 #include <float.h>
