@@ -176,20 +176,60 @@ gather_rope_kernel(const __grid_constant__ GatherArgs a) {
 
   if (warp == kRotWarps) {
     // ---------------------------------------------------------------- loading warp
-    const int chunks_per_query = (int)((a.ctx_cap + a.chunk - 1) / a.chunk);
-    const long long n_items = (long long)a.B * chunks_per_query * a.layer_groups;
+    // A query's chunks that hold a position to gather or to clear, [c0, c0 + n), are all that is dealt out: the capacity
+    // behind a query's last token and the prefix that stays (shot_begin) would cost a step of this warp per chunk
+    // (half a microsecond each: the last 8 of 512 shots of 32 queries of 66 K tokens, four
+    // layers of K: 754 -> 101 us, one layer 200 -> 38).  Lane i knows the i-th of the 32 queries it is at.
     const int group_layers = (a.n_layers_call + a.layer_groups - 1) / a.layer_groups;
+    long long q_len = 0, q_begin = 0, q_end = 0, q_c0 = 0;   // tokens, first position, chunks up to this query's end, c0 - chunks before it
+    int q0 = 0;
+    auto load_queries = [&](int first_query, long long before) {
+      q0 = first_query;
+      long long n = 0, c0 = 0;
+      if (q0 + lane < a.B) {
+        const long long* off = a.ctx_off + (long long)(q0 + lane) * (a.k + 1);
+        q_len = off[a.k];
+        q_begin = off[a.shot_begin];
+        c0 = q_begin / a.chunk;
+        n = (min((q_len + kTile - 1) / kTile * kTile, a.ctx_cap) + a.chunk - 1) / a.chunk - c0;
+        if (n < 0) n = 0;
+      }
+      q_end = n;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const long long o = __shfl_up_sync(0xffffffffu, q_end, d);
+        if (lane >= d) q_end += o;
+      }
+      q_end += before;
+      q_c0 = c0 - (q_end - n);
+    };
+    long long total_chunks = 0;
+    for (int q = 0; q < a.B; q += 32) {
+      load_queries(q, total_chunks);
+      total_chunks = __shfl_sync(0xffffffffu, q_end, 31);
+    }
+    if (a.B > 32) load_queries(0, 0);
     uint32_t it = 0;
     bool ok = true;
-    for (long long item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-      const int l0 = (int)(item % a.layer_groups) * group_layers;
+    // item = (chunk x, layer group lg), the groups of a chunk side by side: neighbouring CTAs take the same chunk's layers
+    long long x = blockIdx.x / a.layer_groups;
+    int lg = blockIdx.x % a.layer_groups;
+    const int step_x = gridDim.x / a.layer_groups, step_lg = gridDim.x % a.layer_groups;
+    for (; x < total_chunks && ok; x += step_x, lg += step_lg) {
+      if (lg >= a.layer_groups) {
+        lg -= a.layer_groups;
+        if (++x >= total_chunks) break;
+      }
+      for (long long e = __shfl_sync(0xffffffffu, q_end, 31); x >= e; e = __shfl_sync(0xffffffffu, q_end, 31))
+        load_queries(q0 + 32, e);
+      const int qi = __popc(__ballot_sync(0xffffffffu, q_end <= x));
+      const int b = q0 + qi;
+      const int l0 = lg * group_layers;
       const int l1 = min(a.n_layers_call, l0 + group_layers);
-      const long long chunk = item / a.layer_groups;
-      const int b = (int)(chunk / chunks_per_query);
-      const long long p0 = (chunk % chunks_per_query) * a.chunk;
+      const long long p0 = (__shfl_sync(0xffffffffu, q_c0, qi) + x) * a.chunk;
       const long long* off = a.ctx_off + (long long)b * (a.k + 1);
-      const long long L = off[a.k];
-      const long long pa = max(p0, off[a.shot_begin]);                 // positions before it stay as they are
+      const long long L = __shfl_sync(0xffffffffu, q_len, qi);
+      const long long pa = max(p0, __shfl_sync(0xffffffffu, q_begin, qi));      // positions before it stay as they are
       const long long pb = min(p0 + a.chunk, min(L, a.ctx_cap));
       // zeros for the rest of the last 128-token tile, so that whole tiles can be read later
       const long long za = max(p0, L), zb = min(p0 + a.chunk, min((L + kTile - 1) / kTile * kTile, a.ctx_cap));
@@ -258,7 +298,7 @@ gather_rope_kernel(const __grid_constant__ GatherArgs a) {
               si.pos0 = pa;
               si.n = (int)(pb - pa);
               si.is_v = v;
-              si.item = item;
+              si.item = x * a.layer_groups + lg;
             }
             if (a.k_pos_mode == 1) {
               bool more = many;

@@ -197,3 +197,36 @@ def test_gather_chunks(dtype, d, hkv, nl, lens, k, shot_begin, k_only, k_pos_mod
             assert (c[b, :, :a] == 7.0).all() and (c[b, :, end:] == 7.0).all() and (c[b, :, L:end] == 0.0).all()
         if not k_only:
             assert np.array_equal(hp.f64(vc[b, :, a:L].cpu()), want_v[:, a:L])
+
+
+@pytest.mark.parametrize("B,nl,shot_begin", [(1, 1, 5), (32, 3, 0), (33, 2, 2), (70, 1, 5)])
+@pytest.mark.parametrize("k_only", [True, False])
+def test_gather_deals_out_what_there_is_to_do(B, nl, shot_begin, k_only):
+    """Contexts far below the capacity, kept prefixes (all of it at shot_begin = k: only the zero fill is left) and
+    more queries than a warp looks at at once: every chunk with work is gathered once, nothing else is touched."""
+    ab = hp.gpu_binding()
+    k = 5
+    w = wl.CONFIGS["cfg2"].scaled(n_layers=nl, n_q_heads=2, n_kv_heads=2, head_dim=64, n_shots=40, len_lo=1, len_hi=90,
+                                  batch=B, k=k, probes=(k,), t_q=1, seed=92)
+    pool = wl.make_pool(w)
+    rng = np.random.default_rng(15)
+    sel_np = np.stack([rng.permutation(40)[:k] for _ in range(B)]).astype(np.int32)
+    off_np = orc.plan_offsets(sel_np, pool["shot_off"])
+    cap = 4 * int(off_np[:, -1].max()) + 3
+    kc = torch.full((B, nl, cap, 2, 64), 7.0, dtype=torch.bfloat16, device="cuda")
+    vc = None if k_only else kc.clone()
+    off, st = torch.zeros((B, k + 1), dtype=torch.int64, device="cuda"), hp.new_status()
+    ab.adapshot_assemble_kv_from(hp.model_of(ab, w), hp.dev_pool(ab, pool), torch.from_numpy(sel_np).cuda(), shot_begin, 0,
+                                 nl, kc, vc, cap, off, st, flags=ab.ASSEMBLE_K_ONLY if k_only else 0)
+    torch.cuda.synchronize()
+    assert st.item() == 0 and np.array_equal(off.cpu().numpy(), off_np)
+    for b in range(B):
+        want_k, want_v, _ = orc.assemble_kv(hp.f64(pool["k"]), hp.f64(pool["v"]), pool["shot_off"], sel_np[b], w.rope_base, 0)
+        a, L = int(off_np[b, shot_begin]), int(off_np[b, -1])
+        end = min(-(-L // 128) * 128, cap)
+        # one rounding to bf16 (half a step, 2^-8 relative) of an fp32 rotation
+        assert (np.abs(hp.f64(kc[b, :, a:L].cpu()) - want_k[:, a:L]) <= 2.0 ** -8 * np.abs(want_k[:, a:L]) + 1e-5).all()
+        if not k_only:
+            assert np.array_equal(hp.f64(vc[b, :, a:L].cpu()), want_v[:, a:L])
+        for c in (kc,) if k_only else (kc, vc):
+            assert (c[b, :, :a] == 7.0).all() and (c[b, :, end:] == 7.0).all() and (c[b, :, L:end] == 0.0).all()
