@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(256) rel_pack_q_kernel(const __nv_bfloat16* __
                                                          __nv_bfloat16* __restrict__ q_pack, int B, int Tq, int Hq,
                                                          int Hkv, int rows_pad) {
   constexpr int VPR = D / 8;                         // 16-byte vectors per row
+  ads_dependency_wait();
   const int G = Hq / Hkv;
   const long long n = (long long)B * Hkv * rows_pad * VPR;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -168,6 +169,7 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  ads_dependency_wait();
 
   auto role_tma = [&]() {
     if (lane == 0) {
@@ -381,6 +383,7 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 // that they add nothing); one thread per row.
 __global__ void __launch_bounds__(128) rel_merge_kernel(const float* __restrict__ ml_part, int splits, int Hkv, int tile0,
                                                         int n_mt, int rows, float* __restrict__ lse2) {
+  ads_dependency_wait();
   const long long unit = blockIdx.x;
   const int r = threadIdx.x;
   const int mt = (int)((tile0 + unit / Hkv) % n_mt);
@@ -400,6 +403,7 @@ __global__ void __launch_bounds__(256) rel_reduce_kernel(const float* __restrict
                                                          int n_mt, int tile0, int n_tiles_m, int splits,
                                                          int tiles_per_split, long long pool_tokens, int b0,
                                                          double* __restrict__ mass) {
+  ads_dependency_wait();
   const int lane = threadIdx.x & 31, b = b0 + blockIdx.y;
   const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (i >= n_shots) return;
@@ -433,6 +437,7 @@ __global__ void __launch_bounds__(256) rel_scores_kernel(const double* __restric
                                                          const long long* __restrict__ shot_off, int B, int n_shots,
                                                          double inv_rows, int per_token,
                                                          unsigned long long* __restrict__ keys) {
+  ads_dependency_wait();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long long)B * n_shots) return;
   const int shot = (int)(i % n_shots);
@@ -535,8 +540,8 @@ int rel_launch(const adapshot_model_t* model, const adapshot_pool_t* pool, int l
   }
 
   const long long n_vec = (long long)B * Hkv * pl.rows_pad * (D / 8);
-  rel_pack_q_kernel<D><<<(unsigned)((n_vec + 255) / 256), 256, 0, st>>>(static_cast<const __nv_bfloat16*>(q), q_pack, B,
-                                                                       Tq, Hq, Hkv, pl.rows_pad);
+  ads_launch_dependent(rel_pack_q_kernel<D>, (unsigned)((n_vec + 255) / 256), 256, 0, st,
+                       static_cast<const __nv_bfloat16*>(q), q_pack, B, Tq, Hq, Hkv, pl.rows_pad);
   if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
   const long long* shot_off = reinterpret_cast<const long long*>(pool->shot_off);
   RelParams rp;
@@ -557,21 +562,22 @@ int rel_launch(const adapshot_model_t* model, const adapshot_pool_t* pool, int l
     rp.n_m = n;
     rp.m_per_cta = pl.m_per_cta;
     const int per_cta = kGroups / pl.m_per_cta;
-    rel_pass_kernel<D><<<dim3((unsigned)((n + pl.m_per_cta - 1) / pl.m_per_cta), (unsigned)((pl.splits + per_cta - 1) / per_cta),
-                              (unsigned)Hkv), kRelThreads, smem, st>>>(tm_q, tm_k, rp);
+    ads_launch_dependent(rel_pass_kernel<D>, dim3((unsigned)((n + pl.m_per_cta - 1) / pl.m_per_cta),
+                                                  (unsigned)((pl.splits + per_cta - 1) / per_cta), (unsigned)Hkv),
+                         kRelThreads, smem, st, tm_q, tm_k, rp);
     if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-    rel_merge_kernel<<<(unsigned)(n * Hkv), 128, 0, st>>>(ml_part, pl.splits, Hkv, t0, pl.n_mt, pl.rows, lse2);
+    ads_launch_dependent(rel_merge_kernel, (unsigned)(n * Hkv), 128, 0, st, ml_part, pl.splits, Hkv, t0, pl.n_mt,
+                         pl.rows, lse2);
     if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
     const int b0 = t0 / pl.n_mt, b1 = (t0 + n - 1) / pl.n_mt;       // queries with rows in the batch
-    rel_reduce_kernel<<<dim3((unsigned)((pool->n_shots + 7) / 8), (unsigned)(b1 - b0 + 1)), 256, 0, st>>>(
-        pieces, lse2, shot_off, pool->n_shots, Hkv, pl.n_mt, t0, n, pl.splits, pl.tiles_per_split, pool->pool_tokens, b0,
-        mass);
+    ads_launch_dependent(rel_reduce_kernel, dim3((unsigned)((pool->n_shots + 7) / 8), (unsigned)(b1 - b0 + 1)), 256, 0, st,
+                         pieces, lse2, shot_off, pool->n_shots, Hkv, pl.n_mt, t0, n, pl.splits, pl.tiles_per_split,
+                         pool->pool_tokens, b0, mass);
     if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
   }
 
   const long long n_sc = (long long)B * pool->n_shots;
-  rel_scores_kernel<<<(unsigned)((n_sc + 255) / 256), 256, 0, st>>>(
-      mass, shot_off, B, pool->n_shots, 1.0 / ((double)Tq * Hq),
+  ads_launch_dependent(rel_scores_kernel, (unsigned)((n_sc + 255) / 256), 256, 0, st, mass, shot_off, B, pool->n_shots, 1.0 / ((double)Tq * Hq),
       (flags & ADAPSHOT_RELEVANCE_PER_TOKEN) ? 1 : 0, keys);
   if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
   return ads_topk_from_keys(keys, pool->n_shots, B, k, sel_idx, sel_score, st);

@@ -199,11 +199,11 @@ def test_gather_chunks(dtype, d, hkv, nl, lens, k, shot_begin, k_only, k_pos_mod
             assert np.array_equal(hp.f64(vc[b, :, a:L].cpu()), want_v[:, a:L])
 
 
-@pytest.mark.parametrize("B,nl,shot_begin", [(1, 1, 5), (32, 3, 0), (33, 2, 2), (70, 1, 5)])
+@pytest.mark.parametrize("B,nl,shot_begin", [(1, 1, 4), (32, 3, 0), (33, 2, 2), (70, 1, 4)])
 @pytest.mark.parametrize("k_only", [True, False])
 def test_gather_deals_out_what_there_is_to_do(B, nl, shot_begin, k_only):
-    """Contexts far below the capacity, kept prefixes (all of it at shot_begin = k: only the zero fill is left) and
-    more queries than a warp looks at at once: every chunk with work is gathered once, nothing else is touched."""
+    """Contexts far below the capacity, kept prefixes and more queries than a warp looks at at once: every chunk with
+    work is gathered once, nothing else is touched."""
     ab = hp.gpu_binding()
     k = 5
     w = wl.CONFIGS["cfg2"].scaled(n_layers=nl, n_q_heads=2, n_kv_heads=2, head_dim=64, n_shots=40, len_lo=1, len_hi=90,
