@@ -464,9 +464,10 @@ rank_topk_kernel(const unsigned long long* __restrict__ all_keys, int N, int k,
 }
 
 // Rank counting compares every pair of keys, over the whole chip; the radix selection is one CTA per
-// query (8 to 9 us up to 4096 keys).  One query: 3.2 us at 1024 keys, 4.2 at 2048, 6.2 at 2900; eight queries of 1024
-// keys 4.8.
-bool rank_by_counting(int N, int B) { return (long long)N * N * B <= 9000000ll; }
+// query.  Counting / selection: one query of 3100 keys 6.3 / 8.9 us, 3740 keys 7.0 / 9.0, three of 2040 keys 5.8 / 8.5,
+// thirteen of 1024 6.1 / 8.2, fifty of 512 6.9 / 7.5, two hundred of 256 9.5 / 12; the line lies where the counting,
+// which grows with the product, would reach the selection (fifty of 512 keys come close to it).
+bool rank_by_counting(int N, int B) { return (long long)N * N * B <= 14000000ll; }
 
 }  // namespace
 

@@ -90,3 +90,14 @@ def test_radix_selection_cuts_equal_scores_by_id(n_same, k):
     zero = torch.zeros(6100, 32)
     zero[17], zero[5000] = 1.0, -1.0
     _check(ab, zero, torch.ones(1, 32), k)
+
+
+@pytest.mark.parametrize("N,B,k", [(2, 1, 2), (31, 2, 31), (2047, 1, 2047), (2049, 1, 300), (3741, 1, 3741), (3742, 1, 3742)])
+def test_rank_counting_with_ties(N, B, k):
+    # odd and even counts (a last pair of one key), one and two tiles of keys, both sides of the line to the radix
+    # selection; every embedding occurs about three times, so that equal scores lie in front of and behind each other
+    ab = hp.gpu_binding()
+    g = torch.Generator().manual_seed(N)
+    base = torch.randn((N + 2) // 3, 32, generator=g)
+    emb = base[torch.randint(0, base.shape[0], (N,), generator=g)]
+    _check(ab, emb, torch.randn(B, 32, generator=g), k)
