@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 from typing import Optional, Sequence
 
 import torch
@@ -190,59 +191,51 @@ class Pool:
                        _ptr(shot_off), _ptr(k), _ptr(v), _ptr(emb))
 
 
-class PassT(C.Structure):
-    _fields_ = [("model", C.POINTER(ModelT)), ("pool", C.POINTER(PoolT)), ("probe_nshots", C.POINTER(_i32)),
-                ("layer_end", C.POINTER(_i32)), ("B", _i32), ("k", _i32), ("P", _i32), ("Tq", _i32), ("n_chunks", _i32),
-                ("variant", _i32), ("V", _i32), ("logits_dtype", _i32), ("logits_stride", _i64), ("ctx_cap", _i64),
-                ("q_emb", _vp), ("q", C.POINTER(_vp)), ("kq", C.POINTER(_vp)), ("vq", C.POINTER(_vp)),
-                ("out", C.POINTER(_vp)), ("logits", _vp), ("sel_idx", _vp), ("sel_score", _vp), ("ctx_off", _vp),
-                ("k_ctx", _vp), ("v_ctx", _vp), ("H", _vp), ("first_ok", _vp), ("ws_select", _vp), ("ws_attn", _vp),
-                ("ws_entropy", _vp), ("ws_select_bytes", _sz), ("ws_attn_bytes", _sz), ("ws_entropy_bytes", _sz),
-                ("status", _vp), ("tau", _f), ("reserved", _i32)]
-
-
 PASS_FULL, PASS_VPOOL, PASS_FUSED = 0, 1, 2
-_reuse_pass = _sig("adapshot_reuse_pass", C.c_int, [C.POINTER(PassT), _vp])
+_reuse_pass = _sig("adapshot_reuse_pass", C.c_int, [_vp, _vp])
+# adapshot_pass_t: model, pool, probe_nshots, layer_end | B, k, P, Tq, n_chunks, variant, V, logits_dtype | logits_stride,
+# ctx_cap | q_emb, q, kq, vq, out, logits | sel_idx, sel_score, ctx_off, k_ctx, v_ctx, H, first_ok, ws_select, ws_attn,
+# ws_entropy | their three sizes | status | tau, reserved
+_PASS_FORMAT = "4P8i2q6P10P3NPfi"
+_PASS_BYTES = struct.calcsize(_PASS_FORMAT)
 
 
-class Pass:
-    """The struct of adapshot_reuse_pass: the fixed part (buffers, sizes) is filled in once; a call sets the pointers
-    of that pass's tensors.  The tensors behind the fixed part belong to the caller, who keeps them."""
-
-    def __init__(self, model: ModelT, pool: Pool, B: int, k: int, probes: Sequence[int], Tq: int, layer_end: Sequence[int],
-                 variant: int, ctx_cap: int, buffers: dict):
-        n = len(layer_end)
-        self.n, self.rows = n, B * len(probes)
-        self._keep = (model, pool, (_i32 * len(probes))(*[int(x) for x in probes]), (_i32 * n)(*[int(x) for x in layer_end]))
-        self.ptrs = {name: (_vp * n)() for name in ("q", "kq", "vq", "out")}
-        layers = [le - lb for lb, le in zip([0, *layer_end[:-1]], layer_end)]
-        row = self.rows * Tq * model.head_dim                       # elements of one head and layer
-        self.sizes = {name: [row * h * l for l in layers] for name, h in
-                      (("q", model.n_q_heads), ("kq", model.n_kv_heads), ("vq", model.n_kv_heads), ("out", model.n_q_heads))}
-        self.c = PassT(model=C.pointer(model), pool=C.pointer(pool.c), probe_nshots=self._keep[2], layer_end=self._keep[3],
-                       B=B, k=k, P=len(probes), Tq=Tq, n_chunks=n, variant=variant, ctx_cap=ctx_cap, **self.ptrs)
-        for name, t in buffers.items():
-            setattr(self.c, name, _ptr(t))
-            if name.startswith("ws_"):
-                setattr(self.c, name + "_bytes", t.numel() * t.element_size())
-        self.ref = C.byref(self.c)
-
-    def __call__(self, q_emb: torch.Tensor, q, kq, vq, out, logits: torch.Tensor, tau: float):
-        c, n = self.c, self.n
-        if logits.stride(1) != 1 or not logits.is_cuda:
-            raise ValueError("logit rows must be contiguous, on the GPU")
-        if logits.shape[0] != self.rows or len(q) < n or len(kq) < n or len(vq) < n or len(out) < n:
-            raise ValueError("one logit row per query and probe, one tensor per layer chunk")
-        for name, ts in (("q", q), ("kq", kq), ("vq", vq), ("out", out)):
-            p, size = self.ptrs[name], self.sizes[name]
-            for i in range(n):
-                if ts[i].numel() != size[i]:
-                    raise ValueError(f"{name}[{i}] has {ts[i].numel()} elements, expected {size[i]}")
-                p[i] = _ptr(ts[i])
-        c.q_emb, c.logits, c.tau = _ptr(q_emb), logits.data_ptr(), tau
-        c.V, c.logits_stride = logits.shape[1], logits.stride(0)
-        c.logits_dtype = F32 if logits.dtype == torch.float32 else BF16
-        _check(_reuse_pass(self.ref, _stream()))
+def adapshot_reuse_pass(model: ModelT, pool: Pool, probe_nshots: Sequence[int], layer_end: Sequence[int], variant: int,
+                        k: int, Tq: int, ctx_cap: int, q_emb: torch.Tensor, q, kq, vq, out, logits: torch.Tensor,
+                        tau: float, sel_idx: torch.Tensor, sel_score: Optional[torch.Tensor], ctx_off: torch.Tensor,
+                        k_ctx: Optional[torch.Tensor], v_ctx: Optional[torch.Tensor], H: torch.Tensor,
+                        first_ok: Optional[torch.Tensor], ws_select: torch.Tensor, ws_attn: torch.Tensor,
+                        ws_entropy: torch.Tensor, status: torch.Tensor):
+    """Steps 1 to 4 of a pass in one call; q, kq, vq and out hold one tensor per chunk of layers (chunk i ends with
+    layer layer_end[i]).  Every pointer is that of this call: nothing is kept."""
+    B, P, n = sel_idx.shape[0], len(probe_nshots), len(layer_end)
+    if not logits.is_cuda or logits.stride(1) != 1:
+        raise ValueError("logit rows must be contiguous, on the GPU")
+    if logits.shape[0] != B * P or not n <= min(len(q), len(kq), len(vq), len(out)):
+        raise ValueError("one logit row per query and probe, one tensor per layer chunk")
+    row, begin = B * P * Tq * model.head_dim, 0                   # elements of one head and layer
+    row_q, row_kv = row * model.n_q_heads, row * model.n_kv_heads
+    for i, end in enumerate(layer_end):
+        n_q, n_kv, begin = row_q * (end - begin), row_kv * (end - begin), end
+        if q[i].numel() != n_q or out[i].numel() != n_q or kq[i].numel() != n_kv or vq[i].numel() != n_kv:
+            raise ValueError(f"a tensor of layer chunk {i} has another size than the pass")
+    tensors = (q_emb, sel_idx, ctx_off, H, ws_select, ws_attn, ws_entropy, status, *q[:n], *kq[:n], *vq[:n], *out[:n])
+    ptrs = [t.data_ptr() for t in tensors if t.is_cuda and t.is_contiguous()]                   # _ptr of each
+    if len(ptrs) != len(tensors):
+        raise ValueError("expected contiguous CUDA tensors")
+    # the struct, the four arrays of pointers, layer_end and probe_nshots, in one piece
+    buf = (C.c_char * (_PASS_BYTES + 36 * n + 4 * P))()
+    at = C.addressof(buf)
+    arrays, step = at + _PASS_BYTES, 8 * n
+    struct.pack_into(
+        f"{_PASS_FORMAT}{4 * n}P{n + P}i", buf, 0,
+        C.addressof(model), C.addressof(pool.c), arrays + 4 * step + 4 * n, arrays + 4 * step, B, k, P, Tq, n, variant,
+        logits.shape[1], F32 if logits.dtype == torch.float32 else BF16, logits.stride(0), ctx_cap,
+        ptrs[0], arrays, arrays + step, arrays + 2 * step, arrays + 3 * step, logits.data_ptr(),
+        ptrs[1], _ptr(sel_score) or 0, ptrs[2], _ptr(k_ctx) or 0, _ptr(v_ctx) or 0, ptrs[3], _ptr(first_ok) or 0,
+        ptrs[4], ptrs[5], ptrs[6], ws_select.nbytes, ws_attn.nbytes, ws_entropy.nbytes, ptrs[7], tau, 0,
+        *ptrs[8:], *layer_end, *probe_nshots)
+    _check(_reuse_pass(at, _stream()))
 
 
 def adapshot_select_workspace_bytes(n_shots: int, B: int, k: int) -> int:

@@ -93,16 +93,6 @@ class ReusePath:
         self.entropy_overlap = bool(entropy_overlap)
         self.side = torch.cuda.Stream(device=device)
         self.ev_begin, self.ev_entropy = torch.cuda.Event(), torch.cuda.Event()
-        buffers = dict(sel_idx=self.sel_idx, sel_score=self.sel_score, ctx_off=self.ctx_off, H=self.H,
-                       first_ok=self.first_ok, ws_select=self.ws_select, ws_attn=self.ws_attn,
-                       ws_entropy=self.ws_entropy, status=self.status)
-        if not self.fused:
-            buffers["k_ctx"] = self.k_bufs[0]
-            if not self.vpool:
-                buffers["v_ctx"] = self.v_bufs[0]
-        self.whole = ab.Pass(model, pool, batch, k, self.probes, t_q, [le for _, le in self.chunks],
-                             ab.PASS_FUSED if self.fused else ab.PASS_VPOOL if self.vpool else ab.PASS_FULL,
-                             self.ctx_cap, buffers)
         if self.overlap:
             self.ev_plan = torch.cuda.Event()
             self.ev_asm = [torch.cuda.Event() for _ in range(2)]
@@ -154,7 +144,13 @@ class ReusePath:
         gathers of a multi-chunk pass on the side stream, ordered by events).
         q_chunks[i] / kq_chunks[i] / vq_chunks[i] belong to layer chunk self.chunks[i]."""
         if not self.entropy_overlap and not self.overlap:      # one stream, the calls in order: one call
-            self.whole(q_emb, q_chunks, kq_chunks, vq_chunks, self.out, logits, tau)
+            variant = ab.PASS_FUSED if self.fused else ab.PASS_VPOOL if self.vpool else ab.PASS_FULL
+            ab.adapshot_reuse_pass(self.model, self.pool, self.probes, [le for _, le in self.chunks], variant, self.k,
+                                   self.t_q, self.ctx_cap, q_emb, q_chunks, kq_chunks, vq_chunks, self.out, logits, tau,
+                                   self.sel_idx, self.sel_score, self.ctx_off,
+                                   None if self.fused else self.k_bufs[0],
+                                   self.v_bufs[0] if variant == ab.PASS_FULL else None, self.H, self.first_ok,
+                                   self.ws_select, self.ws_attn, self.ws_entropy, self.status)
             return self.out, self.H, self.first_ok
         main = torch.cuda.current_stream()
         if self.entropy_overlap:

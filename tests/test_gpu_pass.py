@@ -1,0 +1,60 @@
+"""ReusePath.run: what it reads and writes is what the object and the call hold at that moment."""
+import pytest
+import torch
+
+from paper_2605_03644_b200 import workloads as wl
+from tests import helpers as hp
+
+pytestmark = pytest.mark.gpu
+
+VARIANTS = {"full": dict(vpool=False), "vpool": dict(vpool=True), "fused": dict(fused=True, vpool=False)}
+BUFFERS = ("sel_idx", "sel_score", "ctx_off", "H", "first_ok", "status", "ws_select", "ws_attn", "ws_entropy")
+
+
+def _workload(seed):
+    return wl.CONFIGS["cfg2"].scaled(n_layers=3, n_q_heads=4, n_kv_heads=2, n_shots=20, len_lo=20, len_hi=20, len_dist="const",
+                                     batch=3, k=6, probes=(2, 6), t_q=9, vocab=1000, emb_dim=64, seed=seed)
+
+
+def _path(w, variant):
+    from paper_2605_03644_b200 import binding as ab
+    from paper_2605_03644_b200.pipeline import ReusePath
+    pool = hp.dev_pool(ab, wl.make_pool(w))
+    return ReusePath(hp.model_of(ab, w), pool, w.batch, w.k, w.probes, w.t_q, w.vocab, w.k * w.len_hi, 2, **VARIANTS[variant])
+
+
+def _inputs(path, qs):
+    chunk = lambda x: [x[:, lb:le].contiguous().cuda() for lb, le in path.chunks]
+    return qs["q_emb"].cuda(), chunk(qs["q"]), chunk(qs["kq"]), chunk(qs["vq"]), qs["logits"].cuda(), 6.0
+
+
+@pytest.mark.parametrize("variant", VARIANTS)
+def test_a_pass_uses_the_tensors_and_the_pool_it_has_now(variant):
+    w, other = _workload(41), _workload(42)
+    path, fresh = _path(w, variant), _path(other, variant)
+    args = _inputs(path, wl.make_queries(w))
+    path.run(*args)
+    want_out, want_H, want_ok = ([t.clone() for t in fresh.run(*args)[0]], fresh.H.clone(), fresh.first_ok.clone())
+    torch.cuda.synchronize()
+    # everything the object holds is replaced, the pool among it
+    held = {name: getattr(path, name) for name in BUFFERS}
+    held.update({f"{name}[{i}]": t for name in ("k_bufs", "v_bufs", "out") for i, t in enumerate(getattr(path, name))})
+    for name in BUFFERS:
+        setattr(path, name, torch.zeros_like(held[name]))
+    for name in ("k_bufs", "v_bufs", "out"):
+        setattr(path, name, [torch.zeros_like(t) for t in getattr(path, name)])
+    path.pool, path.model = fresh.pool, fresh.model
+    before = {name: t.clone() for name, t in held.items()}
+    out, H, ok = path.run(*args)
+    torch.cuda.synchronize()
+    assert path.status.item() == 0 and fresh.status.item() == 0
+    assert H is path.H and ok is path.first_ok and torch.equal(H, want_H) and torch.equal(ok, want_ok)
+    assert torch.equal(path.sel_idx, fresh.sel_idx) and torch.equal(path.ctx_off, fresh.ctx_off)
+    assert all(torch.equal(a, b) for a, b in zip(out, want_out))
+    for name, t in held.items():
+        assert torch.equal(t, before[name]), name
+    # probes are read at the call, too
+    path.probes = fresh.probes = [1, 5]
+    a, b = path.run(*args)[0], fresh.run(*args)[0]
+    torch.cuda.synchronize()
+    assert all(torch.equal(x, y) for x, y in zip(a, b)) and not any(torch.equal(x, y) for x, y in zip(a, want_out))
