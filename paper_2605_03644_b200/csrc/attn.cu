@@ -888,8 +888,9 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     // the positions up and mark where a run ends; every run is brought as one or two power-of-two boxes
     // (maps with 128, 64, ..., 1-row boxes over the pool; a box may start at any row, its shared-memory
     // address only has to be 128-byte aligned), one box per lane, all found before the stage is waited
-    // for.  Positions beyond the context continue the last run (their P is exactly zero; rows outside
-    // the pool arrive as zeros).  The probe's own tokens are one run of the own-token tensor.
+    // for.  Positions beyond the context take rows outside the pool, which arrive as zeros: their P is exactly zero,
+    // but 0 times what the next shot of the pool holds need not be.  The probe's own tokens are one run of
+    // the own-token tensor.
     const bool is_k = FUSED && warp != kGatherWarp;
     int* rows_s = reinterpret_cast<int*>(base_ptr + SM::kOffRows + (is_k ? 512 : 0));
     const uint32_t n_st = is_k ? KS : VS;
@@ -931,7 +932,7 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             continue;
           }
           // pool row of positions lane, lane + 32, lane + 64, lane + 96 of the tile (looked up while the
-          // stage may still be in use); beyond the context the last run is continued
+          // stage may still be in use)
           const long long pos0 = (long long)(w.ctx_begin + i) * kTileN;
           const long long L_all = p.ctx_cap;            // (row map entries beyond a query's context are -1)
           int r[4];
@@ -945,15 +946,10 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 #pragma unroll
           for (int q4 = 0; q4 < 4; ++q4) valid_mask[q4] = __ballot_sync(0xffffffffu, r[q4] >= 0);
           const int n_valid = __popc(valid_mask[0]) + __popc(valid_mask[1]) + __popc(valid_mask[2]) + __popc(valid_mask[3]);
-          __syncwarp();
-#pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4) rows_s[lane + 32 * q4] = r[q4];
-          __syncwarp();
-          const int last_row = n_valid > 0 ? rows_s[n_valid - 1] : 0;
 #pragma unroll
           for (int q4 = 0; q4 < 4; ++q4) {
             const int pidx = lane + 32 * q4;
-            if (pidx >= n_valid) r[q4] = last_row + (pidx - n_valid + 1);
+            if (pidx >= n_valid) r[q4] = pidx - 2 * kTileN;       // one run of rows in front of the pool: zeros
           }
           __syncwarp();
 #pragma unroll

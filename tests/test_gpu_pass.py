@@ -58,3 +58,24 @@ def test_a_pass_uses_the_tensors_and_the_pool_it_has_now(variant):
     a, b = path.run(*args)[0], fresh.run(*args)[0]
     torch.cuda.synchronize()
     assert all(torch.equal(x, y) for x, y in zip(a, b)) and not any(torch.equal(x, y) for x, y in zip(a, want_out))
+
+
+@pytest.mark.parametrize("lens", [(20, 20), (90, 150)])
+@pytest.mark.parametrize("variant", VARIANTS)
+def test_what_unselected_shots_hold_does_not_matter(variant, lens):
+    # contexts that end within a 128-key tile, in a pool whose other shots are not numbers (slots that nothing has
+    # filled yet, for instance)
+    w = _workload(43).scaled(len_lo=lens[0], len_hi=lens[1], len_dist="uniform")
+    path = _path(w, variant)
+    args = _inputs(path, wl.make_queries(w))
+    want = [t.clone() for t in path.run(*args)[0]]
+    shot_off, chosen = path.pool.shot_off.tolist(), set(path.sel_idx.flatten().tolist())
+    assert len(chosen) < w.n_shots
+    for i in range(w.n_shots):
+        if i not in chosen:
+            path.pool.k[:, shot_off[i]:shot_off[i + 1]] = float("nan")
+            path.pool.v[:, shot_off[i]:shot_off[i + 1]] = float("inf") if i % 2 else float("nan")
+    got = path.run(*args)[0]
+    torch.cuda.synchronize()
+    assert path.status.item() == 0
+    assert all(torch.isfinite(b).all() and torch.equal(a, b) for a, b in zip(want, got))
