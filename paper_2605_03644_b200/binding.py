@@ -155,6 +155,19 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return t.data_ptr()
 
 
+def _check_q_emb(pool: Pool, q_emb: torch.Tensor, B: int):
+    if q_emb.dtype != torch.float32 or q_emb.numel() != B * pool.c.emb_dim:
+        raise ValueError(f"query embeddings {tuple(q_emb.shape)}, {q_emb.dtype}: expected {B} x {pool.c.emb_dim}, float32")
+
+
+def _logit_dtype(logits: torch.Tensor) -> int:
+    if logits.dtype == torch.float32:
+        return F32
+    if logits.dtype != torch.bfloat16:
+        raise ValueError(f"logits of {logits.dtype}, expected float32 or bfloat16")
+    return BF16
+
+
 # The handle of the current device's current stream, without the Stream object that torch.cuda.current_stream() builds
 # (3 us, paid by every call).
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
@@ -209,6 +222,8 @@ def adapshot_reuse_pass(model: ModelT, pool: Pool, probe_nshots: Sequence[int], 
     """Steps 1 to 4 of a pass in one call; q, kq, vq and out hold one tensor per chunk of layers (chunk i ends with
     layer layer_end[i]).  Every pointer is that of this call: nothing is kept."""
     B, P, n = sel_idx.shape[0], len(probe_nshots), len(layer_end)
+    dtype = torch.float32 if model.dtype == F32 else torch.bfloat16
+    _check_q_emb(pool, q_emb, B)
     if not logits.is_cuda or logits.stride(1) != 1:
         raise ValueError("logit rows must be contiguous, on the GPU")
     if logits.shape[0] != B * P or not n <= min(len(q), len(kq), len(vq), len(out)):
@@ -219,6 +234,8 @@ def adapshot_reuse_pass(model: ModelT, pool: Pool, probe_nshots: Sequence[int], 
         n_q, n_kv, begin = row_q * (end - begin), row_kv * (end - begin), end
         if q[i].numel() != n_q or out[i].numel() != n_q or kq[i].numel() != n_kv or vq[i].numel() != n_kv:
             raise ValueError(f"a tensor of layer chunk {i} has another size than the pass")
+        if q[i].dtype != dtype or out[i].dtype != dtype or kq[i].dtype != dtype or vq[i].dtype != dtype:
+            raise ValueError(f"a tensor of layer chunk {i} is not {dtype}")
     tensors = (q_emb, sel_idx, ctx_off, H, ws_select, ws_attn, ws_entropy, status, *q[:n], *kq[:n], *vq[:n], *out[:n])
     ptrs = [t.data_ptr() for t in tensors if t.is_cuda and t.is_contiguous()]                   # _ptr of each
     if len(ptrs) != len(tensors):
@@ -230,7 +247,7 @@ def adapshot_reuse_pass(model: ModelT, pool: Pool, probe_nshots: Sequence[int], 
     struct.pack_into(
         f"{_PASS_FORMAT}{4 * n}P{n + P}i", buf, 0,
         C.addressof(model), C.addressof(pool.c), arrays + 4 * step + 4 * n, arrays + 4 * step, B, k, P, Tq, n, variant,
-        logits.shape[1], F32 if logits.dtype == torch.float32 else BF16, logits.stride(0), ctx_cap,
+        logits.shape[1], _logit_dtype(logits), logits.stride(0), ctx_cap,
         ptrs[0], arrays, arrays + step, arrays + 2 * step, arrays + 3 * step, logits.data_ptr(),
         ptrs[1], _ptr(sel_score) or 0, ptrs[2], _ptr(k_ctx) or 0, _ptr(v_ctx) or 0, ptrs[3], _ptr(first_ok) or 0,
         ptrs[4], ptrs[5], ptrs[6], ws_select.nbytes, ws_attn.nbytes, ws_entropy.nbytes, ptrs[7], tau, 0,
@@ -245,6 +262,9 @@ def adapshot_select_workspace_bytes(n_shots: int, B: int, k: int) -> int:
 def adapshot_select(pool: Pool, q_emb: torch.Tensor, k: int, sel_idx: torch.Tensor,
                     sel_score: Optional[torch.Tensor], ws: torch.Tensor, status: torch.Tensor):
     B = q_emb.shape[0]
+    _check_q_emb(pool, q_emb, B)
+    if sel_idx.numel() < B * k:
+        raise ValueError(f"room for {sel_idx.numel()} selected shots, {B * k} asked for")
     _check(_select(C.byref(pool.c), _ptr(q_emb), B, k, _ptr(sel_idx), _ptr(sel_score),
                    _ptr(ws), ws.numel() * ws.element_size(), _ptr(status), _stream()))
 
@@ -391,7 +411,7 @@ def adapshot_entropy_workspace_bytes(R: int, V: int) -> int:
 def adapshot_entropy(logits: torch.Tensor, H: torch.Tensor, tau: float, rows_per_group: int,
                      first_ok: Optional[torch.Tensor], ws: torch.Tensor, status: torch.Tensor):
     R, V = logits.shape
-    dt = F32 if logits.dtype == torch.float32 else BF16
+    dt = _logit_dtype(logits)
     if logits.stride(1) != 1:
         raise ValueError("logit rows must be contiguous")
     _check(_entropy(logits.data_ptr(), dt, R, V, logits.stride(0), _ptr(H), tau, rows_per_group,
@@ -402,7 +422,7 @@ def adapshot_entropy_subset(logits: torch.Tensor, subset_ids: torch.Tensor, H: t
                             rows_per_group: int, first_ok: Optional[torch.Tensor], ws: torch.Tensor,
                             status: torch.Tensor, renorm: bool = False):
     R, V = logits.shape
-    dt = F32 if logits.dtype == torch.float32 else BF16
+    dt = _logit_dtype(logits)
     if logits.stride(1) != 1 or subset_ids.dtype != torch.int32:
         raise ValueError("logit rows must be contiguous and subset_ids int32")
     _check(_entropy_subset(logits.data_ptr(), dt, R, V, logits.stride(0), _ptr(subset_ids), subset_ids.numel(),
@@ -417,7 +437,7 @@ def adapshot_entropy_static(logits: torch.Tensor, H: torch.Tensor, tau: float, r
     is a fixed array inside the library.  Raises AdapshotError(ECAPACITY) beyond its
     size.  Calls share that array, so do not let two of them overlap on the GPU."""
     R, V = logits.shape
-    dt = F32 if logits.dtype == torch.float32 else BF16
+    dt = _logit_dtype(logits)
     if logits.stride(1) != 1:
         raise ValueError("logit rows must be contiguous")
     _check(_entropy_static(logits.data_ptr(), dt, R, V, logits.stride(0), _ptr(H), tau, rows_per_group,
