@@ -214,25 +214,28 @@ _PASS_BYTES = struct.calcsize(_PASS_FORMAT)
 
 
 def adapshot_reuse_pass(model: ModelT, pool: Pool, probe_nshots: Sequence[int], layer_end: Sequence[int], variant: int,
-                        k: int, Tq: int, ctx_cap: int, q_emb: torch.Tensor, q, kq, vq, out, logits: torch.Tensor,
+                        k: int, ctx_cap: int, q_emb: torch.Tensor, q, kq, vq, out, logits: torch.Tensor,
                         tau: float, sel_idx: torch.Tensor, sel_score: Optional[torch.Tensor], ctx_off: torch.Tensor,
                         k_ctx: Optional[torch.Tensor], v_ctx: Optional[torch.Tensor], H: torch.Tensor,
                         first_ok: Optional[torch.Tensor], ws_select: torch.Tensor, ws_attn: torch.Tensor,
                         ws_entropy: torch.Tensor, status: torch.Tensor):
-    """Steps 1 to 4 of a pass in one call; q, kq, vq and out hold one tensor per chunk of layers (chunk i ends with
-    layer layer_end[i]).  Every pointer is that of this call: nothing is kept."""
-    B, P, n = sel_idx.shape[0], len(probe_nshots), len(layer_end)
+    """Steps 1 to 4 of a pass of q_emb.shape[0] queries of q[0].shape[3] tokens in one call; q, kq, vq and out hold one
+    tensor per chunk of layers (chunk i ends with layer layer_end[i]).  The other tensors may be those of a larger
+    batch or of longer queries.  Every pointer is that of this call: nothing is kept."""
+    B, P, n, Tq = q_emb.shape[0], len(probe_nshots), len(layer_end), q[0].shape[3]
     dtype = torch.float32 if model.dtype == F32 else torch.bfloat16
     _check_q_emb(pool, q_emb, B)
     if not logits.is_cuda or logits.stride(1) != 1:
         raise ValueError("logit rows must be contiguous, on the GPU")
     if logits.shape[0] != B * P or not n <= min(len(q), len(kq), len(vq), len(out)):
         raise ValueError("one logit row per query and probe, one tensor per layer chunk")
+    if sel_idx.numel() < B * k or H.numel() < B * P:
+        raise ValueError("more queries or probes than there is room for")
     row, begin = B * P * Tq * model.head_dim, 0                   # elements of one head and layer
     row_q, row_kv = row * model.n_q_heads, row * model.n_kv_heads
     for i, end in enumerate(layer_end):
         n_q, n_kv, begin = row_q * (end - begin), row_kv * (end - begin), end
-        if q[i].numel() != n_q or out[i].numel() != n_q or kq[i].numel() != n_kv or vq[i].numel() != n_kv:
+        if q[i].numel() != n_q or out[i].numel() < n_q or kq[i].numel() < n_kv or vq[i].numel() < n_kv:
             raise ValueError(f"a tensor of layer chunk {i} has another size than the pass")
         if q[i].dtype != dtype or out[i].dtype != dtype or kq[i].dtype != dtype or vq[i].dtype != dtype:
             raise ValueError(f"a tensor of layer chunk {i} is not {dtype}")

@@ -118,12 +118,16 @@ class ReusePath:
         ab.adapshot_assemble_kv(self.model, self.pool, self.sel_idx, layer_begin, layer_end,
                                 k_ctx, v_ctx, self.ctx_cap, self.ctx_off, self.status, flags=flags)
 
+    def _selected(self, q):
+        """The selections of q's queries (a batch may hold fewer than were planned for)."""
+        return self.sel_idx if q.shape[0] == self.sel_idx.shape[0] else self.sel_idx[:q.shape[0]]
+
     def attend(self, q, kq, vq, out, layer_begin: int, layer_end: int, buf: int = 0, probes=None):
         """Attention of the probes (default: all of them; a sub-list must be ascending) over the cache."""
         k_ctx, v_ctx = self.k_bufs[buf], (None if self.vpool else self.v_bufs[buf])
         probes = self.probes if probes is None else list(probes)
         if self.vpool:
-            ab.adapshot_query_attn_vpool(self.model, self.pool, self.sel_idx, k_ctx, self.ctx_cap, self.ctx_off,
+            ab.adapshot_query_attn_vpool(self.model, self.pool, self._selected(q), k_ctx, self.ctx_cap, self.ctx_off,
                                          probes, q, kq, vq, layer_begin, layer_end, out, None,
                                          self.ws_attn, self.status)
             return
@@ -132,7 +136,7 @@ class ReusePath:
                                self.ws_attn, self.status)
 
     def attend_fused(self, q, kq, vq, out, layer_begin: int, layer_end: int):
-        ab.adapshot_query_attn_fused(self.model, self.pool, self.sel_idx, self.ctx_off, self.ctx_cap,
+        ab.adapshot_query_attn_fused(self.model, self.pool, self._selected(q), self.ctx_off, self.ctx_cap,
                                      self.probes, q, kq, vq, layer_begin, layer_end, out, None,
                                      self.ws_attn, self.status)
 
@@ -142,11 +146,12 @@ class ReusePath:
     def run(self, q_emb, q_chunks, kq_chunks, vq_chunks, logits, tau: float = 0.65):
         """One pass of the whole path; everything is enqueued on the current stream (the
         gathers of a multi-chunk pass on the side stream, ordered by events).
-        q_chunks[i] / kq_chunks[i] / vq_chunks[i] belong to layer chunk self.chunks[i]."""
+        q_chunks[i] / kq_chunks[i] / vq_chunks[i] belong to layer chunk self.chunks[i].  A batch may hold fewer queries
+        than were planned for, or shorter ones: the results are then packed in front of the buffers returned."""
         if not self.entropy_overlap and not self.overlap:      # one stream, the calls in order: one call
             variant = ab.PASS_FUSED if self.fused else ab.PASS_VPOOL if self.vpool else ab.PASS_FULL
             ab.adapshot_reuse_pass(self.model, self.pool, self.probes, [le for _, le in self.chunks], variant, self.k,
-                                   self.t_q, self.ctx_cap, q_emb, q_chunks, kq_chunks, vq_chunks, self.out, logits, tau,
+                                   self.ctx_cap, q_emb, q_chunks, kq_chunks, vq_chunks, self.out, logits, tau,
                                    self.sel_idx, self.sel_score, self.ctx_off,
                                    None if self.fused else self.k_bufs[0],
                                    self.v_bufs[0] if variant == ab.PASS_FULL else None, self.H, self.first_ok,

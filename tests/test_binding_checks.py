@@ -31,7 +31,7 @@ def _pass_args(ab, B=3, P=2, k=4, t_q=5):
     i32, u8, f32 = dict(dtype=torch.int32), dict(dtype=torch.uint8), dict(dtype=torch.float32)
     rows = lambda h: [_t(B, le - lb, P, t_q, h, d) for lb, le in ((0, 2), (2, 3))]
     return dict(model=ab.make_model(3, hq, hkv, d, "bf16", 1e4), pool=pool, probe_nshots=[2, k], layer_end=ends,
-                variant=ab.PASS_FULL, k=k, Tq=t_q, ctx_cap=40, q_emb=_t(B, 16, **f32), q=rows(hq), kq=rows(hkv),
+                variant=ab.PASS_FULL, k=k, ctx_cap=40, q_emb=_t(B, 16, **f32), q=rows(hq), kq=rows(hkv),
                 vq=rows(hkv), out=rows(hq), logits=_t(B * P, 24, **f32), tau=0.5, sel_idx=_t(B, k, **i32),
                 sel_score=_t(B, k, **f32), ctx_off=_t(B, k + 1, dtype=torch.int64), k_ctx=_t(B * 2 * 40 * hkv * d),
                 v_ctx=_t(B * 2 * 40 * hkv * d), H=_t(B * P, **f32), first_ok=_t(B, **i32), ws_select=_t(256, **u8),

@@ -16,11 +16,11 @@ def _workload(seed):
                                      batch=3, k=6, probes=(2, 6), t_q=9, vocab=1000, emb_dim=64, seed=seed)
 
 
-def _path(w, variant):
+def _path(w, variant, **kw):
     from paper_2605_03644_b200 import binding as ab
     from paper_2605_03644_b200.pipeline import ReusePath
     pool = hp.dev_pool(ab, wl.make_pool(w))
-    return ReusePath(hp.model_of(ab, w), pool, w.batch, w.k, w.probes, w.t_q, w.vocab, w.k * w.len_hi, 2, **VARIANTS[variant])
+    return ReusePath(hp.model_of(ab, w), pool, w.batch, w.k, w.probes, w.t_q, w.vocab, w.k * w.len_hi, 2, **VARIANTS[variant], **kw)
 
 
 def _inputs(path, qs):
@@ -79,3 +79,21 @@ def test_what_unselected_shots_hold_does_not_matter(variant, lens):
     torch.cuda.synchronize()
     assert path.status.item() == 0
     assert all(torch.isfinite(b).all() and torch.equal(a, b) for a, b in zip(want, got))
+
+
+@pytest.mark.parametrize("overlap", [dict(), dict(entropy_overlap=True)])
+@pytest.mark.parametrize("variant", VARIANTS)
+def test_fewer_and_shorter_queries_than_planned(variant, overlap):
+    # two of three queries, five of nine tokens: what a path planned for just that gives
+    w = _workload(44)
+    small = w.scaled(batch=2, t_q=5)
+    path, fresh = _path(w, variant, **overlap), _path(small, variant)
+    path.run(*_inputs(path, wl.make_queries(w)))              # (every query has a selection)
+    args = _inputs(fresh, wl.make_queries(small))
+    out, H, ok = path.run(*args)
+    want_out, want_H, want_ok = fresh.run(*args)
+    torch.cuda.synchronize()
+    assert path.status.item() == 0 and fresh.status.item() == 0
+    assert torch.equal(path.sel_idx[:2], fresh.sel_idx) and torch.equal(path.ctx_off[:2], fresh.ctx_off)
+    assert all(torch.equal(a.flatten()[:b.numel()], b.flatten()) for a, b in zip(out, want_out))
+    assert torch.equal(H[:want_H.numel()], want_H) and torch.equal(ok[:2], want_ok)
