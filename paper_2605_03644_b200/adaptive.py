@@ -66,11 +66,6 @@ class ProbeRounds:
         self.ws_attn = torch.empty(max(256, ab.adapshot_attn_workspace_bytes(model, batch, m, t_q, nl, self.ctx_cap)), **u8)
         self.ws_entropy = torch.empty(max(256, ab.adapshot_entropy_workspace_bytes(batch * m, vocab)), **u8)
 
-        # per round: the selection's prefix (one query's is a view, several queries' are copied round by round) and
-        # the offsets, made once because the GPU waits for the host between rounds
-        self._rounds = [(self.sel_idx[:, :probes[-1]] if batch == 1 else None, self.ctx_off(probes[-1]))
-                        for probes in self.schedule]
-
     def ctx_off(self, k: int) -> torch.Tensor:
         return self._ctx_off[: self.B * (k + 1)].view(self.B, k + 1)
 
@@ -81,9 +76,7 @@ class ProbeRounds:
         probes = self.schedule[r]
         k_r = probes[-1]
         nl = self.model.n_layers
-        sel_r, off_r = self._rounds[r]
-        if sel_r is None:
-            sel_r = self.sel_idx[:, :k_r].contiguous()
+        sel_r, off_r = self.sel_idx[:, :k_r].contiguous(), self.ctx_off(k_r)
         # the earlier rounds' shots are in place already: only the new ones are gathered
         first_new = self.schedule[r - 1][-1] if r > 0 else 0
         ab.adapshot_assemble_kv_from(self.model, self.pool, sel_r, first_new, 0, nl, self.k_ctx, self.v_ctx,
@@ -91,6 +84,16 @@ class ProbeRounds:
         ab.adapshot_query_attn(self.model, self.k_ctx, self.v_ctx, self.ctx_cap, off_r, k_r, probes,
                                q, kq, vq, 0, nl, self.out, None, self.ws_attn, self.status)
         ab.adapshot_entropy(logits, self.H, tau, self.m, self.first_ok, self.ws_entropy, self.status)
+
+    def _verdict_of_round(self):
+        """The status word and first_ok, when the round is done: by one copy while they lie side by side (status and
+        first_ok may have been replaced)."""
+        at = self._verdict.data_ptr()
+        if self.status.data_ptr() != at or self.first_ok.data_ptr() != at + 16:
+            return self.status.item(), self.first_ok.tolist()
+        self._verdict_host.copy_(self._verdict)
+        host = self._verdict_host.tolist()
+        return host[0], host[4:]
 
     def run(self, q_emb: torch.Tensor, round_inputs: Callable[[int, List[int]], tuple], tau: float = 0.65,
             on_round: Optional[Callable[[int, "ProbeRounds"], None]] = None):
@@ -103,11 +106,10 @@ class ProbeRounds:
         for r, probes in enumerate(self.schedule):
             q, kq, vq, logits = round_inputs(r, probes)
             self.run_round(r, q, kq, vq, logits, tau)
-            self._verdict_host.copy_(self._verdict)      # returns when the round is done
-            verdict = self._verdict_host.tolist()
-            if verdict[0] != 0:
-                raise RuntimeError(f"device status {verdict[0]}: {ab.adapshot_strerror(verdict[0])}")
-            per_round.append(verdict[4:])
+            status, first_ok = self._verdict_of_round()
+            if status != 0:
+                raise RuntimeError(f"device status {status}: {ab.adapshot_strerror(status)}")
+            per_round.append(first_ok)
             if on_round is not None:
                 on_round(r, self)
             if all(s != (-1, -1) for s in first_stops(per_round)):

@@ -97,3 +97,30 @@ def test_fewer_and_shorter_queries_than_planned(variant, overlap):
     assert torch.equal(path.sel_idx[:2], fresh.sel_idx) and torch.equal(path.ctx_off[:2], fresh.ctx_off)
     assert all(torch.equal(a.flatten()[:b.numel()], b.flatten()) for a, b in zip(out, want_out))
     assert torch.equal(H[:want_H.numel()], want_H) and torch.equal(ok[:2], want_ok)
+
+
+@pytest.mark.parametrize("batch", [1, 2])
+def test_rounds_of_probes_use_the_tensors_they_have_now(batch):
+    from paper_2605_03644_b200 import binding as ab
+    from paper_2605_03644_b200.adaptive import ProbeRounds
+    w = _workload(45).scaled(batch=batch, n_shots=12)
+    make = lambda seed: ProbeRounds(hp.model_of(ab, w), hp.dev_pool(ab, wl.make_pool(w.scaled(seed=seed))), batch, 1, 2, 2, 2,
+                                    w.t_q, w.vocab, 160)
+    driver, fresh = make(45), make(46)
+    qs = [wl.make_queries(w.scaled(seed=50 + r)) for r in range(2)]
+    inputs = lambda r, probes: tuple(qs[r][name].cuda() for name in ("q", "kq", "vq", "logits"))
+    q_emb = qs[0]["q_emb"].cuda()
+    tau = float(torch.softmax(qs[1]["logits"].double(), 1).log().mul(-torch.softmax(qs[1]["logits"].double(), 1)).sum(1).max()) + 0.01
+    driver.run(q_emb, inputs, 0.0)
+    want = fresh.run(q_emb, inputs, tau)
+    for name in ("sel_idx", "sel_score", "status", "first_ok", "H", "out", "k_ctx", "v_ctx", "_ctx_off"):
+        setattr(driver, name, torch.zeros_like(getattr(driver, name)))
+    driver.pool = fresh.pool
+    assert driver.run(q_emb, inputs, tau) == want and want["n_star"][0] > 0
+    torch.cuda.synchronize()
+    assert torch.equal(driver.sel_idx, fresh.sel_idx) and torch.equal(driver.out, fresh.out)
+    assert torch.equal(driver.first_ok, fresh.first_ok)
+    # an error is seen in the status word it was written to
+    driver.ctx_cap = 32
+    with pytest.raises(RuntimeError, match="capacity"):
+        driver.run(q_emb, inputs, 0.0)
