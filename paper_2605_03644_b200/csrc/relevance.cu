@@ -43,8 +43,9 @@ __device__ __forceinline__ float rel_ex2(float x) {
 
 // 2^x for a pair of scores on the FMA pipe (for x <= 0 or thereabouts; x below -125, -inf included, gives
 // about 2^-125 instead of 0, which no sum here can see):
-// x = n + f with n = round(x) taken from the low mantissa bits of x + 1.5 * 2^23, 2^f by a cubic on
-// [-0.5, 0.5] (relative error 7.5e-5, fitted for this build), n added to the exponent field.  The
+// x = n + f with n = round(x) taken from the low mantissa bits of x + 1.5 * 2^23, 2^f by the quartic on
+// [-0.5, 0.5] whose largest relative error is smallest (2.6e-6; 7e-7 at f = 0, where every row's largest score lies:
+// a cubic, 7.2e-5 there, made the masses of peaked rows wrong by 1.6e-5), n added to the exponent field.  The
 // passes send every fourth pair here: the exponential unit (16 results per clock and SM) is what
 // bounds it together with instruction issue (856 us with none there, 791 with every fourth,
 // 867 with every second pair).
@@ -55,9 +56,10 @@ __device__ __forceinline__ float2 rel_ex2_poly2(float2 x) {
   const float2 t = __fadd2_rn(x, make_float2(kMagic, kMagic));
   const float2 n = __fadd2_rn(t, make_float2(-kMagic, -kMagic));
   const float2 f = __fadd2_rn(x, make_float2(-n.x, -n.y));
-  float2 p = __ffma2_rn(make_float2(0.0551716685f, 0.0551716685f), f, make_float2(0.2426111251f, 0.2426111251f));
-  p = __ffma2_rn(p, f, make_float2(0.6932609677f, 0.6932609677f));
-  p = __ffma2_rn(p, f, make_float2(0.9999280572f, 0.9999280572f));
+  float2 p = __ffma2_rn(make_float2(0.009570102207f, 0.009570102207f), f, make_float2(0.05591785908f, 0.05591785908f));
+  p = __ffma2_rn(p, f, make_float2(0.2402474433f, 0.2402474433f));
+  p = __ffma2_rn(p, f, make_float2(0.6931217909f, 0.6931217909f));
+  p = __ffma2_rn(p, f, make_float2(0.9999992847f, 0.9999992847f));
   return make_float2(__uint_as_float(__float_as_uint(p.x) + (__float_as_uint(t.x) << 23)),
                      __uint_as_float(__float_as_uint(p.y) + (__float_as_uint(t.y) << 23)));
 }

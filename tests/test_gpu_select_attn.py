@@ -128,3 +128,26 @@ def test_m_tiles_and_ranges_per_cta(t_q, batch):
     w = wl.CONFIGS["cfg2"].scaled(n_shots=70, len_lo=10, len_hi=120, batch=batch, k=30, t_q=t_q, n_q_heads=8,
                                   n_kv_heads=2, seed=89)
     _check(w, 1, 0, 30)
+
+
+def _scores_and_masses(gain, t_q):
+    """Keys and queries that lean towards a common direction: logits of about ten times the gain with many shots close to
+    the largest.  Returns the call's scores and the oracle's, in the call's order."""
+    ab = hp.gpu_binding()
+    w = wl.CONFIGS["cfg2"].scaled(n_shots=200, len_lo=16, len_hi=80, batch=1, k=200, t_q=t_q, n_q_heads=8, n_kv_heads=2,
+                                  channel_scale=False, seed=90)
+    pool, qs = wl.make_pool(w, n_layers=1), wl.make_queries(w, n_layers=1, n_probes=1)
+    lean = torch.nn.functional.normalize(torch.randn(2, 128, generator=torch.Generator().manual_seed(3)), dim=1)
+    pool["k"] = (pool["k"].float() + 8.0 * lean).to(torch.bfloat16)
+    q = (qs["q"][:, 0, 0].float() + 8.0 * gain * lean.repeat_interleave(4, 0)).to(torch.bfloat16).contiguous()
+    sel, score = _run(ab, hp.model_of(ab, w, n_layers=1), hp.dev_pool(ab, pool), 0, q, 200)
+    s = orc.relevance_attention(hp.f64(q[0]), hp.f64(pool["k"][0]), pool["shot_off"])
+    return score[0], s[sel[0]]
+
+
+@pytest.mark.parametrize("t_q", [8, 40])
+def test_masses_of_peaked_rows(t_q):
+    # Logits of about 40.  The exponentials are good to 2.6e-6 and so is the normaliser; a score of 40 / ln 2 = 58 carries an
+    # fp32 sum's rounding, 2^-24 * 58 = 3.4e-6 at a time.  (Seen: 4e-7 of the norm.)
+    score, want = _scores_and_masses(4.0, t_q)
+    assert np.linalg.norm(score - want) <= 5e-6 * np.linalg.norm(want)
