@@ -7,11 +7,14 @@
 //
 // One pass over the pool's K of that layer, on the tensor cores (tcgen05, S in TMEM, tiles staged by TMA).  The
 // normaliser of a row is only known after all keys have been seen, so the pass leaves, for every query row and shot,
-// the log2 of the row's un-normalised mass on the shot:
+// the log2 of the row's un-normalised mass on the shot, relative to the row's first maximum in that range of keys:
 //   pass    S = Q K^T, one thread per query row (TMEM lane): running maximum, exponentials, and their sum over
-//           every shot of the CTA's range of keys, written as maximum + log2(sum) at the shot's end;
-//   merge   the ranges' (maximum, sum) pairs -> log2-sum-exp of every row;
-//   reduce  mass of a shot = sum over rows of 2^(its log2 mass - the row's log2-sum-exp), a warp per shot.
+//           every shot of the CTA's range of keys, written as maximum - first maximum + log2(sum) at the shot's end;
+//   merge   the ranges' maxima and sums -> what is left to add to a range's pieces: its first maximum - log2-sum-exp of
+//           the row;
+//   reduce  mass of a shot = sum over rows of 2^(its piece + the row's share), a warp per shot.
+// (Both are small where the mass is, however large the scores are. As maximum + log2(sum) every piece carried the rounding of
+// the maximum, each shot its own: 2.5e-5 of a shot's mass at logits of 2048, now 3e-6 at most.)
 // (A second pass over the keys, with the normalisers known, used to take the reduce step's place: it cost as much as
 // the first: 1842 us for both, 1113 with one, for 2 queries x 128 tokens and 328 K pool tokens.)  What lies between the steps is 4
 // bytes per row and shot; the rows are taken in batches that keep it below kPieceBytes.
@@ -66,8 +69,8 @@ __device__ __forceinline__ float2 rel_ex2_poly2(float2 x) {
 
 // A unit is an M tile (of a query) and a KV head; units of a batch of M tiles are numbered from 0.
 struct RelParams {
-  float* ml_part;               // [unit][split][128][2] (max in log2 units, sum)
-  float* pieces;                // [unit][n_shots + splits][128]: log2 mass of row on shot i in range s, at slot s + i
+  float* ml_part;               // [unit][split][3][128]: max (log2 units), sum, first max; the merge replaces the last
+  float* pieces;                // [unit][n_shots + splits][128]: log2 mass of row on shot i in range s - first max, at slot s + i
   const long long* shot_off;
   int32_t* status;
   long long pool_tokens;
@@ -252,6 +255,7 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const int r = quarter * 32 + lane;                      // TMEM lane: query row
     const uint32_t lane_addr = static_cast<uint32_t>(quarter * 32) << 16;
     float m_run = -1.0e30f, l_run = 0.f, acc = 0.f;         // running maximum, sum of the shots so far, of the current one
+    float m_first = 0.f;                                    // the maximum of the first keys (0 where they have none)
     // the current shot and where it and the next one end (the last one with the pool); the same in every lane
     auto shot_end = [&](int i) -> long long {
       return i + 1 < p.n_shots ? p.shot_off[i + 1] : i + 1 == p.n_shots ? p.pool_tokens : (1ll << 62);
@@ -267,7 +271,7 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     long long end = shot_end(shot), end_next = shot_end(shot + 1);
     float* piece = p.pieces + ((unit * (p.n_shots + p.splits) + split + shot) * kTile + r);
     auto flush = [&]() {                                    // the current shot is complete (in this range)
-      *piece = m_run + __log2f(acc);
+      *piece = (m_run - m_first) + __log2f(acc);
       l_run += acc;
       acc = 0.f;
       piece += kTile;
@@ -308,6 +312,7 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           acc *= keep;
           m_run = mx;
         }
+        if (half == 0 && i == 0 && m_run > -1.0e29f) m_first = m_run;
         // two scores per FMA / add instruction; the exponentials themselves are one MUFU operation each
         const float2 scale2 = make_float2(p.scale_log2, p.scale_log2), neg_m2 = make_float2(-m_run, -m_run);
         float group[kCols / 16];                            // sums of 16 keys
@@ -357,9 +362,10 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     if (ok && n_mine > 0) {
       // the shot that goes on in the next range
       if (shot < p.n_shots && (shot == 0 || (long long)t1 * kTile > p.shot_off[shot])) flush();
-      float* out = p.ml_part + ((unit * p.splits + split) * kTile + r) * 2;
+      float* out = p.ml_part + (unit * p.splits + split) * 3 * kTile + r;
       out[0] = m_run;
-      out[1] = l_run;
+      out[kTile] = l_run;
+      out[2 * kTile] = m_first;
     }
   };
 
@@ -381,26 +387,29 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   if (threadIdx.x == 0 && *abort_flag != 0) ads_set_status(p.status, ADAPSHOT_ETIMEOUT);
 }
 
-// lse2[unit][row] = log2 sum_keys 2^(s c) from the per-range (max, sum) pairs, +inf for rows that do not exist (so
-// that they add nothing); one thread per row.
-__global__ void __launch_bounds__(128) rel_merge_kernel(const float* __restrict__ ml_part, int splits, int Hkv, int tile0,
-                                                        int n_mt, int rows, float* __restrict__ lse2) {
+// What is left to add to the pieces of a row in every range: first max - log2 sum_keys 2^(s c), -inf for rows that do not exist
+// (so that they add nothing); one thread per row.
+__global__ void __launch_bounds__(128) rel_merge_kernel(float* __restrict__ ml_part, int splits, int Hkv, int tile0,
+                                                        int n_mt, int rows) {
   ads_dependency_wait();
   const long long unit = blockIdx.x;
   const int r = threadIdx.x;
   const int mt = (int)((tile0 + unit / Hkv) % n_mt);
+  float* ml = ml_part + unit * splits * 3 * kTile + r;              // a range's figures are 3 * 128 floats
   float M = -1.0e30f;
-  for (int s = 0; s < splits; ++s) M = fmaxf(M, ml_part[((unit * splits + s) * kTile + r) * 2]);
+  for (int s = 0; s < splits; ++s) M = fmaxf(M, ml[s * 3 * kTile]);
   float l = 0.f;
+  for (int s = 0; s < splits; ++s) l += ml[s * 3 * kTile + kTile] * exp2f(ml[s * 3 * kTile] - M);
+  const bool exists = mt * kTile + r < rows;
   for (int s = 0; s < splits; ++s) {
-    const float* ml = ml_part + ((unit * splits + s) * kTile + r) * 2;
-    l += ml[1] * exp2f(ml[0] - M);
+    float* first = ml + s * 3 * kTile + 2 * kTile;
+    *first = !exists ? -INFINITY : l > 0.f ? (*first - M) - log2f(l) : *first;
   }
-  lse2[unit * kTile + r] = mt * kTile + r >= rows ? INFINITY : l > 0.f ? M + log2f(l) : 0.f;
 }
 
-// mass[b][i] (+)= sum over the batch's rows of query b of 2^(piece - lse); grid (shots / 8, queries), a warp per shot.
-__global__ void __launch_bounds__(256) rel_reduce_kernel(const float* __restrict__ pieces, const float* __restrict__ lse2,
+// mass[b][i] (+)= sum over the batch's rows of query b of 2^(piece + the row's share); grid (shots / 8, queries), a warp per
+// shot.
+__global__ void __launch_bounds__(256) rel_reduce_kernel(const float* __restrict__ pieces, const float* __restrict__ ml_part,
                                                          const long long* __restrict__ shot_off, int n_shots, int Hkv,
                                                          int n_mt, int tile0, int n_tiles_m, int splits,
                                                          int tiles_per_split, long long pool_tokens, int b0,
@@ -414,17 +423,17 @@ __global__ void __launch_bounds__(256) rel_reduce_kernel(const float* __restrict
   const int s0 = (int)(o0 / kTile) / tiles_per_split, s1 = (int)((o1 - 1) / kTile) / tiles_per_split;
   double sum = 0.0;
   for (int m = first; m < last; ++m) {
-    const float4* lse = reinterpret_cast<const float4*>(lse2 + (long long)(m - tile0) * Hkv * kTile) + lane;
     for (int s = s0; s <= s1; ++s) {
       const float4* pc = reinterpret_cast<const float4*>(
           pieces + (((long long)(m - tile0) * Hkv * (n_shots + splits)) + s + i) * kTile) + lane;
-      float part = 0.f;
+      const float4* share = reinterpret_cast<const float4*>(
+          ml_part + (((long long)(m - tile0) * Hkv * splits + s) * 3 + 2) * kTile) + lane;
 #pragma unroll 8
       for (int g = 0; g < Hkv; ++g) {
-        const float4 v = pc[(long long)g * (n_shots + splits) * (kTile / 4)], n = lse[g * (kTile / 4)];
-        part += (rel_ex2(v.x - n.x) + rel_ex2(v.y - n.y)) + (rel_ex2(v.z - n.z) + rel_ex2(v.w - n.w));
+        const float4 v = pc[(long long)g * (n_shots + splits) * (kTile / 4)], n = share[(long long)g * splits * 3 * (kTile / 4)];
+        const float part = (rel_ex2(v.x + n.x) + rel_ex2(v.y + n.y)) + (rel_ex2(v.z + n.z) + rel_ex2(v.w + n.w));
+        sum += (double)part;
       }
-      sum += (double)part;
     }
   }
   sum = warp_sum(sum);
@@ -454,7 +463,7 @@ struct RelPlan {
   int G, n_mt, rows, rows_pad, n_tiles, splits, tiles_per_split;
   int batch;                    // M tiles per launch of the pass
   int m_per_cta;                // of which share a CTA
-  size_t off_qpack, off_ml, off_lse, off_pieces, off_mass, off_keys, total;
+  size_t off_qpack, off_ml, off_pieces, off_mass, off_keys, total;
 };
 
 RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int B, int Tq) {
@@ -500,8 +509,7 @@ RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int
   pl.splits = (pl.n_tiles + pl.tiles_per_split - 1) / pl.tiles_per_split;
   size_t off = 0;
   pl.off_qpack = off;   off += ads_round_up((size_t)B * Hkv * pl.rows_pad * D * 2, 256);
-  pl.off_ml = off;      off += ads_round_up((size_t)units * pl.splits * kTile * 2 * 4, 256);
-  pl.off_lse = off;     off += ads_round_up((size_t)units * kTile * 4, 256);
+  pl.off_ml = off;      off += ads_round_up((size_t)units * pl.splits * kTile * 3 * 4, 256);
   pl.off_pieces = off;  off += ads_round_up((size_t)units * ((size_t)pool->n_shots + pl.splits) * kTile * 4, 256);
   pl.off_mass = off;    off += ads_round_up((size_t)B * pool->n_shots * 8, 256);
   pl.off_keys = off;    off += ads_round_up((size_t)B * pool->n_shots * 8, 256);
@@ -522,7 +530,6 @@ int rel_launch(const adapshot_model_t* model, const adapshot_pool_t* pool, int l
   unsigned char* wsb = static_cast<unsigned char*>(ws);
   __nv_bfloat16* q_pack = reinterpret_cast<__nv_bfloat16*>(wsb + pl.off_qpack);
   float* ml_part = reinterpret_cast<float*>(wsb + pl.off_ml);
-  float* lse2 = reinterpret_cast<float*>(wsb + pl.off_lse);
   float* pieces = reinterpret_cast<float*>(wsb + pl.off_pieces);
   double* mass = reinterpret_cast<double*>(wsb + pl.off_mass);
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(wsb + pl.off_keys);
@@ -569,11 +576,11 @@ int rel_launch(const adapshot_model_t* model, const adapshot_pool_t* pool, int l
                          kRelThreads, smem, st, tm_q, tm_k, rp);
     if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
     ads_launch_dependent(rel_merge_kernel, (unsigned)(n * Hkv), 128, 0, st, ml_part, pl.splits, Hkv, t0, pl.n_mt,
-                         pl.rows, lse2);
+                         pl.rows);
     if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
     const int b0 = t0 / pl.n_mt, b1 = (t0 + n - 1) / pl.n_mt;       // queries with rows in the batch
     ads_launch_dependent(rel_reduce_kernel, dim3((unsigned)((pool->n_shots + 7) / 8), (unsigned)(b1 - b0 + 1)), 256, 0, st,
-                         pieces, lse2, shot_off, pool->n_shots, Hkv, pl.n_mt, t0, n, pl.splits, pl.tiles_per_split,
+                         pieces, ml_part, shot_off, pool->n_shots, Hkv, pl.n_mt, t0, n, pl.splits, pl.tiles_per_split,
                          pool->pool_tokens, b0, mass);
     if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
   }

@@ -151,3 +151,20 @@ def test_masses_of_peaked_rows(t_q):
     # fp32 sum's rounding, 2^-24 * 58 = 3.4e-6 at a time.  (Seen: 4e-7 of the norm.)
     score, want = _scores_and_masses(4.0, t_q)
     assert np.linalg.norm(score - want) <= 5e-6 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("big", [0.0, 128.0])
+def test_masses_do_not_carry_the_rounding_of_large_scores(big):
+    # whole numbers, so that the scores are exact; with big = 128 all of them are 2048 larger, which the masses must not show:
+    # the exponentials (2.6e-6) are all that is rounded
+    ab = hp.gpu_binding()
+    w = wl.CONFIGS["cfg2"].scaled(n_shots=150, len_lo=16, len_hi=40, batch=1, k=150, t_q=6, n_q_heads=4, n_kv_heads=2,
+                                  head_dim=64, seed=91)
+    pool = wl.make_pool(w, n_layers=1)
+    g = torch.Generator().manual_seed(4)
+    pool["k"] = torch.randint(-1, 2, pool["k"].shape, generator=g).to(torch.bfloat16)
+    q = torch.randint(-2, 3, (1, 6, 4, 64), generator=g).to(torch.bfloat16)
+    pool["k"][..., 0], q[..., 0] = big, big
+    sel, score = _run(ab, hp.model_of(ab, w, n_layers=1), hp.dev_pool(ab, pool), 0, q, 150)
+    s = orc.relevance_attention(hp.f64(q[0]), hp.f64(pool["k"][0]), pool["shot_off"])
+    assert np.all(np.abs(score[0] - s[sel[0]]) <= 3e-6 * s[sel[0]])
