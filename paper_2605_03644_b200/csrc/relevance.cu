@@ -17,7 +17,8 @@
 // the maximum, each shot its own: 2.5e-5 of a shot's mass at logits of 2048, now 3e-6 at most.)
 // (A second pass over the keys, with the normalisers known, used to take the reduce step's place: it cost as much as
 // the first: 1842 us for both, 1113 with one, for 2 queries x 128 tokens and 328 K pool tokens.)  What lies between the steps is 4
-// bytes per row and shot; the rows are taken in batches that keep it below kPieceBytes.
+// bytes per row and shot; the rows are taken in batches (of M tiles, and of KV heads where one tile is too much) that keep
+// it below kPieceBytes.
 // The scores then go through the same top-k as the embedding selector (ties -> lower shot id).
 #include <float.h>
 
@@ -67,7 +68,8 @@ __device__ __forceinline__ float2 rel_ex2_poly2(float2 x) {
                      __uint_as_float(__float_as_uint(p.y) + (__float_as_uint(t.y) << 23)));
 }
 
-// A unit is an M tile (of a query) and a KV head; units of a batch of M tiles are numbered from 0.
+// A unit is an M tile (of a query) and a KV head; units of a batch (M tiles from tile0 on, heads from head0 on) are numbered
+// from 0.
 struct RelParams {
   float* ml_part;               // [unit][split][3][128]: max (log2 units), sum, first max; the merge replaces the last
   float* pieces;                // [unit][n_shots + splits][128]: log2 mass of row on shot i in range s - first max, at slot s + i
@@ -75,6 +77,7 @@ struct RelParams {
   int32_t* status;
   long long pool_tokens;
   int Hkv, n_mt, n_shots, layer, tile0;     // tile0: first of the batch's M tiles (b * n_mt + mt)
+  int head0, n_heads;           // KV heads of the batch
   int n_tiles, splits, tiles_per_split;
   int n_m, m_per_cta;           // M tiles of the batch; how many of them share a CTA's K tiles (1, 2 or 4)
   float scale_log2;
@@ -114,7 +117,7 @@ struct RelSmem {
   static constexpr uint32_t kTotal = kOffBar + 256 + 1024;      // + alignment slack
 };
 
-// grid (groups of M tiles, groups of key ranges, Hkv).  The four consumer groups of a CTA take m_per_cta M tiles times
+// grid (groups of M tiles, groups of key ranges, KV heads).  The four consumer groups of a CTA take m_per_cta M tiles times
 // 4 / m_per_cta key ranges: group x has M tile x % m_per_cta and range x / m_per_cta.  M tiles of a CTA share
 // every K tile; where there are few of them the ranges keep all groups busy.  CTAs that differ in their M tiles only
 // walk the same key tiles at the same time, so the pool's K layer is read from DRAM about once.
@@ -140,7 +143,7 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + SM::kOffBar + 8 * kRNumBars + 8);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = blockIdx.z;
+  const int g = p.head0 + blockIdx.z;
   const int m0 = blockIdx.x * p.m_per_cta, n_m = min(p.m_per_cta, p.n_m - m0);      // M tiles of this CTA
   const int s0 = blockIdx.y * (kGroups / p.m_per_cta), n_s = min(kGroups / p.m_per_cta, p.splits - s0);   // its ranges
   const int stages = kSmemTiles - p.m_per_cta;
@@ -251,7 +254,7 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const int m = x % p.m_per_cta, j = x / p.m_per_cta;
     if (m >= n_m || j >= n_s) return;                       // fewer M tiles or ranges than the CTA has room for
     const int split = s0 + j, n_mine = range_tiles(j), t0 = split * p.tiles_per_split, t1 = t0 + n_mine;
-    const long long unit = (long long)(m0 + m) * p.Hkv + g;
+    const long long unit = (long long)(m0 + m) * p.n_heads + blockIdx.z;
     const int r = quarter * 32 + lane;                      // TMEM lane: query row
     const uint32_t lane_addr = static_cast<uint32_t>(quarter * 32) << 16;
     float m_run = -1.0e30f, l_run = 0.f, acc = 0.f;         // running maximum, sum of the shots so far, of the current one
@@ -389,12 +392,12 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 
 // What is left to add to the pieces of a row in every range: first max - log2 sum_keys 2^(s c), -inf for rows that do not exist
 // (so that they add nothing); one thread per row.
-__global__ void __launch_bounds__(128) rel_merge_kernel(float* __restrict__ ml_part, int splits, int Hkv, int tile0,
+__global__ void __launch_bounds__(128) rel_merge_kernel(float* __restrict__ ml_part, int splits, int n_heads, int tile0,
                                                         int n_mt, int rows) {
   ads_dependency_wait();
   const long long unit = blockIdx.x;
   const int r = threadIdx.x;
-  const int mt = (int)((tile0 + unit / Hkv) % n_mt);
+  const int mt = (int)((tile0 + unit / n_heads) % n_mt);
   float* ml = ml_part + unit * splits * 3 * kTile + r;              // a range's figures are 3 * 128 floats
   float M = -1.0e30f;
   for (int s = 0; s < splits; ++s) M = fmaxf(M, ml[s * 3 * kTile]);
@@ -407,12 +410,12 @@ __global__ void __launch_bounds__(128) rel_merge_kernel(float* __restrict__ ml_p
   }
 }
 
-// mass[b][i] (+)= sum over the batch's rows of query b of 2^(piece + the row's share); grid (shots / 8, queries), a warp per
+// mass[b][i] (+)= sum over the batch's rows and heads of query b of 2^(piece + the row's share); grid (shots / 8, queries), a warp per
 // shot.
 __global__ void __launch_bounds__(256) rel_reduce_kernel(const float* __restrict__ pieces, const float* __restrict__ ml_part,
-                                                         const long long* __restrict__ shot_off, int n_shots, int Hkv,
+                                                         const long long* __restrict__ shot_off, int n_shots, int n_heads,
                                                          int n_mt, int tile0, int n_tiles_m, int splits,
-                                                         int tiles_per_split, long long pool_tokens, int b0,
+                                                         int tiles_per_split, long long pool_tokens, int b0, int head0,
                                                          double* __restrict__ mass) {
   ads_dependency_wait();
   const int lane = threadIdx.x & 31, b = b0 + blockIdx.y;
@@ -425,11 +428,11 @@ __global__ void __launch_bounds__(256) rel_reduce_kernel(const float* __restrict
   for (int m = first; m < last; ++m) {
     for (int s = s0; s <= s1; ++s) {
       const float4* pc = reinterpret_cast<const float4*>(
-          pieces + (((long long)(m - tile0) * Hkv * (n_shots + splits)) + s + i) * kTile) + lane;
+          pieces + (((long long)(m - tile0) * n_heads * (n_shots + splits)) + s + i) * kTile) + lane;
       const float4* share = reinterpret_cast<const float4*>(
-          ml_part + (((long long)(m - tile0) * Hkv * splits + s) * 3 + 2) * kTile) + lane;
+          ml_part + (((long long)(m - tile0) * n_heads * splits + s) * 3 + 2) * kTile) + lane;
 #pragma unroll 8
-      for (int g = 0; g < Hkv; ++g) {
+      for (int g = 0; g < n_heads; ++g) {
         const float4 v = pc[(long long)g * (n_shots + splits) * (kTile / 4)], n = share[(long long)g * splits * 3 * (kTile / 4)];
         const float part = (rel_ex2(v.x + n.x) + rel_ex2(v.y + n.y)) + (rel_ex2(v.z + n.z) + rel_ex2(v.w + n.w));
         sum += (double)part;
@@ -439,7 +442,7 @@ __global__ void __launch_bounds__(256) rel_reduce_kernel(const float* __restrict
   sum = warp_sum(sum);
   if (lane == 0) {
     double* out = mass + (long long)b * n_shots + i;
-    *out = first == b * n_mt ? sum : *out + sum;
+    *out = first == b * n_mt && head0 == 0 ? sum : *out + sum;
   }
 }
 
@@ -458,10 +461,11 @@ __global__ void __launch_bounds__(256) rel_scores_kernel(const double* __restric
 }
 
 constexpr size_t kPieceBytes = 256u << 20;
+constexpr long long kMaxRanges = 16 * 148 * kGroups;     // (unit, range) pairs of a launch that are worth having: sixteen waves
 
 struct RelPlan {
   int G, n_mt, rows, rows_pad, n_tiles, splits, tiles_per_split;
-  int batch;                    // M tiles per launch of the pass
+  int batch, heads;             // M tiles and KV heads per launch of the pass
   int m_per_cta;                // of which share a CTA
   size_t off_qpack, off_ml, off_pieces, off_mass, off_keys, total;
 };
@@ -475,12 +479,17 @@ RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int
   pl.rows_pad = pl.n_mt * kTile;
   pl.n_tiles = (int)((pool->pool_tokens + kTile - 1) / kTile);
   const int most = (pl.n_tiles + 7) / 8 < 256 ? (pl.n_tiles + 7) / 8 : 256;
-  // M tiles whose pieces fit, in batches of equal size
+  // M tiles whose pieces fit, in batches of equal size; where one tile's do not, KV heads in batches of equal size
   const long long m_tiles = (long long)B * pl.n_mt;
-  const size_t per_tile = (size_t)Hkv * ((size_t)pool->n_shots + most) * kTile * 4;
-  const long long fit = (long long)(kPieceBytes / per_tile) > 1 ? (long long)(kPieceBytes / per_tile) : 1;
+  const size_t per_unit = ((size_t)pool->n_shots + most) * kTile * 4;
+  const long long fit_units = (long long)(kPieceBytes / per_unit), fit = fit_units / Hkv > 1 ? fit_units / Hkv : 1;
   const long long n_batches = (m_tiles + fit - 1) / fit;
   pl.batch = (int)((m_tiles + n_batches - 1) / n_batches);
+  pl.heads = Hkv;
+  if (fit_units < Hkv) {
+    const int n = (int)((Hkv + (fit_units > 1 ? fit_units : 1) - 1) / (fit_units > 1 ? fit_units : 1));
+    pl.heads = (Hkv + n - 1) / n;
+  }
   // M tiles per CTA: as many as share without leaving more than a seventh of the places empty
   pl.m_per_cta = 1;
   for (int m = 4; m > 1; m >>= 1)
@@ -491,12 +500,12 @@ RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int
   // Key ranges: the CTAs run in waves of 148 (a fixed figure, so that the workspace size does not depend on the
   // device), each costs its tiles plus about four tiles' time of start-up; the split with the cheapest waves *
   // (tiles + 4) is taken, every range at least eight key tiles.
-  const long long units = (long long)pl.batch * Hkv;
+  const long long units = (long long)pl.batch * pl.heads;
   const int per_cta = kGroups / pl.m_per_cta;                 // ranges of one CTA
-  const long long ctas = (long long)((pl.batch + pl.m_per_cta - 1) / pl.m_per_cta) * Hkv;
+  const long long ctas = (long long)((pl.batch + pl.m_per_cta - 1) / pl.m_per_cta) * pl.heads;
   int best_s = 1;
   long long best_cost = 0;
-  for (int sp = 1; sp <= most; ++sp) {
+  for (int sp = 1; sp <= most && (sp == 1 || units * sp <= kMaxRanges); ++sp) {
     const long long tiles = (pl.n_tiles + sp - 1) / sp;
     const long long waves = (ctas * ((sp + per_cta - 1) / per_cta) + 147) / 148;
     const long long cost = waves * (tiles + 4);
@@ -507,10 +516,15 @@ RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int
   }
   pl.tiles_per_split = (pl.n_tiles + best_s - 1) / best_s;
   pl.splits = (pl.n_tiles + pl.tiles_per_split - 1) / pl.tiles_per_split;
+  // The sizes are those of the largest batch and split that a call with no more rows than this one can have: a workspace
+  // for the longest query takes the shorter ones, too.
+  const long long most_units = (m_tiles < fit ? m_tiles : fit) * pl.heads;
+  const long long all = most_units * most < kMaxRanges ? most_units * most : kMaxRanges;
+  const size_t ranges = (size_t)(all > most_units ? all : most_units);
   size_t off = 0;
   pl.off_qpack = off;   off += ads_round_up((size_t)B * Hkv * pl.rows_pad * D * 2, 256);
-  pl.off_ml = off;      off += ads_round_up((size_t)units * pl.splits * kTile * 3 * 4, 256);
-  pl.off_pieces = off;  off += ads_round_up((size_t)units * ((size_t)pool->n_shots + pl.splits) * kTile * 4, 256);
+  pl.off_ml = off;      off += ads_round_up(ranges * kTile * 3 * 4, 256);
+  pl.off_pieces = off;  off += ads_round_up(((size_t)most_units * pool->n_shots + ranges) * kTile * 4, 256);
   pl.off_mass = off;    off += ads_round_up((size_t)B * pool->n_shots * 8, 256);
   pl.off_keys = off;    off += ads_round_up((size_t)B * pool->n_shots * 8, 256);
   pl.total = off;
@@ -565,25 +579,27 @@ int rel_launch(const adapshot_model_t* model, const adapshot_pool_t* pool, int l
   static bool attr_done[kAdsMaxDevices] = {false};
   if (ads_set_max_smem(rel_pass_kernel<D>, smem, attr_done) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
   const int m_tiles = B * pl.n_mt;
-  for (int t0 = 0; t0 < m_tiles; t0 += pl.batch) {
-    const int n = m_tiles - t0 < pl.batch ? m_tiles - t0 : pl.batch;
-    rp.tile0 = t0;
-    rp.n_m = n;
-    rp.m_per_cta = pl.m_per_cta;
-    const int per_cta = kGroups / pl.m_per_cta;
-    ads_launch_dependent(rel_pass_kernel<D>, dim3((unsigned)((n + pl.m_per_cta - 1) / pl.m_per_cta),
-                                                  (unsigned)((pl.splits + per_cta - 1) / per_cta), (unsigned)Hkv),
-                         kRelThreads, smem, st, tm_q, tm_k, rp);
-    if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-    ads_launch_dependent(rel_merge_kernel, (unsigned)(n * Hkv), 128, 0, st, ml_part, pl.splits, Hkv, t0, pl.n_mt,
-                         pl.rows);
-    if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-    const int b0 = t0 / pl.n_mt, b1 = (t0 + n - 1) / pl.n_mt;       // queries with rows in the batch
-    ads_launch_dependent(rel_reduce_kernel, dim3((unsigned)((pool->n_shots + 7) / 8), (unsigned)(b1 - b0 + 1)), 256, 0, st,
-                         pieces, ml_part, shot_off, pool->n_shots, Hkv, pl.n_mt, t0, n, pl.splits, pl.tiles_per_split,
-                         pool->pool_tokens, b0, mass);
-    if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-  }
+  for (int t0 = 0; t0 < m_tiles; t0 += pl.batch)
+    for (int h0 = 0; h0 < Hkv; h0 += pl.heads) {
+      const int n = m_tiles - t0 < pl.batch ? m_tiles - t0 : pl.batch, nh = Hkv - h0 < pl.heads ? Hkv - h0 : pl.heads;
+      rp.tile0 = t0;
+      rp.head0 = h0;
+      rp.n_heads = nh;
+      rp.n_m = n;
+      rp.m_per_cta = pl.m_per_cta;
+      const int per_cta = kGroups / pl.m_per_cta;
+      ads_launch_dependent(rel_pass_kernel<D>, dim3((unsigned)((n + pl.m_per_cta - 1) / pl.m_per_cta),
+                                                    (unsigned)((pl.splits + per_cta - 1) / per_cta), (unsigned)nh),
+                           kRelThreads, smem, st, tm_q, tm_k, rp);
+      if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
+      ads_launch_dependent(rel_merge_kernel, (unsigned)(n * nh), 128, 0, st, ml_part, pl.splits, nh, t0, pl.n_mt, pl.rows);
+      if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
+      const int b0 = t0 / pl.n_mt, b1 = (t0 + n - 1) / pl.n_mt;       // queries with rows in the batch
+      ads_launch_dependent(rel_reduce_kernel, dim3((unsigned)((pool->n_shots + 7) / 8), (unsigned)(b1 - b0 + 1)), 256, 0,
+                           st, pieces, ml_part, shot_off, pool->n_shots, nh, pl.n_mt, t0, n, pl.splits,
+                           pl.tiles_per_split, pool->pool_tokens, b0, h0, mass);
+      if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
+    }
 
   const long long n_sc = (long long)B * pool->n_shots;
   ads_launch_dependent(rel_scores_kernel, (unsigned)((n_sc + 255) / 256), 256, 0, st, mass, shot_off, B, pool->n_shots, 1.0 / ((double)Tq * Hq),

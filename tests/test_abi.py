@@ -108,3 +108,21 @@ def test_header_is_plain_c(tmp_path):
     r = subprocess.run([gcc, "-std=c99", "-Wall", "-Werror", "-I", os.path.join(ROOT, "include"), "-c", str(src),
                         "-o", str(tmp_path / "t.o")], capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
+
+
+@pytest.mark.parametrize("n_shots,tokens,hkv", [(20000, 64, 8), (65536, 64, 8), (200000, 64, 8), (600000, 3, 4), (300, 128, 8),
+                                                (64, 16, 1)])
+def test_ranking_workspace_grows_with_the_call_and_is_bounded(ab, n_shots, tokens, hkv):
+    # a workspace for the longest query and the largest batch takes all others; the pieces stay below 256 MiB (512 bytes per
+    # shot and the ranges of one unit where the pool alone asks for more)
+    pool = ab.PoolT(n_shots, 64, n_shots * tokens, 0x1000, 0x1000, None, None)
+    model = ab.make_model(1, 4 * hkv, hkv, 128, "bf16", 5e5)
+    size = lambda B, t_q: ab.lib.adapshot_select_attn_workspace_bytes(C.byref(model), C.byref(pool), B, t_q, 1)
+    for fixed, sizes in ((1, [size(1, t) for t in range(1, 700)]), (2, [size(b, 33) for b in range(1, 140)]),
+                         (3, [size(3, t) for t in range(1, 300, 7)])):
+        assert all(a <= b for a, b in zip(sizes, sizes[1:])), fixed
+    for B, t_q in ((1, 8), (1, 96), (1, 128), (4, 200)):
+        rest = B * hkv * -(-t_q * 4 // 128) * 128 * 256 + 2 * B * n_shots * 8        # packed Q, masses and keys
+        ranges = 16 * 148 * 4 * 128 * 12                                             # (max, sum, first max) of the ranges
+        pieces = max(256 << 20, (n_shots + 256) * 512)
+        assert size(B, t_q) <= rest + ranges + pieces + 4096

@@ -168,3 +168,12 @@ def test_masses_do_not_carry_the_rounding_of_large_scores(big):
     sel, score = _run(ab, hp.model_of(ab, w, n_layers=1), hp.dev_pool(ab, pool), 0, q, 150)
     s = orc.relevance_attention(hp.f64(q[0]), hp.f64(pool["k"][0]), pool["shot_off"])
     assert np.all(np.abs(score[0] - s[sel[0]]) <= 3e-6 * s[sel[0]])
+
+
+@pytest.mark.parametrize("batch,t_q", [(1, 3), (2, 130)])
+def test_heads_in_batches(batch, t_q):
+    # 66000 shots: the pieces of one M tile and all eight KV heads are more than 256 MB, so the heads go four by four, the M
+    # tiles (two per query at 130 tokens) one by one
+    w = wl.CONFIGS["cfg2"].scaled(n_shots=66000, len_lo=1, len_hi=1, batch=batch, k=32, t_q=t_q, n_q_heads=8,
+                                  n_kv_heads=8, head_dim=64, emb_dim=8, seed=92)
+    _check(w, 1, 0, 32)
