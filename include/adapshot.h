@@ -306,7 +306,8 @@ ADAPSHOT_API int adapshot_decode_attn(const adapshot_model_t* model, const void*
  *   R * splits < 2^31, where splits <= 64 is the number of slices (multiples of 8192
  *   entries, one CTA each) a row is cut into; ADAPSHOT_ESHAPE otherwise.
  *   Ask adapshot_entropy_workspace_bytes for the scratch size (12 bytes per row and
- *   slice, rounded up to 256; it depends on R and V only, not on the device).     */
+ *   slice it can be cut into, rounded up to 256; it depends on R and V only, not on the
+ *   device, and serves every smaller R and V).                                    */
 ADAPSHOT_API size_t adapshot_entropy_workspace_bytes(int32_t R, int32_t V);
 ADAPSHOT_API int adapshot_entropy(const void* logits, int32_t dtype, int32_t R, int32_t V, int64_t row_stride,
                      float* H, float tau, int32_t rows_per_group, int32_t* first_ok,

@@ -329,13 +329,14 @@ constexpr int kEntCtaOverhead = 2048;    // fixed cost of a CTA (start, state me
 // minimises waves * (slice + overhead) is taken: 1024 rows of 128 256 run as 2 slices each (2.8
 // waves) rather than whole (1.4 waves, the second one two fifths full), 224 rows as 3 slices (one wave).  `max_states` bounds R * n (the fixed scratch of the static entry point).
 struct EntSplit { int slice, n; };
+constexpr int kEntMaxSlices = 64;        // of a row
 EntSplit ent_split(int R, int V, long long max_states = 0x7fffffffll) {
   const long long unit = kEntSliceUnit;
   const long long kMaxSlice = 0x7fffe000ll;                             // the largest multiple of the unit an int holds
   EntSplit best{(int)((long long)V <= kMaxSlice ? ((long long)V + unit - 1) / unit * unit : kMaxSlice),
                 (long long)V <= kMaxSlice ? 1 : 2};                      // the row in one piece (two beyond 2^31 - 8192)
   double best_cost = 0.0;
-  for (int want = 1; want <= 64; ++want) {
+  for (int want = 1; want <= kEntMaxSlices; ++want) {
     // the shortest slice (a multiple of the unit) that cuts the row into at most `want` pieces
     const long long per = ((long long)V + want - 1) / want;
     long long slice = (per + unit - 1) / unit * unit;
@@ -352,12 +353,16 @@ EntSplit ent_split(int R, int V, long long max_states = 0x7fffffffll) {
   return best;
 }
 int ent_splits(int R, int V) { return ent_split(R, V).n; }
+size_t ent_state_bytes(long long states) { return ads_round_up((size_t)states * 3 * sizeof(float), 256); }
 
 }  // namespace
 
 extern "C" size_t adapshot_entropy_workspace_bytes(int32_t R, int32_t V) {
   if (R <= 0 || V <= 0) return 0;
-  return ads_round_up((size_t)R * ent_splits(R, V) * 3 * sizeof(float), 256);
+  // As many slices as a row of this length is ever cut into: fewer rows are cut into more slices, and a workspace for a
+  // batch has to serve every smaller one.
+  const long long n = ((long long)V + kEntSliceUnit - 1) / kEntSliceUnit;
+  return ent_state_bytes((long long)R * (n < kEntMaxSlices ? n : kEntMaxSlices));
 }
 
 extern "C" int adapshot_entropy(const void* logits, int32_t dtype, int32_t R, int32_t V,
@@ -373,7 +378,7 @@ extern "C" int adapshot_entropy(const void* logits, int32_t dtype, int32_t R, in
   if ((long long)R * ent_splits(R, V) > 0x7fffffffll) return ADAPSHOT_ESHAPE;
   const size_t es = dtype == ADAPSHOT_F32 ? 4 : 2;
   if (!ads_aligned16(logits) || !ads_aligned16(ws) || (row_stride * es) % 16 != 0) return ADAPSHOT_EALIGN;
-  if (ws_bytes < adapshot_entropy_workspace_bytes(R, V)) return ADAPSHOT_ECAPACITY;
+  if (ws_bytes < ent_state_bytes((long long)R * ent_splits(R, V))) return ADAPSHOT_ECAPACITY;
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const EntSplit cut = ent_split(R, V);
@@ -409,7 +414,7 @@ extern "C" int adapshot_entropy_subset(const void* logits, int32_t dtype, int32_
   if (!ads_aligned16(logits) || !ads_aligned16(ws) || (row_stride * es) % 16 != 0 ||
       ((uintptr_t)subset_ids & 3u))
     return ADAPSHOT_EALIGN;
-  if (ws_bytes < adapshot_entropy_workspace_bytes(R, V)) return ADAPSHOT_ECAPACITY;
+  if (ws_bytes < ent_state_bytes((long long)R * ent_splits(R, V))) return ADAPSHOT_ECAPACITY;
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const EntSplit cut = ent_split(R, V);

@@ -159,3 +159,20 @@ def test_entropy_minus_infinity_conventions(dt):
     assert abs(got[1] - want1) < 1e-4 * want1
     assert got[2] == 0.0 and got[3] == 0.0
     assert abs(got[4] - math.log(8192)) < 1e-4 * math.log(8192)
+
+
+@pytest.mark.parametrize("rows", [13 * 7, 25 * 7, 1])
+def test_a_workspace_for_a_batch_serves_smaller_ones(rows):
+    # fewer rows are cut into more slices: 32 queries of seven probes into 3 per row, 25 into 4
+    ab = hp.gpu_binding()
+    V = 128256
+    g = torch.Generator().manual_seed(rows)
+    logits = (torch.randn(rows, V, generator=g) * 2.0).to(torch.bfloat16)
+    ws = torch.empty(ab.adapshot_entropy_workspace_bytes(32 * 7, V), dtype=torch.uint8, device="cuda")
+    H, st = torch.zeros(rows, device="cuda"), hp.new_status()
+    ab.adapshot_entropy(logits.cuda(), H, 0.65, 1, None, ws, st)
+    torch.cuda.synchronize()
+    want = orc.entropy(hp.f64(logits))
+    assert st.item() == 0 and (np.abs(H.cpu().numpy() - want) <= REL_TOL * np.maximum(np.abs(want), 1e-3)).all()
+    sizes = [ab.adapshot_entropy_workspace_bytes(r, V) for r in range(1, 300)]
+    assert sizes == sorted(sizes)
