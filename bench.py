@@ -106,14 +106,14 @@ HEADLINE = "cfg5"            # the largest 8B-shape configuration that fits one 
 SUB_WORKLOADS = ("cfg2", "cfg3")   # reported beside it in the default run, each with its own roofline / clocks / e2e
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, from the ncu captures summarised under
-# profiles/ (file named beside each figure).  A capture of a few layers / queries is scaled to a full
+# profiles/ (the capture is named beside each figure).  A capture of a few layers / queries is scaled to a full
 # launch by the units it holds: (query, layer, kv head) units are independent and equally sized on
 # average, so the traffic grows in proportion.  None = no capture of the kernel as it stands.
 NCU_TRAFFIC = {
     # workload: (attn_main bytes per captured launch, layers x queries in that capture,
     #            gather bytes per captured launch, layers x queries in that capture), for the variant
     #            that `--variant auto` picks for the workload
-    "cfg3": (5.498e8, 4, None, 1),                # profiles/attn_main_kernel.md (1 layer x 4 queries, K-only cache)
+    "cfg3": (5.498e8, 4, None, 1),                # ncu capture of 1 layer x 4 queries, K-only cache
 }
 
 

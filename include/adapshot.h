@@ -93,9 +93,8 @@ typedef struct adapshot_pool {
  * the lower id.  Nested probes use prefixes of sel_idx.
  *   q_emb [B][emb_dim] fp32; sel_idx [B][k] int32 out; sel_score [B][k] fp32 out
  *   or NULL.  Needs 1 <= k <= n_shots (else ADAPSHOT_ESHAPE); a pool of more than
- *   8192 shots (one sort chunk) takes k <= 4096 (else ADAPSHOT_EUNSUPPORTED: the
- *   chunks' candidate lists would not shrink from one merge round to the next).
- *   Scores are compared in fp64.                                                */
+ *   8192 shots (the candidates that one CTA sorts) takes k <= 4096, half of them
+ *   (else ADAPSHOT_EUNSUPPORTED).  Scores are compared in fp64.                  */
 ADAPSHOT_API size_t adapshot_select_workspace_bytes(int32_t n_shots, int32_t B, int32_t k);
 ADAPSHOT_API int adapshot_select(const adapshot_pool_t* pool, const float* q_emb, int32_t B, int32_t k,
                     int32_t* sel_idx, float* sel_score,
@@ -208,9 +207,9 @@ ADAPSHOT_API int adapshot_query_attn(const adapshot_model_t* model,
  * the pool (through sel_idx / ctx_off) and K is re-encoded (Eq. 7) tile by tile in
  * shared memory on its way to the tensor cores, so that no assembled cache is written
  * to or read from HBM.  Results equal adapshot_assemble_kv + adapshot_query_attn up to
- * the rounding of the rotary angles (fp32 (cos, sin) from fp64 angles, sixteen rows further
- * by one fp32 complex multiplication; K' rounded once to bf16 as in the materialised
- * path).  ctx_off: the plan written by adapshot_assemble_kv (plan-only call is enough)
+ * the rounding of the rotary angles (fp32 (cos, sin) from fp64 angles once per 128-row tile,
+ * 16 (d = 128) or 32 (d = 64) rows further by one fp32 complex multiplication; K' rounded
+ * once to bf16 as in the materialised path).  ctx_off: the plan written by adapshot_assemble_kv (plan-only call is enough)
  * for the same sel_idx; ctx_cap: an upper bound of every L (sizes two row maps of
  * B * ctx_cap int32 in the workspace).  Both
  * k_pos_mode values are taken (1: every key of a shot is rotated by the angle of the

@@ -114,7 +114,6 @@ struct GatherArgs {
   int layer_begin, n_layers_call;
   int shot_begin;              // first selected shot to gather (earlier positions of the cache are kept)
   int k_pos_mode;
-  double rope_base;
   int32_t* status;
   double theta[64];            // theta_i = rope_base^(-2i/D), i < D/2, formed on the host
   int chunk;                   // destination tokens per chunk
@@ -515,7 +514,7 @@ extern "C" int adapshot_assemble_kv_from(const adapshot_model_t* model, const ad
   a.n_shots = pool->n_shots; a.B = B; a.k = k; a.n_kv_heads = model->n_kv_heads;
   a.layer_begin = layer_begin; a.n_layers_call = layer_end - layer_begin;
   a.shot_begin = shot_begin;
-  a.k_pos_mode = model->k_pos_mode; a.rope_base = model->rope_base; a.status = status;
+  a.k_pos_mode = model->k_pos_mode; a.status = status;
   for (int i = 0; i < model->head_dim / 2; ++i)
     a.theta[i] = pow(model->rope_base, -2.0 * (double)i / (double)model->head_dim);
 

@@ -119,7 +119,6 @@ struct PrepParams {
   int To;                     // own tokens per probe: the Tq query rows are the last Tq of them
   const int* nshots_dev;      // per-query shot count of the (single) probe, device memory, or null
   int32_t* status;
-  double rope_base;
   double theta[64];           // theta_i = rope_base^(-2i/D), formed on the host
   int nshots[kMaxProbes];
 };
@@ -1528,7 +1527,6 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
   pp.sched = sched; pp.ctx_cap = ctx_cap;
   pp.B = B; pp.k = k; pp.P = P; pp.Tq = Tq; pp.Hq = Hq; pp.Hkv = Hkv; pp.nl = nl; pp.n_gangs = n_gangs;
   pp.To = To; pp.nshots_dev = extra.nshots_dev; pp.status = status;
-  pp.rope_base = model->rope_base;
   for (int i = 0; i < D / 2; ++i) pp.theta[i] = pow(model->rope_base, -2.0 * (double)i / (double)D);
   for (int i = 0; i < kMaxProbes; ++i) pp.nshots[i] = i < P ? probe_nshots[i] : 0;
   const long long n_tok = (long long)B * nl * P * To;

@@ -510,8 +510,9 @@ decode_rows_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   if (threadIdx.x == 0 && *abort_flag != 0) ads_set_status(p.status, ADAPSHOT_ETIMEOUT);
 }
 
-// Block (u, rr) merges row rr of unit u if a range boundary cut the unit.  One request is cut into up to 37
-// pieces: eight warps take every eighth piece each, all their loads in flight at once, and meet in shared memory.
+// Block (u, rr) merges row rr of unit u if a range boundary cut the unit.  One request of eight KV heads is cut into up to
+// 37 pieces per head, one of a single head into up to one per CTA: eight warps take every eighth piece each, five at a
+// time with their loads in flight at once, and meet in shared memory.
 constexpr int kMergeWarps = 8;
 template <int D>
 __global__ void __launch_bounds__(32 * kMergeWarps) decode_combine_kernel(const __grid_constant__ DecodeParams p) {

@@ -490,7 +490,7 @@ int ads_topk_from_keys(const unsigned long long* keys, int N, int B, int k, int3
 
 extern "C" size_t adapshot_select_workspace_bytes(int32_t n_shots, int32_t B, int32_t k) {
   if (n_shots <= 0 || B <= 0 || k <= 0) return 0;
-  // the sort keys; the second term (a norm per shot) is part of the size that the call has always asked for
+  // the sort keys, and room for a norm per shot that no kernel needs any more: the size a call is refused below stays
   return ads_round_up((size_t)B * n_shots * sizeof(unsigned long long), 256) +
          ads_round_up((size_t)n_shots * sizeof(double), 256);
 }
