@@ -263,13 +263,14 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     auto shot_end = [&](int i) -> long long {
       return i + 1 < p.n_shots ? p.shot_off[i + 1] : i + 1 == p.n_shots ? p.pool_tokens : (1ll << 62);
     };
+    // (found by a 32-ary search of the whole warp: the steps of a binary one are a chain of cold loads)
     int shot = 0;
-    {
-      int hi = p.n_shots;
-      while (hi - shot > 1) {
-        const int mid = (shot + hi) >> 1;
-        if (p.shot_off[mid] <= (long long)t0 * kTile) shot = mid; else hi = mid;
-      }
+    for (int seg = p.n_shots; seg > 1;) {
+      const int stride = (seg + 31) / 32, at = shot + lane * stride;
+      const bool le = lane == 0 || (at < shot + seg && p.shot_off[at] <= (long long)t0 * kTile);
+      const int first = shot + (__popc(__ballot_sync(0xffffffffu, le)) - 1) * stride;
+      seg = min(stride, shot + seg - first);
+      shot = first;
     }
     long long end = shot_end(shot), end_next = shot_end(shot + 1);
     float* piece = p.pieces + ((unit * (p.n_shots + p.splits) + split + shot) * kTile + r);
@@ -391,56 +392,89 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 }
 
 // What is left to add to the pieces of a row in every range: first max - log2 sum_keys 2^(s c), -inf for rows that do not exist
-// (so that they add nothing); one thread per row.
-__global__ void __launch_bounds__(128) rel_merge_kernel(float* __restrict__ ml_part, int splits, int n_heads, int tile0,
-                                                        int n_mt, int rows) {
+// (so that they add nothing).  A block per unit: threadIdx.x is the row, every kMergeGroups-th range a thread's.  (One thread
+// per row walked up to 256 ranges: 51 us for 4 units of 71 ranges, 16 for 148 now.)
+constexpr int kMergeGroups = 8;
+__global__ void __launch_bounds__(kTile * kMergeGroups) rel_merge_kernel(float* __restrict__ ml_part, int splits, int n_heads,
+                                                                         int tile0, int n_mt, int rows) {
+  __shared__ float2 part[kMergeGroups][kTile];
   ads_dependency_wait();
   const long long unit = blockIdx.x;
-  const int r = threadIdx.x;
+  const int r = threadIdx.x, y = threadIdx.y;
   const int mt = (int)((tile0 + unit / n_heads) % n_mt);
   float* ml = ml_part + unit * splits * 3 * kTile + r;              // a range's figures are 3 * 128 floats
-  float M = -1.0e30f;
-  for (int s = 0; s < splits; ++s) M = fmaxf(M, ml[s * 3 * kTile]);
-  float l = 0.f;
-  for (int s = 0; s < splits; ++s) l += ml[s * 3 * kTile + kTile] * exp2f(ml[s * 3 * kTile] - M);
+  float M = -1.0e30f, l = 0.f;
+  for (int base = y; base < splits; base += 8 * kMergeGroups) {     // eight ranges' figures on their way at a time
+    float m8[8], l8[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int s = base + e * kMergeGroups;
+      m8[e] = s < splits ? ml[s * 3 * kTile] : -1.0e30f;
+      l8[e] = s < splits ? ml[s * 3 * kTile + kTile] : 0.f;
+    }
+    float m_new = M;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) m_new = fmaxf(m_new, m8[e]);
+    l *= exp2f(M - m_new);
+    M = m_new;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) l += l8[e] * exp2f(m8[e] - M);
+  }
+  part[y][r] = make_float2(M, l);
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kMergeGroups; ++i) M = fmaxf(M, part[i][r].x);
+  l = 0.f;
+#pragma unroll
+  for (int i = 0; i < kMergeGroups; ++i) l += part[i][r].y * exp2f(part[i][r].x - M);
+  const float log_l = log2f(l);
   const bool exists = mt * kTile + r < rows;
-  for (int s = 0; s < splits; ++s) {
+#pragma unroll 8
+  for (int s = y; s < splits; s += kMergeGroups) {
     float* first = ml + s * 3 * kTile + 2 * kTile;
-    *first = !exists ? -INFINITY : l > 0.f ? (*first - M) - log2f(l) : *first;
+    *first = !exists ? -INFINITY : l > 0.f ? (*first - M) - log_l : *first;
   }
 }
 
-// mass[b][i] (+)= sum over the batch's rows and heads of query b of 2^(piece + the row's share); grid (shots / 8, queries), a warp per
-// shot.
+// mass[b][i] (+)= sum over the batch's rows and heads of query b of 2^(piece + the row's share).  A block of eight warps takes
+// 8 / `warps` shots of a query: the (M tile, head) units of the query are dealt out to a shot's warps, whose sums are added in
+// their order.  (With a warp per shot a pool of 64 shots was eight blocks: 57 us for 8 M tiles of 8 heads, 9 now.)
 __global__ void __launch_bounds__(256) rel_reduce_kernel(const float* __restrict__ pieces, const float* __restrict__ ml_part,
                                                          const long long* __restrict__ shot_off, int n_shots, int n_heads,
                                                          int n_mt, int tile0, int n_tiles_m, int splits,
-                                                         int tiles_per_split, long long pool_tokens, int b0, int head0,
+                                                         int tiles_per_split, long long pool_tokens, int b0, int head0, int warps,
                                                          double* __restrict__ mass) {
+  __shared__ double sum_s[8];
   ads_dependency_wait();
-  const int lane = threadIdx.x & 31, b = b0 + blockIdx.y;
-  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (i >= n_shots) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = b0 + blockIdx.y;
+  const int i = blockIdx.x * (8 / warps) + warp / warps, w = warp % warps;
   const int first = max(tile0, b * n_mt), last = min(tile0 + n_tiles_m, (b + 1) * n_mt);   // M tiles of this query
-  const long long o0 = i > 0 ? shot_off[i] : 0, o1 = i + 1 < n_shots ? shot_off[i + 1] : pool_tokens;
-  const int s0 = (int)(o0 / kTile) / tiles_per_split, s1 = (int)((o1 - 1) / kTile) / tiles_per_split;
   double sum = 0.0;
-  for (int m = first; m < last; ++m) {
+  if (i < n_shots) {
+    const long long o0 = i > 0 ? shot_off[i] : 0, o1 = i + 1 < n_shots ? shot_off[i + 1] : pool_tokens;
+    const int s0 = (int)(o0 / kTile) / tiles_per_split, s1 = (int)((o1 - 1) / kTile) / tiles_per_split;
+    const long long u0 = (long long)(first - tile0) * n_heads + w;                         // this warp's first unit, [m][head]
+    const int n_u = ((last - first) * n_heads - w + warps - 1) / warps;
+    const long long piece_step = (long long)warps * (n_shots + splits) * (kTile / 4), share_step = (long long)warps * splits * 3 * (kTile / 4);
     for (int s = s0; s <= s1; ++s) {
-      const float4* pc = reinterpret_cast<const float4*>(
-          pieces + (((long long)(m - tile0) * n_heads * (n_shots + splits)) + s + i) * kTile) + lane;
-      const float4* share = reinterpret_cast<const float4*>(
-          ml_part + (((long long)(m - tile0) * n_heads * splits + s) * 3 + 2) * kTile) + lane;
+      const float4* pc = reinterpret_cast<const float4*>(pieces + (u0 * (n_shots + splits) + s + i) * kTile) + lane;
+      const float4* share = reinterpret_cast<const float4*>(ml_part + ((u0 * splits + s) * 3 + 2) * kTile) + lane;
 #pragma unroll 8
-      for (int g = 0; g < n_heads; ++g) {
-        const float4 v = pc[(long long)g * (n_shots + splits) * (kTile / 4)], n = share[(long long)g * splits * 3 * (kTile / 4)];
+      for (int e = 0; e < n_u; ++e, pc += piece_step, share += share_step) {
+        const float4 v = *pc, n = *share;
         const float part = (rel_ex2(v.x + n.x) + rel_ex2(v.y + n.y)) + (rel_ex2(v.z + n.z) + rel_ex2(v.w + n.w));
         sum += (double)part;
       }
     }
   }
   sum = warp_sum(sum);
-  if (lane == 0) {
+  if (warps > 1) {
+    if (lane == 0) sum_s[warp] = sum;
+    __syncthreads();
+    if (w == 0)
+      for (int e = 1; e < warps; ++e) sum += sum_s[warp + e];
+  }
+  if (lane == 0 && w == 0 && i < n_shots) {
     double* out = mass + (long long)b * n_shots + i;
     *out = first == b * n_mt && head0 == 0 ? sum : *out + sum;
   }
@@ -461,6 +495,7 @@ __global__ void __launch_bounds__(256) rel_scores_kernel(const double* __restric
 }
 
 constexpr size_t kPieceBytes = 256u << 20;
+constexpr int kStartTiles = 4;          // what starting a CTA costs, in tiles (7 and 12 give the same times within 1 %)
 constexpr long long kMaxRanges = 16 * 148 * kGroups;     // (unit, range) pairs of a launch that are worth having: sixteen waves
 
 struct RelPlan {
@@ -478,11 +513,11 @@ RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int
   pl.n_mt = (pl.rows + kTile - 1) / kTile;
   pl.rows_pad = pl.n_mt * kTile;
   pl.n_tiles = (int)((pool->pool_tokens + kTile - 1) / kTile);
-  const int most = (pl.n_tiles + 7) / 8 < 256 ? (pl.n_tiles + 7) / 8 : 256;
+  const int most = (pl.n_tiles + 1) / 2 < 256 ? (pl.n_tiles + 1) / 2 : 256;
   // M tiles whose pieces fit, in batches of equal size; where one tile's do not, KV heads in batches of equal size
   const long long m_tiles = (long long)B * pl.n_mt;
-  const size_t per_unit = ((size_t)pool->n_shots + most) * kTile * 4;
-  const long long fit_units = (long long)(kPieceBytes / per_unit), fit = fit_units / Hkv > 1 ? fit_units / Hkv : 1;
+  const long long fit_units = (long long)((kPieceBytes / (kTile * 4) - kMaxRanges) / (size_t)pool->n_shots);
+  const long long fit = fit_units / Hkv > 1 ? fit_units / Hkv : 1;
   const long long n_batches = (m_tiles + fit - 1) / fit;
   pl.batch = (int)((m_tiles + n_batches - 1) / n_batches);
   pl.heads = Hkv;
@@ -498,8 +533,8 @@ RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int
       break;
     }
   // Key ranges: the CTAs run in waves of 148 (a fixed figure, so that the workspace size does not depend on the
-  // device), each costs its tiles plus about four tiles' time of start-up; the split with the cheapest waves *
-  // (tiles + 4) is taken, every range at least eight key tiles.
+  // device), each costs its tiles and a start; the split with the cheapest waves *
+  // (tiles + kStartTiles) is taken, every range at least two key tiles.
   const long long units = (long long)pl.batch * pl.heads;
   const int per_cta = kGroups / pl.m_per_cta;                 // ranges of one CTA
   const long long ctas = (long long)((pl.batch + pl.m_per_cta - 1) / pl.m_per_cta) * pl.heads;
@@ -508,7 +543,7 @@ RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int
   for (int sp = 1; sp <= most && (sp == 1 || units * sp <= kMaxRanges); ++sp) {
     const long long tiles = (pl.n_tiles + sp - 1) / sp;
     const long long waves = (ctas * ((sp + per_cta - 1) / per_cta) + 147) / 148;
-    const long long cost = waves * (tiles + 4);
+    const long long cost = waves * (tiles + kStartTiles);
     if (sp == 1 || cost < best_cost) {
       best_s = sp;
       best_cost = cost;
@@ -592,12 +627,14 @@ int rel_launch(const adapshot_model_t* model, const adapshot_pool_t* pool, int l
                                                     (unsigned)((pl.splits + per_cta - 1) / per_cta), (unsigned)nh),
                            kRelThreads, smem, st, tm_q, tm_k, rp);
       if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-      ads_launch_dependent(rel_merge_kernel, (unsigned)(n * nh), 128, 0, st, ml_part, pl.splits, nh, t0, pl.n_mt, pl.rows);
+      ads_launch_dependent(rel_merge_kernel, (unsigned)(n * nh), dim3(kTile, kMergeGroups), 0, st, ml_part, pl.splits, nh, t0, pl.n_mt, pl.rows);
       if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
       const int b0 = t0 / pl.n_mt, b1 = (t0 + n - 1) / pl.n_mt;       // queries with rows in the batch
-      ads_launch_dependent(rel_reduce_kernel, dim3((unsigned)((pool->n_shots + 7) / 8), (unsigned)(b1 - b0 + 1)), 256, 0,
-                           st, pieces, ml_part, shot_off, pool->n_shots, nh, pl.n_mt, t0, n, pl.splits,
-                           pl.tiles_per_split, pool->pool_tokens, b0, h0, mass);
+      int warps = 8;                                                  // per shot: one where shots alone fill the chip
+      while (warps > 1 && (long long)pool->n_shots * (b1 - b0 + 1) * warps > 2 * 8 * 148 * 4) warps >>= 1;
+      ads_launch_dependent(rel_reduce_kernel, dim3((unsigned)((pool->n_shots + 8 / warps - 1) / (8 / warps)),
+                           (unsigned)(b1 - b0 + 1)), 256, 0, st, pieces, ml_part, shot_off, pool->n_shots, nh, pl.n_mt, t0,
+                           n, pl.splits, pl.tiles_per_split, pool->pool_tokens, b0, h0, warps, mass);
       if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
     }
 

@@ -177,3 +177,11 @@ def test_heads_in_batches(batch, t_q):
     w = wl.CONFIGS["cfg2"].scaled(n_shots=66000, len_lo=1, len_hi=1, batch=batch, k=32, t_q=t_q, n_q_heads=8,
                                   n_kv_heads=8, head_dim=64, emb_dim=8, seed=92)
     _check(w, 1, 0, 32)
+
+
+@pytest.mark.parametrize("n_shots,lens,t_q,batch", [(5, (40, 70), 300, 1), (64, (16, 48), 17, 2), (700, (100, 140), 3, 1)])
+def test_warps_per_shot_and_many_ranges(n_shots, lens, t_q, batch):
+    # eight warps per shot over nineteen M tiles, over one, and more ranges than a thread of the merge takes at a time
+    w = wl.CONFIGS["cfg2"].scaled(n_shots=n_shots, len_lo=lens[0], len_hi=lens[1], batch=batch, k=n_shots, t_q=t_q, n_q_heads=8,
+                                  n_kv_heads=1, seed=93)
+    _check(w, 1, 0, n_shots)
