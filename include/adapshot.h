@@ -111,10 +111,11 @@ ADAPSHOT_API int adapshot_select(const adapshot_pool_t* pool, const float* q_emb
  * Q and K enter as stored (no rotary rotation is applied here); scale = model->softmax_scale
  * or 1/sqrt(d).  sel_idx[b][r] = id of the r-th most relevant shot, equal scores by lower id.
  *   q [B][T_q][Hq][d] bf16; sel_idx [B][k] int32 out; sel_score [B][k] fp32 out or NULL.
- * bf16 tensor-core kernels (one pass over the layer's K; between it and the reduction the
- * workspace holds 4 bytes per query row and shot, up to 256 MB at a time, or 512 bytes per
- * shot where a pool of more than half a million shots makes that more; a workspace for some
- * B and Tq serves every smaller B and Tq), fp32 exponentials,
+ * bf16 tensor-core kernels (one pass over the layer's K, two where a shot has fewer than 12
+ * tokens on average; between the steps the workspace holds 4 bytes per query row and shot, or
+ * with two passes per query, KV head and key, up to 256 MB at a time: more only for half a
+ * million shots, or 67 million keys, of one tile and head; a workspace for some B and Tq
+ * serves every smaller B and Tq), fp32 exponentials,
  * fp64 accumulation of the masses in a fixed order.  model->dtype must be ADAPSHOT_BF16; limits as adapshot_select,
  * pool_tokens < 2^31 - 256.                                                                 */
 #define ADAPSHOT_RELEVANCE_PER_TOKEN 1u

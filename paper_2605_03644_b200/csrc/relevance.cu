@@ -5,7 +5,7 @@
 // shot's relevance being the attention mass that falls on its tokens, averaged over query tokens
 // and heads (optionally divided by T_i).  Q and K enter as stored; 1/sqrt(d) scaling as in Eq. 5.
 //
-// One pass over the pool's K of that layer, on the tensor cores (tcgen05, S in TMEM, tiles staged by TMA).  The
+// On the tensor cores (tcgen05, S in TMEM, tiles staged by TMA), in one pass over the pool's K of that layer.  The
 // normaliser of a row is only known after all keys have been seen, so the pass leaves, for every query row and shot,
 // the log2 of the row's un-normalised mass on the shot, relative to the row's first maximum in that range of keys:
 //   pass    S = Q K^T, one thread per query row (TMEM lane): running maximum, exponentials, and their sum over
@@ -15,10 +15,17 @@
 //   reduce  mass of a shot = sum over rows of 2^(its piece + the row's share), a warp per shot.
 // (Both are small where the mass is, however large the scores are. As maximum + log2(sum) every piece carried the rounding of
 // the maximum, each shot its own: 2.5e-5 of a shot's mass at logits of 2048, now 3e-6 at most.)
-// (A second pass over the keys, with the normalisers known, used to take the reduce step's place: it cost as much as
-// the first: 1842 us for both, 1113 with one, for 2 queries x 128 tokens and 328 K pool tokens.)  What lies between the steps is 4
-// bytes per row and shot; the rows are taken in batches (of M tiles, and of KV heads where one tile is too much) that keep
-// it below kPieceBytes.
+// What lies between the steps is 4 bytes per row and shot; the rows are taken in batches (of M tiles, and of KV heads where
+// one tile is too much) that keep it below kPieceBytes.
+// Where shots are short (fewer than kShortShot tokens on average) a piece per row and shot costs more than seeing the keys
+// again: there a second pass, with the normalisers known, takes the places of the pieces and of their reduction.  Its score
+// tiles are the other way round, a thread per key, so that a key's masses add up over the rows in its thread:
+//   pass 1  running maximum and sum of every row;  merge  -> maximum and 1 / sum;
+//   pass 2  mass of a key and KV head = sum over the query's rows of 2^(score - maximum) / sum;
+//   keys    mass of a shot = sum over its keys and the heads.
+// One pass / two, 32 / 8 heads, d = 128, 8 queries x 256 tokens: 2.5 tokens per shot (30000 shots) 12061 / 3295 us, 8 tokens
+// (4000) 2248 / 1472, 12 tokens (2000) 1397 / 1279, 24 tokens (3000) 2662 / 3123; one query of 8 tokens 224 / 130, 67 / 64,
+// 48 / 53, 74 / 116.  For 160 tokens per shot two passes cost nearly twice as much (1842 / 912 us before the pieces).
 // The scores then go through the same top-k as the embedding selector (ties -> lower shot id).
 #include <float.h>
 
@@ -71,6 +78,8 @@ __device__ __forceinline__ float2 rel_ex2_poly2(float2 x) {
 // A unit is an M tile (of a query) and a KV head; units of a batch (M tiles from tile0 on, heads from head0 on) are numbered
 // from 0.
 struct RelParams {
+  float2* norm;                 // [unit][128]: (-max, 1 / sum) of every row (two passes)
+  float* key_mass;              // [query of the batch][head of the batch][n_tiles * 128] (two passes)
   float* ml_part;               // [unit][split][3][128]: max (log2 units), sum, first max; the merge replaces the last
   float* pieces;                // [unit][n_shots + splits][128]: log2 mass of row on shot i in range s - first max, at slot s + i
   const long long* shot_off;
@@ -125,7 +134,11 @@ struct RelSmem {
 // instruction issue: sixteen consumer warps keep both busy under each other's latencies.  (Two CTAs per SM with one M
 // tile and four consumer warps each: 1000 us for 2 queries x 128 tokens, 328 K pool tokens; 790 us now, the exponential unit
 // and the issue slots both two thirds busy.)
-template <int D>
+//
+// STEP: what is done with the scores.  In kMasses the operands change places: a CTA keeps up to four K tiles (m_per_cta), a
+// consumer group's rows are the keys of one of them, and the M tiles of the batch stream by.
+enum RelStep { kPieces, kNormalisers, kMasses };
+template <int D, int STEP>
 __global__ void __launch_bounds__(kRelThreads, 1)
 rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                 const __grid_constant__ RelParams p) {
@@ -144,12 +157,16 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = p.head0 + blockIdx.z;
-  const int m0 = blockIdx.x * p.m_per_cta, n_m = min(p.m_per_cta, p.n_m - m0);      // M tiles of this CTA
-  const int s0 = blockIdx.y * (kGroups / p.m_per_cta), n_s = min(kGroups / p.m_per_cta, p.splits - s0);   // its ranges
+  const int m0 = blockIdx.x * p.m_per_cta;          // tiles that stay: M tiles of this CTA (kMasses: K tiles)
+  const int n_m = min(p.m_per_cta, (STEP == kMasses ? p.n_tiles : p.n_m) - m0);
+  const int s0 = blockIdx.y * (kGroups / p.m_per_cta);                                // its ranges
+  const int n_s = STEP == kMasses ? 1 : min(kGroups / p.m_per_cta, p.splits - s0);
+  const int m_stream = blockIdx.y * p.tiles_per_split;                               // kMasses: first M tile that streams by
   const int stages = kSmemTiles - p.m_per_cta;
   const uint32_t k_base = base + p.m_per_cta * kTileBytes;
   // tiles of range s0 + j: the last range of a call may be shorter than the others
   auto range_tiles = [&](int j) {
+    if constexpr (STEP == kMasses) return min(p.n_m - m_stream, p.tiles_per_split);
     return max(0, min(p.n_tiles, (s0 + j + 1) * p.tiles_per_split) - (s0 + j) * p.tiles_per_split);
   };
   const int n_it = range_tiles(0);
@@ -183,11 +200,18 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     if (lane == 0) {
       tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k);
       mbar_arrive_expect_tx(bar(kRQFull), n_m * kTileBytes);
-      for (int m = 0; m < n_m; ++m) {
-        const int b = (p.tile0 + m0 + m) / p.n_mt, mt = (p.tile0 + m0 + m) % p.n_mt;
+      auto load_rows = [&](uint32_t dst, uint32_t full, int m) {         // M tile m of the batch
+        const int b = (p.tile0 + m) / p.n_mt, mt = (p.tile0 + m) % p.n_mt;
 #pragma unroll
-        for (int s = 0; s < SUB; ++s)
-          tma_load_3d(base + m * kTileBytes + s * 16384u, &tm_q, bar(kRQFull), s * 64, mt * kTile, b * p.Hkv + g);
+        for (int s = 0; s < SUB; ++s) tma_load_3d(dst + s * 16384u, &tm_q, full, s * 64, mt * kTile, b * p.Hkv + g);
+      };
+      auto load_keys = [&](uint32_t dst, uint32_t full, int tile) {
+#pragma unroll
+        for (int s = 0; s < SUB; ++s) tma_load_4d(dst + s * 16384u, &tm_k, full, s * 64, g, tile * kTile, p.layer);
+      };
+      for (int m = 0; m < n_m; ++m) {
+        if constexpr (STEP == kMasses) load_keys(base + m * kTileBytes, bar(kRQFull), m0 + m);
+        else load_rows(base + m * kTileBytes, bar(kRQFull), m0 + m);
       }
       bool ok = true;
       int st = 0, n = 0;
@@ -198,10 +222,8 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           ok = mbar_wait(bar(kRKEmpty + st), phase, abort_flag);
           if (!ok) break;
           mbar_arrive_expect_tx(bar(kRKFull + st), kTileBytes);
-#pragma unroll
-          for (int s = 0; s < SUB; ++s)
-            tma_load_4d(k_base + st * kTileBytes + s * 16384u, &tm_k, bar(kRKFull + st), s * 64, g,
-                        ((s0 + j) * p.tiles_per_split + i) * kTile, p.layer);
+          if constexpr (STEP == kMasses) load_rows(k_base + st * kTileBytes, bar(kRKFull + st), m_stream + i);
+          else load_keys(k_base + st * kTileBytes, bar(kRKFull + st), (s0 + j) * p.tiles_per_split + i);
           ++n;
           if (++st == stages) { st = 0; phase ^= 1; }
         }
@@ -249,6 +271,46 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     }
     __syncwarp();
   };
+  auto role_masses = [&]() {
+    const int x = (warp >> 2) - 1, quarter = warp & 3, r = quarter * 32 + lane;      // TMEM lane: key of the tile
+    if (x >= n_m) return;
+    const uint32_t lane_addr = static_cast<uint32_t>(quarter * 32) << 16;
+    float* out = p.key_mass + (long long)blockIdx.z * p.n_tiles * kTile + (long long)(m0 + x) * kTile + r;
+    const long long per_query = (long long)p.n_heads * p.n_tiles * kTile;
+    double sum = 0.0;
+    for (int i = 0; i < n_it; ++i) {
+      if (!__all_sync(0xffffffffu, mbar_wait(bar(kRSFull + x), i & 1, abort_flag))) return;
+      tc_fence_after();
+      const float2 scale2 = make_float2(p.scale_log2, p.scale_log2);
+      float2 part[2] = {{0.f, 0.f}, {0.f, 0.f}};
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        constexpr int kCols = kTile / 2;
+        float s[kCols];
+        tmem_ld2x32(tmem_base + lane_addr + x * kTile + half * kCols, reinterpret_cast<uint32_t*>(s));
+        if (half == 1) {
+          tc_fence_before();
+          mbar_arrive(bar(kRSEmpty + x));
+        }
+        // the rows' normalisers, two rows per load, the same address in every lane
+        const float4* nm = reinterpret_cast<const float4*>(p.norm + ((long long)(m_stream + i) * p.n_heads + blockIdx.z) * kTile + half * kCols);
+#pragma unroll
+        for (int c = 0; c < kCols; c += 2) {
+          const float4 n = nm[c / 2];
+          const float2 a = __ffma2_rn(make_float2(s[c], s[c + 1]), scale2, make_float2(n.x, n.z));
+          const float2 e = ((c >> 1) & 3) == 3 ? rel_ex2_poly2(a) : make_float2(rel_ex2(a.x), rel_ex2(a.y));
+          part[(c >> 1) & 1] = __ffma2_rn(e, make_float2(n.y, n.w), part[(c >> 1) & 1]);
+        }
+      }
+      const float2 both = __fadd2_rn(part[0], part[1]);
+      sum += (double)(both.x + both.y);
+      const int tile = p.tile0 + m_stream + i;
+      if ((tile + 1) % p.n_mt == 0) {                        // the query's last tile (batches and their parts hold whole queries)
+        out[(long long)(tile / p.n_mt - p.tile0 / p.n_mt) * per_query] = (float)sum;
+        sum = 0.0;
+      }
+    }
+  };
   auto role_consume = [&]() {
     const int x = (warp >> 2) - 1, quarter = warp & 3;
     const int m = x % p.m_per_cta, j = x / p.m_per_cta;
@@ -265,13 +327,14 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     };
     // (found by a 32-ary search of the whole warp: the steps of a binary one are a chain of cold loads)
     int shot = 0;
-    for (int seg = p.n_shots; seg > 1;) {
+    for (int seg = STEP == kNormalisers ? 1 : p.n_shots; seg > 1;) {
       const int stride = (seg + 31) / 32, at = shot + lane * stride;
       const bool le = lane == 0 || (at < shot + seg && p.shot_off[at] <= (long long)t0 * kTile);
       const int first = shot + (__popc(__ballot_sync(0xffffffffu, le)) - 1) * stride;
       seg = min(stride, shot + seg - first);
       shot = first;
     }
+    if (STEP == kNormalisers) shot = p.n_shots;             // (nothing ends)
     long long end = shot_end(shot), end_next = shot_end(shot + 1);
     float* piece = p.pieces + ((unit * (p.n_shots + p.splits) + split + shot) * kTile + r);
     auto flush = [&]() {                                    // the current shot is complete (in this range)
@@ -319,38 +382,40 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         if (half == 0 && i == 0 && m_run > -1.0e29f) m_first = m_run;
         // two scores per FMA / add instruction; the exponentials themselves are one MUFU operation each
         const float2 scale2 = make_float2(p.scale_log2, p.scale_log2), neg_m2 = make_float2(-m_run, -m_run);
-        float group[kCols / 16];                            // sums of 16 keys
+        float group[kCols / 8];                             // sums of 8 keys
 #pragma unroll
-        for (int c0 = 0; c0 < kCols; c0 += 16) {
+        for (int c0 = 0; c0 < kCols; c0 += 8) {
           float2 part = make_float2(0.f, 0.f);
 #pragma unroll
-          for (int c = c0; c < c0 + 16; c += 2) {
+          for (int c = c0; c < c0 + 8; c += 2) {
             const float2 a = __ffma2_rn(make_float2(s[c], s[c + 1]), scale2, neg_m2);
             const float2 e = ((c >> 1) & 3) == 3 ? rel_ex2_poly2(a) : make_float2(rel_ex2(a.x), rel_ex2(a.y));
             s[c] = e.x;
             s[c + 1] = e.y;
             part = c == c0 ? e : __fadd2_rn(part, e);
           }
-          group[c0 / 16] = part.x + part.y;
+          group[c0 / 8] = part.x + part.y;
         }
         // sums per shot (the branches are the same in every lane): all keys within one shot, else group by group, the
-        // keys of a group one by one only where a shot ends in it
+        // keys of a group one by one only where a shot ends in it (groups of 16: 6-20 % slower at 16 to 48 tokens per shot)
         const long long left = end - key0;
-        if (left > kCols) {
-          acc += (group[0] + group[1]) + (group[2] + group[3]);
+        if (STEP == kNormalisers) {
+          l_run += ((group[0] + group[1]) + (group[2] + group[3])) + ((group[4] + group[5]) + (group[6] + group[7]));
+        } else if (left > kCols) {
+          acc += ((group[0] + group[1]) + (group[2] + group[3])) + ((group[4] + group[5]) + (group[6] + group[7]));
         } else {
           int ce = (int)left;                               // columns left of the current shot
 #pragma unroll
-          for (int c0 = 0; c0 < kCols; c0 += 16) {
-            if (ce > c0 + 16) {
-              acc += group[c0 / 16];
+          for (int c0 = 0; c0 < kCols; c0 += 8) {
+            if (ce > c0 + 8) {
+              acc += group[c0 / 8];
             } else {
               int from = c0;
-              while (from < c0 + 16) {
-                const int to = min(ce, c0 + 16);
+              while (from < c0 + 8) {
+                const int to = min(ce, c0 + 8);
                 float sum[2] = {0.f, 0.f};
 #pragma unroll
-                for (int c = 0; c < 16; ++c) sum[c & 1] += c0 + c >= from && c0 + c < to ? s[c0 + c] : 0.f;
+                for (int c = 0; c < 8; ++c) sum[c & 1] += c0 + c >= from && c0 + c < to ? s[c0 + c] : 0.f;
                 acc += sum[0] + sum[1];
                 if (to == ce) {
                   flush();
@@ -365,7 +430,7 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     }
     if (ok && n_mine > 0) {
       // the shot that goes on in the next range
-      if (shot < p.n_shots && (shot == 0 || (long long)t1 * kTile > p.shot_off[shot])) flush();
+      if (STEP == kPieces && shot < p.n_shots && (shot == 0 || (long long)t1 * kTile > p.shot_off[shot])) flush();
       float* out = p.ml_part + (unit * p.splits + split) * 3 * kTile + r;
       out[0] = m_run;
       out[kTile] = l_run;
@@ -379,7 +444,8 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     else if (warp == 1) role_mma();
   } else {
     regs_raise<kRelRegsConsumer>();
-    role_consume();
+    if constexpr (STEP == kMasses) role_masses();
+    else role_consume();
   }
 
   tc_fence_before();
@@ -392,11 +458,12 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 }
 
 // What is left to add to the pieces of a row in every range: first max - log2 sum_keys 2^(s c), -inf for rows that do not exist
-// (so that they add nothing).  A block per unit: threadIdx.x is the row, every kMergeGroups-th range a thread's.  (One thread
+// (so that they add nothing).  With norm set (two passes): (-max, 1 / sum) of the row instead, 0 for the latter.  A block per unit: threadIdx.x is the row, every kMergeGroups-th range a thread's.  (One thread
 // per row walked up to 256 ranges: 51 us for 4 units of 71 ranges, 16 for 148 now.)
 constexpr int kMergeGroups = 8;
 __global__ void __launch_bounds__(kTile * kMergeGroups) rel_merge_kernel(float* __restrict__ ml_part, int splits, int n_heads,
-                                                                         int tile0, int n_mt, int rows) {
+                                                                         int tile0, int n_mt, int rows,
+                                                                         float2* __restrict__ norm) {
   __shared__ float2 part[kMergeGroups][kTile];
   ads_dependency_wait();
   const long long unit = blockIdx.x;
@@ -429,6 +496,10 @@ __global__ void __launch_bounds__(kTile * kMergeGroups) rel_merge_kernel(float* 
   for (int i = 0; i < kMergeGroups; ++i) l += part[i][r].y * exp2f(part[i][r].x - M);
   const float log_l = log2f(l);
   const bool exists = mt * kTile + r < rows;
+  if (norm != nullptr) {
+    if (y == 0) norm[unit * kTile + r] = make_float2(-M, exists && l > 0.f ? 1.f / l : 0.f);
+    return;
+  }
 #pragma unroll 8
   for (int s = y; s < splits; s += kMergeGroups) {
     float* first = ml + s * 3 * kTile + 2 * kTile;
@@ -480,6 +551,31 @@ __global__ void __launch_bounds__(256) rel_reduce_kernel(const float* __restrict
   }
 }
 
+// Two passes: mass[b][i] (+)= sum over the batch's heads of the masses of shot i's keys; grid (shots / 8, queries of the batch),
+// a warp per shot.
+__global__ void __launch_bounds__(256) rel_keys_kernel(const float* __restrict__ key_mass, const long long* __restrict__ shot_off,
+                                                       int n_shots, int n_heads, int head0, long long keys_pad,
+                                                       long long pool_tokens, int b0, double* __restrict__ mass) {
+  ads_dependency_wait();
+  const int lane = threadIdx.x & 31, i = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (i >= n_shots) return;
+  const long long o0 = i > 0 ? shot_off[i] : 0, o1 = i + 1 < n_shots ? shot_off[i + 1] : pool_tokens;
+  const float* src = key_mass + (long long)blockIdx.y * n_heads * keys_pad;
+  double sum = 0.0;
+  if (o1 - o0 < 32) {                                // several heads' keys at a time
+    const int len = (int)(o1 - o0);
+    for (int e = lane; e < len * n_heads; e += 32) sum += (double)src[e / len * keys_pad + o0 + e % len];
+  } else {
+    for (int h = 0; h < n_heads; ++h)
+      for (long long k = o0 + lane; k < o1; k += 32) sum += (double)src[h * keys_pad + k];
+  }
+  sum = warp_sum(sum);
+  if (lane == 0) {
+    double* out = mass + (long long)(b0 + blockIdx.y) * n_shots + i;
+    *out = head0 == 0 ? sum : *out + sum;
+  }
+}
+
 // score[b][i] = mass[b][i] / (T_q * Hq) (and / T_i with per_token); writes the sort keys.
 __global__ void __launch_bounds__(256) rel_scores_kernel(const double* __restrict__ mass,
                                                          const long long* __restrict__ shot_off, int B, int n_shots,
@@ -495,14 +591,16 @@ __global__ void __launch_bounds__(256) rel_scores_kernel(const double* __restric
 }
 
 constexpr size_t kPieceBytes = 256u << 20;
+constexpr long long kShortShot = 12;     // tokens per shot on average below which two passes are taken
 constexpr int kStartTiles = 4;          // what starting a CTA costs, in tiles (7 and 12 give the same times within 1 %)
 constexpr long long kMaxRanges = 16 * 148 * kGroups;     // (unit, range) pairs of a launch that are worth having: sixteen waves
 
 struct RelPlan {
+  bool two_passes;
   int G, n_mt, rows, rows_pad, n_tiles, splits, tiles_per_split;
   int batch, heads;             // M tiles and KV heads per launch of the pass
   int m_per_cta;                // of which share a CTA
-  size_t off_qpack, off_ml, off_pieces, off_mass, off_keys, total;
+  size_t off_qpack, off_ml, off_norm, off_pieces, off_mass, off_keys, total;
 };
 
 RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int B, int Tq) {
@@ -514,12 +612,15 @@ RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int
   pl.rows_pad = pl.n_mt * kTile;
   pl.n_tiles = (int)((pool->pool_tokens + kTile - 1) / kTile);
   const int most = (pl.n_tiles + 1) / 2 < 256 ? (pl.n_tiles + 1) / 2 : 256;
-  // M tiles whose pieces fit, in batches of equal size; where one tile's do not, KV heads in batches of equal size
+  // What lies between the steps fits in batches of equal size: M tiles (two passes: whole queries), and KV heads where one of
+  // them is too much.
   const long long m_tiles = (long long)B * pl.n_mt;
-  const long long fit_units = (long long)((kPieceBytes / (kTile * 4) - kMaxRanges) / (size_t)pool->n_shots);
-  const long long fit = fit_units / Hkv > 1 ? fit_units / Hkv : 1;
+  pl.two_passes = pool->pool_tokens < kShortShot * pool->n_shots;
+  const long long step = pl.two_passes ? pl.n_mt : 1;           // M tiles that stay together
+  const long long fit_units = (long long)((kPieceBytes / (kTile * 4) - kMaxRanges) / (pl.two_passes ? (size_t)pl.n_tiles : (size_t)pool->n_shots));
+  const long long fit = (fit_units / Hkv > 1 ? fit_units / Hkv : 1) * step;
   const long long n_batches = (m_tiles + fit - 1) / fit;
-  pl.batch = (int)((m_tiles + n_batches - 1) / n_batches);
+  pl.batch = (int)((m_tiles / step + n_batches - 1) / n_batches * step);
   pl.heads = Hkv;
   if (fit_units < Hkv) {
     const int n = (int)((Hkv + (fit_units > 1 ? fit_units : 1) - 1) / (fit_units > 1 ? fit_units : 1));
@@ -559,7 +660,9 @@ RelPlan rel_plan(const adapshot_model_t* model, const adapshot_pool_t* pool, int
   size_t off = 0;
   pl.off_qpack = off;   off += ads_round_up((size_t)B * Hkv * pl.rows_pad * D * 2, 256);
   pl.off_ml = off;      off += ads_round_up(ranges * kTile * 3 * 4, 256);
-  pl.off_pieces = off;  off += ads_round_up(((size_t)most_units * pool->n_shots + ranges) * kTile * 4, 256);
+  pl.off_norm = off;    off += pl.two_passes ? ads_round_up((size_t)most_units * kTile * sizeof(float2), 256) : 0;
+  pl.off_pieces = off;  off += ads_round_up(
+      (pl.two_passes ? (size_t)(most_units / step) * pl.n_tiles : (size_t)most_units * pool->n_shots + ranges) * kTile * 4, 256);
   pl.off_mass = off;    off += ads_round_up((size_t)B * pool->n_shots * 8, 256);
   pl.off_keys = off;    off += ads_round_up((size_t)B * pool->n_shots * 8, 256);
   pl.total = off;
@@ -603,6 +706,8 @@ int rel_launch(const adapshot_model_t* model, const adapshot_pool_t* pool, int l
   if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
   const long long* shot_off = reinterpret_cast<const long long*>(pool->shot_off);
   RelParams rp;
+  rp.norm = pl.two_passes ? reinterpret_cast<float2*>(wsb + pl.off_norm) : nullptr;
+  rp.key_mass = pieces;
   rp.ml_part = ml_part; rp.pieces = pieces; rp.shot_off = shot_off; rp.status = status;
   rp.pool_tokens = pool->pool_tokens;
   rp.Hkv = Hkv; rp.n_mt = pl.n_mt; rp.n_shots = pool->n_shots; rp.layer = layer;
@@ -611,8 +716,15 @@ int rel_launch(const adapshot_model_t* model, const adapshot_pool_t* pool, int l
   rp.scale_log2 = scale * 1.4426950408889634f;
 
   const int smem = (int)RelSmem<D>::kTotal;
-  static bool attr_done[kAdsMaxDevices] = {false};
-  if (ads_set_max_smem(rel_pass_kernel<D>, smem, attr_done) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
+  static bool attr_done[3][kAdsMaxDevices] = {{false}, {false}, {false}};
+  auto launch_pass = [&](auto kernel, int which, int tiles, int ranges, int heads) -> int {
+    if (ads_set_max_smem(kernel, smem, attr_done[which]) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
+    const int per_cta = kGroups / rp.m_per_cta;
+    ads_launch_dependent(kernel, dim3((unsigned)((tiles + rp.m_per_cta - 1) / rp.m_per_cta),
+                                      (unsigned)((ranges + per_cta - 1) / per_cta), (unsigned)heads),
+                         kRelThreads, smem, st, tm_q, tm_k, rp);
+    return ads_launch_status();
+  };
   const int m_tiles = B * pl.n_mt;
   for (int t0 = 0; t0 < m_tiles; t0 += pl.batch)
     for (int h0 = 0; h0 < Hkv; h0 += pl.heads) {
@@ -622,14 +734,40 @@ int rel_launch(const adapshot_model_t* model, const adapshot_pool_t* pool, int l
       rp.n_heads = nh;
       rp.n_m = n;
       rp.m_per_cta = pl.m_per_cta;
-      const int per_cta = kGroups / pl.m_per_cta;
-      ads_launch_dependent(rel_pass_kernel<D>, dim3((unsigned)((n + pl.m_per_cta - 1) / pl.m_per_cta),
-                                                    (unsigned)((pl.splits + per_cta - 1) / per_cta), (unsigned)nh),
-                           kRelThreads, smem, st, tm_q, tm_k, rp);
-      if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-      ads_launch_dependent(rel_merge_kernel, (unsigned)(n * nh), dim3(kTile, kMergeGroups), 0, st, ml_part, pl.splits, nh, t0, pl.n_mt, pl.rows);
+      const int rc = pl.two_passes ? launch_pass(rel_pass_kernel<D, kNormalisers>, 1, n, pl.splits, nh)
+                                   : launch_pass(rel_pass_kernel<D, kPieces>, 0, n, pl.splits, nh);
+      if (rc != ADAPSHOT_OK) return rc;
+      ads_launch_dependent(rel_merge_kernel, (unsigned)(n * nh), dim3(kTile, kMergeGroups), 0, st, ml_part, pl.splits, nh, t0,
+                           pl.n_mt, pl.rows, rp.norm);
       if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
       const int b0 = t0 / pl.n_mt, b1 = (t0 + n - 1) / pl.n_mt;       // queries with rows in the batch
+      if (pl.two_passes) {
+        // K tiles that stay in a CTA and queries that stream by: the cheapest waves * (steps + start).  A step of four, two or
+        // one K tiles takes about 4, 2.4 or 1.6 times the exponentials of one.
+        const int queries = n / pl.n_mt;
+        double best = 0.0;
+        int per_cta = 4, parts = 1;
+        for (int m = 4; m >= 1; m >>= 1)
+          for (int y = 1; y <= queries && y <= 64; ++y) {
+            const int part = (queries + y - 1) / y;
+            const long long ctas = (long long)((pl.n_tiles + m - 1) / m) * nh * ((queries + part - 1) / part);
+            const double cost = (double)((ctas + 147) / 148) * (part * pl.n_mt * (m == 4 ? 4.0 : m == 2 ? 2.4 : 1.6) + 16.0);
+            if (best == 0.0 || cost < best) {
+              best = cost;
+              per_cta = m;
+              parts = part;
+            }
+          }
+        rp.m_per_cta = per_cta;
+        rp.tiles_per_split = parts * pl.n_mt;
+        if (launch_pass(rel_pass_kernel<D, kMasses>, 2, pl.n_tiles, (queries + parts - 1) / parts * (kGroups / per_cta), nh) != ADAPSHOT_OK)
+          return ADAPSHOT_ECUDA;
+        rp.tiles_per_split = pl.tiles_per_split;
+        ads_launch_dependent(rel_keys_kernel, dim3((unsigned)((pool->n_shots + 7) / 8), (unsigned)(b1 - b0 + 1)), 256, 0, st,
+                             pieces, shot_off, pool->n_shots, nh, h0, (long long)pl.n_tiles * kTile, pool->pool_tokens, b0, mass);
+        if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
+        continue;
+      }
       int warps = 8;                                                  // per shot: one where shots alone fill the chip
       while (warps > 1 && (long long)pool->n_shots * (b1 - b0 + 1) * warps > 2 * 8 * 148 * 4) warps >>= 1;
       ads_launch_dependent(rel_reduce_kernel, dim3((unsigned)((pool->n_shots + 8 / warps - 1) / (8 / warps)),

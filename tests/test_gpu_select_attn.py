@@ -171,9 +171,8 @@ def test_masses_do_not_carry_the_rounding_of_large_scores(big):
 
 
 @pytest.mark.parametrize("batch,t_q", [(1, 3), (2, 130)])
-def test_heads_in_batches(batch, t_q):
-    # 66000 shots: the pieces of one M tile and all eight KV heads are more than 256 MB, so the heads go four by four, the M
-    # tiles (two per query at 130 tokens) one by one
+def test_many_shots_of_one_token(batch, t_q):
+    # 66000 shots of one token: two passes, all heads at once; two M tiles per query at 130 tokens
     w = wl.CONFIGS["cfg2"].scaled(n_shots=66000, len_lo=1, len_hi=1, batch=batch, k=32, t_q=t_q, n_q_heads=8,
                                   n_kv_heads=8, head_dim=64, emb_dim=8, seed=92)
     _check(w, 1, 0, 32)
@@ -185,3 +184,41 @@ def test_warps_per_shot_and_many_ranges(n_shots, lens, t_q, batch):
     w = wl.CONFIGS["cfg2"].scaled(n_shots=n_shots, len_lo=lens[0], len_hi=lens[1], batch=batch, k=n_shots, t_q=t_q, n_q_heads=8,
                                   n_kv_heads=1, seed=93)
     _check(w, 1, 0, n_shots)
+
+
+@pytest.mark.parametrize("lens,n_shots,t_q,batch,hq,hkv", [
+    ((11, 11), 300, 33, 2, 8, 2),       # just below the line of twelve tokens: two passes; K tiles two by two
+    ((12, 12), 300, 33, 2, 8, 2),       # on it: one pass
+    ((1, 6), 9000, 40, 3, 8, 8),        # every CTA keeps four K tiles; two M tiles per query; queries in parts
+    ((1, 3), 50, 5, 1, 4, 1),           # one K tile
+    ((1, 40), 200, 150, 1, 8, 1),       # nineteen M tiles of one query in front of 32 K tiles
+])
+def test_short_shots(lens, n_shots, t_q, batch, hq, hkv):
+    w = wl.CONFIGS["cfg2"].scaled(n_shots=n_shots, len_lo=lens[0], len_hi=lens[1], batch=batch, k=min(n_shots, 50), t_q=t_q,
+                                  n_q_heads=hq, n_kv_heads=hkv, head_dim=64 if hkv == 8 else 128, seed=94)
+    _check(w, 1, 0, w.k)
+
+
+def test_short_shots_with_queries_in_batches():
+    # 210 K keys x 8 heads x 4 bytes: 39 queries at a time, so 40 queries go as two times twenty; those at the seam and the ends
+    ab = hp.gpu_binding()
+    w = wl.CONFIGS["cfg2"].scaled(n_shots=42000, len_lo=5, len_hi=5, batch=40, k=64, t_q=1, n_q_heads=8, n_kv_heads=8,
+                                  head_dim=64, emb_dim=8, seed=95)
+    pool, qs = wl.make_pool(w, n_layers=1), wl.make_queries(w, n_layers=1, n_probes=1)
+    q = qs["q"][:, 0, 0].contiguous()
+    sel, score = _run(ab, hp.model_of(ab, w, n_layers=1), hp.dev_pool(ab, pool), 0, q, 64)
+    k_layer = hp.f64(pool["k"][0])
+    for b in (0, 19, 20, 39):
+        s = orc.relevance_attention(hp.f64(q[b]), k_layer, pool["shot_off"])
+        assert np.all(np.abs(score[b] - s[sel[b]]) <= SCORE_REL * s[sel[b]])
+        assert s[sel[b]].min() >= np.sort(s)[-64] * (1 - 2 * SCORE_REL)
+
+
+@pytest.mark.parametrize("n_shots,t_q,hq,hkv", [
+    (66000, 2, 8, 8),                   # the pieces of one M tile are more than 256 MB: the KV heads go four by four
+    (4000, 550, 32, 8),                 # eighteen M tiles of one query in two batches
+])
+def test_pieces_in_batches(n_shots, t_q, hq, hkv):
+    w = wl.CONFIGS["cfg2"].scaled(n_shots=n_shots, len_lo=12, len_hi=12, batch=1, k=32, t_q=t_q, n_q_heads=hq, n_kv_heads=hkv,
+                                  head_dim=64, emb_dim=8, seed=96)
+    _check(w, 1, 0, 32)
