@@ -281,9 +281,9 @@ ADAPSHOT_API int adapshot_tree_attn(const adapshot_model_t* model, const void* k
  *             outside that range is reported as ADAPSHOT_EINDEX in `status` and clamped
  *   q_new   : [B][nl][T_new][Hq][d];  k_own, v_own : [B][nl][T_own][Hkv][d]  (un-rotated)
  *   out     : [B][nl][T_new][Hq][d];  lse [B][nl][Hq][T_new] or NULL
- * A decode step is bound by the K/V bytes it reads: calls of at most 32 rows per KV head
- * (T_new * G) stream them through a kernel of their own, larger ones take the kernels of
- * adapshot_query_attn.  Limits: B <= 256, T_own >= T_new >= 1.                              */
+ * A decode step is bound by the K/V bytes it reads: calls of at most 16 rows per KV head
+ * (T_new * G; 32 where that is faster) stream them through a kernel of their own, larger
+ * ones take the kernels of adapshot_query_attn.  Limits: B <= 256, T_own >= T_new >= 1.                              */
 ADAPSHOT_API size_t adapshot_decode_workspace_bytes(const adapshot_model_t* model, int32_t B, int32_t T_new,
                                        int32_t T_own, int32_t n_layers_in_call);
 ADAPSHOT_API int adapshot_decode_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_ctx,

@@ -1796,8 +1796,10 @@ extern "C" size_t adapshot_decode_workspace_bytes(const adapshot_model_t* model,
                                                   int32_t T_own, int32_t n_layers_in_call) {
   if (model == nullptr || !attn_shape_ok(model) || B <= 0 || T_new <= 0 || T_own < T_new || n_layers_in_call <= 0)
     return 0;
-  if (ads_decode_rows_fit(model, T_new)) return ads_decode_rows_workspace(model, B);
-  return make_plan(model, B, 1, T_new, n_layers_in_call, 0, T_own).total;
+  const size_t rows = ads_decode_rows_workspace(model, B), plan = make_plan(model, B, 1, T_new, n_layers_in_call, 0, T_own).total;
+  if (!ads_decode_rows_fit(model, T_new)) return plan;
+  // (a larger context only ever speaks for the kernel that streams)
+  return ads_decode_rows_pay(model, B, T_new, T_own, 1) || rows > plan ? rows : plan;
 }
 
 extern "C" int adapshot_decode_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_ctx,
@@ -1820,10 +1822,11 @@ extern "C" int adapshot_decode_attn(const adapshot_model_t* model, const void* k
     return ADAPSHOT_EALIGN;
   if (ctx_cap > (1ll << 31) - 256) return ADAPSHOT_ESHAPE;
   const int nl = layer_end - layer_begin;
-  // Up to 32 rows per KV head: the kernel that streams K/V through warp-level tiles (decode.cu): 256 against
+  // Up to 32 rows per KV head: the kernel that streams K/V through warp-level tiles (decode.cu) where it pays: 256 against
   // 376 us at 4 rows and 32 requests.  The line is where its accumulators stop fitting two CTAs per SM; more rows
-  // fill the 128-row tiles of the prefill kernels better as well.
-  if (ads_decode_rows_fit(model, T_new)) {
+  // fill the 128-row tiles of the prefill kernels better as well.  A workspace that only it can do with is taken, too.
+  if (ads_decode_rows_fit(model, T_new) &&
+      (ads_decode_rows_pay(model, B, T_new, T_own, ctx_cap) || ws_bytes < make_plan(model, B, 1, T_new, nl, 0, T_own).total)) {
     if (ws_bytes < ads_decode_rows_workspace(model, B)) return ADAPSHOT_ECAPACITY;
     return ads_decode_rows(model, k_ctx, v_ctx, ctx_cap, ctx_off, B, k, n_shots, q_new, k_own, v_own, T_new, T_own, nl,
                            out, lse, ws, status, static_cast<cudaStream_t>(stream));

@@ -106,9 +106,10 @@ __device__ __forceinline__ double ads_key_score(unsigned long long k) {
 int ads_topk_from_keys(const unsigned long long* keys, int N, int B, int k, int32_t* sel_idx, float* sel_score,
                        cudaStream_t st);
 
-// Decoding with few rows per KV head (decode.cu): whether a call's rows fit, its scratch, and the call itself
+// Decoding with few rows per KV head (decode.cu): whether a call's rows fit, whether it pays, its scratch, and the call itself
 // (arguments checked by the caller).
 bool ads_decode_rows_fit(const adapshot_model_t* model, int T_new);
+bool ads_decode_rows_pay(const adapshot_model_t* model, int B, int T_new, int T_own, int64_t ctx_cap);
 size_t ads_decode_rows_workspace(const adapshot_model_t* model, int B);
 int ads_decode_rows(const adapshot_model_t* model, const void* k_ctx, const void* v_ctx, int64_t ctx_cap,
                     const int64_t* ctx_off, int B, int k, const int32_t* n_shots, const void* q_new, const void* k_own,

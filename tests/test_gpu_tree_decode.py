@@ -176,3 +176,41 @@ def test_decode_row_counts_and_range_cuts(hq, d, batch, n_shots, t_new, t_own):
                 want.append(o_want)
                 assert abs(float(lse[b, 0, h, t]) - l_want) <= hp.lse_bound()
     hp.assert_attn_close(np.stack(got), np.stack(want))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("hq,hkv,d,batch,k,t_new,t_own,small_ws", [
+    (8, 1, 128, 2, 3, 4, 100, False),      # 32 rows, d = 128: streamed for one KV head and long own sequences
+    (8, 1, 128, 2, 3, 4, 99, False),       # the prefill kernels
+    (8, 1, 128, 2, 3, 4, 99, True),        # streamed, because the workspace has no room for the prefill kernels'
+    (8, 2, 64, 2, 3, 8, 210, False),       # 32 rows, d = 64, a capacity of 216 to 224 and 4 x 210 own tokens: streamed
+    (8, 2, 64, 2, 3, 8, 190, False),       # the prefill kernels
+    (8, 2, 64, 1, 3, 8, 20, True),
+])
+def test_decode_on_both_sides_of_the_line_between_the_kernels(hq, hkv, d, batch, k, t_new, t_own, small_ws):
+    ab = hp.gpu_binding()
+    w = wl.CONFIGS["cfg2"].scaled(n_shots=k, len_lo=63, len_hi=65, batch=batch, k=k, probes=(k,), t_q=t_own, n_q_heads=hq,
+                                  n_kv_heads=hkv, head_dim=d, seed=77)
+    ab, pool, qs, sel_np, off_np, model, cap, kc, vc, off = _setup(w, 1, 14)
+    q_new = qs["q"][:, :, 0, t_own - t_new:].contiguous().cuda()
+    k_own, v_own = qs["kq"][:, :, 0].contiguous().cuda(), qs["vq"][:, :, 0].contiguous().cuda()
+    out, st = torch.full_like(q_new, 9.0), hp.new_status()
+    n_bytes = ab.adapshot_decode_workspace_bytes(model, batch, 1 if small_ws else t_new, t_own, 1)
+    assert not small_ws or n_bytes < ab.adapshot_decode_workspace_bytes(model, batch, t_new, t_own, 1)
+    ws = torch.empty(n_bytes, dtype=torch.uint8, device="cuda")
+    n_star = torch.full((batch,), k, dtype=torch.int32, device="cuda")
+    ab.adapshot_decode_attn(model, kc, vc, cap, off, k, n_star, q_new, k_own, v_own, 0, 1, out, None, ws, st)
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    kp, vp = hp.f64(pool["k"][:1]), hp.f64(pool["v"][:1])
+    got, want = [], []
+    for b in range(batch):
+        k_ctx, v_ctx, _ = orc.assemble_kv(kp, vp, pool["shot_off"], sel_np[b], w.rope_base)
+        for t in range(t_new):
+            u = t_own - t_new + t
+            for h in range(hq):
+                g = h // (hq // hkv)
+                want.append(orc.decode_row(hp.f64(q_new[b, 0, t, h].cpu()), hp.f64(qs["kq"][b, 0, 0])[:u + 1], hp.f64(qs["vq"][b, 0, 0])[:u + 1],
+                                           k_ctx[0], v_ctx[0], int(off_np[b, k]), g, w.rope_base)[0])
+                got.append(out[b, 0, t, h].cpu().double().numpy())
+    hp.assert_attn_close(np.stack(got), np.stack(want))
