@@ -463,18 +463,18 @@ rank_topk_kernel(const unsigned long long* __restrict__ all_keys, int N, int k,
   }
 }
 
-// Rank counting compares every pair of keys, over the whole chip; the radix selection is one CTA per
-// query.  Counting / selection: one query of 3100 keys 6.3 / 8.9 us, 3740 keys 7.0 / 9.0, three of 2040 keys 5.8 / 8.5,
-// thirteen of 1024 6.1 / 8.2, fifty of 512 6.9 / 7.5, two hundred of 256 9.5 / 12; the line lies where the counting,
-// which grows with the product, would reach the selection (fifty of 512 keys come close to it).
-bool rank_by_counting(int N, int B) { return (long long)N * N * B <= 14000000ll; }
+// Rank counting compares every pair of keys, over the whole chip, whatever k; the radix selection is one CTA per query and
+// sorts k candidates at its end.  Counting / selection, us: one query of 3000 keys, k = 1 8.0 / 7.2, k = 128 8.1 / 10.4; 4096 keys,
+// k = 1 9.2 / 7.6, 128 9.2 / 11.0, 1024 9.3 / 17.8, 4096 9.3 / 65; 8192 keys, k = 512 21 / 16, 1024 21 / 20, 4096 21 / 70; 64
+// queries of 512 keys, k = 32 10.7 / 8.4, k = 128 10.7 / 10.3; the line follows the points where the two meet.
+bool rank_by_counting(int N, int B, int k) { return (long long)N * N * B <= 11000000ll + 48000ll * k; }
 
 }  // namespace
 
 int ads_topk_from_keys(const unsigned long long* keys, int N, int B, int k, int32_t* sel_idx, float* sel_score,
                        cudaStream_t st) {
   if (N > kSortCap && k > kSortCap / 2) return ADAPSHOT_EUNSUPPORTED;
-  if (rank_by_counting(N, B)) {
+  if (rank_by_counting(N, B, k)) {
     dim3 grid((N + kRankCand - 1) / kRankCand, B);
     ads_launch_dependent(rank_topk_kernel, grid, kRankThreads, 0, st, keys, N, k, sel_idx, sel_score);
     return ads_launch_status();

@@ -101,3 +101,13 @@ def test_rank_counting_with_ties(N, B, k):
     base = torch.randn((N + 2) // 3, 32, generator=g)
     emb = base[torch.randint(0, base.shape[0], (N,), generator=g)]
     _check(ab, emb, torch.randn(B, 32, generator=g), k)
+
+
+@pytest.mark.parametrize("N,B,k", [(3751, 1, 64), (3752, 1, 64), (6100, 1, 600), (6400, 1, 600), (8192, 1, 4096), (8192, 3, 4096)])
+def test_both_sides_of_the_line_between_counting_and_selection(N, B, k):
+    # N^2 B against 11 million and 48000 k; every embedding occurs about three times
+    ab = hp.gpu_binding()
+    g = torch.Generator().manual_seed(N + B)
+    base = torch.randn((N + 2) // 3, 32, generator=g)
+    emb = base[torch.randint(0, base.shape[0], (N,), generator=g)]
+    _check(ab, emb, torch.randn(B, 32, generator=g), k)
