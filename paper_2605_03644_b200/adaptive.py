@@ -76,11 +76,12 @@ class ProbeRounds:
         probes = self.schedule[r]
         k_r = probes[-1]
         nl = self.model.n_layers
-        sel_r, off_r = self.sel_idx[:, :k_r].contiguous(), self.ctx_off(k_r)
+        # (no views of them while the GPU waits: one query's prefix begins where its selection does, and so do the offsets)
+        sel_r, off_r = self.sel_idx if self.B == 1 else self.sel_idx[:, :k_r].contiguous(), self._ctx_off
         # the earlier rounds' shots are in place already: only the new ones are gathered
         first_new = self.schedule[r - 1][-1] if r > 0 else 0
         ab.adapshot_assemble_kv_from(self.model, self.pool, sel_r, first_new, 0, nl, self.k_ctx, self.v_ctx,
-                                     self.ctx_cap, off_r, self.status)
+                                     self.ctx_cap, off_r, self.status, k=k_r)
         ab.adapshot_query_attn(self.model, self.k_ctx, self.v_ctx, self.ctx_cap, off_r, k_r, probes,
                                q, kq, vq, 0, nl, self.out, None, self.ws_attn, self.status)
         ab.adapshot_entropy(logits, self.H, tau, self.m, self.first_ok, self.ws_entropy, self.status)

@@ -227,7 +227,7 @@ def adapshot_reuse_pass(model: ModelT, pool: Pool, probe_nshots: Sequence[int], 
     _check_q_emb(pool, q_emb, B)
     if not logits.is_cuda or logits.stride(1) != 1:
         raise ValueError("logit rows must be contiguous, on the GPU")
-    if logits.shape[0] != B * P or not n <= min(len(q), len(kq), len(vq), len(out)):
+    if logits.shape[0] != B * P or len(q) < n or len(kq) < n or len(vq) < n or len(out) < n:
         raise ValueError("one logit row per query and probe, one tensor per layer chunk")
     if sel_idx.numel() < B * k or H.numel() < B * P:
         raise ValueError("more queries or probes than there is room for")
@@ -239,22 +239,22 @@ def adapshot_reuse_pass(model: ModelT, pool: Pool, probe_nshots: Sequence[int], 
             raise ValueError(f"a tensor of layer chunk {i} has another size than the pass")
         if q[i].dtype != dtype or out[i].dtype != dtype or kq[i].dtype != dtype or vq[i].dtype != dtype:
             raise ValueError(f"a tensor of layer chunk {i} is not {dtype}")
-    tensors = (q_emb, sel_idx, ctx_off, H, ws_select, ws_attn, ws_entropy, status, *q[:n], *kq[:n], *vq[:n], *out[:n])
-    ptrs = [t.data_ptr() for t in tensors if t.is_cuda and t.is_contiguous()]                   # _ptr of each
+    tensors = (q_emb, sel_idx, sel_score, ctx_off, k_ctx, v_ctx, H, first_ok, ws_select, ws_attn, ws_entropy, status,
+               *q[:n], *kq[:n], *vq[:n], *out[:n])
+    ptrs = [0 if t is None else t.data_ptr() for t in tensors if t is None or t.is_cuda and t.is_contiguous()]   # _ptr of each
     if len(ptrs) != len(tensors):
         raise ValueError("expected contiguous CUDA tensors")
     # the struct, the four arrays of pointers, layer_end and probe_nshots, in one piece
     buf = (C.c_char * (_PASS_BYTES + 36 * n + 4 * P))()
     at = C.addressof(buf)
-    arrays, step = at + _PASS_BYTES, 8 * n
+    q_at, step = at + _PASS_BYTES, 8 * n
+    ends_at = q_at + 4 * step
     struct.pack_into(
         f"{_PASS_FORMAT}{4 * n}P{n + P}i", buf, 0,
-        C.addressof(model), C.addressof(pool.c), arrays + 4 * step + 4 * n, arrays + 4 * step, B, k, P, Tq, n, variant,
-        logits.shape[1], _logit_dtype(logits), logits.stride(0), ctx_cap,
-        ptrs[0], arrays, arrays + step, arrays + 2 * step, arrays + 3 * step, logits.data_ptr(),
-        ptrs[1], _ptr(sel_score) or 0, ptrs[2], _ptr(k_ctx) or 0, _ptr(v_ctx) or 0, ptrs[3], _ptr(first_ok) or 0,
-        ptrs[4], ptrs[5], ptrs[6], ws_select.nbytes, ws_attn.nbytes, ws_entropy.nbytes, ptrs[7], tau, 0,
-        *ptrs[8:], *layer_end, *probe_nshots)
+        C.addressof(model), C.addressof(pool.c), ends_at + 4 * n, ends_at, B, k, P, Tq, n, variant, logits.shape[1],
+        _logit_dtype(logits), logits.stride(0), ctx_cap, ptrs[0], q_at, q_at + step, q_at + 2 * step, q_at + 3 * step,
+        logits.data_ptr(), *ptrs[1:11], ws_select.nbytes, ws_attn.nbytes, ws_entropy.nbytes, ptrs[11], tau, 0, *ptrs[12:],
+        *layer_end, *probe_nshots)
     _check(_reuse_pass(at, _stream()))
 
 
@@ -296,8 +296,14 @@ def adapshot_assemble_kv(model: ModelT, pool: Pool, sel_idx: torch.Tensor, layer
 
 def adapshot_assemble_kv_from(model: ModelT, pool: Pool, sel_idx: torch.Tensor, shot_begin: int,
                               layer_begin: int, layer_end: int, k_ctx: torch.Tensor, v_ctx: torch.Tensor,
-                              ctx_cap: int, ctx_off: torch.Tensor, status: torch.Tensor, flags: int = 0):
-    B, k = sel_idx.shape
+                              ctx_cap: int, ctx_off: torch.Tensor, status: torch.Tensor, flags: int = 0,
+                              k: Optional[int] = None):
+    """k: how many shots of the selection are meant (default: all; fewer only of a single query's)."""
+    B, n_sel = sel_idx.shape
+    if k is None:
+        k = n_sel
+    elif k > n_sel or (B > 1 and k != n_sel):
+        raise ValueError(f"{k} shots per query of a selection of {tuple(sel_idx.shape)}")
     _check(_assemble_from(C.byref(model), C.byref(pool.c), _ptr(sel_idx), B, k, shot_begin, layer_begin,
                           layer_end, _ptr(k_ctx), _ptr(v_ctx), ctx_cap, _ptr(ctx_off), flags, _ptr(status),
                           _stream()))

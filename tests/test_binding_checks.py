@@ -71,3 +71,17 @@ def test_select_and_entropy_refuse_other_shapes_and_types(ab):
     ab.adapshot_select(a["pool"], a["q_emb"], a["k"], a["sel_idx"], None, a["ws_select"], a["status"])
     ab.adapshot_entropy(a["logits"], a["H"], 0.5, 2, None, a["ws_entropy"], a["status"])
     assert ab.calls == ["_select", "_entropy"]
+
+
+def test_a_prefix_of_the_selection_is_taken_of_one_query_alone(ab, monkeypatch):
+    got = []
+    monkeypatch.setattr(ab, "_assemble_from", lambda *a: got.append((a[3], a[4])) or 0)
+    a = _pass_args(ab)
+    call = lambda sel, k: ab.adapshot_assemble_kv_from(a["model"], a["pool"], sel, 0, 0, 3, a["k_ctx"], a["v_ctx"], 40,
+                                                       a["ctx_off"], a["status"], k=k)
+    one, three = a["sel_idx"][:1].contiguous(), a["sel_idx"]
+    call(one, 2), call(one, None), call(three, 4), call(three, None)
+    assert got == [(1, 2), (1, 4), (3, 4), (3, 4)]
+    for sel, k in ((one, 5), (three, 2)):
+        with pytest.raises(ValueError):
+            call(sel, k)
