@@ -58,13 +58,13 @@ static inline int ads_set_max_smem(Kernel kernel, int bytes, bool* done) {
 }
 
 // Programmatic dependent launch: the kernel may be started while the one in front of it in the stream still
-// ends, so that its launch and its set-up cost no gap (a pass of a few short shots, nine kernels: 45.9 -> 28.3 us;
-// two rounds of probes 637 -> 622; a ranking by attention over 64 shots 56 -> 45, over 2048 912 -> 906).  Every kernel launched this way calls ads_dependency_wait()
-// before it touches global memory (in every block: what completes a kernel is the completion of its blocks, and a
-// block that did not wait would not stand for the kernels before).  ads_dependency_trigger() lets the next kernel
-// in earlier, once all blocks have called it; only the decode kernels do: elsewhere the early blocks took
-// room from the kernel they waited for (one layer of one query 132 -> 139 us with triggers in every kernel, of which the
-// selection's alone account for all).
+// ends, so that its launch and its set-up cost no gap (a pass of a few short shots, nine kernels: 45.9 -> 28.3 us; two rounds
+// of probes 637 -> 622; a ranking by attention over 2048 shots 912 -> 906).  Every kernel launched this way calls
+// ads_dependency_wait() before it touches global memory (in every block: what completes a kernel is the completion of its
+// blocks, and a block that did not wait would not stand for the kernels before).  ads_dependency_trigger() lets the next
+// kernel in earlier, once all blocks have called it; only the decode kernels do: elsewhere the early blocks took room from
+// the kernel they waited for (one layer of one query 132 -> 139 us with triggers in every kernel, the selection's alone
+// account for all of it).
 template <typename... KArgs, typename... Args>
 static inline void ads_launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                         const Args&... args) {
