@@ -8,6 +8,7 @@ stream is passed to every call.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 import struct
 from typing import Optional, Sequence
@@ -213,6 +214,13 @@ _PASS_FORMAT = "4P8i2q6P10P3NPfi"
 _PASS_BYTES = struct.calcsize(_PASS_FORMAT)
 
 
+@functools.lru_cache(maxsize=256)
+def _pass_layout(n: int, P: int):
+    """The struct, the four arrays of pointers, layer_end and probe_nshots in one piece: its format and a buffer type."""
+    form = struct.Struct(f"{_PASS_FORMAT}{4 * n}P{n + P}i")
+    return form.pack_into, C.c_char * form.size
+
+
 def adapshot_reuse_pass(model: ModelT, pool: Pool, probe_nshots: Sequence[int], layer_end: Sequence[int], variant: int,
                         k: int, ctx_cap: int, q_emb: torch.Tensor, q, kq, vq, out, logits: torch.Tensor,
                         tau: float, sel_idx: torch.Tensor, sel_score: Optional[torch.Tensor], ctx_off: torch.Tensor,
@@ -225,9 +233,10 @@ def adapshot_reuse_pass(model: ModelT, pool: Pool, probe_nshots: Sequence[int], 
     B, P, n, Tq = q_emb.shape[0], len(probe_nshots), len(layer_end), q[0].shape[3]
     dtype = torch.float32 if model.dtype == F32 else torch.bfloat16
     _check_q_emb(pool, q_emb, B)
-    if not logits.is_cuda or logits.stride(1) != 1:
+    (n_rows, V), (row_stride, one) = logits.shape, logits.stride()
+    if not logits.is_cuda or one != 1:
         raise ValueError("logit rows must be contiguous, on the GPU")
-    if logits.shape[0] != B * P or len(q) < n or len(kq) < n or len(vq) < n or len(out) < n:
+    if n_rows != B * P or len(q) < n or len(kq) < n or len(vq) < n or len(out) < n:
         raise ValueError("one logit row per query and probe, one tensor per layer chunk")
     if sel_idx.numel() < B * k or H.numel() < B * P:
         raise ValueError("more queries or probes than there is room for")
@@ -244,15 +253,14 @@ def adapshot_reuse_pass(model: ModelT, pool: Pool, probe_nshots: Sequence[int], 
     ptrs = [0 if t is None else t.data_ptr() for t in tensors if t is None or t.is_cuda and t.is_contiguous()]   # _ptr of each
     if len(ptrs) != len(tensors):
         raise ValueError("expected contiguous CUDA tensors")
-    # the struct, the four arrays of pointers, layer_end and probe_nshots, in one piece
-    buf = (C.c_char * (_PASS_BYTES + 36 * n + 4 * P))()
+    pack_into, buffer = _pass_layout(n, P)
+    buf = buffer()
     at = C.addressof(buf)
     q_at, step = at + _PASS_BYTES, 8 * n
     ends_at = q_at + 4 * step
-    struct.pack_into(
-        f"{_PASS_FORMAT}{4 * n}P{n + P}i", buf, 0,
-        C.addressof(model), C.addressof(pool.c), ends_at + 4 * n, ends_at, B, k, P, Tq, n, variant, logits.shape[1],
-        _logit_dtype(logits), logits.stride(0), ctx_cap, ptrs[0], q_at, q_at + step, q_at + 2 * step, q_at + 3 * step,
+    pack_into(
+        buf, 0, C.addressof(model), C.addressof(pool.c), ends_at + 4 * n, ends_at, B, k, P, Tq, n, variant, V,
+        _logit_dtype(logits), row_stride, ctx_cap, ptrs[0], q_at, q_at + step, q_at + 2 * step, q_at + 3 * step,
         logits.data_ptr(), *ptrs[1:11], ws_select.nbytes, ws_attn.nbytes, ws_entropy.nbytes, ptrs[11], tau, 0, *ptrs[12:],
         *layer_end, *probe_nshots)
     _check(_reuse_pass(at, _stream()))

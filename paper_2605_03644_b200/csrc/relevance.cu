@@ -12,7 +12,7 @@
 //           every shot of the CTA's range of keys, written as maximum - first maximum + log2(sum) at the shot's end;
 //   merge   the ranges' maxima and sums -> what is left to add to a range's pieces: its first maximum - log2-sum-exp of
 //           the row;
-//   reduce  mass of a shot = sum over rows of 2^(its piece + the row's share), a warp per shot.
+//   reduce  mass of a shot = sum over rows of 2^(its piece + the row's share), one to eight warps per shot.
 // (Both are small where the mass is, however large the scores are. As maximum + log2(sum) every piece carried the rounding of
 // the maximum, each shot its own: 2.5e-5 of a shot's mass at logits of 2048, now 3e-6 at most.)
 // What lies between the steps is 4 bytes per row and shot; the rows are taken in batches (of M tiles, and of KV heads where
@@ -25,7 +25,8 @@
 //   keys    mass of a shot = sum over its keys and the heads.
 // One pass / two, 32 / 8 heads, d = 128, 8 queries x 256 tokens: 2.5 tokens per shot (30000 shots) 12061 / 3295 us, 8 tokens
 // (4000) 2248 / 1472, 12 tokens (2000) 1397 / 1279, 24 tokens (3000) 2662 / 3123; one query of 8 tokens 224 / 130, 67 / 64,
-// 48 / 53, 74 / 116.  For 160 tokens per shot two passes cost nearly twice as much (1842 / 912 us before the pieces).
+// 48 / 53, 74 / 116.  2 queries x 128 tokens over 328 K keys in shots of 160 tokens: 912 us with one pass, 1842 with two (the
+// form before the pieces).
 // The scores then go through the same top-k as the embedding selector (ties -> lower shot id).
 #include <float.h>
 
@@ -458,8 +459,9 @@ rel_pass_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 }
 
 // What is left to add to the pieces of a row in every range: first max - log2 sum_keys 2^(s c), -inf for rows that do not exist
-// (so that they add nothing).  With norm set (two passes): (-max, 1 / sum) of the row instead, 0 for the latter.  A block per unit: threadIdx.x is the row, every kMergeGroups-th range a thread's.  (One thread
-// per row walked up to 256 ranges: 51 us for 4 units of 71 ranges, 16 for 148 now.)
+// (so that they add nothing).  With norm set (two passes): (-max, 1 / sum) of the row instead, 0 for the latter.  A block per
+// unit: threadIdx.x is the row, every kMergeGroups-th range a thread's.  (One thread per row walked up to 256 ranges: 51 us for 4
+// units of 71 ranges, 16 for 148 now.)
 constexpr int kMergeGroups = 8;
 __global__ void __launch_bounds__(kTile * kMergeGroups) rel_merge_kernel(float* __restrict__ ml_part, int splits, int n_heads,
                                                                          int tile0, int n_mt, int rows,
