@@ -31,6 +31,7 @@
 #include <float.h>
 
 #include "common.cuh"
+#include "entropy.cuh"
 #include "sm100_ptx.cuh"
 #include "tma_host.cuh"
 
@@ -107,6 +108,19 @@ struct AttnParams {
   double theta[64];
 };
 
+// V-from-pool and fused variants, once per call: the pool token behind every context position of every query
+// (the gather's plan lookup, stored instead of applied) and, for keys stored rotated, the first position of its
+// shot.  Positions from L to the end of the last 128-token tile get -1; nothing beyond them is read.
+struct RowMapParams {
+  const long long* ctx_off;   // [B][k+1]
+  const int32_t* sel_idx;     // [B][k]
+  const long long* shot_off;  // [n_shots+1]
+  int* row_map;               // [B][ctx_cap]
+  int* off_map;               // [B][ctx_cap] or null
+  long long ctx_cap;
+  int B, k, n_shots;
+};
+
 struct PrepParams {
   const __nv_bfloat16* q;     // [B][nl][P][Tq][Hq][D]
   const __nv_bfloat16* kq;    // [B][nl][P][To][Hkv][D]
@@ -121,6 +135,10 @@ struct PrepParams {
   int32_t* status;
   double theta[64];           // theta_i = rope_base^(-2i/D), formed on the host
   int nshots[kMaxProbes];
+  // what else the launch does: its blocks are the schedule's, then these, then the tokens'
+  AdsEntropyJob ent;          // entropy of the probes' logits, first step
+  RowMapParams map;
+  int map_blocks;             // eight selected shots each; 0: no row map
 };
 
 __device__ __forceinline__ void bf16x8_unpack(const uint4& r, float* x) {
@@ -159,13 +177,39 @@ __device__ __forceinline__ int probe_shots(const PrepParams& p, int b, int j) {
   return n;
 }
 
+// One warp (w) per selected shot: its run of positions is written with whole lines (a search per position
+// took 38 us for 32 queries of 66 K positions and 8.3 us for 8 of 33 K; 3 us for those now).
+__device__ __forceinline__ void row_map_warp(const RowMapParams& p, long long w, int lane) {
+  if (w >= (long long)p.B * p.k) return;
+  const int b = (int)(w / p.k), r = (int)(w % p.k);
+  const long long* off = p.ctx_off + (long long)b * (p.k + 1);
+  const long long o0 = off[r], o1 = off[r + 1];
+  const int s = p.sel_idx[w];
+  int* rows = p.row_map + (long long)b * p.ctx_cap;
+  int* firsts = p.off_map == nullptr ? nullptr : p.off_map + (long long)b * p.ctx_cap;
+  const long long end = min(o1, p.ctx_cap);
+  const bool known = s >= 0 && s < p.n_shots;        // (an unknown shot is reported by the plan and has no positions)
+  const long long src = known ? p.shot_off[s] - o0 : 0;
+  for (long long pos = o0 + lane; pos < end; pos += 32) {
+    rows[pos] = known ? (int)(src + pos) : -1;
+    if (firsts != nullptr) firsts[pos] = (int)o0;
+  }
+  if (r == p.k - 1) {
+    const long long pad = min((o1 + kTileN - 1) / kTileN * kTileN, p.ctx_cap);
+    for (long long pos = o1 + lane; pos < pad; pos += 32) {
+      rows[pos] = -1;
+      if (firsts != nullptr) firsts[pos] = 0;
+    }
+  }
+}
+
 // kPrepParts warps per own token (b, l, j, u): all Hq query heads and Hkv key heads of the token rotate by the same
 // angles (L_j + u) * theta_i, which the block forms once for its tokens, half an angle per thread, while the first
 // rows are on their way.  (Every lane forming its eight angles itself was what bound the kernel: 4096 tokens of 32
 // + 8 heads, 84 MB, 27 us and 14336 tokens 82-90 us; now 20 and 73.)  The first block writes the schedule instead: started
 // first, its chain of dependent steps lies under the others' copies.
 template <int D>
-__global__ void __launch_bounds__(256, 3) attn_prep_kernel(const PrepParams p) {
+__global__ void __launch_bounds__(256, 3) attn_prep_kernel(const __grid_constant__ PrepParams p) {
   constexpr int VPH = D / 8, HALF_V = VPH / 2;
   const int lane = threadIdx.x & 31;
   ads_dependency_wait();
@@ -265,10 +309,25 @@ __global__ void __launch_bounds__(256, 3) attn_prep_kernel(const PrepParams p) {
     if (threadIdx.x == 0) sc->n_cut = s_ncut;
     return;
   }
+  int blk = (int)blockIdx.x - 1;
+  if (blk < p.ent.blocks) {
+    if (p.ent.f32)
+      ent_partial_block(static_cast<const float*>(p.ent.logits), p.ent.V, p.ent.row_stride, p.ent.slice, p.ent.n_split, p.ent.partial, blk);
+    else
+      ent_partial_block(static_cast<const __nv_bfloat16*>(p.ent.logits), p.ent.V, p.ent.row_stride, p.ent.slice, p.ent.n_split,
+                        p.ent.partial, blk);
+    return;
+  }
+  blk -= p.ent.blocks;
+  if (blk < p.map_blocks) {
+    row_map_warp(p.map, blk * 8ll + (threadIdx.x >> 5), lane);
+    return;
+  }
+  blk -= p.map_blocks;
   constexpr int kTokens = 8 / kPrepParts;           // of a block
   __shared__ float2 angle_s[kTokens][D / 2];        // (cos, sin)
   // (tokens and rows fit 32 bits: 2^31 of them would not fit the device's memory)
-  const int n_tok = p.B * p.nl * p.P * p.To, tok0 = (int)(blockIdx.x - 1) * kTokens;
+  const int n_tok = p.B * p.nl * p.P * p.To, tok0 = blk * kTokens;
   const int warp = threadIdx.x >> 5, slot = warp / kPrepParts, part = warp % kPrepParts;
   const int tok = tok0 + slot;
   const bool live = tok < n_tok;
@@ -337,48 +396,6 @@ __global__ void __launch_bounds__(256, 3) attn_prep_kernel(const PrepParams p) {
       }
       dst[0] = bf16x8_pack(xr);
       dst[HALF_V] = bf16x8_pack(yr);
-    }
-  }
-}
-
-// V-from-pool and fused variants, once per call: the pool token behind every context position of every query
-// (the gather's plan lookup, stored instead of applied) and, for keys stored rotated, the first position of its
-// shot.  Positions from L to the end of the last 128-token tile get -1; nothing beyond them is read.
-struct RowMapParams {
-  const long long* ctx_off;   // [B][k+1]
-  const int32_t* sel_idx;     // [B][k]
-  const long long* shot_off;  // [n_shots+1]
-  int* row_map;               // [B][ctx_cap]
-  int* off_map;               // [B][ctx_cap] or null
-  long long ctx_cap;
-  int B, k, n_shots;
-};
-
-// One warp per selected shot: its run of positions is written with whole lines (a search per position
-// took 38 us for 32 queries of 66 K positions and 8.3 us for 8 of 33 K; 3 us for those now).
-__global__ void __launch_bounds__(256) attn_row_map_kernel(const RowMapParams p) {
-  ads_dependency_wait();
-  const int lane = threadIdx.x & 31;
-  const long long w = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (w >= (long long)p.B * p.k) return;
-  const int b = (int)(w / p.k), r = (int)(w % p.k);
-  const long long* off = p.ctx_off + (long long)b * (p.k + 1);
-  const long long o0 = off[r], o1 = off[r + 1];
-  const int s = p.sel_idx[w];
-  int* rows = p.row_map + (long long)b * p.ctx_cap;
-  int* firsts = p.off_map == nullptr ? nullptr : p.off_map + (long long)b * p.ctx_cap;
-  const long long end = min(o1, p.ctx_cap);
-  const bool known = s >= 0 && s < p.n_shots;        // (an unknown shot is reported by the plan and has no positions)
-  const long long src = known ? p.shot_off[s] - o0 : 0;
-  for (long long pos = o0 + lane; pos < end; pos += 32) {
-    rows[pos] = known ? (int)(src + pos) : -1;
-    if (firsts != nullptr) firsts[pos] = (int)o0;
-  }
-  if (r == p.k - 1) {
-    const long long pad = min((o1 + kTileN - 1) / kTileN * kTileN, p.ctx_cap);
-    for (long long pos = o1 + lane; pos < pad; pos += 32) {
-      rows[pos] = -1;
-      if (firsts != nullptr) firsts[pos] = 0;
     }
   }
 }
@@ -1286,10 +1303,12 @@ struct CombineParams {
   __nv_bfloat16* out;   // [B][nl][P][Tq][Hq][D]
   float* lse;           // [B][nl][P][Hq][Tq] or null
   int Tq, Hq, G, n_mp;
+  int nx, ny, blocks;         // its grid: nx units, ny groups of rows, D / (16 kCombineSteps) column steps; in all
+  AdsEntropyJob ent;          // the entropy's second step: a block per group of rows behind them
 };
 
 constexpr int kCombineRows = 8;      // rows per warp
-constexpr int kCombineSteps = 2;     // 16-column steps per warp (blockIdx.z covers the others)
+constexpr int kCombineSteps = 2;     // 16-column steps per warp (other blocks cover the rest)
 
 // Block x merges the x-th of the units that a range boundary cut (listed by the schedule block, so that
 // nothing has to be searched for here).  Latency- and L2-bound: one query of one layer (26 MB of partials)
@@ -1298,14 +1317,21 @@ constexpr int kCombineSteps = 2;     // 16-column steps per warp (blockIdx.z cov
 // so that a load is 8 rows x 16 bytes contiguous per chunk in the partial layout ([D/4][128 rows][4] per
 // M tile) and a store fills one 32-byte sector per row.
 template <int D>
-__global__ void __launch_bounds__(256) attn_combine_kernel(const CombineParams p) {
+__global__ void __launch_bounds__(256) attn_combine_kernel(const __grid_constant__ CombineParams p) {
   ads_dependency_wait();
+  if ((int)blockIdx.x >= p.blocks) {
+    __shared__ float sh_h[kMaxProbes];               // (a group is a query's probes)
+    ent_finish_block(p.ent.partial, p.ent.n_split, p.ent.R, p.ent.rows_per_group, p.ent.tau, p.ent.H, p.ent.first_ok,
+                     (int)blockIdx.x - p.blocks, sh_h);
+    return;
+  }
+  const int bx = blockIdx.x % p.nx, byz = blockIdx.x / p.nx, by = byz % p.ny, bz = byz / p.ny;
   const Sched* sc = p.sched;
-  if (blockIdx.x >= sc->n_cut) return;
-  const Sched::Cut c = sc->cut[blockIdx.x];
+  if (bx >= sc->n_cut) return;
+  const Sched::Cut c = sc->cut[bx];
   const int lane = threadIdx.x & 31;
   const int r_sub = lane & 7, c_sub = lane >> 3;
-  const int m = (blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kCombineRows + r_sub;
+  const int m = (by * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kCombineRows + r_sub;
   if (m >= p.Tq * p.G) return;
   const int mt = m / kTileM, r = m % kTileM, mp = mt >> 1, x = mt & 1;
   const int t = m / p.G, hh = m % p.G, h = c.g * p.G + hh;
@@ -1314,7 +1340,7 @@ __global__ void __launch_bounds__(256) attn_combine_kernel(const CombineParams p
     return ((long long)(2 * (c.gang + i) + (i == 0 ? c.which : 0)) * p.n_mp + mp) * 2 + x;
   };
   const float4* o4 = reinterpret_cast<const float4*>(p.o_part);
-  const int it0 = blockIdx.z * kCombineSteps;
+  const int it0 = bz * kCombineSteps;
   float4 acc[kCombineSteps];
 #pragma unroll
   for (int it = 0; it < kCombineSteps; ++it) acc[it] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1360,7 +1386,7 @@ __global__ void __launch_bounds__(256) attn_combine_kernel(const CombineParams p
     packed.y = pack_bf16x2(acc[it].z * inv, acc[it].w * inv);
     *reinterpret_cast<uint2*>(dst + ((it0 + it) * 4 + c_sub) * 4) = packed;
   }
-  if (p.lse != nullptr && c_sub == 0 && blockIdx.z == 0)
+  if (p.lse != nullptr && c_sub == 0 && bz == 0)
     p.lse[(bpj * p.Hq + h) * p.Tq + t] = (M + log2f(lsum)) * kLn2;
 }
 
@@ -1404,10 +1430,11 @@ struct AttnPlan {
   size_t off_qrot, off_kqrot, off_sched, off_opart, off_ml, off_rowmap, off_offmap, total;
 };
 
-// Own tokens beyond the query rows, and a per-query shot count on the device (decode calls).
+// Own tokens beyond the query rows, and a per-query shot count on the device (decode calls); an entropy call to run beside.
 struct AttnExtra {
   int To = 0;                        // 0: as many own tokens as query rows
   const int32_t* nshots_dev = nullptr;
+  const AdsEntropyJob* ent = nullptr;      // the entropy of the probes' logits, beside the attention
 };
 
 // What the fused variant reads instead of an assembled cache.
@@ -1504,11 +1531,15 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
     }
   }
 
-  // ---- K or V from the pool: row map
+  // ---- rotate Q and the probe's own K, write the schedule and, for K or V from the pool, the row map
   int* row_map = reinterpret_cast<int*>(wsb + pl.off_rowmap);
   int* off_map = reinterpret_cast<int*>(wsb + pl.off_offmap);
+  PrepParams pp;
+  pp.ent = extra.ent != nullptr ? *extra.ent : AdsEntropyJob{};
+  pp.map = RowMapParams{};
+  pp.map_blocks = 0;
   if (fused != nullptr) {
-    RowMapParams rm;
+    RowMapParams& rm = pp.map;
     rm.ctx_off = reinterpret_cast<const long long*>(ctx_off);
     rm.sel_idx = fused->sel_idx;
     rm.shot_off = reinterpret_cast<const long long*>(fused->pool->shot_off);
@@ -1516,12 +1547,8 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
     rm.off_map = mode == kModeFused && model->k_pos_mode == 1 ? off_map : nullptr;
     rm.ctx_cap = ctx_cap;
     rm.B = B; rm.k = k; rm.n_shots = fused->pool->n_shots;
-    ads_launch_dependent(attn_row_map_kernel, (unsigned)(((long long)B * k + 7) / 8), 256, 0, st, rm);
-    if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
+    pp.map_blocks = (int)(((long long)B * k + 7) / 8);
   }
-
-  // ---- rotate Q and the probe's own K, write the schedule
-  PrepParams pp;
   pp.q = static_cast<const __nv_bfloat16*>(q); pp.kq = static_cast<const __nv_bfloat16*>(kq);
   pp.q_rot = q_rot; pp.kq_rot = kq_rot; pp.ctx_off = reinterpret_cast<const long long*>(ctx_off);
   pp.sched = sched; pp.ctx_cap = ctx_cap;
@@ -1530,7 +1557,7 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
   for (int i = 0; i < D / 2; ++i) pp.theta[i] = pow(model->rope_base, -2.0 * (double)i / (double)D);
   for (int i = 0; i < kMaxProbes; ++i) pp.nshots[i] = i < P ? probe_nshots[i] : 0;
   const long long n_tok = (long long)B * nl * P * To;
-  ads_launch_dependent(attn_prep_kernel<D>, (unsigned)((n_tok * kPrepParts + 7) / 8) + 1, 256, 0, st, pp);   // + the schedule block
+  ads_launch_dependent(attn_prep_kernel<D>, (unsigned)((n_tok * kPrepParts + 7) / 8) + 1 + pp.ent.blocks + pp.map_blocks, 256, 0, st, pp);
   if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
 
   // ---- main kernel
@@ -1577,10 +1604,12 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
   cp.Tq = Tq; cp.Hq = Hq; cp.G = G; cp.n_mp = pl.n_mp;
   // (at most one cut unit per range, and no more than there are units: a small call would launch mostly empty blocks)
   const long long units = (long long)B * P * nl * Hkv;
-  const dim3 grid((unsigned)(units < n_gangs ? units : n_gangs),
-                  (unsigned)((Tq * G + 8 * kCombineRows - 1) / (8 * kCombineRows)),
-                  D / (16 * kCombineSteps));
-  ads_launch_dependent(attn_combine_kernel<D>, grid, 256, 0, st, cp);
+  cp.nx = (int)(units < n_gangs ? units : n_gangs);
+  cp.ny = (Tq * G + 8 * kCombineRows - 1) / (8 * kCombineRows);
+  cp.blocks = cp.nx * cp.ny * (D / (16 * kCombineSteps));
+  cp.ent = pp.ent;
+  const int finish = cp.ent.blocks > 0 ? cp.ent.R / cp.ent.rows_per_group : 0;
+  ads_launch_dependent(attn_combine_kernel<D>, (unsigned)(cp.blocks + finish), 256, 0, st, cp);
   return ads_launch_status();
 }
 
@@ -1594,12 +1623,12 @@ extern "C" size_t adapshot_attn_workspace_bytes(const adapshot_model_t* model, i
   return make_plan(model, B, P, Tq, n_layers_in_call).total;
 }
 
-extern "C" int adapshot_query_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_ctx,
+int ads_query_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_ctx,
                                    int64_t ctx_cap, const int64_t* ctx_off, int32_t B, int32_t k,
                                    const int32_t* probe_nshots, int32_t P, const void* q, const void* kq,
                                    const void* vq, int32_t Tq, int32_t layer_begin, int32_t layer_end,
                                    void* out, float* lse, uint32_t flags, void* ws, size_t ws_bytes,
-                                   int32_t* status, void* stream) {
+                                   int32_t* status, void* stream, const AdsEntropyJob* ent) {
   if (model == nullptr || k_ctx == nullptr || v_ctx == nullptr || ctx_off == nullptr || probe_nshots == nullptr ||
       q == nullptr || kq == nullptr || vq == nullptr || out == nullptr || ws == nullptr)
     return ADAPSHOT_EINVAL;
@@ -1620,11 +1649,22 @@ extern "C" int adapshot_query_attn(const adapshot_model_t* model, const void* k_
   const AttnPlan pl = make_plan(model, B, P, Tq, nl);
   if (ws_bytes < pl.total) return ADAPSHOT_ECAPACITY;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  AttnExtra extra;
+  extra.ent = ent;
   if (model->head_dim == 128)
     return launch_attn<128>(model, k_ctx, v_ctx, ctx_cap, ctx_off, B, k, probe_nshots, P, q, kq, vq, Tq, nl, out,
-                            lse, pl, ws, status, st);
+                            lse, pl, ws, status, st, nullptr, kModeCache, extra);
   return launch_attn<64>(model, k_ctx, v_ctx, ctx_cap, ctx_off, B, k, probe_nshots, P, q, kq, vq, Tq, nl, out,
-                         lse, pl, ws, status, st);
+                         lse, pl, ws, status, st, nullptr, kModeCache, extra);
+}
+
+extern "C" int adapshot_query_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_ctx,
+                                   int64_t ctx_cap, const int64_t* ctx_off, int32_t B, int32_t k,
+                                   const int32_t* probe_nshots, int32_t P, const void* q, const void* kq,
+                                   const void* vq, int32_t Tq, int32_t layer_begin, int32_t layer_end,
+                                   void* out, float* lse, uint32_t flags, void* ws, size_t ws_bytes,
+                                   int32_t* status, void* stream) {
+  return ads_query_attn(model, k_ctx, v_ctx, ctx_cap, ctx_off, B, k, probe_nshots, P, q, kq, vq, Tq, layer_begin, layer_end, out, lse, flags, ws, ws_bytes, status, stream, nullptr);
 }
 
 extern "C" size_t adapshot_attn_fused_workspace_bytes(const adapshot_model_t* model, int32_t B, int32_t P,
@@ -1635,13 +1675,13 @@ extern "C" size_t adapshot_attn_fused_workspace_bytes(const adapshot_model_t* mo
   return make_plan(model, B, P, Tq, n_layers_in_call, ctx_cap).total;
 }
 
-extern "C" int adapshot_query_attn_fused(const adapshot_model_t* model, const adapshot_pool_t* pool,
+int ads_query_attn_fused(const adapshot_model_t* model, const adapshot_pool_t* pool,
                                          const int32_t* sel_idx, const int64_t* ctx_off, int64_t ctx_cap,
                                          int32_t B, int32_t k, const int32_t* probe_nshots, int32_t P,
                                          const void* q, const void* kq, const void* vq, int32_t Tq,
                                          int32_t layer_begin, int32_t layer_end, void* out, float* lse,
                                          uint32_t flags, void* ws, size_t ws_bytes, int32_t* status,
-                                         void* stream) {
+                                         void* stream, const AdsEntropyJob* ent) {
   if (model == nullptr || pool == nullptr || sel_idx == nullptr || ctx_off == nullptr || probe_nshots == nullptr ||
       q == nullptr || kq == nullptr || vq == nullptr || out == nullptr || ws == nullptr)
     return ADAPSHOT_EINVAL;
@@ -1666,13 +1706,25 @@ extern "C" int adapshot_query_attn_fused(const adapshot_model_t* model, const ad
   const AttnPlan pl = make_plan(model, B, P, Tq, nl, ctx_cap);
   if (ws_bytes < pl.total) return ADAPSHOT_ECAPACITY;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  AttnExtra extra;
+  extra.ent = ent;
   FusedSrc src;
   src.pool = pool; src.sel_idx = sel_idx; src.layer_begin = layer_begin;
   if (model->head_dim == 128)
     return launch_attn<128>(model, nullptr, nullptr, ctx_cap, ctx_off, B, k, probe_nshots, P, q, kq, vq, Tq, nl,
-                            out, lse, pl, ws, status, st, &src, kModeFused);
+                            out, lse, pl, ws, status, st, &src, kModeFused, extra);
   return launch_attn<64>(model, nullptr, nullptr, ctx_cap, ctx_off, B, k, probe_nshots, P, q, kq, vq, Tq, nl, out,
-                         lse, pl, ws, status, st, &src, kModeFused);
+                         lse, pl, ws, status, st, &src, kModeFused, extra);
+}
+
+extern "C" int adapshot_query_attn_fused(const adapshot_model_t* model, const adapshot_pool_t* pool,
+                                         const int32_t* sel_idx, const int64_t* ctx_off, int64_t ctx_cap,
+                                         int32_t B, int32_t k, const int32_t* probe_nshots, int32_t P,
+                                         const void* q, const void* kq, const void* vq, int32_t Tq,
+                                         int32_t layer_begin, int32_t layer_end, void* out, float* lse,
+                                         uint32_t flags, void* ws, size_t ws_bytes, int32_t* status,
+                                         void* stream) {
+  return ads_query_attn_fused(model, pool, sel_idx, ctx_off, ctx_cap, B, k, probe_nshots, P, q, kq, vq, Tq, layer_begin, layer_end, out, lse, flags, ws, ws_bytes, status, stream, nullptr);
 }
 
 extern "C" size_t adapshot_attn_vpool_workspace_bytes(const adapshot_model_t* model, int32_t B, int32_t P,
@@ -1683,13 +1735,13 @@ extern "C" size_t adapshot_attn_vpool_workspace_bytes(const adapshot_model_t* mo
   return make_plan(model, B, P, Tq, n_layers_in_call, ctx_cap).total;
 }
 
-extern "C" int adapshot_query_attn_vpool(const adapshot_model_t* model, const adapshot_pool_t* pool,
+int ads_query_attn_vpool(const adapshot_model_t* model, const adapshot_pool_t* pool,
                                          const int32_t* sel_idx, const void* k_ctx, int64_t ctx_cap,
                                          const int64_t* ctx_off, int32_t B, int32_t k,
                                          const int32_t* probe_nshots, int32_t P, const void* q, const void* kq,
                                          const void* vq, int32_t Tq, int32_t layer_begin, int32_t layer_end,
                                          void* out, float* lse, uint32_t flags, void* ws, size_t ws_bytes,
-                                         int32_t* status, void* stream) {
+                                         int32_t* status, void* stream, const AdsEntropyJob* ent) {
   if (model == nullptr || pool == nullptr || sel_idx == nullptr || k_ctx == nullptr || ctx_off == nullptr ||
       probe_nshots == nullptr || q == nullptr || kq == nullptr || vq == nullptr || out == nullptr || ws == nullptr)
     return ADAPSHOT_EINVAL;
@@ -1712,13 +1764,25 @@ extern "C" int adapshot_query_attn_vpool(const adapshot_model_t* model, const ad
   const AttnPlan pl = make_plan(model, B, P, Tq, nl, ctx_cap);
   if (ws_bytes < pl.total) return ADAPSHOT_ECAPACITY;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  AttnExtra extra;
+  extra.ent = ent;
   FusedSrc src;
   src.pool = pool; src.sel_idx = sel_idx; src.layer_begin = layer_begin;
   if (model->head_dim == 128)
     return launch_attn<128>(model, k_ctx, nullptr, ctx_cap, ctx_off, B, k, probe_nshots, P, q, kq, vq, Tq, nl, out,
-                            lse, pl, ws, status, st, &src, kModeVPool);
+                            lse, pl, ws, status, st, &src, kModeVPool, extra);
   return launch_attn<64>(model, k_ctx, nullptr, ctx_cap, ctx_off, B, k, probe_nshots, P, q, kq, vq, Tq, nl, out, lse,
-                         pl, ws, status, st, &src, kModeVPool);
+                         pl, ws, status, st, &src, kModeVPool, extra);
+}
+
+extern "C" int adapshot_query_attn_vpool(const adapshot_model_t* model, const adapshot_pool_t* pool,
+                                         const int32_t* sel_idx, const void* k_ctx, int64_t ctx_cap,
+                                         const int64_t* ctx_off, int32_t B, int32_t k,
+                                         const int32_t* probe_nshots, int32_t P, const void* q, const void* kq,
+                                         const void* vq, int32_t Tq, int32_t layer_begin, int32_t layer_end,
+                                         void* out, float* lse, uint32_t flags, void* ws, size_t ws_bytes,
+                                         int32_t* status, void* stream) {
+  return ads_query_attn_vpool(model, pool, sel_idx, k_ctx, ctx_cap, ctx_off, B, k, probe_nshots, P, q, kq, vq, Tq, layer_begin, layer_end, out, lse, flags, ws, ws_bytes, status, stream, nullptr);
 }
 
 // ---------------------------------------------------------------- literal tree layout

@@ -106,6 +106,36 @@ __device__ __forceinline__ double ads_key_score(unsigned long long k) {
 int ads_topk_from_keys(const unsigned long long* keys, int N, int B, int k, int32_t* sel_idx, float* sel_score,
                        cudaStream_t st);
 
+// One entropy call, checked and cut into blocks (entropy.cu): what a kernel needs that runs it beside its own work.
+struct AdsEntropyJob {
+  const void* logits;
+  float* partial;              // [blocks][3]
+  float* H;
+  int32_t* first_ok;
+  long long row_stride;
+  int f32, R, V, slice, n_split, rows_per_group;
+  float tau;
+  int blocks;                  // R * n_split; 0: no job
+};
+int ads_entropy_job(const void* logits, int32_t dtype, int32_t R, int32_t V, int64_t row_stride, float* H, float tau,
+                    int32_t rows_per_group, int32_t* first_ok, void* ws, size_t ws_bytes, AdsEntropyJob* job);
+
+// The three attention calls (attn.cu), with the entropy of the same probes' logits beside them when `ent` is given.
+int ads_query_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_ctx, int64_t ctx_cap,
+                   const int64_t* ctx_off, int32_t B, int32_t k, const int32_t* probe_nshots, int32_t P, const void* q,
+                   const void* kq, const void* vq, int32_t Tq, int32_t layer_begin, int32_t layer_end, void* out, float* lse,
+                   uint32_t flags, void* ws, size_t ws_bytes, int32_t* status, void* stream, const AdsEntropyJob* ent);
+int ads_query_attn_fused(const adapshot_model_t* model, const adapshot_pool_t* pool, const int32_t* sel_idx,
+                         const int64_t* ctx_off, int64_t ctx_cap, int32_t B, int32_t k, const int32_t* probe_nshots,
+                         int32_t P, const void* q, const void* kq, const void* vq, int32_t Tq, int32_t layer_begin,
+                         int32_t layer_end, void* out, float* lse, uint32_t flags, void* ws, size_t ws_bytes,
+                         int32_t* status, void* stream, const AdsEntropyJob* ent);
+int ads_query_attn_vpool(const adapshot_model_t* model, const adapshot_pool_t* pool, const int32_t* sel_idx,
+                         const void* k_ctx, int64_t ctx_cap, const int64_t* ctx_off, int32_t B, int32_t k,
+                         const int32_t* probe_nshots, int32_t P, const void* q, const void* kq, const void* vq, int32_t Tq,
+                         int32_t layer_begin, int32_t layer_end, void* out, float* lse, uint32_t flags, void* ws,
+                         size_t ws_bytes, int32_t* status, void* stream, const AdsEntropyJob* ent);
+
 // Decoding with few rows per KV head (decode.cu): whether a call's rows fit, whether it pays, its scratch, and the call itself
 // (arguments checked by the caller).
 bool ads_decode_rows_fit(const adapshot_model_t* model, int T_new);

@@ -99,6 +99,39 @@ def test_fewer_and_shorter_queries_than_planned(variant, overlap):
     assert torch.equal(H[:want_H.numel()], want_H) and torch.equal(ok[:2], want_ok)
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("vocab", [7, 1000, 20003])          # less than a vector, one slice per row, several with a ragged tail
+@pytest.mark.parametrize("variant", VARIANTS)
+def test_entropy_beside_the_attention_equals_its_own_call(variant, vocab, dtype):
+    # own workspaces: beside the attention; one workspace for every step: after it, as calls in turn would have it
+    w = _workload(47).scaled(vocab=vocab, t_q=70)
+    path, steps = _path(w, variant), _path(w, variant)
+    args = list(_inputs(path, wl.make_queries(w)))
+    stride = -(-vocab // 8) * 8
+    args[4] = torch.nn.functional.pad(args[4].to(dtype), (0, stride - vocab))[:, :vocab]
+    tau = 0.9 * torch.log(torch.tensor(float(vocab))).item()
+    steps.select(args[0])
+    if variant == "fused":
+        steps.plan()
+    for i, (lb, le) in enumerate(steps.chunks):
+        if variant == "fused":
+            steps.attend_fused(args[1][i], args[2][i], args[3][i], steps.out[i], lb, le)
+        else:
+            steps.assemble(lb, le, keep_plan=i > 0)
+            steps.attend(args[1][i], args[2][i], args[3][i], steps.out[i], lb, le)
+    steps.entropy(args[4], tau)
+    for shared in (False, True):
+        if shared:
+            path.ws_entropy = path.ws_select = path.ws_attn
+        path.H.fill_(-1)
+        path.first_ok.fill_(-7)
+        out, H, ok = path.run(*args[:5], tau)
+        torch.cuda.synchronize()
+        assert path.status.item() == 0 and steps.status.item() == 0
+        assert torch.equal(H, steps.H) and torch.equal(ok, steps.first_ok)
+        assert all(torch.equal(a, b) for a, b in zip(out, steps.out))
+
+
 @pytest.mark.parametrize("batch", [1, 2])
 def test_rounds_of_probes_use_the_tensors_they_have_now(batch):
     from paper_2605_03644_b200 import binding as ab
