@@ -46,7 +46,8 @@ constexpr int kMaxGang = 8;          // CTAs that share one range of K/V tiles
 constexpr int kUnitCost = 4;          // fixed cost of starting a unit, in tiles (measured: about 10 k clocks)
 constexpr int kTileM = 128;          // query rows per M tile (TMEM lanes)
 constexpr int kTileN = 128;          // keys per tile
-constexpr int kAttnThreads = 384;    // warp 0 TMA, warp 1 MMA, warp 2 gathers V (V from the pool), softmax of M tile A on warps 4-7, B on 8-11
+constexpr int kAttnThreads = 384;    // warp 0 TMA and items, warp 1 MMA, warp 2 gathers V (V from the pool), softmax of M tile A on
+                                     // warps 4-7, B on 8-11
 constexpr int kFusedThreads = 512;   // fused variant: warps 2-3 gather V and K, softmax on warps 4-11, K rotated by warps 12-15
 constexpr int kModeCache = 0;        // K and V tiles by TMA from the assembled cache
 constexpr int kModeFused = 1;        // K and V tiles from the pool, K re-encoded in shared memory
@@ -99,6 +100,7 @@ struct AttnParams {
   int To;                     // own tokens per probe (>= Tq): the Tq rows are the last Tq of them
   int n_mt, n_mp, gang, n_gangs;
   float scale_log2;           // softmax_scale * log2(e)
+  unsigned long long g_magic; // ceil(2^32 / G)
   // K or V from the pool
   const int* row_map;            // [B][ctx_cap]: pool token of every context position, -1 beyond L
   const int* off_map;            // [B][ctx_cap]: first position of the shot a position lies in (k_pos_mode 1)
@@ -404,8 +406,10 @@ __global__ void __launch_bounds__(256, 3) attn_prep_kernel(const __grid_constant
 // written by TMA with the 128-byte swizzle; D = 128 needs two of them per tile.
 // The fused variant has a third K stage (one tile landing, one being rotated, one in use) in the place of
 // the read-out staging.
-__host__ __device__ constexpr int sched_cache_pairs(int mode) { return mode == kModeFused ? 16 : 40; }
-__host__ __device__ constexpr uint32_t sched_cache_bytes(int mode) { return mode == kModeFused ? 512 : 1024; }
+constexpr int kCachePairs = 12;
+constexpr uint32_t kCacheBytes = 320;
+constexpr uint32_t kBarBytes = 384;                  // barriers, TMEM slot, abort flags
+constexpr int kItems = 4;                            // items published ahead of the roles that work on them
 template <int D, int MODE>
 struct AttnSmem {
   static constexpr int kKStages = MODE == kModeFused ? 3 : 2;
@@ -417,7 +421,9 @@ struct AttnSmem {
   static constexpr uint32_t kOffV = kOffK + kKStages * kTileBytes;
   static constexpr uint32_t kOffStage = kOffV + kVStages * kTileBytes;    // read-out staging of the 8 softmax warps
   static constexpr uint32_t kOffBar = kOffStage + 8 * kStageBytes;
-  static constexpr uint32_t kOffRows = kOffBar + 256 + sched_cache_bytes(MODE);   // pool rows of a tile, per gather warp
+  static constexpr uint32_t kOffItems = kOffBar + kBarBytes;
+  static constexpr uint32_t kOffCache = kOffItems + kItems * 64;
+  static constexpr uint32_t kOffRows = kOffCache + kCacheBytes;                   // pool rows of a tile, per gather warp
   static constexpr uint32_t kTotal = kOffRows + (MODE == kModeVPool ? 512 : MODE == kModeFused ? 1024 : 0) + 1024;   // + alignment slack
 };
 
@@ -426,8 +432,10 @@ enum Bar {
   kBarQFull = 0, kBarQEmpty = 2, kBarKFull = 4, kBarKEmpty = 7, kBarVFull = 10, kBarVEmpty = 13,
   kBarSFull = 16, kBarPFull = 18, kBarOFull = 20, kBarOEmpty = 22, kBarDrain = 24,
   kBarKRot = 25,                 // fused variant: K tile rotated
-  kNumBars = 28
+  kBarItemFull = 28, kBarItemEmpty = 28 + kItems,
+  kNumBars = 28 + 2 * kItems
 };
+static_assert(8 * kNumBars + 16 <= kBarBytes, "room of the barriers");
 
 // A piece = the part of one unit (pair, layer, kv head) that falls into a gang's range.
 struct Piece {
@@ -444,7 +452,6 @@ struct Walker {
 // The part of the schedule a CTA walks, copied to shared memory once: the pairs from the
 // one its range starts in.  Pairs beyond the copy (a range that spans more than
 // kCachePairs pairs) are read from the workspace.
-template <int kCachePairs>
 struct SchedCache {
   long long prefix[kCachePairs + 1];
   long long Lj[kCachePairs];
@@ -453,14 +460,12 @@ struct SchedCache {
   long long begin, end;
   int p0, n;
 };
-static_assert(sizeof(SchedCache<sched_cache_pairs(kModeCache)>) <= sched_cache_bytes(kModeCache) &&
-              sizeof(SchedCache<sched_cache_pairs(kModeFused)>) <= sched_cache_bytes(kModeFused), "room of the schedule cache");
+static_assert(sizeof(SchedCache) <= kCacheBytes, "room of the schedule cache");
 struct PairInfo {
   long long prefix, next_prefix, Lj;
   int n_ctx, n_su;
 };
-template <typename Cache>
-__device__ __forceinline__ PairInfo pair_info(const Sched* sc, const Cache* c, int pair) {
+__device__ __forceinline__ PairInfo pair_info(const Sched* sc, const SchedCache* c, int pair) {
   PairInfo pi;
   const int k = pair - c->p0;
   if (k >= 0 && k < c->n) {
@@ -473,8 +478,7 @@ __device__ __forceinline__ PairInfo pair_info(const Sched* sc, const Cache* c, i
   return pi;
 }
 
-template <typename Cache>
-__device__ __forceinline__ bool next_piece(const Sched* sc, const Cache* cache, int n_pairs, Walker& wk,
+__device__ __forceinline__ bool next_piece(const Sched* sc, const SchedCache* cache, int n_pairs, Walker& wk,
                                            Piece& pc) {
   if (wk.x >= wk.end) return false;
   PairInfo pi = pair_info(sc, cache, wk.pair);
@@ -483,8 +487,9 @@ __device__ __forceinline__ bool next_piece(const Sched* sc, const Cache* cache, 
   const int nsu = pi.n_su;
   const long long rel = wk.x - pi.prefix;
   pc.pair = lo;
-  pc.su = (int)(rel / nsu);
-  pc.t0 = (int)(rel % nsu);
+  // (a 32-bit division where the position allows it: the 64-bit one is some hundred dependent instructions)
+  pc.su = (rel >> 32) == 0 ? (int)((uint32_t)rel / (uint32_t)nsu) : (int)(rel / nsu);
+  pc.t0 = (int)(rel - (long long)pc.su * nsu);
   const long long room = wk.end - wk.x;
   pc.t1 = (int)(room < (long long)(nsu - pc.t0) ? pc.t0 + room : nsu);
   pc.n_su = nsu;
@@ -495,25 +500,30 @@ __device__ __forceinline__ bool next_piece(const Sched* sc, const Cache* cache, 
   return true;
 }
 
-// One M pair of one piece: what a CTA works on between two read-outs of O.
-struct Item {
-  int b, l, j, g, mp;
-  bool has_b, whole;
-  int ctx_begin, n_ctx, own_begin, n_own, n_tiles;
-  long long Lj;
+// One M pair of one piece: what a CTA works on between two read-outs of O.  One thread walks the schedule and publishes the
+// items in shared memory, a few ahead: each of ten roles walking it by itself paid 3000 clocks of dependent divisions between
+// two items, and the issuing thread's and the softmax warps' were in the chain (four probes of 4 to 16 shots, 16 layers: 603 -> 582 us
+// with the rounds' other kernels, no cache 343 -> 308; seven probes of 32 queries 6240 -> 6150).
+struct __align__(64) Item {
+  int n_tiles;                   // -1: no more items
+  int n_ctx, ctx_begin, own_begin;
+  int b, l, g, mp;
+  int flags;                     // 1: there is an M tile B; 2: the piece covers its unit
   int outer_ctx, outer_own, outer_q;
-  long long slot;
+  int Lj, slot;
+  __device__ bool has_b() const { return (flags & 1) != 0; }
+  __device__ bool whole() const { return (flags & 2) != 0; }
 };
+static_assert(sizeof(Item) == 64, "room of an item");
 
 __device__ __forceinline__ void make_item(const AttnParams& p, const Piece& pc, int gang_id, int mp, Item& w) {
-  w.j = p.P - 1 - pc.pair / p.B;
+  const int j = p.P - 1 - pc.pair / p.B;
   w.b = pc.pair % p.B;
   w.l = pc.su / p.Hkv;
-  w.g = pc.su % p.Hkv;
+  w.g = pc.su - w.l * p.Hkv;
   w.mp = mp;
-  w.has_b = 2 * mp + 1 < p.n_mt;
-  w.whole = pc.t0 == 0 && pc.t1 == pc.n_su;
-  w.Lj = pc.Lj;
+  w.flags = (2 * mp + 1 < p.n_mt ? 1 : 0) | (pc.t0 == 0 && pc.t1 == pc.n_su ? 2 : 0);
+  w.Lj = (int)pc.Lj;
   const int ctx_end = min(pc.t1, pc.n_ctx);
   w.ctx_begin = pc.t0;
   w.n_ctx = max(0, ctx_end - pc.t0);
@@ -522,12 +532,19 @@ __device__ __forceinline__ void make_item(const AttnParams& p, const Piece& pc, 
   const int own_need = (p.To - p.Tq + row_hi / p.G) / kTileN + 1;
   w.own_begin = max(pc.t0, pc.n_ctx) - pc.n_ctx;
   const int own_end = min(pc.t1 - pc.n_ctx, own_need);
-  w.n_own = max(0, own_end - w.own_begin);
-  w.n_tiles = w.n_ctx + w.n_own;
+  const int n_own = max(0, own_end - w.own_begin);
+  w.n_tiles = w.n_ctx + n_own;
   w.outer_ctx = w.b * p.nl + w.l;
-  w.outer_own = w.outer_ctx * p.P + w.j;
+  w.outer_own = w.outer_ctx * p.P + j;
   w.outer_q = w.outer_own * p.Hkv + w.g;
-  w.slot = ((long long)(2 * gang_id + (pc.first_of_gang ? 0 : 1)) * p.n_mp + mp);
+  w.slot = (2 * gang_id + (pc.first_of_gang ? 0 : 1)) * p.n_mp + mp;
+}
+
+// m / G for 0 <= m < 2^32 with g_magic = ceil(2^32 / G)
+__device__ __forceinline__ int div_g(const AttnParams& p, int m) {
+  uint32_t q = (uint32_t)(((unsigned long long)(uint32_t)m * p.g_magic) >> 32);     // at most one too large
+  if (q * (uint32_t)p.G > (uint32_t)m) --q;
+  return (int)q;
 }
 
 // Maps over the pool's V (or K) with boxes of 1, 2, 4, ..., 128 rows, from which a tile is stitched run by
@@ -557,6 +574,7 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   constexpr uint32_t kTmemS = 0, kTmemO = 256;
   constexpr int kSoftmaxWarp0 = 4;          // first of the eight softmax warps
   constexpr int kGatherWarp = 2;   // the warp that gathers the V tiles (fused: K by the next one)
+  constexpr int kItemReaders = 8 + (FUSED ? 3 + kRotateWarps : VPOOL ? 2 : 1);     // every role's warps but the TMA thread's
   constexpr int kBarKReady = FUSED ? kBarKRot : kBarKFull;
 
   extern __shared__ unsigned char smem_raw[];
@@ -578,10 +596,11 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       mbar_init(bar(kBarQFull + i), 1);
       mbar_init(bar(kBarQEmpty + i), 1);
       mbar_init(bar(kBarSFull + i), 1);
-      mbar_init(bar(kBarPFull + i), 128);
+      mbar_init(bar(kBarPFull + i), 4);
       mbar_init(bar(kBarOFull + i), 1);
-      mbar_init(bar(kBarOEmpty + i), 128);
+      mbar_init(bar(kBarOEmpty + i), 4);
     }
+    mbar_init(bar(kBarDrain), 1);
     for (int i = 0; i < 3; ++i) {
       mbar_init(bar(kBarKFull + i), 1);
       mbar_init(bar(kBarKEmpty + i), 1);
@@ -589,7 +608,10 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       mbar_init(bar(kBarKRot + i), kRotateWarps);
       mbar_init(bar(kBarVEmpty + i), 1);
     }
-    mbar_init(bar(kBarDrain), 1);
+    for (int i = 0; i < kItems; ++i) {
+      mbar_init(bar(kBarItemFull + i), 1);
+      mbar_init(bar(kBarItemEmpty + i), kItemReaders);
+    }
     abort_flag[0] = 0;
     abort_flag[1] = 0;
     mbar_fence_init();
@@ -599,9 +621,8 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     tmem_relinquish();
   }
   ads_dependency_wait();
-  // the CTA's part of the schedule, fetched by two otherwise idle warps while the rest is set up
-  constexpr int kCachePairs = sched_cache_pairs(MODE);
-  SchedCache<kCachePairs>* cache = reinterpret_cast<SchedCache<kCachePairs>*>(base_ptr + SM::kOffBar + 256);
+  // the CTA's part of the schedule, fetched by two warps while the rest is set up
+  SchedCache* cache = reinterpret_cast<SchedCache*>(base_ptr + SM::kOffCache);
   if (warp >= 2 && warp < 4) {
     const int p0 = sc->first_pair[gang_id];
     const int n = min(kCachePairs, n_pairs - p0);
@@ -625,63 +646,91 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  Walker wk0;
-  wk0.begin = cache->begin;
-  wk0.end = cache->end;
-  wk0.x = wk0.begin;
-  wk0.pair = cache->p0;
+  // ---- items: published by the TMA thread, read by a warp (or one thread of it) at a time
+  Item* items = reinterpret_cast<Item*>(base_ptr + SM::kOffItems);
+  // The n-th item; false at the end, or when the wait was given up (ok).  whole_warp: every lane calls and gets the item.
+  auto read_item = [&](uint32_t n, Item& w, bool& ok, bool whole_warp) -> bool {
+    const uint32_t slot = n % kItems;
+    ok = mbar_wait(bar(kBarItemFull + slot), (n / kItems) & 1, abort_flag);
+    if (whole_warp) ok = __all_sync(0xffffffffu, ok);
+    if (!ok) return false;
+    w = items[slot];
+    if (whole_warp) __syncwarp();
+    if (!whole_warp || lane == 0) mbar_arrive(bar(kBarItemEmpty + slot));
+    return w.n_tiles >= 0;
+  };
 
   auto role_tma = [&]() {
-    // ------------------------------------------------------------ TMA producer
+    // ------------------------------------------- TMA producer, and the walk through the schedule
     if (lane == 0) {
+      Walker wk;
+      wk.x = wk.begin = cache->begin;
+      wk.end = cache->end;
+      wk.pair = cache->p0;
+      Piece pc;
+      int mp = p.n_mp;                     // M pair of the next item; n_mp: the next piece's first
+      uint32_t n_pub = 0;
+      auto publish = [&](Item& w) -> bool {
+        const uint32_t slot = n_pub % kItems;
+        w.n_tiles = -1;
+        if (mp >= p.n_mp && next_piece(sc, cache, n_pairs, wk, pc)) mp = rank;
+        if (mp < p.n_mp) {
+          make_item(p, pc, gang_id, mp, w);
+          mp += p.gang;
+        }
+        if (!mbar_wait(bar(kBarItemEmpty + slot), ((n_pub / kItems) & 1) ^ 1, abort_flag)) return false;
+        items[slot] = w;
+        mbar_arrive(bar(kBarItemFull + slot));
+        ++n_pub;
+        return true;
+      };
       tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_kctx); tma_prefetch_desc(&tm_vctx);
       uint32_t tk = 0, tv = 0, nq[2] = {0, 0};
-      bool ok = true;
-      Walker wk = wk0;
-      Piece pc;
-      while (ok && next_piece(sc, cache, n_pairs, wk, pc)) {
-        for (int mp = rank; mp < p.n_mp && ok; mp += p.gang) {
-          Item w;
-          make_item(p, pc, gang_id, mp, w);
-          if (w.n_tiles == 0) continue;
-          for (int x = 0; x < (w.has_b ? 2 : 1) && ok; ++x) {
-            ok = mbar_wait(bar(kBarQEmpty + x), (nq[x] & 1) ^ 1, abort_flag);
-            if (!ok) break;
-            mbar_arrive_expect_tx(bar(kBarQFull + x), kTileBytes);
+      Item w, next;
+      bool ok = publish(w);
+      while (ok && w.n_tiles >= 0) {
+        for (int x = 0; x < (w.has_b() ? 2 : 1) && ok && w.n_tiles > 0; ++x) {
+          ok = mbar_wait(bar(kBarQEmpty + x), (nq[x] & 1) ^ 1, abort_flag);
+          if (!ok) break;
+          mbar_arrive_expect_tx(bar(kBarQFull + x), kTileBytes);
 #pragma unroll
-            for (int s = 0; s < SUB; ++s)
-              tma_load_3d(base + SM::kOffQ + x * kTileBytes + s * 16384u, &tm_q, bar(kBarQFull + x), s * 64,
-                          (2 * mp + x) * kTileM, w.outer_q);
-            ++nq[x];
-          }
-          for (int i = 0; i < (FUSED ? 0 : w.n_tiles) && ok; ++i) {
-            const bool own = i >= w.n_ctx;
-            const CUtensorMap* mk = own ? &tm_kown : &tm_kctx;
-            const CUtensorMap* mv = own ? &tm_vown : &tm_vctx;
-            const int row = own ? (w.own_begin + i - w.n_ctx) * kTileN : (w.ctx_begin + i) * kTileN;
-            const int outer = own ? w.outer_own : w.outer_ctx;
-            const int sk = tk % KS;
-            ok = mbar_wait(bar(kBarKEmpty + sk), ((tk / KS) & 1) ^ 1, abort_flag);
-            if (!ok) break;
-            mbar_arrive_expect_tx(bar(kBarKFull + sk), kTileBytes);
-#pragma unroll
-            for (int s = 0; s < SUB; ++s)
-              tma_load_4d(base + SM::kOffK + sk * kTileBytes + s * 16384u, mk, bar(kBarKFull + sk), s * 64, w.g, row,
-                          outer);
-            ++tk;
-            if constexpr (!VPOOL) {
-              const int sv = tv % VS;
-              ok = mbar_wait(bar(kBarVEmpty + sv), ((tv / VS) & 1) ^ 1, abort_flag);
-              if (!ok) break;
-              mbar_arrive_expect_tx(bar(kBarVFull + sv), kTileBytes);
-#pragma unroll
-              for (int s = 0; s < SUB; ++s)
-                tma_load_4d(base + SM::kOffV + sv * kTileBytes + s * 16384u, mv, bar(kBarVFull + sv), s * 64, w.g,
-                            row, outer);
-              ++tv;
-            }
-          }
+          for (int s = 0; s < SUB; ++s)
+            tma_load_3d(base + SM::kOffQ + x * kTileBytes + s * 16384u, &tm_q, bar(kBarQFull + x), s * 64,
+                        (2 * w.mp + x) * kTileM, w.outer_q);
+          ++nq[x];
         }
+        // the next item is worked out while the first tiles of this one are on their way
+        const int n_load = FUSED ? 0 : w.n_tiles;
+        if (ok && n_load == 0) ok = publish(next);
+        for (int i = 0; i < n_load && ok; ++i) {
+          const bool own = i >= w.n_ctx;
+          const CUtensorMap* mk = own ? &tm_kown : &tm_kctx;
+          const CUtensorMap* mv = own ? &tm_vown : &tm_vctx;
+          const int row = own ? (w.own_begin + i - w.n_ctx) * kTileN : (w.ctx_begin + i) * kTileN;
+          const int outer = own ? w.outer_own : w.outer_ctx;
+          const int sk = tk % KS;
+          ok = mbar_wait(bar(kBarKEmpty + sk), ((tk / KS) & 1) ^ 1, abort_flag);
+          if (!ok) break;
+          mbar_arrive_expect_tx(bar(kBarKFull + sk), kTileBytes);
+#pragma unroll
+          for (int s = 0; s < SUB; ++s)
+            tma_load_4d(base + SM::kOffK + sk * kTileBytes + s * 16384u, mk, bar(kBarKFull + sk), s * 64, w.g, row,
+                        outer);
+          ++tk;
+          if constexpr (!VPOOL) {
+            const int sv = tv % VS;
+            ok = mbar_wait(bar(kBarVEmpty + sv), ((tv / VS) & 1) ^ 1, abort_flag);
+            if (!ok) break;
+            mbar_arrive_expect_tx(bar(kBarVFull + sv), kTileBytes);
+#pragma unroll
+            for (int s = 0; s < SUB; ++s)
+              tma_load_4d(base + SM::kOffV + sv * kTileBytes + s * 16384u, mv, bar(kBarVFull + sv), s * 64, w.g,
+                          row, outer);
+            ++tv;
+          }
+          if (i == min(1, n_load - 1)) ok = publish(next);
+        }
+        w = next;
       }
       if (!ok && !FUSED) {
         // gave up: let the copies already in flight land before the CTA retires
@@ -698,41 +747,41 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     }
     __syncwarp();
   };
+  // Descriptors as a constant high half plus a low half = (address >> 4) with an immediate per k-step.
+  constexpr uint32_t kHi = smem_desc_hi_sw128(1024);
+  const uint32_t q_lo0 = smem_desc_lo(base + SM::kOffQ, 16);
+  const uint32_t k_lo0 = smem_desc_lo(base + SM::kOffK, 16);
+  const uint32_t v_lo0 = smem_desc_lo(base + SM::kOffV, 16384);
+  auto qk_step = [&](const int x, uint32_t k_lo, int ks) {
+    const uint32_t o = ((ks / 4) * 16384u + (ks % 4) * 32u) >> 4;
+    umma_ss_lohi(tmem_base + kTmemS + x * kTileN, q_lo0 + x * (kTileBytes >> 4) + o, kHi, k_lo + o, kHi, kIdescQK,
+                 ks > 0 ? 1u : 0u);
+  };
+  auto issue_pv = [&](const int x, uint32_t v_stage, bool first) {
+    const uint32_t v_lo = v_lo0 + v_stage * (kTileBytes >> 4);
+    const uint32_t d = tmem_base + kTmemO + x * 128;
+    const uint32_t a = tmem_base + kTmemS + x * kTileN;
+    // A = P from TMEM: 16 bf16 keys of one k-step occupy 8 packed columns
+    umma_ts_lohi(d, a, v_lo, kHi, kIdescPV, first ? 0u : 1u);
+#pragma unroll
+    for (int ks = 1; ks < kTileN / 16; ++ks)
+      umma_ts_lohi(d, a + ks * 8, v_lo + ((ks * 2048u) >> 4), kHi, kIdescPV, 1u);
+  };
   auto role_mma = [&]() {
     // -------------------------------------------------------------- MMA issuer
     if (lane == 0) {
-      // The tensor pipe takes only a few UMMAs ahead of the one it runs: whatever this thread
-      // does between two issues is time the pipe may idle, so the per-tile path is kept short
-      // (scalar counters, no indexed arrays, descriptors as a constant high half plus a low
-      // half = (address >> 4) with an immediate per k-step).
-      uint32_t tk = 0, tv = 0, np0 = 0, np1 = 0, ni0 = 0, ni1 = 0;
+      // The tensor pipe takes only a few UMMAs ahead of the one it runs: whatever this thread does between two issues is
+      // time the pipe may idle, so the per-tile path is kept short.  (A thread per M tile that takes turns with the other,
+      // so that each waits and commits under the other's UMMAs, is slower: one layer of one query 119.9 -> 126.9 us, eight
+      // queries of 33 K tokens, four layers, 2765 -> 2880.)
+      uint32_t tk = 0, tv = 0, np0 = 0, np1 = 0, ni0 = 0, ni1 = 0, n_item = 0;
       bool ok = true;
-      Walker wk = wk0;
-      Piece pc;
-      constexpr uint32_t kHi = smem_desc_hi_sw128(1024);
-      const uint32_t q_lo0 = smem_desc_lo(base + SM::kOffQ, 16);
-      const uint32_t k_lo0 = smem_desc_lo(base + SM::kOffK, 16);
-      const uint32_t v_lo0 = smem_desc_lo(base + SM::kOffV, 16384);
+      Item w;
       auto issue_qk = [&](const int x, uint32_t k_stage) {
-        const uint32_t q_lo = q_lo0 + x * (kTileBytes >> 4);
         const uint32_t k_lo = k_lo0 + k_stage * (kTileBytes >> 4);
-        const uint32_t d = tmem_base + kTmemS + x * kTileN;
 #pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-          const uint32_t o = ((ks / 4) * 16384u + (ks % 4) * 32u) >> 4;
-          umma_ss_lohi(d, q_lo + o, kHi, k_lo + o, kHi, kIdescQK, ks > 0 ? 1u : 0u);
-        }
+        for (int ks = 0; ks < D / 16; ++ks) qk_step(x, k_lo, ks);
         umma_commit(bar(kBarSFull + x));
-      };
-      auto issue_pv = [&](const int x, uint32_t v_stage, bool first) {
-        const uint32_t v_lo = v_lo0 + v_stage * (kTileBytes >> 4);
-        const uint32_t d = tmem_base + kTmemO + x * 128;
-        const uint32_t a = tmem_base + kTmemS + x * kTileN;
-        // A = P from TMEM: 16 bf16 keys of one k-step occupy 8 packed columns
-        umma_ts_lohi(d, a, v_lo, kHi, kIdescPV, first ? 0u : 1u);
-#pragma unroll
-        for (int ks = 1; ks < kTileN / 16; ++ks)
-          umma_ts_lohi(d, a + ks * 8, v_lo + ((ks * 2048u) >> 4), kHi, kIdescPV, 1u);
       };
       // one M tile's share of tile i: O += P V, then S of the next tile (in place of P: the
       // tensor pipe runs its operations in order)
@@ -752,43 +801,42 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         }
         return true;
       };
-      while (ok && next_piece(sc, cache, n_pairs, wk, pc)) {
-        for (int mp = rank; mp < p.n_mp && ok; mp += p.gang) {
-          Item w;
-          make_item(p, pc, gang_id, mp, w);
-          if (w.n_tiles == 0) continue;
-          // S of the first tile for both M tiles
-          ok = mbar_wait(bar(kBarQFull + 0), ni0 & 1, abort_flag);
-          if (ok && w.has_b) ok = mbar_wait(bar(kBarQFull + 1), ni1 & 1, abort_flag);
-          if (ok) ok = mbar_wait(bar(kBarKReady + tk % KS), (tk / KS) & 1, abort_flag);
-          if (!ok) break;
-          tc_fence_after();
-          issue_qk(0, tk % KS);
-          if (w.n_tiles == 1) umma_commit(bar(kBarQEmpty + 0));
-          if (w.has_b) {
-            issue_qk(1, tk % KS);
-            if (w.n_tiles == 1) umma_commit(bar(kBarQEmpty + 1));
-          }
-          umma_commit(bar(kBarKEmpty + tk % KS));
-          ++tk;
-          for (int i = 0; i < w.n_tiles && ok; ++i) {
-            const bool next = i + 1 < w.n_tiles;
-            const uint32_t k_stage = tk % KS, v_stage = tv % VS;
-            if (next) ok = mbar_wait(bar(kBarKReady + k_stage), (tk / KS) & 1, abort_flag);
-            if (ok) ok = mbar_wait(bar(kBarVFull + v_stage), (tv / VS) & 1, abort_flag);
-            if (ok) ok = chain(0, np0, ni0, i, w.n_tiles, k_stage, v_stage);
-            if (ok && w.has_b) ok = chain(1, np1, ni1, i, w.n_tiles, k_stage, v_stage);
-            if (!ok) break;
-            umma_commit(bar(kBarVEmpty + v_stage));
-            ++tv;
-            if (next) {
-              umma_commit(bar(kBarKEmpty + k_stage));
-              ++tk;
-            }
-          }
-          ++ni0;
-          if (w.has_b) ++ni1;
+      while (read_item(n_item, w, ok, false)) {
+        ++n_item;
+        if (w.n_tiles == 0) continue;
+        const bool has_b = w.has_b();
+        // S of the first tile for both M tiles
+        ok = mbar_wait(bar(kBarQFull + 0), ni0 & 1, abort_flag);
+        if (ok && has_b) ok = mbar_wait(bar(kBarQFull + 1), ni1 & 1, abort_flag);
+        if (ok) ok = mbar_wait(bar(kBarKReady + tk % KS), (tk / KS) & 1, abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+        issue_qk(0, tk % KS);
+        if (w.n_tiles == 1) umma_commit(bar(kBarQEmpty + 0));
+        if (has_b) {
+          issue_qk(1, tk % KS);
+          if (w.n_tiles == 1) umma_commit(bar(kBarQEmpty + 1));
         }
+        umma_commit(bar(kBarKEmpty + tk % KS));
+        ++tk;
+        for (int i = 0; i < w.n_tiles && ok; ++i) {
+          const bool next = i + 1 < w.n_tiles;
+          const uint32_t k_stage = tk % KS, v_stage = tv % VS;
+          if (next) ok = mbar_wait(bar(kBarKReady + k_stage), (tk / KS) & 1, abort_flag);
+          if (ok) ok = mbar_wait(bar(kBarVFull + v_stage), (tv / VS) & 1, abort_flag);
+          if (ok) ok = chain(0, np0, ni0, i, w.n_tiles, k_stage, v_stage);
+          if (ok && has_b) ok = chain(1, np1, ni1, i, w.n_tiles, k_stage, v_stage);
+          if (!ok) break;
+          umma_commit(bar(kBarVEmpty + v_stage));
+          ++tv;
+          if (next) {
+            umma_commit(bar(kBarKEmpty + k_stage));
+            ++tk;
+          }
+        }
+        if (!ok) break;
+        ++ni0;
+        if (has_b) ++ni1;
       }
       if (!ok) {
         umma_commit(bar(kBarDrain));
@@ -855,45 +903,40 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     };
     uint32_t tk = 0;
     bool ok = true;
-    Walker wk = wk0;
-    Piece pc;
-    while (ok && next_piece(sc, cache, n_pairs, wk, pc)) {
-      for (int mp = rank; mp < p.n_mp && ok; mp += p.gang) {
-        Item w;
-        make_item(p, pc, gang_id, mp, w);
-        const int* omap = p.off_map + (long long)w.b * p.ctx_cap;
-        auto first_of = [&](int i) -> int {           // first position of the shot that map_row of tile i lies in
-          const long long pos = (long long)(w.ctx_begin + i) * kTileN + map_row;
-          return per_shot && i < w.n_ctx && pos < p.ctx_cap ? omap[pos] : 0;
-        };
-        int first = first_of(0), first_cur = -1;
-        for (int i = 0; i < w.n_tiles; ++i, ++tk) {
-          const uint32_t sk = tk % KS;
-          unsigned char* kt = base_ptr + SM::kOffK + sk * kTileBytes;
-          const bool ctx = i < w.n_ctx;               // (the probe's own keys were rotated by the prep kernel)
-          const int first_next = first_of(i + 1);
-          if (ctx && !per_shot) set_angles((double)((long long)(w.ctx_begin + i) * kTileN + row0));
-          ok = __all_sync(0xffffffffu, mbar_wait(bar(kBarKFull + sk), (tk / KS) & 1, abort_flag));
-          if (!ok) break;
-          if (ctx && !per_shot) {
+    Item w;
+    for (uint32_t n_item = 0; ok && read_item(n_item, w, ok, true); ++n_item) {
+      const int* omap = p.off_map + (long long)w.b * p.ctx_cap;
+      auto first_of = [&](int i) -> int {           // first position of the shot that map_row of tile i lies in
+        const long long pos = (long long)(w.ctx_begin + i) * kTileN + map_row;
+        return per_shot && i < w.n_ctx && pos < p.ctx_cap ? omap[pos] : 0;
+      };
+      int first = first_of(0), first_cur = -1;
+      for (int i = 0; i < w.n_tiles; ++i, ++tk) {
+        const uint32_t sk = tk % KS;
+        unsigned char* kt = base_ptr + SM::kOffK + sk * kTileBytes;
+        const bool ctx = i < w.n_ctx;               // (the probe's own keys were rotated by the prep kernel)
+        const int first_next = first_of(i + 1);
+        if (ctx && !per_shot) set_angles((double)((long long)(w.ctx_begin + i) * kTileN + row0));
+        ok = __all_sync(0xffffffffu, mbar_wait(bar(kBarKFull + sk), (tk / KS) & 1, abort_flag));
+        if (!ok) break;
+        if (ctx && !per_shot) {
 #pragma unroll
-            for (int u = 0; u < kUnits; ++u) rotate_unit(kt, u, u + 1 < kUnits);
-          } else if (ctx) {
+          for (int u = 0; u < kUnits; ++u) rotate_unit(kt, u, u + 1 < kUnits);
+        } else if (ctx) {
 #pragma unroll 2
-            for (int u = 0; u < kUnits; ++u) {
-              const int o = __shfl_sync(0xffffffffu, first, u * RPW + lane / PPR);
-              if (o != first_cur) {
-                set_angles((double)o);
-                first_cur = o;
-              }
-              rotate_unit(kt, u, false);
+          for (int u = 0; u < kUnits; ++u) {
+            const int o = __shfl_sync(0xffffffffu, first, u * RPW + lane / PPR);
+            if (o != first_cur) {
+              set_angles((double)o);
+              first_cur = o;
             }
+            rotate_unit(kt, u, false);
           }
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar(kBarKRot + sk));
-          first = first_next;
         }
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(kBarKRot + sk));
+        first = first_next;
       }
     }
   };
@@ -917,142 +960,137 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     uint32_t sv = 0, phase = 0;                  // stage and parity of tile tv
     uint32_t tv = 0;
     bool ok = true;
-    Walker wk = wk0;
-    Piece pc;
+    Item w;
     if (lane == 0) {
       tma_prefetch_desc(own_map);
 #pragma unroll
       for (int e = 0; e < 8; ++e) tma_prefetch_desc(&maps->m[e]);
     }
-    while (ok && next_piece(sc, cache, n_pairs, wk, pc)) {
-      for (int mp = rank; mp < p.n_mp && ok; mp += p.gang) {
-        Item w;
-        make_item(p, pc, gang_id, mp, w);
-        for (int i = 0; i < w.n_tiles; ++i, ++tv, phase ^= (sv + 1 == n_st), sv = sv + 1 == n_st ? 0 : sv + 1) {
-          const uint32_t v_dst = tiles0 + sv * kTileBytes;
-          const uint32_t full = full0 + 8u * sv;
-          if (i >= w.n_ctx) {
-            // own tokens: one tiled box (rows beyond the last own token arrive as zeros)
-            if (lane == 0) {
-              ok = mbar_wait(empty0 + 8u * sv, phase ^ 1, abort_flag);
-              if (ok) {
-                mbar_arrive_expect_tx(full, kTileBytes);
-#pragma unroll
-                for (int s2 = 0; s2 < SUB; ++s2)
-                  tma_load_4d(v_dst + s2 * 16384u, own_map, full, s2 * 64, w.g,
-                              (w.own_begin + i - w.n_ctx) * kTileN, w.outer_own);
-              }
-            }
-            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-            if (!ok) break;
-            continue;
-          }
-          // pool row of positions lane, lane + 32, lane + 64, lane + 96 of the tile (looked up while the
-          // stage may still be in use)
-          const long long pos0 = (long long)(w.ctx_begin + i) * kTileN;
-          const long long L_all = p.ctx_cap;            // (row map entries beyond a query's context are -1)
-          int r[4];
-#pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4) {
-            const long long pos = pos0 + lane + 32 * q4;
-            r[q4] = pos < L_all ? p.row_map[(long long)w.b * p.ctx_cap + pos] : -1;
-          }
-          // the number of valid positions of the tile: they form a prefix (valid positions are 0 .. L-1)
-          unsigned valid_mask[4];
-#pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4) valid_mask[q4] = __ballot_sync(0xffffffffu, r[q4] >= 0);
-          const int n_valid = __popc(valid_mask[0]) + __popc(valid_mask[1]) + __popc(valid_mask[2]) + __popc(valid_mask[3]);
-#pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4) {
-            const int pidx = lane + 32 * q4;
-            if (pidx >= n_valid) r[q4] = pidx - 2 * kTileN;       // one run of rows in front of the pool: zeros
-          }
-          __syncwarp();
-#pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4) rows_s[lane + 32 * q4] = r[q4];
-          // a run ends after position pidx when the next position is not the next pool row
-          unsigned brk[4];
-#pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4) {
-            int nxt = __shfl_down_sync(0xffffffffu, r[q4], 1);
-            const int wrap = __shfl_sync(0xffffffffu, q4 < 3 ? r[q4 + 1 < 4 ? q4 + 1 : 3] : 0, 0);
-            if (lane == 31) nxt = wrap;
-            const bool last = lane == 31 && q4 == 3;
-            brk[q4] = __ballot_sync(0xffffffffu, last || nxt != r[q4] + 1);
-          }
-          // the run ends as one 128-bit mask in every lane; lane j then finds the j-th box on its own.
-          // A run of n rows takes the largest power-of-two box that fits, once from its first row and,
-          // unless n is that power of two, once more ending at its last row: the two overlap, both write
-          // the same values there, and no run needs more than two copy instructions (the copy engine's
-          // time goes with the number of instructions, not with the bytes)
-          __syncwarp();
-          int my_pidx = -1, my_row = 0, my_lg = 0, n_boxes = 0;
-          uint32_t tile_bytes = 0;                 // what the boxes deliver in all (overlaps are copied twice)
-          {
-            int pidx = 0;
-            while (pidx < kTileN) {
-              int e = pidx;                       // end of the run that starts at pidx: first set bit at or after it
-              for (;;) {
-                const unsigned word = (e < 32 ? brk[0] : e < 64 ? brk[1] : e < 96 ? brk[2] : brk[3]) >> (e & 31);
-                if (word != 0) { e += __ffs(word) - 1; break; }
-                e = (e | 31) + 1;
-              }
-              const int n = e - pidx + 1;
-              const int lg = 31 - __clz(n);        // the largest power-of-two box that fits
-              if (n_boxes == lane) { my_pidx = pidx; my_lg = lg; }
-              ++n_boxes;
-              if (n > (1 << lg)) {                 // the rest of the run: the same box once more, ending at the run's end
-                if (n_boxes == lane) { my_pidx = e + 1 - (1 << lg); my_lg = lg; }
-                ++n_boxes;
-              }
-              tile_bytes += (n > (1 << lg) ? 2u : 1u) * ((uint32_t)SUB << (lg + 7));
-              pidx = e + 1;
-            }
-          }
-          if (my_pidx >= 0) my_row = rows_s[my_pidx];
-          // (tiles of more than 32 boxes - many one-token shots - take further rounds of the same walk)
+    for (uint32_t n_item = 0; ok && read_item(n_item, w, ok, true); ++n_item) {
+      for (int i = 0; i < w.n_tiles; ++i, ++tv, phase ^= (sv + 1 == n_st), sv = sv + 1 == n_st ? 0 : sv + 1) {
+        const uint32_t v_dst = tiles0 + sv * kTileBytes;
+        const uint32_t full = full0 + 8u * sv;
+        if (i >= w.n_ctx) {
+          // own tokens: one tiled box (rows beyond the last own token arrive as zeros)
           if (lane == 0) {
             ok = mbar_wait(empty0 + 8u * sv, phase ^ 1, abort_flag);
-            if (ok) mbar_arrive_expect_tx(full, tile_bytes);
+            if (ok) {
+              mbar_arrive_expect_tx(full, kTileBytes);
+#pragma unroll
+              for (int s2 = 0; s2 < SUB; ++s2)
+                tma_load_4d(v_dst + s2 * 16384u, own_map, full, s2 * 64, w.g,
+                            (w.own_begin + i - w.n_ctx) * kTileN, w.outer_own);
+            }
           }
           ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
           if (!ok) break;
-          const int layer = p.layer_begin + w.l;
-          if (my_pidx >= 0) {
+          continue;
+        }
+        // pool row of positions lane, lane + 32, lane + 64, lane + 96 of the tile (looked up while the
+        // stage may still be in use)
+        const long long pos0 = (long long)(w.ctx_begin + i) * kTileN;
+        const long long L_all = p.ctx_cap;            // (row map entries beyond a query's context are -1)
+        int r[4];
+#pragma unroll
+        for (int q4 = 0; q4 < 4; ++q4) {
+          const long long pos = pos0 + lane + 32 * q4;
+          r[q4] = pos < L_all ? p.row_map[(long long)w.b * p.ctx_cap + pos] : -1;
+        }
+        // the number of valid positions of the tile: they form a prefix (valid positions are 0 .. L-1)
+        unsigned valid_mask[4];
+#pragma unroll
+        for (int q4 = 0; q4 < 4; ++q4) valid_mask[q4] = __ballot_sync(0xffffffffu, r[q4] >= 0);
+        const int n_valid = __popc(valid_mask[0]) + __popc(valid_mask[1]) + __popc(valid_mask[2]) + __popc(valid_mask[3]);
+#pragma unroll
+        for (int q4 = 0; q4 < 4; ++q4) {
+          const int pidx = lane + 32 * q4;
+          if (pidx >= n_valid) r[q4] = pidx - 2 * kTileN;       // one run of rows in front of the pool: zeros
+        }
+        __syncwarp();
+#pragma unroll
+        for (int q4 = 0; q4 < 4; ++q4) rows_s[lane + 32 * q4] = r[q4];
+        // a run ends after position pidx when the next position is not the next pool row
+        unsigned brk[4];
+#pragma unroll
+        for (int q4 = 0; q4 < 4; ++q4) {
+          int nxt = __shfl_down_sync(0xffffffffu, r[q4], 1);
+          const int wrap = __shfl_sync(0xffffffffu, q4 < 3 ? r[q4 + 1 < 4 ? q4 + 1 : 3] : 0, 0);
+          if (lane == 31) nxt = wrap;
+          const bool last = lane == 31 && q4 == 3;
+          brk[q4] = __ballot_sync(0xffffffffu, last || nxt != r[q4] + 1);
+        }
+        // the run ends as one 128-bit mask in every lane; lane j then finds the j-th box on its own.
+        // A run of n rows takes the largest power-of-two box that fits, once from its first row and,
+        // unless n is that power of two, once more ending at its last row: the two overlap, both write
+        // the same values there, and no run needs more than two copy instructions (the copy engine's
+        // time goes with the number of instructions, not with the bytes)
+        __syncwarp();
+        int my_pidx = -1, my_row = 0, my_lg = 0, n_boxes = 0;
+        uint32_t tile_bytes = 0;                 // what the boxes deliver in all (overlaps are copied twice)
+        {
+          int pidx = 0;
+          while (pidx < kTileN) {
+            int e = pidx;                       // end of the run that starts at pidx: first set bit at or after it
+            for (;;) {
+              const unsigned word = (e < 32 ? brk[0] : e < 64 ? brk[1] : e < 96 ? brk[2] : brk[3]) >> (e & 31);
+              if (word != 0) { e += __ffs(word) - 1; break; }
+              e = (e | 31) + 1;
+            }
+            const int n = e - pidx + 1;
+            const int lg = 31 - __clz(n);        // the largest power-of-two box that fits
+            if (n_boxes == lane) { my_pidx = pidx; my_lg = lg; }
+            ++n_boxes;
+            if (n > (1 << lg)) {                 // the rest of the run: the same box once more, ending at the run's end
+              if (n_boxes == lane) { my_pidx = e + 1 - (1 << lg); my_lg = lg; }
+              ++n_boxes;
+            }
+            tile_bytes += (n > (1 << lg) ? 2u : 1u) * ((uint32_t)SUB << (lg + 7));
+            pidx = e + 1;
+          }
+        }
+        if (my_pidx >= 0) my_row = rows_s[my_pidx];
+        // (tiles of more than 32 boxes - many one-token shots - take further rounds of the same walk)
+        if (lane == 0) {
+          ok = mbar_wait(empty0 + 8u * sv, phase ^ 1, abort_flag);
+          if (ok) mbar_arrive_expect_tx(full, tile_bytes);
+        }
+        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+        if (!ok) break;
+        const int layer = p.layer_begin + w.l;
+        if (my_pidx >= 0) {
+#pragma unroll
+          for (int s2 = 0; s2 < SUB; ++s2)
+            tma_load_4d(v_dst + s2 * 16384u + (uint32_t)my_pidx * 128u, &maps->m[my_lg], full, s2 * 64,
+                        w.g, my_row, layer);
+        }
+        for (int round = 1; round * 32 < n_boxes; ++round) {      // rare: more than 32 boxes in the tile
+          int pidx = 0, idx = 0, bp = -1, bl = 0;
+          while (pidx < kTileN) {
+            int e = pidx;
+            for (;;) {
+              const unsigned word = (e < 32 ? brk[0] : e < 64 ? brk[1] : e < 96 ? brk[2] : brk[3]) >> (e & 31);
+              if (word != 0) { e += __ffs(word) - 1; break; }
+              e = (e | 31) + 1;
+            }
+            const int n = e - pidx + 1;
+            const int lg = 31 - __clz(n);
+            if (idx == round * 32 + lane) { bp = pidx; bl = lg; }
+            ++idx;
+            if (n > (1 << lg)) {
+              if (idx == round * 32 + lane) { bp = e + 1 - (1 << lg); bl = lg; }
+              ++idx;
+            }
+            pidx = e + 1;
+          }
+          if (bp >= 0) {
+            const int brow = rows_s[bp];
 #pragma unroll
             for (int s2 = 0; s2 < SUB; ++s2)
-              tma_load_4d(v_dst + s2 * 16384u + (uint32_t)my_pidx * 128u, &maps->m[my_lg], full, s2 * 64,
-                          w.g, my_row, layer);
+              tma_load_4d(v_dst + s2 * 16384u + (uint32_t)bp * 128u, &maps->m[bl], full, s2 * 64, w.g,
+                          brow, layer);
           }
-          for (int round = 1; round * 32 < n_boxes; ++round) {      // rare: more than 32 boxes in the tile
-            int pidx = 0, idx = 0, bp = -1, bl = 0;
-            while (pidx < kTileN) {
-              int e = pidx;
-              for (;;) {
-                const unsigned word = (e < 32 ? brk[0] : e < 64 ? brk[1] : e < 96 ? brk[2] : brk[3]) >> (e & 31);
-                if (word != 0) { e += __ffs(word) - 1; break; }
-                e = (e | 31) + 1;
-              }
-              const int n = e - pidx + 1;
-              const int lg = 31 - __clz(n);
-              if (idx == round * 32 + lane) { bp = pidx; bl = lg; }
-              ++idx;
-              if (n > (1 << lg)) {
-                if (idx == round * 32 + lane) { bp = e + 1 - (1 << lg); bl = lg; }
-                ++idx;
-              }
-              pidx = e + 1;
-            }
-            if (bp >= 0) {
-              const int brow = rows_s[bp];
-#pragma unroll
-              for (int s2 = 0; s2 < SUB; ++s2)
-                tma_load_4d(v_dst + s2 * 16384u + (uint32_t)bp * 128u, &maps->m[bl], full, s2 * 64, w.g,
-                            brow, layer);
-            }
-          }
-          __syncwarp();
         }
+        __syncwarp();
       }
     }
     if (!ok && lane == 0) {
@@ -1072,18 +1110,29 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     const uint32_t o_addr = tmem_base + lane_addr + kTmemO + x * 128;
     uint32_t ns = 0, ni = 0;
     bool ok = true;
-    Walker wk = wk0;
-    Piece pc;
-    while (ok && next_piece(sc, cache, n_pairs, wk, pc)) {
-      for (int mp = rank; mp < p.n_mp && ok; mp += p.gang) {
-        Item w;
-        make_item(p, pc, gang_id, mp, w);
-        if (x == 1 && !w.has_b) continue;
-        const int mt = 2 * mp + x;
+    auto warp_arrive = [&](uint32_t b) {             // this warp's share of a barrier that four warps complete
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(b);
+    };
+    for (uint32_t n_item = 0; ok; ++n_item) {
+      // (the item is read where it lies: its fields would cost registers over the whole tile loop)
+      const uint32_t islot = n_item % kItems;
+      ok = __all_sync(0xffffffffu, mbar_wait(bar(kBarItemFull + islot), (n_item / kItems) & 1, abort_flag));
+      if (!ok) break;
+      const Item& w = items[islot];
+      const int n_tiles = w.n_tiles;
+      if (n_tiles < 0) break;
+      if (x == 0 || w.has_b()) {
+        const int mt = 2 * w.mp + x;
         const int m = mt * kTileM + r;               // row of the unit: token m / G, head m % G
-        const int t_row = m / p.G;
+        const int t_row = div_g(p, m);
         float m_used = kNegSentinel, l_sum = 0.f;
-        for (int i = 0; i < w.n_tiles; ++i, ++ns) {
+        // columns below a limit are visible, 128 fewer with every tile: context keys before L_j, own keys up to the row's token
+        const int n_ctx = w.n_ctx;
+        const int ctx_limit = w.Lj - w.ctx_begin * kTileN;
+        const int own_limit = p.To - p.Tq + min(t_row, p.Tq - 1) + 1 + (n_ctx - w.own_begin) * kTileN;
+        for (int i = 0; i < n_tiles; ++i, ++ns) {
           ok = __all_sync(0xffffffffu, mbar_wait(bar(kBarSFull + x), ns & 1, abort_flag));
           if (!ok) break;
           tc_fence_after();
@@ -1091,15 +1140,8 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           if constexpr (FUSED) tmem_ld4x32(s_addr, reinterpret_cast<uint32_t*>(s));
           else tmem_ld128(s_addr, reinterpret_cast<uint32_t*>(s));
 
-          // mask: context keys at or beyond L_j; own keys after the row's token (causal).
-          // Only the last context tile and the own-token tiles can hide anything.
-          int limit = kTileN;                          // columns < limit are visible
-          if (i < w.n_ctx) {
-            const long long first = (long long)(w.ctx_begin + i) * kTileN;
-            if (first + kTileN > w.Lj) limit = (int)(w.Lj - first);
-          } else {
-            limit = p.To - p.Tq + min(t_row, p.Tq - 1) - (w.own_begin + i - w.n_ctx) * kTileN + 1;   // <= 0: all hidden
-          }
+          // mask: only the last context tile and the own-token tiles can hide anything (limit <= 0: all of it)
+          const int limit = (i < n_ctx ? ctx_limit : own_limit) - i * kTileN;
           if (__any_sync(0xffffffffu, limit < kTileN)) {
 #pragma unroll
             for (int cidx = 0; cidx < kTileN; ++cidx) s[cidx] = cidx < limit ? s[cidx] : -INFINITY;
@@ -1161,115 +1203,107 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
               tmem_st32(o_addr + q4 * 32, reinterpret_cast<const uint32_t*>(o));
             }
           }
-          tc_fence_before();
-          mbar_arrive(bar(kBarPFull + x));
+          warp_arrive(bar(kBarPFull + x));
         }
         if (!ok) break;
         const bool row_ok = m < p.Tq * p.G;
-        if (w.n_tiles == 0) {
+        if (n_tiles == 0) {
           // nothing of this M pair falls into the piece: a neutral partial (a whole unit is never empty)
-          float4* otile = reinterpret_cast<float4*>(p.o_part) + (w.slot * 2 + x) * (long long)(D / 4) * kTileM + r;
+          float4* otile = reinterpret_cast<float4*>(p.o_part) + (w.slot * 2 + x) * ((long long)(D / 4) * kTileM) + r;
 #pragma unroll
           for (int c4 = 0; c4 < D / 4; ++c4) otile[c4 * kTileM] = make_float4(0.f, 0.f, 0.f, 0.f);
-          float* ml = p.ml_part + ((w.slot * 2 + x) * kTileM + r) * 2;
+          float* ml = p.ml_part + ((long long)(w.slot * 2 + x) * kTileM + r) * 2;
           ml[0] = kNegSentinel;
           ml[1] = 0.f;
-          continue;
-        }
-        ok = __all_sync(0xffffffffu, mbar_wait(bar(kBarOFull + x), ni & 1, abort_flag));
-        if (!ok) break;
-        tc_fence_after();
-        if (w.whole) {
-          // The piece covers the unit: normalise and store the final rows.  A thread owns a
-          // row, and rows are far apart in the output, so a direct store would touch 32 lines
-          // per instruction; instead the warp passes 64 columns at a time through its staging
-          // area (16-byte chunks swizzled by the row) and writes four rows' 128-byte segments
-          // per instruction.
-          const float inv = 1.f / l_sum;
-          const long long bpj = w.outer_own;
-          unsigned char* stg = base_ptr + SM::kOffStage + (warp - kSoftmaxWarp0) * SM::kStageBytes;
-          const int sub = lane >> 3, ch = lane & 7;            // read-back: row 4 j + sub, chunk ch
-          const int m0 = mt * kTileM + quarter * 32;
-          if constexpr (FUSED) {
-            // (no staging area in the fused variant's shared-memory plan: one row per thread)
-            const int hq = w.g * p.G + m % p.G;
-            __nv_bfloat16* dst = p.out + (((bpj * p.Tq + t_row) * p.Hq) + hq) * (long long)D;
+        } else {
+          ok = __all_sync(0xffffffffu, mbar_wait(bar(kBarOFull + x), ni & 1, abort_flag));
+          if (!ok) break;
+          tc_fence_after();
+          if (w.whole()) {
+            // The piece covers the unit: normalise and store the final rows.  A thread owns a
+            // row, and rows are far apart in the output, so a direct store would touch 32 lines
+            // per instruction; instead the warp passes 64 columns at a time through its staging
+            // area (16-byte chunks swizzled by the row) and writes four rows' 128-byte segments
+            // per instruction.
+            const float inv = 1.f / l_sum;
+            const long long bpj = w.outer_own;
+            unsigned char* stg = base_ptr + SM::kOffStage + (warp - kSoftmaxWarp0) * SM::kStageBytes;
+            const int sub = lane >> 3, ch = lane & 7;            // read-back: row 4 j + sub, chunk ch
+            const int m0 = mt * kTileM + quarter * 32;
+            if constexpr (FUSED) {
+              // (no staging area in the fused variant's shared-memory plan: one row per thread)
+              const int hq = w.g * p.G + m - t_row * p.G;
+              __nv_bfloat16* dst = p.out + (((bpj * p.Tq + t_row) * p.Hq) + hq) * (long long)D;
+#pragma unroll
+              for (int q4 = 0; q4 < D / 32; ++q4) {
+                float o[32];
+                tmem_ld32(o_addr + q4 * 32, reinterpret_cast<uint32_t*>(o));
+                if (q4 == D / 32 - 1) warp_arrive(bar(kBarOEmpty + x));
+                if (row_ok) {
+#pragma unroll
+                  for (int e = 0; e < 32; e += 8) {
+                    float v8[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) v8[u] = o[e + u] * inv;
+                    *reinterpret_cast<uint4*>(dst + q4 * 32 + e) = bf16x8_pack(v8);
+                  }
+                }
+              }
+            } else {
+#pragma unroll
+            for (int h = 0; h < D / 64; ++h) {
+              float o[64];
+              tmem_ld32(o_addr + h * 64, reinterpret_cast<uint32_t*>(o));
+              tmem_ld32(o_addr + h * 64 + 32, reinterpret_cast<uint32_t*>(o + 32));
+              if (h == D / 64 - 1) warp_arrive(bar(kBarOEmpty + x));     // O is in registers: the next item may overwrite it
+#pragma unroll
+              for (int c = 0; c < 8; ++c) {
+                float v8[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v8[u] = o[c * 8 + u] * inv;
+                *reinterpret_cast<uint4*>(stg + lane * 128 + ((c ^ (lane & 7)) << 4)) = bf16x8_pack(v8);
+              }
+              __syncwarp();
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                const int row = 4 * j + sub;
+                const int mm = m0 + row;
+                const uint4 v = *reinterpret_cast<const uint4*>(stg + row * 128 + ((ch ^ (row & 7)) << 4));
+                if (mm < p.Tq * p.G) {
+                  const int tt = div_g(p, mm), hq = w.g * p.G + mm - tt * p.G;
+                  __nv_bfloat16* dst = p.out + (((bpj * p.Tq + tt) * p.Hq) + hq) * (long long)D;
+                  *reinterpret_cast<uint4*>(dst + h * 64 + ch * 8) = v;
+                }
+              }
+              __syncwarp();
+            }
+            }
+            if (row_ok && p.lse != nullptr) {
+              const int hh = m - t_row * p.G, hq = w.g * p.G + hh;
+              p.lse[(bpj * p.Hq + hq) * p.Tq + t_row] = (m_used + log2f(l_sum)) * kLn2;
+            }
+          } else {
+            // un-normalised partial, four columns of 128 rows at a time ([D/4][128][4] per M tile):
+            // a warp's 32 rows are 512 contiguous bytes per store
+            float4* otile = reinterpret_cast<float4*>(p.o_part) + (w.slot * 2 + x) * ((long long)(D / 4) * kTileM) + r;
 #pragma unroll
             for (int q4 = 0; q4 < D / 32; ++q4) {
               float o[32];
               tmem_ld32(o_addr + q4 * 32, reinterpret_cast<uint32_t*>(o));
-              if (q4 == D / 32 - 1) {
-                tc_fence_before();
-                mbar_arrive(bar(kBarOEmpty + x));
-              }
-              if (row_ok) {
+              if (q4 == D / 32 - 1) warp_arrive(bar(kBarOEmpty + x));
 #pragma unroll
-                for (int e = 0; e < 32; e += 8) {
-                  float v8[8];
-#pragma unroll
-                  for (int u = 0; u < 8; ++u) v8[u] = o[e + u] * inv;
-                  *reinterpret_cast<uint4*>(dst + q4 * 32 + e) = bf16x8_pack(v8);
-                }
-              }
+              for (int e = 0; e < 32; e += 4)
+                otile[(q4 * 8 + e / 4) * kTileM] = make_float4(o[e], o[e + 1], o[e + 2], o[e + 3]);
             }
-          } else {
-#pragma unroll
-          for (int h = 0; h < D / 64; ++h) {
-            float o[64];
-            tmem_ld32(o_addr + h * 64, reinterpret_cast<uint32_t*>(o));
-            tmem_ld32(o_addr + h * 64 + 32, reinterpret_cast<uint32_t*>(o + 32));
-            if (h == D / 64 - 1) {             // O is in registers: the next item may overwrite it
-              tc_fence_before();
-              mbar_arrive(bar(kBarOEmpty + x));
-            }
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-              float v8[8];
-#pragma unroll
-              for (int u = 0; u < 8; ++u) v8[u] = o[c * 8 + u] * inv;
-              *reinterpret_cast<uint4*>(stg + lane * 128 + ((c ^ (lane & 7)) << 4)) = bf16x8_pack(v8);
-            }
-            __syncwarp();
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const int row = 4 * j + sub;
-              const int mm = m0 + row;
-              const uint4 v = *reinterpret_cast<const uint4*>(stg + row * 128 + ((ch ^ (row & 7)) << 4));
-              if (mm < p.Tq * p.G) {
-                const int tt = mm / p.G, hq = w.g * p.G + mm % p.G;
-                __nv_bfloat16* dst = p.out + (((bpj * p.Tq + tt) * p.Hq) + hq) * (long long)D;
-                *reinterpret_cast<uint4*>(dst + h * 64 + ch * 8) = v;
-              }
-            }
-            __syncwarp();
+            float* ml = p.ml_part + ((long long)(w.slot * 2 + x) * kTileM + r) * 2;
+            ml[0] = m_used;
+            ml[1] = l_sum;
           }
-          }
-          if (row_ok && p.lse != nullptr) {
-            const int hh = m % p.G, hq = w.g * p.G + hh;
-            p.lse[(bpj * p.Hq + hq) * p.Tq + t_row] = (m_used + log2f(l_sum)) * kLn2;
-          }
-        } else {
-          // un-normalised partial, four columns of 128 rows at a time ([D/4][128][4] per M tile):
-          // a warp's 32 rows are 512 contiguous bytes per store
-          float4* otile = reinterpret_cast<float4*>(p.o_part) + (w.slot * 2 + x) * (long long)(D / 4) * kTileM + r;
-#pragma unroll
-          for (int q4 = 0; q4 < D / 32; ++q4) {
-            float o[32];
-            tmem_ld32(o_addr + q4 * 32, reinterpret_cast<uint32_t*>(o));
-            if (q4 == D / 32 - 1) {
-              tc_fence_before();
-              mbar_arrive(bar(kBarOEmpty + x));
-            }
-#pragma unroll
-            for (int e = 0; e < 32; e += 4)
-              otile[(q4 * 8 + e / 4) * kTileM] = make_float4(o[e], o[e + 1], o[e + 2], o[e + 3]);
-          }
-          float* ml = p.ml_part + ((w.slot * 2 + x) * kTileM + r) * 2;
-          ml[0] = m_used;
-          ml[1] = l_sum;
+          ++ni;
         }
-        ++ni;
       }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(kBarItemEmpty + islot));
     }
   };
 
@@ -1277,8 +1311,8 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   if (warp < 4) {
     regs_lower<FUSED ? kFusedRegsIssue : kRegsIssue>();
     if (warp == 0) role_tma();
+    else if (FUSED ? warp != 1 : VPOOL && warp == kGatherWarp) role_gather();
     else if (warp == 1) role_mma();
-    else if (FUSED || (VPOOL && warp == kGatherWarp)) role_gather();
   } else if (!FUSED || warp < kRotateWarp0) {
     regs_raise<FUSED ? kFusedRegsSoftmax : kRegsSoftmax>();
     role_softmax();
@@ -1565,6 +1599,7 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
   ap.sched = sched; ap.o_part = o_part; ap.ml_part = ml_part;
   ap.out = static_cast<__nv_bfloat16*>(out); ap.lse = lse; ap.status = status;
   ap.B = B; ap.P = P; ap.Tq = Tq; ap.Hq = Hq; ap.Hkv = Hkv; ap.G = G; ap.nl = nl; ap.To = To;
+  ap.g_magic = ((1ull << 32) + G - 1) / G;
   ap.n_mt = pl.n_mt; ap.n_mp = pl.n_mp; ap.gang = pl.gang; ap.n_gangs = n_gangs;
   const float scale = model->softmax_scale > 0.f ? model->softmax_scale : 1.0f / sqrtf((float)D);
   ap.scale_log2 = scale * 1.4426950408889634f;
