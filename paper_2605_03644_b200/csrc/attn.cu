@@ -141,6 +141,7 @@ struct PrepParams {
   AdsEntropyJob ent;          // entropy of the probes' logits, first step
   RowMapParams map;
   int map_blocks;             // eight selected shots each; 0: no row map
+  int tok_blocks;
 };
 
 __device__ __forceinline__ void bf16x8_unpack(const uint4& r, float* x) {
@@ -208,7 +209,9 @@ __device__ __forceinline__ void row_map_warp(const RowMapParams& p, long long w,
 // kPrepParts warps per own token (b, l, j, u): all Hq query heads and Hkv key heads of the token rotate by the same
 // angles (L_j + u) * theta_i, which the block forms once for its tokens, half an angle per thread, while the first
 // rows are on their way.  (Every lane forming its eight angles itself was what bound the kernel: 4096 tokens of 32
-// + 8 heads, 84 MB, 27 us and 14336 tokens 82-90 us; now 20 and 73.)  The first block writes the schedule instead: started
+// + 8 heads, 84 MB, 27 us and 14336 tokens 82-90 us; 20 and 73 then.)  The blocks stay for the whole call: the angles of their next
+// tokens, a chain of two loads and fp64 arithmetic, are formed while this group's rows are on their way (a block per two tokens: 21.2 and
+// 73 us, 17.2 and 60 now).  The first block writes the schedule instead: started
 // first, its chain of dependent steps lies under the others' copies.
 template <int D>
 __global__ void __launch_bounds__(256, 3) attn_prep_kernel(const __grid_constant__ PrepParams p) {
@@ -326,79 +329,90 @@ __global__ void __launch_bounds__(256, 3) attn_prep_kernel(const __grid_constant
     return;
   }
   blk -= p.map_blocks;
-  constexpr int kTokens = 8 / kPrepParts;           // of a block
-  __shared__ float2 angle_s[kTokens][D / 2];        // (cos, sin)
+  constexpr int kTokens = 8 / kPrepParts;           // of a block at a time
+  __shared__ float2 angle_s[2][kTokens][D / 2];     // (cos, sin)
   // (tokens and rows fit 32 bits: 2^31 of them would not fit the device's memory)
-  const int n_tok = p.B * p.nl * p.P * p.To, tok0 = blk * kTokens;
+  const int n_tok = p.B * p.nl * p.P * p.To, n_groups = (n_tok + kTokens - 1) / kTokens;
   const int warp = threadIdx.x >> 5, slot = warp / kPrepParts, part = warp % kPrepParts;
-  const int tok = tok0 + slot;
-  const bool live = tok < n_tok;
-  const int bpj = tok / p.To;                       // (b*nl + l)*P + j
-  const int u_own = tok - bpj * p.To;               // own token u sits at position L_j + u
-  const int G = p.Hq / p.Hkv;
-  const int t = u_own - (p.To - p.Tq);              // query row of this token (the last Tq own tokens have one)
-  const bool has_q = t >= 0;
-  const int jcol = lane % HALF_V;
-  const uint4* qsrc = reinterpret_cast<const uint4*>(p.q) + ((long long)bpj * p.Tq + (has_q ? t : 0)) * p.Hq * VPH;
-  const uint4* ksrc = reinterpret_cast<const uint4*>(p.kq) + (long long)tok * p.Hkv * VPH;
-  uint4* kdst = reinterpret_cast<uint4*>(p.kq_rot) + (long long)tok * p.Hkv * VPH;
-  uint4* qdst_base = reinterpret_cast<uint4*>(p.q_rot);
-  const int units = live ? (p.Hq + p.Hkv) * HALF_V : 0;
+  const int G = p.Hq / p.Hkv, jcol = lane % HALF_V;
   constexpr int kFly = 3;                           // units of a lane loaded at once (the 8B shape has 2.5 per lane)
   uint4 lo[kFly], hi[kFly];
+  int tok, bpj, t, units;                           // of this thread's token
+  auto take = [&](int group) {
+    tok = group * kTokens + slot;
+    bpj = tok / p.To;                               // (b*nl + l)*P + j
+    t = tok - bpj * p.To - (p.To - p.Tq);           // query row of this token (the last Tq own tokens have one), or negative
+    units = tok < n_tok ? (p.Hq + p.Hkv) * HALF_V : 0;
+  };
   auto load = [&](int u0) {
+    const uint4* qsrc = reinterpret_cast<const uint4*>(p.q) + ((long long)bpj * p.Tq + max(t, 0)) * p.Hq * VPH + jcol;
+    const uint4* ksrc = reinterpret_cast<const uint4*>(p.kq) + (long long)tok * p.Hkv * VPH + jcol;
 #pragma unroll
     for (int e = 0; e < kFly; ++e) {
       const int u = u0 + e * 32 * kPrepParts, head = u / HALF_V;       // column == jcol since 32 % HALF_V == 0
-      if (u >= units || (head < p.Hq && !has_q)) continue;
-      const uint4* src = head < p.Hq ? qsrc + head * VPH + jcol : ksrc + (head - p.Hq) * VPH + jcol;
+      if (u >= units || (head < p.Hq && t < 0)) continue;
+      const uint4* src = head < p.Hq ? qsrc + head * VPH : ksrc + (head - p.Hq) * VPH;
       lo[e] = src[0];
       hi[e] = src[HALF_V];
     }
   };
-  load(part * 32 + lane);
-  for (int i = threadIdx.x; i < kTokens * (D / 2); i += 256) {
-    const int tk = tok0 + i / (D / 2);
-    if (tk < n_tok) {
-      const int x = tk / p.To, bl = x / p.P, j = x - bl * p.P, b = bl / p.nl;
-      const long long Lj = p.ctx_off[(long long)b * (p.k + 1) + probe_shots(p, b, j)];
-      float sn, cs;
-      rope_sincos((double)(Lj + tk - x * p.To), p.theta[i % (D / 2)], &sn, &cs);
-      angle_s[i / (D / 2)][i % (D / 2)] = make_float2(cs, sn);
+  auto angles = [&](int group, int buf) {
+    for (int i = threadIdx.x; i < kTokens * (D / 2); i += 256) {
+      const int tk = group * kTokens + i / (D / 2);
+      if (tk < n_tok) {
+        const int x = tk / p.To, bl = x / p.P, j = x - bl * p.P, b = bl / p.nl;
+        const long long Lj = p.ctx_off[(long long)b * (p.k + 1) + probe_shots(p, b, j)];
+        float sn, cs;
+        rope_sincos((double)(Lj + tk - x * p.To), p.theta[i % (D / 2)], &sn, &cs);
+        angle_s[buf][i / (D / 2)][i % (D / 2)] = make_float2(cs, sn);
+      }
     }
-  }
+  };
+  const int u_first = part * 32 + lane;
+  take(blk);
+  load(u_first);
+  angles(blk, 0);
   __syncthreads();
-  float sn[8], cs[8];
+  for (int group = blk, buf = 0; group < n_groups; group += p.tok_blocks, buf ^= 1) {
+    const int next = group + p.tok_blocks;
+    if (next < n_groups) angles(next, buf ^ 1);      // (under the loads of this group's rows)
+    float sn[8], cs[8];
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const float4 v = *reinterpret_cast<const float4*>(&angle_s[slot][jcol * 8 + 2 * e]);
-    cs[2 * e] = v.x; sn[2 * e] = v.y; cs[2 * e + 1] = v.z; sn[2 * e + 1] = v.w;
-  }
-  for (int u0 = part * 32 + lane; u0 < units; u0 += kFly * 32 * kPrepParts) {
-    if (u0 >= kFly * 32 * kPrepParts) load(u0);
-#pragma unroll
-    for (int e = 0; e < kFly; ++e) {
-      const int u = u0 + e * 32 * kPrepParts, head = u / HALF_V;
-      if (u >= units || (head < p.Hq && !has_q)) continue;
-      float x[8], y[8], xr[8], yr[8];
-      bf16x8_unpack(lo[e], x);
-      bf16x8_unpack(hi[e], y);
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        xr[c] = x[c] * cs[c] - y[c] * sn[c];
-        yr[c] = y[c] * cs[c] + x[c] * sn[c];
-      }
-      uint4* dst;
-      if (head < p.Hq) {
-        const int g = head / G, hh = head % G;
-        const long long row = ((long long)bpj * p.Hkv + g) * (p.Tq * G) + t * G + hh;
-        dst = qdst_base + row * VPH + jcol;
-      } else {
-        dst = kdst + (head - p.Hq) * VPH + jcol;
-      }
-      dst[0] = bf16x8_pack(xr);
-      dst[HALF_V] = bf16x8_pack(yr);
+    for (int e = 0; e < 4; ++e) {
+      const float4 v = *reinterpret_cast<const float4*>(&angle_s[buf][slot][jcol * 8 + 2 * e]);
+      cs[2 * e] = v.x; sn[2 * e] = v.y; cs[2 * e + 1] = v.z; sn[2 * e + 1] = v.w;
     }
+    for (int u0 = u_first; u0 < units; u0 += kFly * 32 * kPrepParts) {
+      if (u0 >= kFly * 32 * kPrepParts) load(u0);
+#pragma unroll
+      for (int e = 0; e < kFly; ++e) {
+        const int u = u0 + e * 32 * kPrepParts, head = u / HALF_V;
+        if (u >= units || (head < p.Hq && t < 0)) continue;
+        float x[8], y[8], xr[8], yr[8];
+        bf16x8_unpack(lo[e], x);
+        bf16x8_unpack(hi[e], y);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          xr[c] = x[c] * cs[c] - y[c] * sn[c];
+          yr[c] = y[c] * cs[c] + x[c] * sn[c];
+        }
+        uint4* dst;
+        if (head < p.Hq) {
+          const int g = head / G, hh = head - g * G;
+          const long long row = ((long long)bpj * p.Hkv + g) * (p.Tq * G) + t * G + hh;
+          dst = reinterpret_cast<uint4*>(p.q_rot) + row * VPH + jcol;
+        } else {
+          dst = reinterpret_cast<uint4*>(p.kq_rot) + (long long)tok * p.Hkv * VPH + (head - p.Hq) * VPH + jcol;
+        }
+        dst[0] = bf16x8_pack(xr);
+        dst[HALF_V] = bf16x8_pack(yr);
+      }
+    }
+    if (next < n_groups) {
+      take(next);
+      load(u_first);
+    }
+    __syncthreads();
   }
 }
 
@@ -1591,7 +1605,9 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
   for (int i = 0; i < D / 2; ++i) pp.theta[i] = pow(model->rope_base, -2.0 * (double)i / (double)D);
   for (int i = 0; i < kMaxProbes; ++i) pp.nshots[i] = i < P ? probe_nshots[i] : 0;
   const long long n_tok = (long long)B * nl * P * To;
-  ads_launch_dependent(attn_prep_kernel<D>, (unsigned)((n_tok * kPrepParts + 7) / 8) + 1 + pp.ent.blocks + pp.map_blocks, 256, 0, st, pp);
+  const long long n_groups = (n_tok * kPrepParts + 7) / 8;
+  pp.tok_blocks = (int)(n_groups < 3 * n_sm ? n_groups : 3 * n_sm);       // what is resident at a time
+  ads_launch_dependent(attn_prep_kernel<D>, (unsigned)(1 + pp.ent.blocks + pp.map_blocks + pp.tok_blocks), 256, 0, st, pp);
   if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
 
   // ---- main kernel
