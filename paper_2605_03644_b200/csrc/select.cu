@@ -200,27 +200,29 @@ __device__ __forceinline__ bool pair_less(unsigned long long ka, int ia, unsigne
 }
 
 // Top k by radix selection, one CTA per query.  The keys' interval is narrowed, 4096 bins at a time, until
-// the bin that holds the k-th key and everything in front of it fit the candidate area; the candidates are
-// then sorted by (key, id).  The first pass bins by the score's sign, exponent and five bits more (cosines and
-// attention masses both spread over many of them), the following ones divide the bin's interval evenly, so two
-// passes nearly always do; equal keys without end are cut by id.  Latency-bound: a pass reads the keys once
-// (the second one from L1) with eight loads in flight per thread.  A cluster of eight CTAs per query that
-// added their histograms up through distributed shared memory was slower (40 us against 21 at 20000 keys): the
-// cluster barriers cost more than the counting.  (One 8192-entry bitonic sort per chunk took 79 us per launch;
-// 20000 keys, k = 512, 16 queries: 159 -> 21 us, 8192 keys, k = 512, 32 queries: 145 -> 13 us.)
+// the bin that holds the k-th key and everything in front of it fit the candidate area; up to 1024 candidates are then
+// put in order by dealing them out to 4096 bins once more, more of them by a bitonic sort.  The first pass bins by the score's
+// sign, exponent and five bits more (cosines and attention masses both spread over many of them), the following ones
+// divide the bin's interval evenly, so two passes nearly always do; equal keys without end are cut by id.  Bound by the
+// instructions of one SM per query: a pass reads the keys once (the second one from L1) with eight loads in flight per
+// thread.  A cluster of eight CTAs per query that added their histograms up through distributed shared memory was slower
+// (40 us against 21 at 20000 keys): the cluster barriers cost more than the counting.  (20000 keys, k = 512, 16 queries: one
+// 8192-entry bitonic sort per chunk 159 us, candidates sorted in 55 steps and bins by compares and selects 20.8, now 16.3; 8192
+// keys, k = 512, 32 queries 145, 14.6 and 11.2; 4096 keys, k = 256, 8 queries 11.0 and 9.6.)
 constexpr int kSelThreads = 1024;
 constexpr int kSelBins = 4096;
+constexpr int kBinMost = 32;          // candidates in one bin that are ordered by comparing each with all
 
 // First-pass bins, ascending with the key: 0 = scores of 2 and more, 1 .. 2040 = positive scores below that in 32nds
 // of an octave (63 octaves), 2041 = smaller ones, then the negative scores in the same way.
 constexpr int kBinHi = (1023 + 1) << 5, kBinLo = kBinHi - 2040;
 constexpr int kBinShift = 47;                     // leaves the sign, the exponent and 5 bits
 __device__ __forceinline__ int first_bin(unsigned long long key) {
-  const int v = (int)(key >> kBinShift);          // 17 bits: those of a positive score count down
-  const int m = v < 0x10000 ? 0xffff - v : v - 0x10000;
-  const int mid = m - kBinLo;                     // 0 .. 2039
-  if (v < 0x10000) return m >= kBinHi ? 0 : (mid < 0 ? 2041 : 2040 - mid);
-  return m >= kBinHi ? 4083 : (mid < 0 ? 2042 : 2043 + mid);
+  const int v = (int)((uint32_t)(key >> 32) >> (kBinShift - 32));     // 17 bits: those of a positive score count down
+  const bool neg = v >= 0x10000;
+  const int m = neg ? v - 0x10000 : 0xffff - v;
+  const int mid = min(max(m - kBinLo, -1), 2040);
+  return neg ? 2043 + mid : 2040 - mid;
 }
 __device__ __forceinline__ void first_bin_interval(int bin, unsigned long long* lo, unsigned long long* hi) {
   int a, b;                                       // first and last v of the bin
@@ -242,12 +244,28 @@ radix_topk_kernel(const unsigned long long* __restrict__ all_keys, int N, int k,
   int* cid = reinterpret_cast<int*>(ckey + want);                                 // [want]
   int* hist = cid + want;                                                         // [kSelBins]
   __shared__ int warp_sum_s[32], bin_s, before_s, inside_s, n_s;
+  __shared__ unsigned long long warp_min_s[32], warp_max_s[32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x;
   const unsigned long long* keys = all_keys + (long long)b * N;
   ads_dependency_wait();
   constexpr int kFly = 8;
 
+  // This thread's four bins and how many entries lie in front of them (a barrier in between: the caller writes before it).
+  auto bins_before = [&](int (&h)[4]) -> int {
+    const int4 h4 = *reinterpret_cast<const int4*>(hist + 4 * tid);
+    h[0] = h4.x; h[1] = h4.y; h[2] = h4.z; h[3] = h4.w;
+    const int sum = h[0] + h[1] + h[2] + h[3];
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    if (lane == 31) warp_sum_s[warp] = incl;
+    __syncthreads();
+    return incl - sum + __reduce_add_sync(0xffffffffu, lane < warp ? warp_sum_s[lane] : 0);
+  };
   unsigned long long lo = 0, hi = ~0ull;           // keys below lo: taken; above hi: out
   int before = 0, inside = N;                       // how many are below lo, how many in [lo, hi]
   if (tid == 0) n_s = 0;
@@ -260,25 +278,20 @@ radix_topk_kernel(const unsigned long long* __restrict__ all_keys, int N, int k,
       unsigned long long key[kFly];
 #pragma unroll
       for (int u = 0; u < kFly; ++u) key[u] = i0 + u * kSelThreads < N ? keys[i0 + u * kSelThreads] : ~0ull;
+      if (pass == 0) {
 #pragma unroll
-      for (int u = 0; u < kFly; ++u)
-        if (i0 + u * kSelThreads < N && key[u] >= lo && key[u] <= hi)
-          atomicAdd(hist + (pass == 0 ? first_bin(key[u]) : (int)((key[u] - lo) >> shift)), 1);
+        for (int u = 0; u < kFly; ++u)
+          if (i0 + u * kSelThreads < N) atomicAdd(hist + first_bin(key[u]), 1);
+      } else {
+#pragma unroll
+        for (int u = 0; u < kFly; ++u)
+          if (i0 + u * kSelThreads < N && key[u] >= lo && key[u] <= hi) atomicAdd(hist + (int)((key[u] - lo) >> shift), 1);
+      }
     }
     __syncthreads();
     // the bin that holds rank k - 1
-    const int4 h4 = *reinterpret_cast<const int4*>(hist + 4 * tid);
-    const int h[4] = {h4.x, h4.y, h4.z, h4.w};
-    const int sum = h[0] + h[1] + h[2] + h[3];
-    int incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int u = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += u;
-    }
-    if (lane == 31) warp_sum_s[warp] = incl;
-    __syncthreads();
-    int at = before + incl - sum + __reduce_add_sync(0xffffffffu, lane < warp ? warp_sum_s[lane] : 0);
+    int h[4];
+    int at = before + bins_before(h);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       if (at < k && at + h[u] >= k) {
@@ -336,44 +349,61 @@ radix_topk_kernel(const unsigned long long* __restrict__ all_keys, int N, int k,
   }
   __syncthreads();
   const int n = n_s;
+  if (want <= kSelThreads) {
+    // One candidate per thread, dealt out to 4096 bins of equal width between the smallest and the largest key; its place is what lies in
+    // front of its bin and what precedes it there.  (The bitonic sort below takes 55 steps for 1024 candidates.)
+    unsigned long long* skey = reinterpret_cast<unsigned long long*>(hist + kSelBins);     // [want], by bin
+    int* sid = reinterpret_cast<int*>(skey + want);
+    const unsigned long long key = tid < n ? ckey[tid] : ~0ull;
+    const int id = tid < n ? cid[tid] : 0x7fffffff;
+    unsigned long long least = key, most = tid < n ? key : 0;
+    auto across = [&]() {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long a = __shfl_xor_sync(0xffffffffu, least, o), c = __shfl_xor_sync(0xffffffffu, most, o);
+        least = a < least ? a : least;
+        most = c > most ? c : most;
+      }
+    };
+    across();
+    if (lane == 0) { warp_min_s[warp] = least; warp_max_s[warp] = most; }
+    *reinterpret_cast<int4*>(hist + 4 * tid) = make_int4(0, 0, 0, 0);
+    __syncthreads();
+    least = warp_min_s[lane];
+    most = warp_max_s[lane];
+    across();
+    int shift = 64 - __clzll((long long)(most - least)) - 12;
+    if (shift < 0) shift = 0;
+    int bin = 0, nth = 0;
+    if (tid < n) {
+      bin = (int)((key - least) >> shift);
+      nth = atomicAdd(hist + bin, 1);
+    }
+    if (!__syncthreads_or(nth >= kBinMost)) {
+      int h[4];
+      int at = bins_before(h);
+      *reinterpret_cast<int4*>(hist + 4 * tid) = make_int4(at, at + h[0], at + h[0] + h[1], at + h[0] + h[1] + h[2]);
+      __syncthreads();
+      int first = 0, last = 0;
+      if (tid < n) {
+        first = hist[bin];
+        last = bin + 1 < kSelBins ? hist[bin + 1] : n;
+        skey[first + nth] = key;
+        sid[first + nth] = id;
+      }
+      __syncthreads();
+      int place = first;
+      for (int i = first; i < last; ++i) place += pair_less(skey[i], sid[i], key, id) ? 1 : 0;
+      if (tid < n && place < k) {
+        final_idx[(long long)b * k + place] = id;
+        if (final_score != nullptr) final_score[(long long)b * k + place] = (float)key_score(key);
+      }
+      return;
+    }
+  }
+  // bitonic sort, ascending on (key, id); ids are unique so the order is total
   int n_pow2 = 32;
   while (n_pow2 < n) n_pow2 <<= 1;
-  // bitonic sort, ascending on (key, id); ids are unique so the order is total
-  if (n_pow2 <= kSelThreads) {
-    // one candidate per thread: exchanges within a warp by shuffles, the others through shared memory
-    if (tid >= n_pow2) return;                      // (whole warps)
-    auto sync = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(n_pow2) : "memory"); };
-    unsigned long long key = tid < n ? ckey[tid] : ~0ull;      // padding sorts last
-    int id = tid < n ? cid[tid] : 0x7fffffff;
-    sync();
-    for (int size = 2; size <= n_pow2; size <<= 1) {
-      for (int stride = size >> 1; stride > 0; stride >>= 1) {
-        unsigned long long ko;
-        int io;
-        if (stride >= 32) {
-          ckey[tid] = key;
-          cid[tid] = id;
-          sync();
-          ko = ckey[tid ^ stride];
-          io = cid[tid ^ stride];
-          sync();
-        } else {
-          ko = __shfl_xor_sync(0xffffffffu, key, stride);
-          io = __shfl_xor_sync(0xffffffffu, id, stride);
-        }
-        const bool keep_low = ((tid & stride) == 0) == ((tid & size) == 0);
-        if (pair_less(ko, io, key, id) == keep_low) {
-          key = ko;
-          id = io;
-        }
-      }
-    }
-    if (tid < min(k, n)) {
-      final_idx[(long long)b * k + tid] = id;
-      if (final_score != nullptr) final_score[(long long)b * k + tid] = (float)key_score(key);
-    }
-    return;
-  }
   for (int i = n + tid; i < n_pow2; i += kSelThreads) {
     ckey[i] = ~0ull;
     cid[i] = 0x7fffffff;
@@ -484,7 +514,8 @@ int ads_topk_from_keys(const unsigned long long* keys, int N, int B, int k, int3
   while (want < k) want <<= 1;
   static bool attr_set[kAdsMaxDevices] = {false};
   if (ads_set_max_smem(radix_topk_kernel, kSortCap * (8 + 4) + kSelBins * 4, attr_set) != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
-  ads_launch_dependent(radix_topk_kernel, (unsigned)B, kSelThreads, want * (8 + 4) + kSelBins * 4, st, keys, N, k, want, sel_idx, sel_score);
+  const int smem = want * (8 + 4) * (want <= kSelThreads ? 2 : 1) + kSelBins * 4;
+  ads_launch_dependent(radix_topk_kernel, (unsigned)B, kSelThreads, smem, st, keys, N, k, want, sel_idx, sel_score);
   return ads_launch_status();
 }
 

@@ -56,6 +56,20 @@ def test_select_ties_and_zero_norm():
     assert sel[1, :4].tolist() == [40, 41, 42, 43]
 
 
+@pytest.mark.parametrize("k", [1, 33, 128, 512, 1000])
+@pytest.mark.parametrize("copies", [1, 31, 33, 700])       # below and above what a bin of candidates may hold; more than k of them
+def test_select_by_bins_and_by_sorting(copies, k):
+    # a pool large enough for the selection, whose best shots are copies of one another and whose scores span many octaves
+    ab = hp.gpu_binding()
+    g = torch.Generator().manual_seed(copies + k)
+    emb = torch.randn(9000, 32, generator=g)
+    q = torch.randn(4, 32, generator=g)
+    emb[:3000] += 3.0 * q[0]
+    at = torch.randperm(9000, generator=g)[:copies]
+    emb[at] = q[0] + 0.01 * torch.randn(32, generator=g)
+    _check(ab, emb, q, k)
+
+
 def test_nested_probes_are_prefixes():
     ab = hp.gpu_binding()
     g = torch.Generator().manual_seed(6)
