@@ -120,6 +120,44 @@ def test_decode_step_over_the_chosen_prefix(t_new, t_own, d):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("batch", [1, 33])
+def test_decode_right_behind_the_kernel_that_writes_its_lengths(batch):
+    # offsets, shot counts and a workspace of arbitrary content, written on the stream right in front of every call
+    nl, t_own = 1, 70
+    w = wl.CONFIGS["cfg2"].scaled(n_shots=40, len_lo=20, len_hi=200, batch=batch, k=20, probes=(20,), t_q=t_own, seed=77,
+                                  n_q_heads=4, n_kv_heads=1)
+    ab, pool, qs, sel_np, off_np, model, cap, kc, vc, off = _setup(w, nl, 14)
+    dev_pool = hp.dev_pool(ab, pool)
+    kc.normal_(), vc.normal_()                     # (whatever the lengths, every position holds a number)
+    q_new = qs["q"][:, :, 0, t_own - 1:].contiguous().cuda()
+    k_own, v_own = qs["kq"][:, :, 0].contiguous().cuda(), qs["vq"][:, :, 0].contiguous().cuda()
+    rng = np.random.default_rng(15)
+    sels = [torch.from_numpy(np.stack([rng.permutation(w.n_shots)[:w.k] for _ in range(batch)]).astype(np.int32)).cuda() for _ in range(2)]
+    counts = [torch.from_numpy(rng.integers(1, w.k + 1, size=batch).astype(np.int32)).cuda() for _ in range(2)]
+    off, n_dev, st = torch.empty_like(off), torch.empty_like(counts[0]), hp.new_status()
+    ws = torch.empty(ab.adapshot_decode_workspace_bytes(model, batch, 1, t_own, nl), dtype=torch.uint8, device="cuda")
+
+    def step(i, out, wait):
+        n_dev.copy_(counts[i])
+        ws.random_(0, 256)
+        ab.adapshot_assemble_kv(model, dev_pool, sels[i], 0, nl, None, None, cap, off, st)        # the plan alone
+        if wait:
+            torch.cuda.synchronize()
+        ab.adapshot_decode_attn(model, kc, vc, cap, off, w.k, n_dev, q_new, k_own, v_own, 0, nl, out, None, ws, st)
+
+    want = [torch.empty_like(q_new) for _ in range(2)]
+    for i in range(2):
+        step(i, want[i], True)
+    torch.cuda.synchronize()
+    got = [torch.zeros_like(q_new) for _ in range(10)]
+    for i, out in enumerate(got):
+        step(i % 2, out, False)
+    torch.cuda.synchronize()
+    assert not torch.equal(want[0], want[1])
+    assert all(torch.equal(out, want[i % 2]) for i, out in enumerate(got))
+
+
+@pytest.mark.gpu
 def test_decode_reports_a_shot_count_outside_the_selection():
     nl = 1
     w = wl.CONFIGS["cfg2"].scaled(n_shots=16, len_lo=5, len_hi=20, batch=2, k=6, probes=(6,), t_q=4, seed=75)
