@@ -633,6 +633,14 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   if (warp == 0) {
     tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
     tmem_relinquish();
+  } else if (warp == 3) {                    // the maps the mode uses: parameters of the kernel, so ahead of the wait
+    if (lane == 0) tma_prefetch_desc(&tm_q);
+    if (lane == 1) tma_prefetch_desc(&tm_kown);
+    if (lane == 2) tma_prefetch_desc(&tm_vown);
+    if (lane == 3 && !FUSED) tma_prefetch_desc(&tm_kctx);
+    if (lane == 4 && MODE == kModeCache) tma_prefetch_desc(&tm_vctx);
+    if (lane >= 8 && lane < 16 && MODE != kModeCache) tma_prefetch_desc(&vmaps.m[lane - 8]);
+    if (lane >= 16 && lane < 24 && FUSED) tma_prefetch_desc(&kmaps.m[lane - 16]);
   }
   ads_dependency_wait();
   // the CTA's part of the schedule, fetched by two warps while the rest is set up
@@ -698,7 +706,6 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         ++n_pub;
         return true;
       };
-      tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_kctx); tma_prefetch_desc(&tm_vctx);
       uint32_t tk = 0, tv = 0, nq[2] = {0, 0};
       Item w, next;
       bool ok = publish(w);
@@ -975,11 +982,6 @@ attn_main_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     uint32_t tv = 0;
     bool ok = true;
     Item w;
-    if (lane == 0) {
-      tma_prefetch_desc(own_map);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) tma_prefetch_desc(&maps->m[e]);
-    }
     for (uint32_t n_item = 0; ok && read_item(n_item, w, ok, true); ++n_item) {
       for (int i = 0; i < w.n_tiles; ++i, ++tv, phase ^= (sv + 1 == n_st), sv = sv + 1 == n_st ? 0 : sv + 1) {
         const uint32_t v_dst = tiles0 + sv * kTileBytes;
@@ -1351,12 +1353,12 @@ struct CombineParams {
   __nv_bfloat16* out;   // [B][nl][P][Tq][Hq][D]
   float* lse;           // [B][nl][P][Hq][Tq] or null
   int Tq, Hq, G, n_mp;
-  int nx, ny, blocks;         // its grid: nx units, ny groups of rows, D / (16 kCombineSteps) column steps; in all
-  AdsEntropyJob ent;          // the entropy's second step: a block per group of rows behind them
+  int units;                  // of the grid (units, groups of rows, column steps); the blocks beyond them:
+  AdsEntropyJob ent;          // the entropy's second step, a block per group of rows
 };
 
 constexpr int kCombineRows = 8;      // rows per warp
-constexpr int kCombineSteps = 2;     // 16-column steps per warp (other blocks cover the rest)
+constexpr int kCombineSteps = 2;     // 16-column steps per warp (blockIdx.z covers the others)
 
 // Block x merges the x-th of the units that a range boundary cut (listed by the schedule block, so that
 // nothing has to be searched for here).  Latency- and L2-bound: one query of one layer (26 MB of partials)
@@ -1367,19 +1369,19 @@ constexpr int kCombineSteps = 2;     // 16-column steps per warp (other blocks c
 template <int D>
 __global__ void __launch_bounds__(256) attn_combine_kernel(const __grid_constant__ CombineParams p) {
   ads_dependency_wait();
-  if ((int)blockIdx.x >= p.blocks) {
+  if ((int)blockIdx.x >= p.units) {
     __shared__ float sh_h[kMaxProbes];               // (a group is a query's probes)
+    if (blockIdx.y != 0 || blockIdx.z != 0) return;
     ent_finish_block(p.ent.partial, p.ent.n_split, p.ent.R, p.ent.rows_per_group, p.ent.tau, p.ent.H, p.ent.first_ok,
-                     (int)blockIdx.x - p.blocks, sh_h);
+                     (int)blockIdx.x - p.units, sh_h);
     return;
   }
-  const int bx = blockIdx.x % p.nx, byz = blockIdx.x / p.nx, by = byz % p.ny, bz = byz / p.ny;
   const Sched* sc = p.sched;
-  if (bx >= sc->n_cut) return;
-  const Sched::Cut c = sc->cut[bx];
+  if (blockIdx.x >= sc->n_cut) return;
+  const Sched::Cut c = sc->cut[blockIdx.x];
   const int lane = threadIdx.x & 31;
   const int r_sub = lane & 7, c_sub = lane >> 3;
-  const int m = (by * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kCombineRows + r_sub;
+  const int m = (blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kCombineRows + r_sub;
   if (m >= p.Tq * p.G) return;
   const int mt = m / kTileM, r = m % kTileM, mp = mt >> 1, x = mt & 1;
   const int t = m / p.G, hh = m % p.G, h = c.g * p.G + hh;
@@ -1388,7 +1390,7 @@ __global__ void __launch_bounds__(256) attn_combine_kernel(const __grid_constant
     return ((long long)(2 * (c.gang + i) + (i == 0 ? c.which : 0)) * p.n_mp + mp) * 2 + x;
   };
   const float4* o4 = reinterpret_cast<const float4*>(p.o_part);
-  const int it0 = bz * kCombineSteps;
+  const int it0 = blockIdx.z * kCombineSteps;
   float4 acc[kCombineSteps];
 #pragma unroll
   for (int it = 0; it < kCombineSteps; ++it) acc[it] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1434,7 +1436,7 @@ __global__ void __launch_bounds__(256) attn_combine_kernel(const __grid_constant
     packed.y = pack_bf16x2(acc[it].z * inv, acc[it].w * inv);
     *reinterpret_cast<uint2*>(dst + ((it0 + it) * 4 + c_sub) * 4) = packed;
   }
-  if (p.lse != nullptr && c_sub == 0 && bz == 0)
+  if (p.lse != nullptr && c_sub == 0 && blockIdx.z == 0)
     p.lse[(bpj * p.Hq + h) * p.Tq + t] = (M + log2f(lsum)) * kLn2;
 }
 
@@ -1655,12 +1657,12 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
   cp.Tq = Tq; cp.Hq = Hq; cp.G = G; cp.n_mp = pl.n_mp;
   // (at most one cut unit per range, and no more than there are units: a small call would launch mostly empty blocks)
   const long long units = (long long)B * P * nl * Hkv;
-  cp.nx = (int)(units < n_gangs ? units : n_gangs);
-  cp.ny = (Tq * G + 8 * kCombineRows - 1) / (8 * kCombineRows);
-  cp.blocks = cp.nx * cp.ny * (D / (16 * kCombineSteps));
+  cp.units = (int)(units < n_gangs ? units : n_gangs);
   cp.ent = pp.ent;
   const int finish = cp.ent.blocks > 0 ? cp.ent.R / cp.ent.rows_per_group : 0;
-  ads_launch_dependent(attn_combine_kernel<D>, (unsigned)(cp.blocks + finish), 256, 0, st, cp);
+  const dim3 grid((unsigned)(cp.units + finish), (unsigned)((Tq * G + 8 * kCombineRows - 1) / (8 * kCombineRows)),
+                  D / (16 * kCombineSteps));
+  ads_launch_dependent(attn_combine_kernel<D>, grid, 256, 0, st, cp);
   return ads_launch_status();
 }
 
