@@ -101,50 +101,50 @@ __device__ __forceinline__ void mma_f64(double (&c)[4], const double (&a)[4], co
                : "d"(a[0]), "d"(a[1]), "d"(a[2]), "d"(a[3]), "d"(b[0]), "d"(b[1]));
 }
 
-// The same for batches: a CTA takes 32 shots and 8 NB queries, its eight warps share the embedding's length
+// The same for batches: a CTA takes 16 RB shots and 8 NB queries, its eight warps share the embedding's length
 // and are summed in a fixed order through shared memory.  Bound by the fp64 units; the operands come straight
 // from memory as fp32 (a lane's four consecutive elements are the k slots lane % 4 and lane % 4 + 4 of two
-// instructions), so an element is widened once per 16 queries or 32 shots instead of once per product, which is
+// instructions), so an element is widened once per 8 NB queries or 16 RB shots instead of once per product, which is
 // what the warp-per-shot form above spends its time on.  Norms are summed from the same registers.  E % 16 == 0.
-// (20000 shots x 768, 16 queries: 140 -> 26 us; 8192 x 1024, 32 queries: 115 -> 27 us.)
+// (20000 shots x 768, 16 queries: 140 -> 24 us; 8192 x 1024, 32 queries: 115 -> 25 us.)
 constexpr int kMmaWarps = 8;
-template <int NB>
-__global__ void __launch_bounds__(32 * kMmaWarps, 2)
+template <int NB, int RB>
+__global__ void __launch_bounds__(32 * kMmaWarps, RB == 2 ? 2 : 3)
 cosine_mma_kernel(const float* __restrict__ emb, const float* __restrict__ q_emb, int N, int E, int B,
                   unsigned long long* __restrict__ keys) {
-  __shared__ double dot_s[kMmaWarps][8 * NB][33];
-  __shared__ double nn_s[kMmaWarps][32], qq_s[kMmaWarps][8 * NB];
+  __shared__ double dot_s[kMmaWarps][8 * NB][16 * RB + 1];
+  __shared__ double nn_s[kMmaWarps][16 * RB], qq_s[kMmaWarps][8 * NB];
   ads_dependency_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
-  const int row0 = blockIdx.x * 32, q0 = blockIdx.y * 8 * NB;
+  const int row0 = blockIdx.x * 16 * RB, q0 = blockIdx.y * 8 * NB;
   const int steps = E / 16, s0 = warp * steps / kMmaWarps, s1 = (warp + 1) * steps / kMmaWarps;
-  const float4* ap[4];
+  const float4* ap[2 * RB];
   const float4* bp[NB];
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+  for (int r = 0; r < 2 * RB; ++r)
     ap[r] = reinterpret_cast<const float4*>(emb + (long long)min(row0 + 8 * r + g, N - 1) * E) + s0 * 4 + t;
 #pragma unroll
   for (int n = 0; n < NB; ++n)
     bp[n] = reinterpret_cast<const float4*>(q_emb + (long long)min(q0 + 8 * n + g, B - 1) * E) + s0 * 4 + t;
-  double c[2][NB][4] = {}, nn[4] = {}, qq[NB] = {};
-  float4 av[4], bv[NB];
+  double c[RB][NB][4] = {}, nn[2 * RB] = {}, qq[NB] = {};
+  float4 av[2 * RB], bv[NB];
   auto load = [&]() {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) { av[r] = __ldg(ap[r]); ap[r] += 4; }
+    for (int r = 0; r < 2 * RB; ++r) { av[r] = __ldg(ap[r]); ap[r] += 4; }
 #pragma unroll
     for (int n = 0; n < NB; ++n) { bv[n] = __ldg(bp[n]); bp[n] += 4; }
   };
   if (s0 < s1) load();
   for (int s = s0; s < s1; ++s) {
-    double a[4][4], b[NB][4];
+    double a[2 * RB][4], b[NB][4];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) { a[r][0] = av[r].x; a[r][1] = av[r].y; a[r][2] = av[r].z; a[r][3] = av[r].w; }
+    for (int r = 0; r < 2 * RB; ++r) { a[r][0] = av[r].x; a[r][1] = av[r].y; a[r][2] = av[r].z; a[r][3] = av[r].w; }
 #pragma unroll
     for (int n = 0; n < NB; ++n) { b[n][0] = bv[n].x; b[n][1] = bv[n].y; b[n][2] = bv[n].z; b[n][3] = bv[n].w; }
     if (s + 1 < s1) load();
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < 2 * RB; ++r)
 #pragma unroll
       for (int e = 0; e < 4; ++e) nn[r] += a[r][e] * a[r][e];
 #pragma unroll
@@ -154,7 +154,7 @@ cosine_mma_kernel(const float* __restrict__ emb, const float* __restrict__ q_emb
 #pragma unroll
     for (int h = 0; h < 2; ++h)
 #pragma unroll
-      for (int m = 0; m < 2; ++m)
+      for (int m = 0; m < RB; ++m)
 #pragma unroll
         for (int n = 0; n < NB; ++n) {
           const double aa[4] = {a[2 * m][2 * h], a[2 * m + 1][2 * h], a[2 * m][2 * h + 1], a[2 * m + 1][2 * h + 1]};
@@ -163,13 +163,13 @@ cosine_mma_kernel(const float* __restrict__ emb, const float* __restrict__ q_emb
         }
   }
 #pragma unroll
-  for (int m = 0; m < 2; ++m)
+  for (int m = 0; m < RB; ++m)
 #pragma unroll
     for (int n = 0; n < NB; ++n)
 #pragma unroll
       for (int e = 0; e < 4; ++e) dot_s[warp][8 * n + 2 * t + (e & 1)][16 * m + 8 * (e >> 1) + g] = c[m][n][e];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
+  for (int r = 0; r < 2 * RB; ++r) {
     nn[r] += __shfl_xor_sync(0xffffffffu, nn[r], 1);
     nn[r] += __shfl_xor_sync(0xffffffffu, nn[r], 2);
     if (t == 0) nn_s[warp][8 * r + g] = nn[r];
@@ -181,8 +181,8 @@ cosine_mma_kernel(const float* __restrict__ emb, const float* __restrict__ q_emb
     if (t == 0) qq_s[warp][8 * n + g] = qq[n];
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < 32 * 8 * NB; i += 32 * kMmaWarps) {
-    const int r = i & 31, q = i >> 5;
+  for (int i = threadIdx.x; i < 16 * RB * 8 * NB; i += 32 * kMmaWarps) {
+    const int r = i % (16 * RB), q = i / (16 * RB);
     if (row0 + r >= N || q0 + q >= B) continue;
     double d = 0.0, n2 = 0.0, q2 = 0.0;
 #pragma unroll
@@ -541,11 +541,16 @@ extern "C" int adapshot_select(const adapshot_pool_t* pool, const float* q_emb, 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   unsigned long long* keys = static_cast<unsigned long long*>(ws);
   if (B > 2 && E % 16 == 0) {          // (4096 x 384: 4.7 us for two queries by warps, 3.4 for four by matrix tiles)
-    const unsigned rows = (unsigned)((N + 31) / 32);
-    if (B <= 8)
-      ads_launch_dependent(cosine_mma_kernel<1>, dim3(rows, 1), 32 * kMmaWarps, 0, st, pool->emb, q_emb, N, E, B, keys);
-    else
-      ads_launch_dependent(cosine_mma_kernel<2>, dim3(rows, (unsigned)((B + 15) / 16)), 32 * kMmaWarps, 0, st, pool->emb, q_emb, N, E, B, keys);
+    auto run = [&](auto kernel, int rows, int queries) {
+      ads_launch_dependent(kernel, dim3((unsigned)((N + rows - 1) / rows), (unsigned)((B + queries - 1) / queries)), 32 * kMmaWarps, 0, st,
+                           pool->emb, q_emb, N, E, B, keys);
+    };
+    // 16 shots per CTA (three per SM) leave a shorter last wave than 32 (two per SM): 20000 x 768, 16 queries 41.1 -> 39.1 us for the
+    // call, 8192 x 1024, 32 queries 35.2 -> 33.0, 40000 x 384, 32 queries 75.8 -> 72.3.  Up to 8 queries the element widened once per 32
+    // shots matters as much, unless there are SMs to fill: 2048 x 1024, 8 queries 10.5 -> 9.4, 4096 x 1024 13.3 / 13.6, 30000 x 768 35.1 / 35.9.
+    if (B > 8) run(cosine_mma_kernel<2, 1>, 16, 16);
+    else if (N <= 3000) run(cosine_mma_kernel<1, 1>, 16, 8);
+    else run(cosine_mma_kernel<1, 2>, 32, 8);
   } else {
     const unsigned grid = (unsigned)((N + 7) / 8);
     auto run = [&](auto kernel) { ads_launch_dependent(kernel, grid, 256, 0, st, pool->emb, q_emb, N, E, B, keys); };
