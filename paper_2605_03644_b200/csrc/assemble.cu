@@ -515,8 +515,7 @@ extern "C" int adapshot_assemble_kv_from(const adapshot_model_t* model, const ad
   a.layer_begin = layer_begin; a.n_layers_call = layer_end - layer_begin;
   a.shot_begin = shot_begin;
   a.k_pos_mode = model->k_pos_mode; a.status = status;
-  for (int i = 0; i < model->head_dim / 2; ++i)
-    a.theta[i] = pow(model->rope_base, -2.0 * (double)i / (double)model->head_dim);
+  memcpy(a.theta, ads_theta(model->rope_base, model->head_dim), model->head_dim / 2 * sizeof(double));
 
   const bool f32 = model->dtype == ADAPSHOT_F32;
   if (model->head_dim == 128)
