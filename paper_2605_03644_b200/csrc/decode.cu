@@ -38,6 +38,7 @@ constexpr int kMaxB = 256;
 constexpr int kMaxCtas = 320;                // two per SM, at most this many
 constexpr int kUnitCost = 1;                 // fixed cost of a unit (rotate Q, merge the warps), in tiles
 constexpr int kMinRange = 3;                 // shortest range, in tiles (fixed cost included)
+constexpr int kPrefetchRange = 16;           // ranges of up to this many tiles have their first ones prefetched (32 long requests: 536.7 with, 535.2 without)
 constexpr int kPrefetchTiles = 3;            // of a range, brought to L2 ahead (none / 3 / 6 / 12: 67.1 / 63.9 / 64 / 64 us; 32 requests 537 / 537 / 538 / 541)
 constexpr int kRows = 32;                    // rows a partial has room for
 constexpr int kMergeRows = 4;                // rows whose states the warps merge at a time
@@ -259,7 +260,7 @@ decode_rows_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   if (warp == 0) lengths(true);
   __syncthreads();
   find_range();
-  if (threadIdx.x == 32 * kWarps) {
+  if (threadIdx.x == 32 * kWarps && x1 - x0 <= kPrefetchRange) {
     int left = kPrefetchTiles;
     walk([&](int b, int l, int g, int t0, int t1, int, int n_ctx, bool) {
       for (int t = t0; t < min(t1, n_ctx) && left > 0; ++t, --left)
@@ -564,7 +565,8 @@ decode_rows_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
 // 37 pieces per head, one of a single head into up to one per CTA: eight warps take every eighth piece each, five at a
 // time with their loads in flight at once, and meet in shared memory.
 constexpr int kMergeWarps = 8;
-template <int D>
+// AHEAD: see below.
+template <int D, bool AHEAD>
 __global__ void __launch_bounds__(32 * kMergeWarps) decode_combine_kernel(const __grid_constant__ DecodeParams p) {
   __shared__ float4 o_s[kMergeWarps][D / 4];
   __shared__ float2 ml_s[kMergeWarps];
@@ -598,30 +600,40 @@ __global__ void __launch_bounds__(32 * kMergeWarps) decode_combine_kernel(const 
       }
     }
   };
-  // Where the pieces lie follows from the lengths, which the kernel in front wrote when it began: read past the L1 as a guess
-  // before the wait, so that behind it the lengths and the pieces are fetched together instead of one after the other
-  // (63.6 -> 57.9 us for the four calls above).
-  // (Whatever lies there: 0 <= begin < end <= total < 2^31 keeps every range and so every address of the guess within bounds.)
-  p0 = __ldcg(p.prefix + b);
-  const long long p1 = __ldcg(p.prefix + b + 1);
-  total = __ldcg(p.prefix + p.B);
-  const bool guess = 0 <= p0 && p0 < p1 && p1 <= total && total < (1ll << 31);
-  len = guess ? p1 - p0 : 0;
-  if (guess) find();
-  ads_dependency_wait();
-  const long long q0 = p.prefix[b], q1 = p.prefix[b + 1], q2 = p.prefix[p.B];
-  if (guess && c0 < c1) fetch(c0 + warp);
-  if (!guess || q0 != p0 || q1 - q0 != len || q2 != total) {
-    p0 = q0;
-    len = q1 - q0;
-    total = q2;
+  if constexpr (AHEAD) {
+    // Where the pieces lie follows from the lengths, which the kernel in front wrote when it began: read past the L1 as a guess
+    // before the wait, so that behind it the lengths and the pieces are fetched together instead of one after the other
+    // (63.7 -> 58.4 us for four calls of one request of 12 K tokens; with more blocks than the GPU holds at a time the registers this
+    // takes cost more: 32 requests 537 -> 542).  Whatever lies there: 0 <= begin < end <= total < 2^31 keeps every range and so every
+    // address of the guess within bounds.
+    p0 = __ldcg(p.prefix + b);
+    const long long p1 = __ldcg(p.prefix + b + 1);
+    total = __ldcg(p.prefix + p.B);
+    const bool guess = 0 <= p0 && p0 < p1 && p1 <= total && total < (1ll << 31);
+    len = guess ? p1 - p0 : 0;
+    if (guess) find();
+    ads_dependency_wait();
+    const long long q0 = p.prefix[b], q1 = p.prefix[b + 1], q2 = p.prefix[p.B];
+    if (guess && c0 < c1) fetch(c0 + warp);
+    if (!guess || q0 != p0 || q1 - q0 != len || q2 != total) {
+      p0 = q0;
+      len = q1 - q0;
+      total = q2;
+      find();
+      if (c0 < c1) fetch(c0 + warp);
+    }
+  } else {
+    ads_dependency_wait();
+    p0 = p.prefix[b];
+    len = p.prefix[b + 1] - p0;
+    total = p.prefix[p.B];
     find();
-    if (c0 < c1) fetch(c0 + warp);
   }
   if (c0 >= c1) return;                             // one range held all of them and stored the result
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   float M = kNegSentinel, lsum = 0.f;
-  for (int i = c0 + warp;;) {
+  for (int i = c0 + warp; i <= c1; i += 5 * kMergeWarps) {
+    if (!AHEAD || i != c0 + warp) fetch(i);
     float m_new = M;
 #pragma unroll
     for (int e = 0; e < 5; ++e) m_new = fmaxf(m_new, ml[e].x);
@@ -635,9 +647,6 @@ __global__ void __launch_bounds__(32 * kMergeWarps) decode_combine_kernel(const 
       lsum += ml[e].y * w;
       acc.x += v[e].x * w; acc.y += v[e].y * w; acc.z += v[e].z * w; acc.w += v[e].w * w;
     }
-    i += 5 * kMergeWarps;
-    if (i > c1) break;
-    fetch(i);
   }
   if (lane < D / 4) o_s[warp][lane] = acc;
   if (lane == 0) ml_s[warp] = make_float2(M, lsum);
@@ -683,7 +692,8 @@ int launch(const CUtensorMap* m, const DecodeParams& p, cudaStream_t st) {
   ads_launch_dependent(decode_rows_kernel<D, MB>, (unsigned)p.n_cta, kThreads, smem, st, m[0], m[1], m[2], m[3], p);
   if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
   const dim3 grid((unsigned)((long long)p.B * p.nl * p.Hkv), (unsigned)p.rows);
-  ads_launch_dependent(decode_combine_kernel<D>, grid, 32 * kMergeWarps, 0, st, p);
+  if ((long long)grid.x * grid.y <= 2ll * p.n_cta) ads_launch_dependent(decode_combine_kernel<D, true>, grid, 32 * kMergeWarps, 0, st, p);
+  else ads_launch_dependent(decode_combine_kernel<D, false>, grid, 32 * kMergeWarps, 0, st, p);
   return ads_launch_status();
 }
 
