@@ -413,10 +413,10 @@ def measure(args, name: str, steps: int, warmup: int, dev, peaks, dist, rank: in
     del qs
     flush = torch.empty(L2_FLUSH_BYTES, dtype=torch.uint8, device=dev)
     n_sel = 2             # scores as sort keys, top-k
-    if fused or vpool:
-        launches_per_step = n_sel + 1 + len(path.chunks) * ((1 if vpool else 0) + 4) + 2
-    else:
-        launches_per_step = n_sel + 1 + len(path.chunks) * (1 + 3) + 2
+    # per chunk: gather (none without a cache), preparation, main and merge; the entropy of up to 16 MB of logits has no launches of
+    # its own in a pass that is one call
+    beside = not path.entropy_overlap and logits.numel() * logits.element_size() <= 16 << 20
+    launches_per_step = n_sel + 1 + len(path.chunks) * (3 if fused else 4) + (0 if beside else 2)
 
     use_graph = args.graph == "on" or (args.graph == "auto" and w.n_layers == 1)
     if use_graph:
@@ -644,6 +644,7 @@ def measure(args, name: str, steps: int, warmup: int, dev, peaks, dist, rank: in
                    "ctx_cap": ctx_cap, "layers_per_call": lpc, "layer_chunks": [le - lb for lb, le in path.chunks],
                    "gather_overlaps_attention": path.overlap,
                    "entropy": "side stream, overlapped with the pass" if path.entropy_overlap
+                   else "beside the last attention call (its logits are an input)" if beside
                    else "after the last attention call (serial)",
                    "l2": "flushed between steps (512 MiB write)"})
     res = {

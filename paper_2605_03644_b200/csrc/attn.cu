@@ -19,7 +19,7 @@
 //                 memory into whole row segments); a range that cuts a unit stores
 //                 un-normalised partials;
 //   attn_combine  log-sum-exp merge of the partials of the cut units.
-// Two variants take tiles straight from the pool, through a row map written once per call (attn_row_map): the
+// Two variants take tiles straight from the pool, through a row map that the preparation writes once per call: the
 // V-from-pool variant (adapshot_query_attn_vpool) reads K from a cache that holds the re-encoded K only and
 // V, which Eq. 7 leaves as it is, from the pool, so that the gather moves half the bytes; the fused variant
 // (adapshot_query_attn_fused) reads both from the pool and re-encodes K (Eq. 7) in shared memory.  One warp per
