@@ -359,7 +359,9 @@ ADAPSHOT_API int adapshot_entropy_static(const void* logits, int32_t dtype, int3
  * pointers, layer_end HOST int32 [n_chunks] (ascending, chunk i begins where chunk i-1 ends).
  * k_ctx / v_ctx hold one chunk at a time.  variant: ADAPSHOT_PASS_FULL (K and V assembled),
  * _VPOOL (K only, V from the pool; v_ctx unused) or _FUSED (nothing assembled).  The struct is
- * read during the call only.  Returns the first error; steps before it have been enqueued.   */
+ * read during the call only.  Returns the first error; steps before it have been enqueued.
+ * The entropy of up to 16 MB of logits runs beside the last attention call (the logits are an
+ * input); where its buffers share memory with the pass's, after it.                          */
 #define ADAPSHOT_PASS_FULL  0
 #define ADAPSHOT_PASS_VPOOL 1
 #define ADAPSHOT_PASS_FUSED 2

@@ -87,8 +87,9 @@ class ReusePath:
         self.ws_attn = torch.empty(max(256, ws_fn(model, batch, self.P, t_q, self.lpc, self.ctx_cap)), **u8)
         self.ws_entropy = torch.empty(max(256, ab.adapshot_entropy_workspace_bytes(batch * self.P, vocab)), **u8)
         # In the method the probe's logits come out of the model after the probe attention (Eq. 2
-        # follows Eq. 1), so the entropy step runs after the last attention call.  With
-        # entropy_overlap=True it runs on a second stream beside the pass instead (for callers
+        # follows Eq. 1), so a driver that steps through the calls ends with the entropy.  run() is given them
+        # with the queries: up to 16 MB of them go beside the last attention call, more after it.  With
+        # entropy_overlap=True the step runs on a second stream beside the pass instead (for callers
         # whose logits are already there, e.g. those of the previous round of probes).
         self.entropy_overlap = bool(entropy_overlap)
         self.side = torch.cuda.Stream(device=device)
