@@ -515,7 +515,7 @@ extern "C" int adapshot_assemble_kv_from(const adapshot_model_t* model, const ad
   a.layer_begin = layer_begin; a.n_layers_call = layer_end - layer_begin;
   a.shot_begin = shot_begin;
   a.k_pos_mode = model->k_pos_mode; a.status = status;
-  memcpy(a.theta, ads_theta(model->rope_base, model->head_dim), model->head_dim / 2 * sizeof(double));
+  ads_rope_theta(model->rope_base, model->head_dim, a.theta);
 
   const bool f32 = model->dtype == ADAPSHOT_F32;
   if (model->head_dim == 128)

@@ -1604,7 +1604,7 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
   pp.sched = sched; pp.ctx_cap = ctx_cap;
   pp.B = B; pp.k = k; pp.P = P; pp.Tq = Tq; pp.Hq = Hq; pp.Hkv = Hkv; pp.nl = nl; pp.n_gangs = n_gangs;
   pp.To = To; pp.nshots_dev = extra.nshots_dev; pp.status = status;
-  memcpy(pp.theta, ads_theta(model->rope_base, D), D / 2 * sizeof(double));
+  ads_rope_theta(model->rope_base, D, pp.theta);
   for (int i = 0; i < kMaxProbes; ++i) pp.nshots[i] = i < P ? probe_nshots[i] : 0;
   const long long n_tok = (long long)B * nl * P * To;
   const long long n_groups = (n_tok * kPrepParts + 7) / 8;

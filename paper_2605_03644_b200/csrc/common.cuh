@@ -3,11 +3,10 @@
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
-#include <math.h>
 #include <stdint.h>
-#include <string.h>
 
 #include "adapshot.h"
+#include "rope_theta.h"
 
 #define ADAPSHOT_VERSION_NUMBER 100
 
@@ -57,23 +56,6 @@ static inline int ads_set_max_smem(Kernel kernel, int bytes, bool* done) {
     done[dev] = true;
   }
   return ADAPSHOT_OK;
-}
-
-// theta_i = rope_base^(-2i/D), i < D/2 <= 64.  A thread keeps the table it formed last: 64 calls of pow are some 3 us of host time, a
-// sixth of what a small decode call takes there (one short request, four calls: 48.6 -> 45.5 us).
-static inline const double* ads_theta(double rope_base, int D) {
-  struct Table {
-    double base = 0.0;
-    int D = 0;
-    double theta[64];
-  };
-  static thread_local Table t;
-  if (t.base != rope_base || t.D != D) {
-    for (int i = 0; i < D / 2; ++i) t.theta[i] = pow(rope_base, -2.0 * (double)i / (double)D);
-    t.base = rope_base;
-    t.D = D;
-  }
-  return t.theta;
 }
 
 // Programmatic dependent launch: the kernel may be started while the one in front of it in the stream still

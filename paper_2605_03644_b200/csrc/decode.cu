@@ -743,7 +743,7 @@ int ads_decode_rows(const adapshot_model_t* model, const void* k_ctx, const void
   p.n_cta = 2 * n_sm < kMaxCtas ? 2 * n_sm : kMaxCtas;
   const float scale = model->softmax_scale > 0.f ? model->softmax_scale : 1.0f / sqrtf((float)D);
   p.scale_log2 = scale * 1.4426950408889634f;
-  memcpy(p.theta, ads_theta(model->rope_base, D), D / 2 * sizeof(double));
+  ads_rope_theta(model->rope_base, D, p.theta);
 
   CUtensorMap m[4];
   const void* src[4] = {k_ctx, v_ctx, k_own, v_own};
