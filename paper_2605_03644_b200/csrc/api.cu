@@ -32,9 +32,9 @@ bool meet(const void* a, size_t na, const void* b, size_t nb) {
 // is bound by bandwidth on either side.
 constexpr size_t kBesideBytes = 16u << 20;
 
-// Whether the entropy of a pass may run beside its last attention call instead of behind it: a valid call whose logits and
-// states share no memory with what the pass writes or the attention still reads from its workspace (one workspace for every
-// step is fine for calls in turn), nor its results with what the pass reads.
+// Whether the entropy of a pass may run beside its last attention call instead of behind it: a valid call whose logits, states
+// and results share no memory with what that attention call still reads (the pool among it, where it takes tiles from there) or
+// writes.  Calls in turn may share it, one workspace for every step for instance.
 bool entropy_beside(const adapshot_pass_t* p, AdsEntropyJob* job) {
   if (p->model == nullptr || p->B <= 0 || p->P <= 0 || p->Tq <= 0 || p->V <= 0) return false;
   if (ads_entropy_job(p->logits, p->logits_dtype, p->B * p->P, p->V, p->logits_stride, p->H, p->tau, p->P, p->first_ok,
@@ -53,6 +53,7 @@ bool entropy_beside(const adapshot_pass_t* p, AdsEntropyJob* job) {
   if (nl <= 0) return false;
   const size_t tok = rows * nl * (size_t)p->Tq, row_kv = (size_t)p->model->n_kv_heads * p->model->head_dim * 2;
   const size_t cache = (size_t)p->B * nl * (size_t)p->ctx_cap * row_kv;
+  const size_t pool_bytes = (size_t)p->model->n_layers * (size_t)p->pool->pool_tokens * row_kv;
   for (const auto& m : mine) {
     if (meet(m.at, m.n, p->ws_attn, p->ws_attn_bytes) || meet(m.at, m.n, p->out[last], tok * row_q) ||
         meet(m.at, m.n, p->q[last], tok * row_q) || meet(m.at, m.n, p->kq[last], tok * row_kv) ||
@@ -61,6 +62,10 @@ bool entropy_beside(const adapshot_pass_t* p, AdsEntropyJob* job) {
       return false;
     if (p->variant != ADAPSHOT_PASS_FUSED && meet(m.at, m.n, p->k_ctx, cache)) return false;
     if (p->variant == ADAPSHOT_PASS_FULL && meet(m.at, m.n, p->v_ctx, cache)) return false;
+    if (p->variant != ADAPSHOT_PASS_FULL &&
+        (meet(m.at, m.n, p->pool->v, pool_bytes) || meet(m.at, m.n, p->pool->shot_off, ((size_t)p->pool->n_shots + 1) * 8)))
+      return false;
+    if (p->variant == ADAPSHOT_PASS_FUSED && meet(m.at, m.n, p->pool->k, pool_bytes)) return false;
   }
   return true;
 }

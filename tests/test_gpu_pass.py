@@ -132,6 +132,23 @@ def test_entropy_beside_the_attention_equals_its_own_call(variant, vocab, dtype)
         assert all(torch.equal(a, b) for a, b in zip(out, steps.out))
 
 
+@pytest.mark.parametrize("variant,tensor", [("vpool", "v"), ("fused", "v"), ("fused", "k")])
+def test_entropy_states_in_the_pool_do_not_meet_the_attention(variant, tensor):
+    # a workspace that lies on a selected shot of the last layer: written after the attention has read the shot
+    w = _workload(48).scaled(vocab=20003, t_q=70)
+    path = _path(w, variant)
+    args = list(_inputs(path, wl.make_queries(w)))
+    args[4] = torch.nn.functional.pad(args[4], (0, 20008 - w.vocab))[:, :w.vocab]
+    want = [t.clone() for t in path.run(*args)[0]]
+    want_H, want_ok = path.H.clone(), path.first_ok.clone()
+    shot = path.sel_idx[0, 0].item()
+    path.ws_entropy = getattr(path.pool, tensor)[w.n_layers - 1, path.pool.shot_off[shot].item():].flatten().view(torch.uint8)
+    got, H, ok = path.run(*args)
+    torch.cuda.synchronize()
+    assert path.status.item() == 0 and torch.equal(H, want_H) and torch.equal(ok, want_ok)
+    assert all(torch.equal(a, b) for a, b in zip(want, got))
+
+
 @pytest.mark.parametrize("batch", [1, 2])
 def test_rounds_of_probes_use_the_tensors_they_have_now(batch):
     from paper_2605_03644_b200 import binding as ab
