@@ -59,6 +59,7 @@ struct DecodeParams {
   int32_t* status;
   long long ctx_cap;
   int B, k, Hq, Hkv, G, nl, T_new, T_own, rows, n_cta;
+  int ahead;                   // whether lengths, ranges and first tiles are taken ahead of the dependency wait
   float scale_log2;
   double theta[64];
 };
@@ -210,14 +211,25 @@ decode_rows_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
       }
     }
   };
-  // Whether the guess holds: both loads of a request at once, instead of one after the other.
+  // Whether the guess holds: both loads of every request at once, instead of one after the other.
   auto guess_holds = [&]() -> bool {
+    int n[kMaxB / 32];
+    long long L[kMaxB / 32];
+#pragma unroll
+    for (int e = 0; e < kMaxB / 32; ++e) {
+      const int b = e * 32 + lane;
+      if (e * 32 >= p.B) break;
+      if (b < p.B) {
+        n[e] = p.n_shots[b];
+        L[e] = p.ctx_off[(long long)b * (p.k + 1) + n_s[b]];
+      }
+    }
     bool same = true;
-    for (int b = lane; b < p.B; b += 32) {
-      const int n = n_s[b];
-      const int is = p.n_shots[b];
-      const long long L = p.ctx_off[(long long)b * (p.k + 1) + n];
-      same = same && is == n && clamp_len(L) == len_s[b];
+#pragma unroll
+    for (int e = 0; e < kMaxB / 32; ++e) {
+      const int b = e * 32 + lane;
+      if (e * 32 >= p.B) break;
+      if (b < p.B) same = same && n[e] == n_s[b] && clamp_len(L[e]) == len_s[b];
     }
     return same;
   };
@@ -257,10 +269,12 @@ decode_rows_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   // before the wait, so the lengths are a guess until then, right unless one of those kernels changes them.  (From the wait to the
   // first copy 3.3 us when everything followed it, 1.0 now; four calls of one request of 12 K tokens 68.2 -> 63.6 us.  Forming the angles
   // of Q here as well is slower, 70.8: the CTAs enter too late for it to be hidden.)
-  if (warp == 0) lengths(true);
-  __syncthreads();
-  find_range();
-  if (threadIdx.x == 32 * kWarps && x1 - x0 <= kPrefetchRange) {
+  if (p.ahead) {
+    if (warp == 0) lengths(true);
+    __syncthreads();
+    find_range();
+  }
+  if (threadIdx.x == 32 * kWarps && p.ahead && x1 - x0 <= kPrefetchRange) {
     int left = kPrefetchTiles;
     walk([&](int b, int l, int g, int t0, int t1, int, int n_ctx, bool) {
       for (int t = t0; t < min(t1, n_ctx) && left > 0; ++t, --left)
@@ -273,7 +287,7 @@ decode_rows_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
     });
   }
   ads_dependency_wait();
-  if (!__syncthreads_and(warp != 0 || guess_holds())) {
+  if (!p.ahead || !__syncthreads_and(warp != 0 || guess_holds())) {
     if (warp == 0) lengths(false);
     __syncthreads();
     find_range();
@@ -565,7 +579,6 @@ decode_rows_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
 // 37 pieces per head, one of a single head into up to one per CTA: eight warps take every eighth piece each, five at a
 // time with their loads in flight at once, and meet in shared memory.
 constexpr int kMergeWarps = 8;
-// AHEAD: see below.
 template <int D, bool AHEAD>
 __global__ void __launch_bounds__(32 * kMergeWarps) decode_combine_kernel(const __grid_constant__ DecodeParams p) {
   __shared__ float4 o_s[kMergeWarps][D / 4];
@@ -603,8 +616,8 @@ __global__ void __launch_bounds__(32 * kMergeWarps) decode_combine_kernel(const 
   if constexpr (AHEAD) {
     // Where the pieces lie follows from the lengths, which the kernel in front wrote when it began: read past the L1 as a guess
     // before the wait, so that behind it the lengths and the pieces are fetched together instead of one after the other
-    // (63.7 -> 58.4 us for four calls of one request of 12 K tokens; with more blocks than the GPU holds at a time the registers this
-    // takes cost more: 32 requests 537 -> 542).  Whatever lies there: 0 <= begin < end <= total < 2^31 keeps every range and so every
+    // (63.7 -> 58.4 us for four calls of one request of 12 K tokens; not with more blocks, whose registers cost more than that: 32
+    // requests 537 -> 542).  Whatever lies there: 0 <= begin < end <= total < 2^31 keeps every range and so every
     // address of the guess within bounds.
     p0 = __ldcg(p.prefix + b);
     const long long p1 = __ldcg(p.prefix + b + 1);
@@ -692,7 +705,7 @@ int launch(const CUtensorMap* m, const DecodeParams& p, cudaStream_t st) {
   ads_launch_dependent(decode_rows_kernel<D, MB>, (unsigned)p.n_cta, kThreads, smem, st, m[0], m[1], m[2], m[3], p);
   if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
   const dim3 grid((unsigned)((long long)p.B * p.nl * p.Hkv), (unsigned)p.rows);
-  if ((long long)grid.x * grid.y <= 2ll * p.n_cta) ads_launch_dependent(decode_combine_kernel<D, true>, grid, 32 * kMergeWarps, 0, st, p);
+  if (p.ahead) ads_launch_dependent(decode_combine_kernel<D, true>, grid, 32 * kMergeWarps, 0, st, p);
   else ads_launch_dependent(decode_combine_kernel<D, false>, grid, 32 * kMergeWarps, 0, st, p);
   return ads_launch_status();
 }
@@ -741,6 +754,10 @@ int ads_decode_rows(const adapshot_model_t* model, const void* k_ctx, const void
   const int n_sm = ads_sm_count();
   if (n_sm <= 0) return ADAPSHOT_ECUDA;
   p.n_cta = 2 * n_sm < kMaxCtas ? 2 * n_sm : kMaxCtas;
+  // The kernel in front of a layer's call is mostly the merge of the layer before.  With more than three of its blocks per SM this call's
+  // CTAs enter too late to hide anything, and lengths taken twice cost what they would have saved (not ahead / ahead, us per call of short
+  // contexts: 100 requests of one head 11.8 / 11.3, 148 12.3 / 12.8, 256 15.4 / 15.9; 12 of eight heads 12.9 / 12.3, 16 12.8 / 13.4, 64 22.8 / 23.6).
+  p.ahead = 2ll * B * nl * Hkv * p.rows <= 3ll * p.n_cta;
   const float scale = model->softmax_scale > 0.f ? model->softmax_scale : 1.0f / sqrtf((float)D);
   p.scale_log2 = scale * 1.4426950408889634f;
   ads_rope_theta(model->rope_base, D, p.theta);
