@@ -81,6 +81,12 @@ extern "C" int adapshot_reuse_pass(const adapshot_pass_t* p, void* stream) {
   if (rc == ADAPSHOT_OK && p->variant == ADAPSHOT_PASS_FUSED)
     rc = adapshot_assemble_kv(p->model, p->pool, p->sel_idx, p->B, p->k, 0, 1, nullptr, nullptr, p->ctx_cap, p->ctx_off, 0,
                               p->status, stream);
+  AdsPass pass = {};
+  double theta[64];
+  if (p->model != nullptr && (p->model->head_dim == 64 || p->model->head_dim == 128)) {      // (anything else is refused below)
+    ads_rope_theta(p->model->rope_base, p->model->head_dim, theta);
+    pass.theta = theta;
+  }
   // The logits are an input of the call: where nothing forbids it, their entropy runs in blocks of the last attention call's small
   // kernels (the states beside the preparation, the rule beside the merge) instead of two launches behind it.
   AdsEntropyJob job;
@@ -88,26 +94,26 @@ extern "C" int adapshot_reuse_pass(const adapshot_pass_t* p, void* stream) {
   int lb = 0;
   for (int i = 0; rc == ADAPSHOT_OK && i < p->n_chunks; ++i) {
     const int le = p->layer_end[i];
-    const AdsEntropyJob* ent = beside && i + 1 == p->n_chunks ? &job : nullptr;
+    pass.ent = beside && i + 1 == p->n_chunks ? &job : nullptr;
     if (p->variant != ADAPSHOT_PASS_FUSED) {
       const uint32_t flags = (i > 0 ? ADAPSHOT_ASSEMBLE_KEEP_PLAN : 0u) |
                              (p->variant == ADAPSHOT_PASS_VPOOL ? ADAPSHOT_ASSEMBLE_K_ONLY : 0u);
-      rc = adapshot_assemble_kv(p->model, p->pool, p->sel_idx, p->B, p->k, lb, le, p->k_ctx, p->v_ctx, p->ctx_cap,
-                                p->ctx_off, flags, p->status, stream);
+      rc = ads_assemble_kv(p->model, p->pool, p->sel_idx, p->B, p->k, 0, lb, le, p->k_ctx, p->v_ctx, p->ctx_cap,
+                           p->ctx_off, flags, p->status, stream, &pass);
       if (rc != ADAPSHOT_OK) break;
     }
     if (p->variant == ADAPSHOT_PASS_FULL)
       rc = ads_query_attn(p->model, p->k_ctx, p->v_ctx, p->ctx_cap, p->ctx_off, p->B, p->k, p->probe_nshots, p->P,
-                               p->q[i], p->kq[i], p->vq[i], p->Tq, lb, le, p->out[i], nullptr, 0, p->ws_attn,
-                               p->ws_attn_bytes, p->status, stream, ent);
+                          p->q[i], p->kq[i], p->vq[i], p->Tq, lb, le, p->out[i], nullptr, 0, p->ws_attn,
+                          p->ws_attn_bytes, p->status, stream, &pass);
     else if (p->variant == ADAPSHOT_PASS_VPOOL)
       rc = ads_query_attn_vpool(p->model, p->pool, p->sel_idx, p->k_ctx, p->ctx_cap, p->ctx_off, p->B, p->k,
-                                     p->probe_nshots, p->P, p->q[i], p->kq[i], p->vq[i], p->Tq, lb, le, p->out[i],
-                                     nullptr, 0, p->ws_attn, p->ws_attn_bytes, p->status, stream, ent);
+                                p->probe_nshots, p->P, p->q[i], p->kq[i], p->vq[i], p->Tq, lb, le, p->out[i], nullptr,
+                                0, p->ws_attn, p->ws_attn_bytes, p->status, stream, &pass);
     else
       rc = ads_query_attn_fused(p->model, p->pool, p->sel_idx, p->ctx_off, p->ctx_cap, p->B, p->k, p->probe_nshots,
-                                     p->P, p->q[i], p->kq[i], p->vq[i], p->Tq, lb, le, p->out[i], nullptr, 0,
-                                     p->ws_attn, p->ws_attn_bytes, p->status, stream, ent);
+                                p->P, p->q[i], p->kq[i], p->vq[i], p->Tq, lb, le, p->out[i], nullptr, 0, p->ws_attn,
+                                p->ws_attn_bytes, p->status, stream, &pass);
     lb = le;
   }
   if (rc != ADAPSHOT_OK || beside) return rc;

@@ -10,6 +10,8 @@
 // its few (sin, cos) pairs once per chunk, in fp64 before the fp32 sincos, and reuses them.
 #include <math.h>
 
+#include <string.h>
+
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -454,20 +456,9 @@ int launch_gather(GatherArgs a, cudaStream_t st) {
 
 }  // namespace
 
-extern "C" int adapshot_assemble_kv(const adapshot_model_t* model, const adapshot_pool_t* pool,
-                                    const int32_t* sel_idx, int32_t B, int32_t k,
-                                    int32_t layer_begin, int32_t layer_end, void* k_ctx, void* v_ctx,
-                                    int64_t ctx_cap, int64_t* ctx_off, uint32_t flags,
-                                    int32_t* status, void* stream) {
-  return adapshot_assemble_kv_from(model, pool, sel_idx, B, k, 0, layer_begin, layer_end, k_ctx, v_ctx, ctx_cap,
-                                   ctx_off, flags, status, stream);
-}
-
-extern "C" int adapshot_assemble_kv_from(const adapshot_model_t* model, const adapshot_pool_t* pool,
-                                         const int32_t* sel_idx, int32_t B, int32_t k, int32_t shot_begin,
-                                         int32_t layer_begin, int32_t layer_end, void* k_ctx, void* v_ctx,
-                                         int64_t ctx_cap, int64_t* ctx_off, uint32_t flags,
-                                         int32_t* status, void* stream) {
+int ads_assemble_kv(const adapshot_model_t* model, const adapshot_pool_t* pool, const int32_t* sel_idx, int32_t B, int32_t k,
+                    int32_t shot_begin, int32_t layer_begin, int32_t layer_end, void* k_ctx, void* v_ctx, int64_t ctx_cap,
+                    int64_t* ctx_off, uint32_t flags, int32_t* status, void* stream, const AdsPass* pass) {
   if (model == nullptr || pool == nullptr || sel_idx == nullptr || ctx_off == nullptr) return ADAPSHOT_EINVAL;
   if (shot_begin < 0 || shot_begin >= k) return ADAPSHOT_ESHAPE;
   if (B <= 0 || (flags & ~(ADAPSHOT_ASSEMBLE_KEEP_PLAN | ADAPSHOT_ASSEMBLE_K_ONLY)) != 0 ||
@@ -515,10 +506,29 @@ extern "C" int adapshot_assemble_kv_from(const adapshot_model_t* model, const ad
   a.layer_begin = layer_begin; a.n_layers_call = layer_end - layer_begin;
   a.shot_begin = shot_begin;
   a.k_pos_mode = model->k_pos_mode; a.status = status;
-  ads_rope_theta(model->rope_base, model->head_dim, a.theta);
+  if (pass != nullptr && pass->theta != nullptr) memcpy(a.theta, pass->theta, model->head_dim / 2 * sizeof(double));
+  else ads_rope_theta(model->rope_base, model->head_dim, a.theta);
 
   const bool f32 = model->dtype == ADAPSHOT_F32;
   if (model->head_dim == 128)
     return f32 ? launch_gather<float, 128>(a, st) : launch_gather<__nv_bfloat16, 128>(a, st);
   return f32 ? launch_gather<float, 64>(a, st) : launch_gather<__nv_bfloat16, 64>(a, st);
+}
+
+extern "C" int adapshot_assemble_kv(const adapshot_model_t* model, const adapshot_pool_t* pool,
+                                    const int32_t* sel_idx, int32_t B, int32_t k,
+                                    int32_t layer_begin, int32_t layer_end, void* k_ctx, void* v_ctx,
+                                    int64_t ctx_cap, int64_t* ctx_off, uint32_t flags,
+                                    int32_t* status, void* stream) {
+  return ads_assemble_kv(model, pool, sel_idx, B, k, 0, layer_begin, layer_end, k_ctx, v_ctx, ctx_cap, ctx_off, flags, status,
+                         stream, nullptr);
+}
+
+extern "C" int adapshot_assemble_kv_from(const adapshot_model_t* model, const adapshot_pool_t* pool,
+                                         const int32_t* sel_idx, int32_t B, int32_t k, int32_t shot_begin,
+                                         int32_t layer_begin, int32_t layer_end, void* k_ctx, void* v_ctx,
+                                         int64_t ctx_cap, int64_t* ctx_off, uint32_t flags,
+                                         int32_t* status, void* stream) {
+  return ads_assemble_kv(model, pool, sel_idx, B, k, shot_begin, layer_begin, layer_end, k_ctx, v_ctx, ctx_cap, ctx_off, flags,
+                         status, stream, nullptr);
 }

@@ -29,6 +29,7 @@
 // registers (16 KB in flight per SM, latency-bound), 325 us as it is now.)
 #include <cuda.h>
 #include <float.h>
+#include <string.h>
 
 #include "common.cuh"
 #include "entropy.cuh"
@@ -1480,11 +1481,11 @@ struct AttnPlan {
   size_t off_qrot, off_kqrot, off_sched, off_opart, off_ml, off_rowmap, off_offmap, total;
 };
 
-// Own tokens beyond the query rows, and a per-query shot count on the device (decode calls); an entropy call to run beside.
+// Own tokens beyond the query rows, and a per-query shot count on the device (decode calls).
 struct AttnExtra {
   int To = 0;                        // 0: as many own tokens as query rows
   const int32_t* nshots_dev = nullptr;
-  const AdsEntropyJob* ent = nullptr;      // the entropy of the probes' logits, beside the attention
+  AdsPass pass = {};                 // what a pass in one call shares
 };
 
 // What the fused variant reads instead of an assembled cache.
@@ -1585,7 +1586,7 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
   int* row_map = reinterpret_cast<int*>(wsb + pl.off_rowmap);
   int* off_map = reinterpret_cast<int*>(wsb + pl.off_offmap);
   PrepParams pp;
-  pp.ent = extra.ent != nullptr ? *extra.ent : AdsEntropyJob{};
+  pp.ent = extra.pass.ent != nullptr ? *extra.pass.ent : AdsEntropyJob{};
   pp.map = RowMapParams{};
   pp.map_blocks = 0;
   if (fused != nullptr) {
@@ -1604,7 +1605,8 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
   pp.sched = sched; pp.ctx_cap = ctx_cap;
   pp.B = B; pp.k = k; pp.P = P; pp.Tq = Tq; pp.Hq = Hq; pp.Hkv = Hkv; pp.nl = nl; pp.n_gangs = n_gangs;
   pp.To = To; pp.nshots_dev = extra.nshots_dev; pp.status = status;
-  ads_rope_theta(model->rope_base, D, pp.theta);
+  if (extra.pass.theta != nullptr) memcpy(pp.theta, extra.pass.theta, D / 2 * sizeof(double));
+  else ads_rope_theta(model->rope_base, D, pp.theta);
   for (int i = 0; i < kMaxProbes; ++i) pp.nshots[i] = i < P ? probe_nshots[i] : 0;
   const long long n_tok = (long long)B * nl * P * To;
   const long long n_groups = (n_tok * kPrepParts + 7) / 8;
@@ -1676,12 +1678,11 @@ extern "C" size_t adapshot_attn_workspace_bytes(const adapshot_model_t* model, i
   return make_plan(model, B, P, Tq, n_layers_in_call).total;
 }
 
-int ads_query_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_ctx,
-                                   int64_t ctx_cap, const int64_t* ctx_off, int32_t B, int32_t k,
-                                   const int32_t* probe_nshots, int32_t P, const void* q, const void* kq,
-                                   const void* vq, int32_t Tq, int32_t layer_begin, int32_t layer_end,
-                                   void* out, float* lse, uint32_t flags, void* ws, size_t ws_bytes,
-                                   int32_t* status, void* stream, const AdsEntropyJob* ent) {
+int ads_query_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_ctx, int64_t ctx_cap,
+                   const int64_t* ctx_off, int32_t B, int32_t k, const int32_t* probe_nshots, int32_t P, const void* q,
+                   const void* kq, const void* vq, int32_t Tq, int32_t layer_begin, int32_t layer_end, void* out,
+                   float* lse, uint32_t flags, void* ws, size_t ws_bytes, int32_t* status, void* stream,
+                   const AdsPass* pass) {
   if (model == nullptr || k_ctx == nullptr || v_ctx == nullptr || ctx_off == nullptr || probe_nshots == nullptr ||
       q == nullptr || kq == nullptr || vq == nullptr || out == nullptr || ws == nullptr)
     return ADAPSHOT_EINVAL;
@@ -1703,7 +1704,7 @@ int ads_query_attn(const adapshot_model_t* model, const void* k_ctx, const void*
   if (ws_bytes < pl.total) return ADAPSHOT_ECAPACITY;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   AttnExtra extra;
-  extra.ent = ent;
+  if (pass != nullptr) extra.pass = *pass;
   if (model->head_dim == 128)
     return launch_attn<128>(model, k_ctx, v_ctx, ctx_cap, ctx_off, B, k, probe_nshots, P, q, kq, vq, Tq, nl, out,
                             lse, pl, ws, status, st, nullptr, kModeCache, extra);
@@ -1711,13 +1712,13 @@ int ads_query_attn(const adapshot_model_t* model, const void* k_ctx, const void*
                          lse, pl, ws, status, st, nullptr, kModeCache, extra);
 }
 
-extern "C" int adapshot_query_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_ctx,
-                                   int64_t ctx_cap, const int64_t* ctx_off, int32_t B, int32_t k,
-                                   const int32_t* probe_nshots, int32_t P, const void* q, const void* kq,
-                                   const void* vq, int32_t Tq, int32_t layer_begin, int32_t layer_end,
-                                   void* out, float* lse, uint32_t flags, void* ws, size_t ws_bytes,
+extern "C" int adapshot_query_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_ctx, int64_t ctx_cap,
+                                   const int64_t* ctx_off, int32_t B, int32_t k, const int32_t* probe_nshots, int32_t P,
+                                   const void* q, const void* kq, const void* vq, int32_t Tq, int32_t layer_begin,
+                                   int32_t layer_end, void* out, float* lse, uint32_t flags, void* ws, size_t ws_bytes,
                                    int32_t* status, void* stream) {
-  return ads_query_attn(model, k_ctx, v_ctx, ctx_cap, ctx_off, B, k, probe_nshots, P, q, kq, vq, Tq, layer_begin, layer_end, out, lse, flags, ws, ws_bytes, status, stream, nullptr);
+  return ads_query_attn(model, k_ctx, v_ctx, ctx_cap, ctx_off, B, k, probe_nshots, P, q, kq, vq, Tq, layer_begin,
+                        layer_end, out, lse, flags, ws, ws_bytes, status, stream, nullptr);
 }
 
 extern "C" size_t adapshot_attn_fused_workspace_bytes(const adapshot_model_t* model, int32_t B, int32_t P,
@@ -1728,13 +1729,11 @@ extern "C" size_t adapshot_attn_fused_workspace_bytes(const adapshot_model_t* mo
   return make_plan(model, B, P, Tq, n_layers_in_call, ctx_cap).total;
 }
 
-int ads_query_attn_fused(const adapshot_model_t* model, const adapshot_pool_t* pool,
-                                         const int32_t* sel_idx, const int64_t* ctx_off, int64_t ctx_cap,
-                                         int32_t B, int32_t k, const int32_t* probe_nshots, int32_t P,
-                                         const void* q, const void* kq, const void* vq, int32_t Tq,
-                                         int32_t layer_begin, int32_t layer_end, void* out, float* lse,
-                                         uint32_t flags, void* ws, size_t ws_bytes, int32_t* status,
-                                         void* stream, const AdsEntropyJob* ent) {
+int ads_query_attn_fused(const adapshot_model_t* model, const adapshot_pool_t* pool, const int32_t* sel_idx,
+                         const int64_t* ctx_off, int64_t ctx_cap, int32_t B, int32_t k, const int32_t* probe_nshots,
+                         int32_t P, const void* q, const void* kq, const void* vq, int32_t Tq, int32_t layer_begin,
+                         int32_t layer_end, void* out, float* lse, uint32_t flags, void* ws, size_t ws_bytes,
+                         int32_t* status, void* stream, const AdsPass* pass) {
   if (model == nullptr || pool == nullptr || sel_idx == nullptr || ctx_off == nullptr || probe_nshots == nullptr ||
       q == nullptr || kq == nullptr || vq == nullptr || out == nullptr || ws == nullptr)
     return ADAPSHOT_EINVAL;
@@ -1760,7 +1759,7 @@ int ads_query_attn_fused(const adapshot_model_t* model, const adapshot_pool_t* p
   if (ws_bytes < pl.total) return ADAPSHOT_ECAPACITY;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   AttnExtra extra;
-  extra.ent = ent;
+  if (pass != nullptr) extra.pass = *pass;
   FusedSrc src;
   src.pool = pool; src.sel_idx = sel_idx; src.layer_begin = layer_begin;
   if (model->head_dim == 128)
@@ -1771,13 +1770,13 @@ int ads_query_attn_fused(const adapshot_model_t* model, const adapshot_pool_t* p
 }
 
 extern "C" int adapshot_query_attn_fused(const adapshot_model_t* model, const adapshot_pool_t* pool,
-                                         const int32_t* sel_idx, const int64_t* ctx_off, int64_t ctx_cap,
-                                         int32_t B, int32_t k, const int32_t* probe_nshots, int32_t P,
-                                         const void* q, const void* kq, const void* vq, int32_t Tq,
-                                         int32_t layer_begin, int32_t layer_end, void* out, float* lse,
-                                         uint32_t flags, void* ws, size_t ws_bytes, int32_t* status,
-                                         void* stream) {
-  return ads_query_attn_fused(model, pool, sel_idx, ctx_off, ctx_cap, B, k, probe_nshots, P, q, kq, vq, Tq, layer_begin, layer_end, out, lse, flags, ws, ws_bytes, status, stream, nullptr);
+                                         const int32_t* sel_idx, const int64_t* ctx_off, int64_t ctx_cap, int32_t B,
+                                         int32_t k, const int32_t* probe_nshots, int32_t P, const void* q,
+                                         const void* kq, const void* vq, int32_t Tq, int32_t layer_begin,
+                                         int32_t layer_end, void* out, float* lse, uint32_t flags, void* ws,
+                                         size_t ws_bytes, int32_t* status, void* stream) {
+  return ads_query_attn_fused(model, pool, sel_idx, ctx_off, ctx_cap, B, k, probe_nshots, P, q, kq, vq, Tq, layer_begin,
+                              layer_end, out, lse, flags, ws, ws_bytes, status, stream, nullptr);
 }
 
 extern "C" size_t adapshot_attn_vpool_workspace_bytes(const adapshot_model_t* model, int32_t B, int32_t P,
@@ -1788,13 +1787,11 @@ extern "C" size_t adapshot_attn_vpool_workspace_bytes(const adapshot_model_t* mo
   return make_plan(model, B, P, Tq, n_layers_in_call, ctx_cap).total;
 }
 
-int ads_query_attn_vpool(const adapshot_model_t* model, const adapshot_pool_t* pool,
-                                         const int32_t* sel_idx, const void* k_ctx, int64_t ctx_cap,
-                                         const int64_t* ctx_off, int32_t B, int32_t k,
-                                         const int32_t* probe_nshots, int32_t P, const void* q, const void* kq,
-                                         const void* vq, int32_t Tq, int32_t layer_begin, int32_t layer_end,
-                                         void* out, float* lse, uint32_t flags, void* ws, size_t ws_bytes,
-                                         int32_t* status, void* stream, const AdsEntropyJob* ent) {
+int ads_query_attn_vpool(const adapshot_model_t* model, const adapshot_pool_t* pool, const int32_t* sel_idx,
+                         const void* k_ctx, int64_t ctx_cap, const int64_t* ctx_off, int32_t B, int32_t k,
+                         const int32_t* probe_nshots, int32_t P, const void* q, const void* kq, const void* vq,
+                         int32_t Tq, int32_t layer_begin, int32_t layer_end, void* out, float* lse, uint32_t flags,
+                         void* ws, size_t ws_bytes, int32_t* status, void* stream, const AdsPass* pass) {
   if (model == nullptr || pool == nullptr || sel_idx == nullptr || k_ctx == nullptr || ctx_off == nullptr ||
       probe_nshots == nullptr || q == nullptr || kq == nullptr || vq == nullptr || out == nullptr || ws == nullptr)
     return ADAPSHOT_EINVAL;
@@ -1818,7 +1815,7 @@ int ads_query_attn_vpool(const adapshot_model_t* model, const adapshot_pool_t* p
   if (ws_bytes < pl.total) return ADAPSHOT_ECAPACITY;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   AttnExtra extra;
-  extra.ent = ent;
+  if (pass != nullptr) extra.pass = *pass;
   FusedSrc src;
   src.pool = pool; src.sel_idx = sel_idx; src.layer_begin = layer_begin;
   if (model->head_dim == 128)
@@ -1830,12 +1827,12 @@ int ads_query_attn_vpool(const adapshot_model_t* model, const adapshot_pool_t* p
 
 extern "C" int adapshot_query_attn_vpool(const adapshot_model_t* model, const adapshot_pool_t* pool,
                                          const int32_t* sel_idx, const void* k_ctx, int64_t ctx_cap,
-                                         const int64_t* ctx_off, int32_t B, int32_t k,
-                                         const int32_t* probe_nshots, int32_t P, const void* q, const void* kq,
-                                         const void* vq, int32_t Tq, int32_t layer_begin, int32_t layer_end,
-                                         void* out, float* lse, uint32_t flags, void* ws, size_t ws_bytes,
-                                         int32_t* status, void* stream) {
-  return ads_query_attn_vpool(model, pool, sel_idx, k_ctx, ctx_cap, ctx_off, B, k, probe_nshots, P, q, kq, vq, Tq, layer_begin, layer_end, out, lse, flags, ws, ws_bytes, status, stream, nullptr);
+                                         const int64_t* ctx_off, int32_t B, int32_t k, const int32_t* probe_nshots,
+                                         int32_t P, const void* q, const void* kq, const void* vq, int32_t Tq,
+                                         int32_t layer_begin, int32_t layer_end, void* out, float* lse, uint32_t flags,
+                                         void* ws, size_t ws_bytes, int32_t* status, void* stream) {
+  return ads_query_attn_vpool(model, pool, sel_idx, k_ctx, ctx_cap, ctx_off, B, k, probe_nshots, P, q, kq, vq, Tq,
+                              layer_begin, layer_end, out, lse, flags, ws, ws_bytes, status, stream, nullptr);
 }
 
 // ---------------------------------------------------------------- literal tree layout

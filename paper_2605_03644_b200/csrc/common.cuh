@@ -121,21 +121,30 @@ struct AdsEntropyJob {
 int ads_entropy_job(const void* logits, int32_t dtype, int32_t R, int32_t V, int64_t row_stride, float* H, float tau,
                     int32_t rows_per_group, int32_t* first_ok, void* ws, size_t ws_bytes, AdsEntropyJob* job);
 
-// The three attention calls (attn.cu), with the entropy of the same probes' logits beside them when `ent` is given.
+// What the calls of a pass share (null, or a null member: nothing).
+struct AdsPass {
+  const double* theta;         // the model's rotary frequencies
+  const AdsEntropyJob* ent;    // the entropy of the probes' logits, to run beside the attention call
+};
+
+// The gather (assemble.cu) and the three attention calls (attn.cu) behind their entry points.
+int ads_assemble_kv(const adapshot_model_t* model, const adapshot_pool_t* pool, const int32_t* sel_idx, int32_t B, int32_t k,
+                    int32_t shot_begin, int32_t layer_begin, int32_t layer_end, void* k_ctx, void* v_ctx, int64_t ctx_cap,
+                    int64_t* ctx_off, uint32_t flags, int32_t* status, void* stream, const AdsPass* pass);
 int ads_query_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_ctx, int64_t ctx_cap,
                    const int64_t* ctx_off, int32_t B, int32_t k, const int32_t* probe_nshots, int32_t P, const void* q,
                    const void* kq, const void* vq, int32_t Tq, int32_t layer_begin, int32_t layer_end, void* out, float* lse,
-                   uint32_t flags, void* ws, size_t ws_bytes, int32_t* status, void* stream, const AdsEntropyJob* ent);
+                   uint32_t flags, void* ws, size_t ws_bytes, int32_t* status, void* stream, const AdsPass* pass);
 int ads_query_attn_fused(const adapshot_model_t* model, const adapshot_pool_t* pool, const int32_t* sel_idx,
                          const int64_t* ctx_off, int64_t ctx_cap, int32_t B, int32_t k, const int32_t* probe_nshots,
                          int32_t P, const void* q, const void* kq, const void* vq, int32_t Tq, int32_t layer_begin,
                          int32_t layer_end, void* out, float* lse, uint32_t flags, void* ws, size_t ws_bytes,
-                         int32_t* status, void* stream, const AdsEntropyJob* ent);
+                         int32_t* status, void* stream, const AdsPass* pass);
 int ads_query_attn_vpool(const adapshot_model_t* model, const adapshot_pool_t* pool, const int32_t* sel_idx,
                          const void* k_ctx, int64_t ctx_cap, const int64_t* ctx_off, int32_t B, int32_t k,
                          const int32_t* probe_nshots, int32_t P, const void* q, const void* kq, const void* vq, int32_t Tq,
                          int32_t layer_begin, int32_t layer_end, void* out, float* lse, uint32_t flags, void* ws,
-                         size_t ws_bytes, int32_t* status, void* stream, const AdsEntropyJob* ent);
+                         size_t ws_bytes, int32_t* status, void* stream, const AdsPass* pass);
 
 // Decoding with few rows per KV head (decode.cu): whether a call's rows fit, whether it pays, its scratch, and the call itself
 // (arguments checked by the caller).
