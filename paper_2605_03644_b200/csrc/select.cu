@@ -201,7 +201,7 @@ __device__ __forceinline__ bool pair_less(unsigned long long ka, int ia, unsigne
 
 // Top k by radix selection, one CTA per query.  The keys' interval is narrowed, 4096 bins at a time, until
 // the bin that holds the k-th key and everything in front of it fit the candidate area; up to 1024 candidates are then
-// put in order by dealing them out to 4096 bins once more, more of them by a bitonic sort.  The first pass bins by the score's
+// put in order by dealing them out to 4096 bins once more, more of them, or those that crowd a bin, by a bitonic sort.  The first pass bins by the score's
 // sign, exponent and five bits more (cosines and attention masses both spread over many of them), the following ones
 // divide the bin's interval evenly, so two passes nearly always do; equal keys without end are cut by id.  Bound by the
 // instructions of one SM per query: a pass reads the keys once (the second one from L1) with eight loads in flight per
@@ -211,7 +211,7 @@ __device__ __forceinline__ bool pair_less(unsigned long long ka, int ia, unsigne
 // keys, k = 512, 32 queries 145, 14.6 and 11.2; 4096 keys, k = 256, 8 queries 11.0 and 9.6.)
 constexpr int kSelThreads = 1024;
 constexpr int kSelBins = 4096;
-constexpr int kBinMost = 32;          // candidates in one bin that are ordered by comparing each with all
+constexpr int kBinMost = 128;         // candidates in one bin that are ordered by comparing each with all (40 copies of every shot: 21.6 us, 25.2 by sorting)
 
 // First-pass bins, ascending with the key: 0 = scores of 2 and more, 1 .. 2040 = positive scores below that in 32nds
 // of an octave (63 octaves), 2041 = smaller ones, then the negative scores in the same way.
@@ -234,6 +234,44 @@ __device__ __forceinline__ void first_bin_interval(int bin, unsigned long long* 
   else { a = 0x10000 + kBinHi; b = 0x1ffff; }
   *lo = (unsigned long long)a << kBinShift;
   *hi = ((unsigned long long)b << kBinShift) | ((1ull << kBinShift) - 1);
+}
+
+// The candidates of a query one of whose bins is crowded, by a bitonic sort, ascending on (key, id), one per thread (padding: the largest
+// key and id), exchanged within a warp by shuffles.  (Calls of 16 queries over 8192 shots, all scores equal, k = 512: 25.0 us, 30.5
+// where every exchange goes through shared memory as below.  Not inlined: the calls without a crowded bin 13.72 us, 13.95 with it inlined.)
+__device__ __noinline__ void sort_candidates(unsigned long long key, int id, int n, int n_out, unsigned long long* ckey, int* cid,
+                                             int32_t* idx, float* score) {
+  int n_pow2 = 32;
+  while (n_pow2 < n) n_pow2 <<= 1;
+  const int tid = threadIdx.x;
+  if (tid >= n_pow2) return;                        // (whole warps)
+  auto sync = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(n_pow2) : "memory"); };
+  for (int size = 2; size <= n_pow2; size <<= 1) {
+    for (int stride = size >> 1; stride > 0; stride >>= 1) {
+      unsigned long long ko;
+      int io;
+      if (stride >= 32) {
+        sync();
+        ckey[tid] = key;
+        cid[tid] = id;
+        sync();
+        ko = ckey[tid ^ stride];
+        io = cid[tid ^ stride];
+      } else {
+        ko = __shfl_xor_sync(0xffffffffu, key, stride);
+        io = __shfl_xor_sync(0xffffffffu, id, stride);
+      }
+      const bool keep_low = ((tid & stride) == 0) == ((tid & size) == 0);
+      if (pair_less(ko, io, key, id) == keep_low) {
+        key = ko;
+        id = io;
+      }
+    }
+  }
+  if (tid < n_out) {
+    idx[tid] = id;
+    if (score != nullptr) score[tid] = (float)key_score(key);
+  }
 }
 
 __global__ void __launch_bounds__(kSelThreads)
@@ -350,8 +388,9 @@ radix_topk_kernel(const unsigned long long* __restrict__ all_keys, int N, int k,
   __syncthreads();
   const int n = n_s;
   if (want <= kSelThreads) {
-    // One candidate per thread, dealt out to 4096 bins of equal width between the smallest and the largest key; its place is what lies in
-    // front of its bin and what precedes it there.  (The bitonic sort below takes 55 steps for 1024 candidates.)
+    // One candidate per thread, dealt out to 4096 bins; its place is what lies in front of its bin and what precedes it there.  The bins
+    // are of equal width between the smallest and the largest key, or, where that would leave an octave fewer than 32 of them (scores on
+    // both sides of zero; 32 queries of 2048 shots, k = 1000: 24.6 us when they crowded a few bins, 10.7 now), those of the first pass.
     unsigned long long* skey = reinterpret_cast<unsigned long long*>(hist + kSelBins);     // [want], by bin
     int* sid = reinterpret_cast<int*>(skey + want);
     const unsigned long long key = tid < n ? ckey[tid] : ~0ull;
@@ -376,7 +415,8 @@ radix_topk_kernel(const unsigned long long* __restrict__ all_keys, int N, int k,
     if (shift < 0) shift = 0;
     int bin = 0, nth = 0;
     if (tid < n) {
-      bin = (int)((key - least) >> shift);
+      if (shift <= kBinShift) bin = (int)((key - least) >> shift);
+      else bin = first_bin(key);
       nth = atomicAdd(hist + bin, 1);
     }
     if (!__syncthreads_or(nth >= kBinMost)) {
@@ -400,6 +440,9 @@ radix_topk_kernel(const unsigned long long* __restrict__ all_keys, int N, int k,
       }
       return;
     }
+    sort_candidates(key, id, n, min(k, n), ckey, cid, final_idx + (long long)b * k,
+                    final_score == nullptr ? nullptr : final_score + (long long)b * k);
+    return;
   }
   // bitonic sort, ascending on (key, id); ids are unique so the order is total
   int n_pow2 = 32;

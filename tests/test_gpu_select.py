@@ -57,7 +57,7 @@ def test_select_ties_and_zero_norm():
 
 
 @pytest.mark.parametrize("k", [1, 33, 128, 512, 1000])
-@pytest.mark.parametrize("copies", [1, 31, 33, 700])       # below and above what a bin of candidates may hold; more than k of them
+@pytest.mark.parametrize("copies", [1, 31, 33, 127, 129, 700])       # below and above what a bin of candidates may hold; more than k of them
 def test_select_by_bins_and_by_sorting(copies, k):
     # a pool large enough for the selection, whose best shots are copies of one another and whose scores span many octaves
     ab = hp.gpu_binding()
@@ -82,7 +82,7 @@ def test_nested_probes_are_prefixes():
 
 
 @pytest.mark.parametrize("N,E,B,k", [(33, 16, 3, 33), (97, 48, 8, 13), (3001, 64, 9, 1500), (4096, 768, 17, 1025),
-                                     (8192, 32, 4, 5000), (9000, 112, 33, 1024)])
+                                     (8192, 32, 4, 5000), (9000, 112, 33, 1024), (2048, 64, 32, 1000), (2100, 32, 16, 1024)])
 def test_select_batches(N, E, B, k):
     # fp64 matrix tiles: remainders of 32 shots, 8 and 16 queries, embeddings of one step, of fewer steps than warps
     # and of unequal shares; rank counting and radix selection with few and with many candidates; k beyond the
