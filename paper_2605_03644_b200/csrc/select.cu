@@ -536,11 +536,16 @@ rank_topk_kernel(const unsigned long long* __restrict__ all_keys, int N, int k,
   }
 }
 
-// Rank counting compares every pair of keys, over the whole chip, whatever k; the radix selection is one CTA per query and
-// sorts k candidates at its end.  Counting / selection, us: one query of 3000 keys, k = 1 8.0 / 7.2, k = 128 8.1 / 10.4; 4096 keys,
-// k = 1 9.2 / 7.6, 128 9.2 / 11.0, 1024 9.3 / 17.8, 4096 9.3 / 65; 8192 keys, k = 512 21 / 16, 1024 21 / 20, 4096 21 / 70; 64
-// queries of 512 keys, k = 32 10.7 / 8.4, k = 128 10.7 / 10.3; the line follows the points where the two meet.
-bool rank_by_counting(int N, int B, int k) { return (long long)N * N * B <= 11000000ll + 48000ll * k; }
+// Rank counting compares every pair of keys, over the whole chip, whatever k; the radix selection is one CTA per query whose time
+// grows with k: up to 32 candidates hardly cost anything, 128 to 1024 are dealt out to bins, more are sorted.  Counting / selection, us:
+// one query of 3000 keys, k = 1 8.2 / 8.2, 4096 keys, k = 1 9.6 / 8.4, 128 9.7 / 10.9, 512 9.4 / 11.3, 1024 9.7 / 12.5, 6144 keys 14.7 / 9.4,
+// 12.1, 12.8 and 13.7; two of 3000, k = 128 10.3 / 11.3, 512 10.3 / 11.6; of 4096, 13.6 / 11.9, 12.5 and (1024) 13.3; eight of 2048, k = 128
+// 10.9 / 9.4, 512 10.9 / 9.8, 1024 10.9 / 10.7; 32 of 1024, k = 1 12.1 / 7.6, 512 12.1 / 10.1; sorted: one of 4096, k = 4096 9.3 / 65, of 8192 21 / 70.
+bool rank_by_counting(int N, int B, int k) {
+  const long long pairs = (long long)N * N * B;
+  if (k > kSelThreads) return pairs <= 11000000ll + 48000ll * k;
+  return pairs <= 11000000ll + 100000ll * (k < 128 ? k : 128) + 6000ll * (k < 128 ? 0 : k - 128);
+}
 
 }  // namespace
 

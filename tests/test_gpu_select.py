@@ -108,8 +108,7 @@ def test_radix_selection_cuts_equal_scores_by_id(n_same, k):
 
 @pytest.mark.parametrize("N,B,k", [(2, 1, 2), (31, 2, 31), (2047, 1, 2047), (2049, 1, 300), (3741, 1, 3741), (3742, 1, 3742)])
 def test_rank_counting_with_ties(N, B, k):
-    # odd and even counts (a last pair of one key), one and two tiles of keys, both sides of the line to the radix
-    # selection; every embedding occurs about three times, so that equal scores lie in front of and behind each other
+    # odd and even counts (a last pair of one key), one and two tiles of keys; every embedding occurs about three times, so that equal scores lie in front of and behind each other
     ab = hp.gpu_binding()
     g = torch.Generator().manual_seed(N)
     base = torch.randn((N + 2) // 3, 32, generator=g)
@@ -117,9 +116,11 @@ def test_rank_counting_with_ties(N, B, k):
     _check(ab, emb, torch.randn(B, 32, generator=g), k)
 
 
-@pytest.mark.parametrize("N,B,k", [(3751, 1, 64), (3752, 1, 64), (6100, 1, 600), (6400, 1, 600), (8192, 1, 4096), (8192, 3, 4096)])
+@pytest.mark.parametrize("N,B,k", [(3751, 1, 64), (3752, 1, 64), (6100, 1, 600), (6400, 1, 600), (8192, 1, 4096), (8192, 3, 4096),
+                                   (4171, 1, 64), (4172, 1, 64), (5160, 1, 600), (5161, 1, 600), (5401, 1, 1024), (5402, 1, 1024),
+                                   (7758, 1, 1025), (7759, 1, 1025)])
 def test_both_sides_of_the_line_between_counting_and_selection(N, B, k):
-    # N^2 B against 11 million and 48000 k; every embedding occurs about three times
+    # N^2 B against 11 million and what k adds, up to 1024 and beyond; every embedding occurs about three times
     ab = hp.gpu_binding()
     g = torch.Generator().manual_seed(N + B)
     base = torch.randn((N + 2) // 3, 32, generator=g)
