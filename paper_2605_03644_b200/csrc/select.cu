@@ -595,9 +595,12 @@ extern "C" int adapshot_select(const adapshot_pool_t* pool, const float* q_emb, 
     };
     // 16 shots per CTA (three per SM) leave a shorter last wave than 32 (two per SM): 20000 x 768, 16 queries 41.1 -> 39.1 us for the
     // call, 8192 x 1024, 32 queries 35.2 -> 33.0, 40000 x 384, 32 queries 75.8 -> 72.3.  Up to 8 queries the element widened once per 32
-    // shots matters as much, unless there are SMs to fill: 2048 x 1024, 8 queries 10.5 -> 9.4, 4096 x 1024 13.3 / 13.6, 30000 x 768 35.1 / 35.9.
+    // shots matters as much, unless CTAs of 16 shots find an SM each (16 / 32 shots, E = 1024, 4 queries: 1024 shots 6.7 / 7.9, 2368 11.1 /
+    // 12.3; beyond that 2500 14.1 / 13.7, 3000 16.4 / 16.0, 4096 20.7 / 20.3, 8192 62.0 / 61.0, 16384 212.5 / 213.5).
+    const int n_sm = ads_sm_count();
+    if (n_sm <= 0) return ADAPSHOT_ECUDA;
     if (B > 8) run(cosine_mma_kernel<2, 1>, 16, 16);
-    else if (N <= 3000) run(cosine_mma_kernel<1, 1>, 16, 8);
+    else if (N <= 16 * n_sm) run(cosine_mma_kernel<1, 1>, 16, 8);
     else run(cosine_mma_kernel<1, 2>, 32, 8);
   } else {
     const unsigned grid = (unsigned)((N + 7) / 8);
