@@ -714,14 +714,13 @@ int launch(const CUtensorMap* m, const DecodeParams& p, cudaStream_t st) {
 
 // Whether a call whose rows fit is better off here than with the prefill kernels.  Up to 16 rows always (one block of rows:
 // 1.7 to 12 times as fast).  With 17 to 32 the second block of accumulators and the read-out of 32 rows per unit cost what
-// the prefill kernels' empty rows do; prefill / here, geometric mean (range) over 1248 calls of 1 to 200 requests, contexts of 128
-// to 16 K tokens, 3 to 300 own tokens, one and four layers: d = 64, eight KV heads, ctx + 4 own >= 1024 tokens 1.19 (0.89 to 1.54),
-// below 0.83 (0.51 to 1.16); one head, ctx + 16 own >= 1024 1.41 (0.89 to 4.9: what preparing the own tokens costs there), below
-// 1.00 (0.64 to 1.5); d = 128, eight heads 0.79 (0.46 to 1.20); one head, several requests of 100 own tokens or more 1.28 (0.73
-// to 3.8), else 0.82.
+// the prefill kernels' empty rows do; prefill / here, geometric mean (range) over 127 calls of 1 to 200 requests, contexts of 32
+// to 24 K tokens, 5 to 300 own tokens: d = 64, eight KV heads, ctx + 4 own >= 1024 tokens 1.13 (1.00 to 1.24), below 0.71 (0.59 to
+// 0.81); one head, ctx + 16 own >= 1024 1.37 (1.05 to 1.67), below 1.12 (1.03, 1.23); d = 128, eight heads 0.74 (0.52 to 0.93); one head,
+// where the prefill kernels have 16000 own tokens or more to prepare 1.21 (0.95 to 1.96), fewer 0.81 (0.57 to 1.14).
 bool ads_decode_rows_pay(const adapshot_model_t* model, int B, int T_new, int T_own, int64_t ctx_cap) {
   if ((long long)T_new * (model->n_q_heads / model->n_kv_heads) <= 16) return true;
-  if (model->head_dim == 128) return model->n_kv_heads == 1 && B > 1 && T_own >= 100;
+  if (model->head_dim == 128) return model->n_kv_heads == 1 && (long long)B * T_own >= 16000;
   return ctx_cap + (model->n_kv_heads == 1 ? 16ll : 4ll) * T_own >= 1024;
 }
 bool ads_decode_rows_fit(const adapshot_model_t* model, int T_new) {

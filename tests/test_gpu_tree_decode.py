@@ -218,8 +218,10 @@ def test_decode_row_counts_and_range_cuts(hq, d, batch, n_shots, t_new, t_own):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("hq,hkv,d,batch,k,t_new,t_own,small_ws", [
-    (8, 1, 128, 2, 3, 4, 100, False),      # 32 rows, d = 128: streamed for one KV head and long own sequences
-    (8, 1, 128, 2, 3, 4, 99, False),       # the prefill kernels
+    (8, 1, 128, 54, 3, 4, 297, False),     # 32 rows, d = 128, one KV head: streamed from 16000 own tokens of all requests on
+    (8, 1, 128, 54, 3, 4, 296, False),     # the prefill kernels
+    (8, 1, 128, 2, 3, 4, 100, False),
+    (8, 1, 128, 2, 3, 4, 99, False),
     (8, 1, 128, 2, 3, 4, 99, True),        # streamed, because the workspace has no room for the prefill kernels'
     (8, 2, 64, 2, 3, 8, 210, False),       # 32 rows, d = 64, a capacity of 216 to 224 and 4 x 210 own tokens: streamed
     (8, 2, 64, 2, 3, 8, 190, False),       # the prefill kernels
