@@ -1355,7 +1355,7 @@ struct CombineParams {
   float* lse;           // [B][nl][P][Hq][Tq] or null
   int Tq, Hq, G, n_mp;
   int units;                  // of the grid (units, groups of rows, column steps); the blocks beyond them:
-  AdsEntropyJob ent;          // the entropy's second step, a block per group of rows
+  AdsEntropyJob ent;          // the entropy's second step, a block per query
 };
 
 constexpr int kCombineRows = 8;      // rows per warp
@@ -1372,9 +1372,9 @@ __global__ void __launch_bounds__(256) attn_combine_kernel(const __grid_constant
   ads_dependency_wait();
   if ((int)blockIdx.x >= p.units) {
     __shared__ float sh_h[kMaxProbes];               // (a group is a query's probes)
-    if (blockIdx.y != 0 || blockIdx.z != 0) return;
-    ent_finish_block(p.ent.partial, p.ent.n_split, p.ent.R, p.ent.rows_per_group, p.ent.tau, p.ent.H, p.ent.first_ok,
-                     (int)blockIdx.x - p.units, sh_h);
+    const int group = (((int)blockIdx.x - p.units) * (int)gridDim.y + (int)blockIdx.y) * (int)gridDim.z + (int)blockIdx.z;
+    if (group < p.ent.R / p.ent.rows_per_group)
+      ent_finish_block(p.ent.partial, p.ent.n_split, p.ent.R, p.ent.rows_per_group, p.ent.tau, p.ent.H, p.ent.first_ok, group, sh_h);
     return;
   }
   const Sched* sc = p.sched;
@@ -1661,9 +1661,11 @@ int launch_attn(const adapshot_model_t* model, const void* k_ctx, const void* v_
   const long long units = (long long)B * P * nl * Hkv;
   cp.units = (int)(units < n_gangs ? units : n_gangs);
   cp.ent = pp.ent;
-  const int finish = cp.ent.blocks > 0 ? cp.ent.R / cp.ent.rows_per_group : 0;
-  const dim3 grid((unsigned)(cp.units + finish), (unsigned)((Tq * G + 8 * kCombineRows - 1) / (8 * kCombineRows)),
-                  D / (16 * kCombineSteps));
+  dim3 grid((unsigned)cp.units, (unsigned)((Tq * G + 8 * kCombineRows - 1) / (8 * kCombineRows)), D / (16 * kCombineSteps));
+  if (cp.ent.blocks > 0) {             // as many more columns of the grid as hold a block for every query
+    const unsigned column = grid.y * grid.z;
+    grid.x += ((unsigned)(cp.ent.R / cp.ent.rows_per_group) + column - 1) / column;
+  }
   ads_launch_dependent(attn_combine_kernel<D>, grid, 256, 0, st, cp);
   return ads_launch_status();
 }

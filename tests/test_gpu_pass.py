@@ -132,6 +132,23 @@ def test_entropy_beside_the_attention_equals_its_own_call(variant, vocab, dtype)
         assert all(torch.equal(a, b) for a, b in zip(out, steps.out))
 
 
+@pytest.mark.parametrize("batch,t_q", [(1, 9), (4, 9), (5, 9), (13, 40)])      # one column of the merge's grid holds 4 queries, or 8
+def test_every_query_of_a_pass_has_its_entropy(batch, t_q):
+    w = _workload(52).scaled(batch=batch, t_q=t_q)
+    path = _path(w, "full")
+    args = _inputs(path, wl.make_queries(w))
+    p = torch.softmax(args[4].double(), 1)
+    want = -(p * p.log()).sum(1)
+    tau = float(want.view(batch, -1).max(1).values.median()) + 1e-4
+    path.H.fill_(-1)
+    path.first_ok.fill_(-7)
+    _, H, ok = path.run(*args[:5], tau)
+    torch.cuda.synchronize()
+    torch.testing.assert_close(H.double(), want, rtol=1e-5, atol=1e-5)
+    good = (H <= tau).view(batch, -1)
+    assert torch.equal(ok, torch.where(good.any(1), good.int().argmax(1), -1).int())
+
+
 @pytest.mark.parametrize("variant,tensor", [("vpool", "v"), ("fused", "v"), ("fused", "k")])
 def test_entropy_states_in_the_pool_do_not_meet_the_attention(variant, tensor):
     # a workspace that lies on a selected shot of the last layer: written after the attention has read the shot
