@@ -59,7 +59,6 @@ struct DecodeParams {
   int32_t* status;
   long long ctx_cap;
   int B, k, Hq, Hkv, G, nl, T_new, T_own, rows, n_cta;
-  int ahead;                   // whether lengths, ranges and first tiles are taken ahead of the dependency wait
   float scale_log2;
   double theta[64];
 };
@@ -269,12 +268,10 @@ decode_rows_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   // before the wait, so the lengths are a guess until then, right unless one of those kernels changes them.  (From the wait to the
   // first copy 3.3 us when everything followed it, 1.0 now; four calls of one request of 12 K tokens 68.2 -> 63.6 us.  Forming the angles
   // of Q here as well is slower, 70.8: the CTAs enter too late for it to be hidden.)
-  if (p.ahead) {
-    if (warp == 0) lengths(true);
-    __syncthreads();
-    find_range();
-  }
-  if (threadIdx.x == 32 * kWarps && p.ahead && x1 - x0 <= kPrefetchRange) {
+  if (warp == 0) lengths(true);
+  __syncthreads();
+  find_range();
+  if (threadIdx.x == 32 * kWarps && x1 - x0 <= kPrefetchRange) {
     int left = kPrefetchTiles;
     walk([&](int b, int l, int g, int t0, int t1, int, int n_ctx, bool) {
       for (int t = t0; t < min(t1, n_ctx) && left > 0; ++t, --left)
@@ -287,7 +284,7 @@ decode_rows_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
     });
   }
   ads_dependency_wait();
-  if (!p.ahead || !__syncthreads_and(warp != 0 || guess_holds())) {
+  if (!__syncthreads_and(warp != 0 || guess_holds())) {
     if (warp == 0) lengths(false);
     __syncthreads();
     find_range();
@@ -616,8 +613,9 @@ __global__ void __launch_bounds__(32 * kMergeWarps) decode_combine_kernel(const 
   if constexpr (AHEAD) {
     // Where the pieces lie follows from the lengths, which the kernel in front wrote when it began: read past the L1 as a guess
     // before the wait, so that behind it the lengths and the pieces are fetched together instead of one after the other
-    // (63.7 -> 58.4 us for four calls of one request of 12 K tokens; not with more blocks, whose registers cost more than that: 32
-    // requests 537 -> 542).  Whatever lies there: 0 <= begin < end <= total < 2^31 keeps every range and so every
+    // (four calls of one request of 12 K tokens 63.7 -> 58.4 us).  With more than three of these blocks per SM the registers this
+    // takes cost more (after the wait / ahead, us per call and layer, 8 KV heads: 8 requests of 4 K tokens 26.8 / 26.2, 12 of 16 K 95.4 / 94.1,
+    // 16 of 1 K 19.5 / 20.4, 20 of 13 K 133.9 / 136.6).  Whatever lies there: 0 <= begin < end <= total < 2^31 keeps every range and so every
     // address of the guess within bounds.
     p0 = __ldcg(p.prefix + b);
     const long long p1 = __ldcg(p.prefix + b + 1);
@@ -705,7 +703,7 @@ int launch(const CUtensorMap* m, const DecodeParams& p, cudaStream_t st) {
   ads_launch_dependent(decode_rows_kernel<D, MB>, (unsigned)p.n_cta, kThreads, smem, st, m[0], m[1], m[2], m[3], p);
   if (ads_launch_status() != ADAPSHOT_OK) return ADAPSHOT_ECUDA;
   const dim3 grid((unsigned)((long long)p.B * p.nl * p.Hkv), (unsigned)p.rows);
-  if (p.ahead) ads_launch_dependent(decode_combine_kernel<D, true>, grid, 32 * kMergeWarps, 0, st, p);
+  if (2ll * grid.x * grid.y <= 3ll * p.n_cta) ads_launch_dependent(decode_combine_kernel<D, true>, grid, 32 * kMergeWarps, 0, st, p);
   else ads_launch_dependent(decode_combine_kernel<D, false>, grid, 32 * kMergeWarps, 0, st, p);
   return ads_launch_status();
 }
@@ -753,10 +751,6 @@ int ads_decode_rows(const adapshot_model_t* model, const void* k_ctx, const void
   const int n_sm = ads_sm_count();
   if (n_sm <= 0) return ADAPSHOT_ECUDA;
   p.n_cta = 2 * n_sm < kMaxCtas ? 2 * n_sm : kMaxCtas;
-  // The kernel in front of a layer's call is mostly the merge of the layer before.  With more than three of its blocks per SM this call's
-  // CTAs enter too late to hide anything, and lengths taken twice cost what they would have saved (not ahead / ahead, us per call of short
-  // contexts: 100 requests of one head 11.8 / 11.3, 148 12.3 / 12.8, 256 15.4 / 15.9; 12 of eight heads 12.9 / 12.3, 16 12.8 / 13.4, 64 22.8 / 23.6).
-  p.ahead = 2ll * B * nl * Hkv * p.rows <= 3ll * p.n_cta;
   const float scale = model->softmax_scale > 0.f ? model->softmax_scale : 1.0f / sqrtf((float)D);
   p.scale_log2 = scale * 1.4426950408889634f;
   ads_rope_theta(model->rope_base, D, p.theta);
