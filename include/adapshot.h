@@ -414,6 +414,12 @@ ADAPSHOT_API float adapshot_profile_attn_main_ms(void);
  * ends normally; the context stays usable.                                               */
 ADAPSHOT_API int adapshot_selftest_wait_timeout(int32_t* status, long long* cycles, void* stream);
 
+/* ---- Test aid: a kernel in front of another one (no counterpart in the paper).  It lets the kernel launched
+ * behind it in at once, idles for `cycles` SM cycles (at most ADAPSHOT_SELFTEST_MAX_CYCLES, about a
+ * millisecond) and then copies n 32-bit words: what such a kernel reads before it waits is the old content. */
+#define ADAPSHOT_SELFTEST_MAX_CYCLES 2000000
+ADAPSHOT_API int adapshot_selftest_late_copy(int32_t* dst, const int32_t* src, int32_t n, int64_t cycles, void* stream);
+
 ADAPSHOT_API const char* adapshot_strerror(int code);
 ADAPSHOT_API int adapshot_version(void);
 

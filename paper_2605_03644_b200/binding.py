@@ -37,6 +37,7 @@ EXPORTS = [
     "adapshot_entropy_workspace_bytes", "adapshot_entropy", "adapshot_entropy_subset",
     "adapshot_entropy_static", "adapshot_reuse_pass",
     "adapshot_profile", "adapshot_profile_attn_main_ms", "adapshot_selftest_wait_timeout",
+    "adapshot_selftest_late_copy",
     "adapshot_strerror", "adapshot_version",
 ]
 
@@ -128,6 +129,16 @@ def adapshot_profile_attn_main_ms() -> float:
 
 
 _selftest = _sig("adapshot_selftest_wait_timeout", C.c_int, [_vp, _vp, _vp])
+
+
+_late_copy = _sig("adapshot_selftest_late_copy", C.c_int, [_vp, _vp, C.c_int32, C.c_int64, _vp])
+
+
+def adapshot_selftest_late_copy(dst: torch.Tensor, src: torch.Tensor, cycles: int):
+    """Lets the next kernel in, idles, then copies src to dst (whole 32-bit words)."""
+    if dst.nbytes != src.nbytes or dst.nbytes % 4 != 0:
+        raise ValueError("tensors of equal size, in 32-bit words")
+    _check(_late_copy(_ptr(dst), _ptr(src), dst.nbytes // 4, cycles, _stream()))
 
 
 def adapshot_selftest_wait_timeout(status: torch.Tensor, cycles: torch.Tensor):

@@ -683,6 +683,16 @@ __global__ void __launch_bounds__(32 * kMergeWarps) decode_combine_kernel(const 
   if (p.lse != nullptr && threadIdx.x == 0) p.lse[(bl * p.Hq + h) * p.T_new + t] = (M + log2f(lsum)) * kLn2;
 }
 
+// Test aid: stands for a kernel in front of a decode call that writes its lengths late.
+__global__ void __launch_bounds__(256) late_copy_selftest_kernel(int32_t* dst, const int32_t* src, int n, long long cycles) {
+  ads_dependency_trigger();
+  ads_dependency_wait();
+  const long long t0 = clock64();
+  while (clock64() - t0 < cycles) {
+  }
+  for (int i = threadIdx.x; i < n; i += 256) dst[i] = src[i];
+}
+
 struct DecodeLayout {
   size_t off_o, off_ml, off_pre, total;
 };
@@ -766,4 +776,10 @@ int ads_decode_rows(const adapshot_model_t* model, const void* k_ctx, const void
   }
   if (D == 128) return p.rows <= 16 ? launch<128, 1>(m, p, st) : launch<128, 2>(m, p, st);
   return p.rows <= 16 ? launch<64, 1>(m, p, st) : launch<64, 2>(m, p, st);
+}
+
+extern "C" int adapshot_selftest_late_copy(int32_t* dst, const int32_t* src, int32_t n, int64_t cycles, void* stream) {
+  if (dst == nullptr || src == nullptr || n <= 0 || cycles < 0 || cycles > ADAPSHOT_SELFTEST_MAX_CYCLES) return ADAPSHOT_EINVAL;
+  ads_launch_dependent(late_copy_selftest_kernel, 1, 256, 0, static_cast<cudaStream_t>(stream), dst, src, n, (long long)cycles);
+  return ads_launch_status();
 }

@@ -46,6 +46,12 @@ def test_workspace_sizes(ab):
     assert ab.adapshot_entropy_workspace_bytes(4, 32000) % 256 == 0
 
 
+def test_the_late_copy_refuses_what_would_not_end(ab):
+    late, fake = ab.lib.adapshot_selftest_late_copy, C.c_void_p(0x1000)
+    for dst, src, n, cycles in ((None, fake, 4, 0), (fake, None, 4, 0), (fake, fake, 0, 0), (fake, fake, 4, -1), (fake, fake, 4, 2000001)):
+        assert late(dst, src, n, cycles, None) == ab.EINVAL
+
+
 def test_host_side_argument_checks_launch_nothing(ab):
     # all of these return before any CUDA call, so they run without a device
     pool = ab.PoolT(16, 8, 100, 0x1000, 0x1000, 0x1000, 0x1000)

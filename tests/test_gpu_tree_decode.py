@@ -120,27 +120,37 @@ def test_decode_step_over_the_chosen_prefix(t_new, t_own, d):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("batch", [1, 33])
-def test_decode_right_behind_the_kernel_that_writes_its_lengths(batch):
-    # offsets, shot counts and a workspace of arbitrary content, written on the stream right in front of every call
+@pytest.mark.parametrize("idle", [0, 40000])               # SM cycles (20 us) between the call's launch and its lengths
+@pytest.mark.parametrize("arbitrary_ws", [True, False])    # arbitrary content, or what the call before left: another call's ranges
+@pytest.mark.parametrize("batch", [1, 33, 160])            # 4 and 132 blocks in the merge: pieces taken ahead; 640: after the wait
+def test_decode_right_behind_the_kernel_that_writes_its_lengths(batch, arbitrary_ws, idle):
+    # offsets and shot counts of two kinds in turn, written on the stream right in front of every call by a kernel that lets the
+    # call in before it writes
     nl, t_own = 1, 70
     w = wl.CONFIGS["cfg2"].scaled(n_shots=40, len_lo=20, len_hi=200, batch=batch, k=20, probes=(20,), t_q=t_own, seed=77,
                                   n_q_heads=4, n_kv_heads=1)
     ab, pool, qs, sel_np, off_np, model, cap, kc, vc, off = _setup(w, nl, 14)
     dev_pool = hp.dev_pool(ab, pool)
-    kc.normal_(), vc.normal_()                     # (whatever the lengths, every position holds a number)
+    cap = w.k * w.len_hi
+    kc, vc = (torch.randn(batch, nl, cap, 1, w.head_dim, dtype=torch.bfloat16, device="cuda") for _ in range(2))
     q_new = qs["q"][:, :, 0, t_own - 1:].contiguous().cuda()
     k_own, v_own = qs["kq"][:, :, 0].contiguous().cuda(), qs["vq"][:, :, 0].contiguous().cuda()
     rng = np.random.default_rng(15)
     sels = [torch.from_numpy(np.stack([rng.permutation(w.n_shots)[:w.k] for _ in range(batch)]).astype(np.int32)).cuda() for _ in range(2)]
     counts = [torch.from_numpy(rng.integers(1, w.k + 1, size=batch).astype(np.int32)).cuda() for _ in range(2)]
-    off, n_dev, st = torch.empty_like(off), torch.empty_like(counts[0]), hp.new_status()
+    st = hp.new_status()
+    lengths = [torch.empty(off.nbytes + 4 * batch, dtype=torch.uint8, device="cuda") for _ in range(3)]      # two kinds, the one in use
+    views = [(t[:off.nbytes].view(torch.int64).view(off.shape), t[off.nbytes:].view(torch.int32)) for t in lengths]
+    for i in range(2):
+        ab.adapshot_assemble_kv(model, dev_pool, sels[i], 0, nl, None, None, cap, views[i][0], st)           # the plan alone
+        views[i][1].copy_(counts[i])
+    off, n_dev = views[2]
     ws = torch.empty(ab.adapshot_decode_workspace_bytes(model, batch, 1, t_own, nl), dtype=torch.uint8, device="cuda")
 
     def step(i, out, wait):
-        n_dev.copy_(counts[i])
-        ws.random_(0, 256)
-        ab.adapshot_assemble_kv(model, dev_pool, sels[i], 0, nl, None, None, cap, off, st)        # the plan alone
+        if arbitrary_ws:
+            ws.random_(0, 256)
+        ab.adapshot_selftest_late_copy(lengths[2], lengths[i], 0 if wait else idle)
         if wait:
             torch.cuda.synchronize()
         ab.adapshot_decode_attn(model, kc, vc, cap, off, w.k, n_dev, q_new, k_own, v_own, 0, nl, out, None, ws, st)
@@ -153,7 +163,7 @@ def test_decode_right_behind_the_kernel_that_writes_its_lengths(batch):
     for i, out in enumerate(got):
         step(i % 2, out, False)
     torch.cuda.synchronize()
-    assert not torch.equal(want[0], want[1])
+    assert st.item() == 0 and not torch.equal(want[0], want[1])
     assert all(torch.equal(out, want[i % 2]) for i, out in enumerate(got))
 
 
