@@ -1,4 +1,6 @@
 """ReusePath.run: what it reads and writes is what the object and the call hold at that moment."""
+import ctypes
+
 import pytest
 import torch
 
@@ -147,6 +149,89 @@ def test_every_query_of_a_pass_has_its_entropy(batch, t_q):
     torch.testing.assert_close(H.double(), want, rtol=1e-5, atol=1e-5)
     good = (H <= tau).view(batch, -1)
     assert torch.equal(ok, torch.where(good.any(1), good.int().argmax(1), -1).int())
+
+
+def _launches(path, args):
+    """Kernels of one pass, counted in a captured graph."""
+    path.run(*args)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        path.run(*args)
+    n = ctypes.c_size_t()
+    assert ctypes.CDLL("libcudart.so.12").cudaGraphGetNodes(ctypes.c_void_p(graph.raw_cuda_graph()), None, ctypes.byref(n)) == 0
+    return n.value
+
+
+@pytest.mark.parametrize("variant", VARIANTS)
+def test_entropy_has_launches_of_its_own_only_where_it_has_to(variant):
+    # two chunks of layers: scores, top-k, per chunk (gather,) preparation, attention and merge; the fused form has a plan instead
+    w = _workload(49)
+    path = _path(w, variant)
+    args = _inputs(path, wl.make_queries(w))
+    beside = 2 + (1 + 2 * 3 if variant == "fused" else 1 + 2 * 4)
+    assert _launches(path, args) == beside
+    # a tensor of the entropy step in memory that the last attention call reads or writes: the calls in turn
+    shared = {"ws_attn": path.ws_attn, "out": path.out[-1], "q": args[1][-1], "kq": args[2][-1], "vq": args[3][-1],
+              "sel_idx": path.sel_idx, "ctx_off": path.ctx_off}
+    if variant != "fused":
+        shared["k_ctx"] = path.k_bufs[0]
+    if variant == "full":
+        shared["v_ctx"] = path.v_bufs[0]
+    for name, n_bytes in (("H", 4), ("first_ok", 4), ("ws_entropy", 256)):
+        own = getattr(path, name)
+        for where, memory in shared.items():
+            room = memory.flatten().view(torch.uint8)
+            if room.numel() < max(n_bytes, own.nbytes):
+                continue
+            setattr(path, name, room[:own.nbytes].view(own.dtype))
+            assert _launches(path, args) == beside + 2, (name, where)
+        setattr(path, name, own)
+    assert _launches(path, args) == beside
+
+
+@pytest.mark.parametrize("vocab,own", [(699048, 0), (699056, 2)])          # 16 MB of logits less 64 bytes, and 128 bytes more
+def test_entropy_of_large_logits_comes_after_the_attention(vocab, own):
+    w = _workload(50).scaled(vocab=8)
+    path = _path(w, "full")
+    path.ws_entropy = torch.empty(1 << 20, dtype=torch.uint8, device="cuda")
+    args = list(_inputs(path, wl.make_queries(w)))
+    args[4] = torch.randn(w.batch * len(w.probes), vocab, generator=torch.Generator("cuda").manual_seed(1), device="cuda")
+    assert _launches(path, args) == 11 + own
+    p = torch.softmax(args[4].double(), 1)
+    torch.testing.assert_close(path.H.double(), -(p * p.log()).sum(1), rtol=1e-5, atol=1e-5)
+
+
+@pytest.mark.parametrize("variant,where", [("full", "out"), ("full", "k_ctx"), ("full", "v_ctx"), ("vpool", "out"), ("vpool", "k_ctx"),
+                                           ("fused", "out")])
+def test_logits_that_the_pass_writes_are_read_behind_it(variant, where):
+    # logits in the cache or in the last output: what the pass leaves there, as the calls in turn have it
+    w = _workload(51)
+    path, steps = _path(w, variant), _path(w, variant)
+    args = list(_inputs(path, wl.make_queries(w)))
+
+    def logits_of(p):
+        memory = {"out": p.out[-1], "k_ctx": p.k_bufs and p.k_bufs[0], "v_ctx": p.v_bufs and p.v_bufs[0]}[where]
+        memory.zero_()
+        return memory.flatten()[:w.batch * len(w.probes) * w.vocab].view(-1, w.vocab)
+
+    args[4] = logits_of(steps)
+    steps.select(args[0])
+    if variant == "fused":
+        steps.plan()
+    for i, (lb, le) in enumerate(steps.chunks):
+        if variant == "fused":
+            steps.attend_fused(args[1][i], args[2][i], args[3][i], steps.out[i], lb, le)
+        else:
+            steps.assemble(lb, le, keep_plan=i > 0)
+            steps.attend(args[1][i], args[2][i], args[3][i], steps.out[i], lb, le)
+    steps.entropy(args[4], 6.0)
+    args[4] = logits_of(path)
+    out, H, ok = path.run(*args[:5], 6.0)
+    torch.cuda.synchronize()
+    assert path.status.item() == 0 and steps.status.item() == 0
+    assert torch.equal(H, steps.H) and torch.equal(ok, steps.first_ok) and H.std() > 0
+    assert all(torch.equal(a, b) for a, b in zip(out, steps.out))
 
 
 @pytest.mark.parametrize("variant,tensor", [("vpool", "v"), ("fused", "v"), ("fused", "k")])
