@@ -44,7 +44,10 @@ constexpr int kMaxProbes = 16;
 constexpr int kMaxPairs = 256;       // (probe, query) pairs one call may hold: B * P <= 256
 constexpr int kMaxCtas = 160;        // persistent grid: one CTA per SM, at most this many
 constexpr int kMaxGang = 8;          // CTAs that share one range of K/V tiles
-constexpr int kUnitCost = 4;          // fixed cost of starting a unit, in tiles (measured: about 10 k clocks)
+// Fixed cost of starting a unit, in tiles.  (10 k clocks when every role walked the schedule by itself, 3 k of them the walk that one thread does
+// ahead now.  2 / 3 / 4 / 6, us: one layer of one query, four probes 122.8 / 122.9 / 123.9 / 124.9, two rounds of probes 569 / 567 / 572 / 572, 28 queries
+// of seven short probes 217 / 221 / 226 / 238, seven queries of four, eight layers 682 / 663 / 650 / 680: flat from 2 to 4.)
+constexpr int kUnitCost = 4;
 constexpr int kTileM = 128;          // query rows per M tile (TMEM lanes)
 constexpr int kTileN = 128;          // keys per tile
 constexpr int kAttnThreads = 384;    // warp 0 TMA and items, warp 1 MMA, warp 2 gathers V (V from the pool), softmax of M tile A on
@@ -421,7 +424,7 @@ __global__ void __launch_bounds__(256, 3) attn_prep_kernel(const __grid_constant
 // written by TMA with the 128-byte swizzle; D = 128 needs two of them per tile.
 // The fused variant has a third K stage (one tile landing, one being rotated, one in use) in the place of
 // the read-out staging.
-constexpr int kCachePairs = 12;
+constexpr int kCachePairs = 12;       // (30 of them: no faster, 192 short pairs in one range 2234.5 / 2234.7 us)
 constexpr uint32_t kCacheBytes = 320;
 constexpr uint32_t kBarBytes = 384;                  // barriers, TMEM slot, abort flags
 constexpr int kItems = 4;                            // items published ahead of the roles that work on them

@@ -61,8 +61,11 @@ static inline int ads_set_max_smem(Kernel kernel, int bytes, bool* done) {
 // Programmatic dependent launch: the kernel may be started while the one in front of it in the stream still
 // ends, so that its launch and its set-up cost no gap (a pass of a few short shots, nine kernels: 45.9 -> 28.3 us; two rounds
 // of probes 637 -> 622; a ranking by attention over 2048 shots 912 -> 906).  Every kernel launched this way calls
-// ads_dependency_wait() before it touches global memory (in every block: what completes a kernel is the completion of its
-// blocks, and a block that did not wait would not stand for the kernels before).  ads_dependency_trigger() lets the next
+// ads_dependency_wait(), in every block (what completes a kernel is the completion of its blocks, and a block that did not wait
+// would not stand for the kernels before), and before the wait it writes no memory and relies on none.  Only the two decode
+// kernels read any there, as a guess: past the L1, so that no old line is left in it for the reads behind the wait; clamped or
+// checked so that no address leaves its buffer whatever they find, tiles by L2 prefetches alone; and compared behind the wait with
+// what is read there before a result depends on it.  ads_dependency_trigger() lets the next
 // kernel in earlier, once all blocks have called it; only the decode kernels do: elsewhere the early blocks took room from
 // the kernel they waited for (one layer of one query 132 -> 139 us with triggers in every kernel, the selection's alone
 // account for all of it).

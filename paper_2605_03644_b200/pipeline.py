@@ -41,10 +41,11 @@ def layer_chunks(n_layers: int, lpc: int, ramp: bool = False):
 def v_from_pool_pays(cache_bytes: float, mean_shot_tokens: float) -> bool:
     """The measured choice between a K-only cache, V tiles taken from the pool, and a full cache (`cache_bytes` of
     K and V per call).  Leaving V where it is saves half of the gather and costs the attention 2-3 % (V tiles stitched
-    from runs of pool rows) and one small launch.  One query of one layer: full / K-only 59 / 60 us at 16 shots of 160
-    tokens, 67.6 / 67.5 at 32 (33 MB), 82.7 / 79.3 at 64, 109 / 101 at 128; three layers of 64 K tokens 1712 / 1640.
-    Short shots make many runs per tile: at 24 tokens on average 90 / 95 us (one query, 12 K tokens) and 1395 / 1401
-    (32 queries), at 36 tokens 1042 / 978, at 48 2689 / 2405; at 12 744 / 946."""
+    from runs of pool rows).  One query of one layer: full / K-only 43.1 / 43.1 us at 16 shots of 160 tokens, 49.3 / 47.2
+    at 32 (21 MB), 58.9 / 53.3 at 48 (31 MB), 68.0 / 59.7 at 64, 98.3 / 84.5 at 128; four queries of 8 shots 57.2 / 53.6.
+    The line was drawn when the row map took a launch of its own and stays on its safe side: callers below it find V in
+    the cache.  Short shots make many runs per tile: 512 of 16 tokens on average 61.8 / 67.7 us (one query) and 262 / 321
+    (eight), of 20 69.5 / 72.6 and 320 / 355, of 24 80.3 / 78.1 and 387 / 392, of 32 86.9 / 83.1."""
     return cache_bytes > (32 << 20) and mean_shot_tokens >= 32
 
 
